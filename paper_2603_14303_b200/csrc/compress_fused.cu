@@ -1,43 +1,45 @@
 // Fused bf16 compress kernel (d = 128), sm_100a: Eq. 2 + Algorithm 1 + Eq. 3 in one pass over K, V.
 //
-// Persistent blocks (as many as fit on the GPU at once) draw work tiles from a global ticket
-// counter.  A tile is a run of whole segments of at most SC_TILE_ROWS tokens of one (sequence, KV
-// head) -- K and V both staged in shared memory -- or one longer segment alone (K staged, then V
-// in a second pass over the same buffer).  Per tile:
-//   1. the rows are staged by TMA (cp.async.bulk.tensor, boxes of 32 rows x 64 columns, 128-byte
-//      swizzle so that ldmatrix is conflict free, completion on an mbarrier), issued by the block's
-//      ninth "service" warp;
-//   2. Eq. 2 + Algorithm 1, one warp per segment.  Up to 32 tokens (the usual case) everything
-//      stays in registers: mma.m16n8k16 tiles laid over the segment's own rows give the upper
-//      triangle of its Gram matrix (bf16 products are exact in fp32), the diagonal gives the norms,
-//      Sim > tau is decided as G_ij > tau*|k_i|*|k_j|, each lane ends up with one row's adjacency
-//      word, and the greedy pass costs one shuffle and a few word operations per seed;
-//   3. the rows of segments of more than 32 tokens get their similarities from the tensor core: one thread issues
-//      eight tcgen05.mma (128 x 128 x 128, bf16) on the staged rows -- the 128-byte-swizzled layout the TMA boxes
-//      wrote is the K-major operand layout -- into tensor memory (three such blocks for a tile of 129..256 tokens,
-//      the diagonal ones first: they give the norms); the warps that own such rows read the accumulator one row per
-//      thread and keep, as bits in registers, which EARLIER tokens of its segment each row is similar to.
-//      Algorithm 1 is then settled for all those rows at once, in rounds: a row with an earlier neighbour that is
-//      a seed is a member, a row whose earlier neighbours are all members is a seed (the lowest open row is decided
-//      in every round, so the rounds end; chunks that are unions of cliques take two).  A member joins the earliest
-//      seed among its neighbours, which is what the sequential pass does; the lanes of a warp that name the same
-//      seed are found with match.any and write that word of the seed's member mask.  Warps without such rows do
-//      the short segments meanwhile (segments are claimed from a counter, not dealt by warp number);
-//   4. the tile's cluster count enters a prefix sum over the tiles of its (sequence, head): a
-//      decoupled look-back over per-tile status words (tickets are handed out in order, so every
-//      predecessor is held by a running block and the bounded wait cannot starve), or, in
-//      two-pass mode, a count pass followed by a write pass;
-//   5. Eq. 3, beside the service warp's look-back: every token belongs to exactly one cluster, so a
-//      cluster's mean can overwrite its seed's staged row.  The clusters are dealt to the compute
-//      warps in seed order; a lane owns eight columns of the K or of the V row, sums the member
-//      rows in fp32 in token order, scales by 1/|S| and rounds once to bf16; clusters of one token
-//      are left as they are.  The cores then leave in seed order with 16-byte coalesced stores.
-//      The service warp draws the block's next ticket during step 2.
-// The last block to finish zeroes the status words and counters, so a workspace that was zero
-// before the call is zero again after it.
-// One launch may serve several layers (sc_compress_layers): the tickets then go round the (layer, sequence,
-// head) units, which puts L*B*Hkv tickets between consecutive tiles of a head instead of B*Hkv; with few heads
-// per layer that is what keeps one late tile from holding up every tile of its head that is in flight.
+// Persistent blocks (three per SM) draw work tiles from a global ticket counter.  A tile is a run of whole segments of
+// at most SC_TILE_ROWS tokens of one (layer, sequence, KV head) -- K and V both staged in shared memory -- or one longer
+// segment alone (K staged, then V in its place).  A block has four compute warps and a service warp; they meet
+// through mbarriers only.  The service warp stages a tile as soon as the buffer is free, looks back for the tile's output
+// offset, publishes the tile's prefix and draws the next ticket while the tile is pooled.
+// Compute warps, per tile:
+//   1. similarities (Eq. 2): the Gram matrix of the tile's keys is one 128 x 128 x 128 tcgen05.mma product in tensor
+//      memory (the 128-byte-swizzled layout the TMA boxes wrote is the K-major operand layout; three such products, one
+//      after the other, for a tile of 129..256 tokens).  Thread i owns row i; it reads only the columns its warp's rows
+//      can need and keeps, as bits in registers, which EARLIER tokens of its segment it is similar to (Sim > tau decided as
+//      |k_c| (tau |k_i|) - G < 0: one fma and one funnel shift that collects its sign per pair).
+//   2. Algorithm 1 for all rows at once, in rounds: a row with an earlier neighbour that is a seed is a member, a row
+//      whose earlier neighbours are all members is a seed.  Both facts are final once true, the lowest open row is
+//      decided in every round, so the rounds end and give exactly the sequential pass's partition; chunks that are unions
+//      of cliques take two.  A member joins the earliest seed among its earlier neighbours.  The tile's cluster count is
+//      published at once; every token's cluster number (rank of its seed) goes to shared memory.
+//   3. Eq. 3: the members' sum of a cluster is a row of M V, M the 0/1 matrix clusters x tokens; M's fragments are made
+//      from the cluster numbers, K and V come transposed from their staged rows (ldmatrix.trans), mma.m16n8k16 adds up in
+//      fp32 (products with 1 and 0 are exact).  Sixteen clusters at a time, over the tokens from their first seed to the
+//      end of their last segment only; each warp takes a quarter of the columns.  Sums are scaled by 1/|S|, rounded once
+//      and stored.  Clusters of one token are copied bit for bit; a sum that is not finite (0 * inf would reach other
+//      clusters) sends the sixteen clusters to a loop over their members.
+//
+// What bounds it: the length of a tile's chain of steps with three 64 KB tiles in flight per SM (issue slots a quarter
+// used).  The kernel before this one clustered every segment with one warp's mma.sync tiles and greedy pass and added up
+// member rows on the CUDA cores, nine warps and five block barriers a tile, 13 K warp instructions per 128 tokens; here
+// 7.4 K.  32 layers x 8 heads x 32K tokens in one launch: 1395 -> 1115 us (3.9 -> 4.8 TB/s); 16 sequences x 16K, lognormal
+// chunks, 8 heads, per layer: 500 -> 310 us.  Measured on the way: sums over member rows in cluster order instead of
+// the product, 1245 us / 475 us (single-token chains of shared loads are longer than the products); keys and values
+// released and pooled separately so that the next keys load earlier, +13 %; L2 prefetch of the next tile, +5 %; only
+// clusters of more than one token in the product, +5 %; a second service warp (96 registers a thread), worse throughout.
+// Long tiles by mma.sync blocks instead of tcgen05: 16 x 16K +8 %.
+//
+// Offsets: a prefix sum over the tiles of each head by decoupled look-back over per-tile status words; tickets are handed
+// out in order, so every predecessor is held by a running block and the bounded wait cannot starve.  A block draws its
+// next ticket only when its tile's count is out and its offset known: drawn with the staging, one tile earlier, a tile
+// waited unstarted in a block that itself waited, and held up its successors (16 x 16K: 711 -> 666 us for two layers; chunks of
+// 128 tokens: 884 -> 781).  Tickets go round the (layer, sequence, head) units.  The last block to finish zeroes the
+// status words and counters, so a workspace that was zero before the call is zero again after it.  One launch may
+// serve several layers (sc_compress_layers).
 #include <cuda.h>
 
 #include <mutex>
@@ -49,95 +51,52 @@ namespace sc {
 
 namespace cf {
 
-constexpr int kWarps = 8;                         // compute warps
-constexpr int kThreads = (kWarps + 1) * 32;       // plus one service warp: next ticket, look-back
+constexpr int kWarps = 4;                         // compute warps
+constexpr int kThreads = (kWarps + 1) * 32;       // plus one service warp
+constexpr int kTeam = kWarps * 32;
 constexpr int kD = 128;
-constexpr int kRowBytes = 256;                    // one K or V row in global memory
 constexpr int kHalfRow = 128;                     // a staged row is two 128-byte halves (64 columns each), see tile_addr
 constexpr int kBoxRows = 32;                      // rows per TMA box
 constexpr int kBoxBytes = kBoxRows * kHalfRow;    // 4096
 constexpr int kMaxRows = SC_MAX_CHUNK_LEN;        // 256: a long tile
 constexpr int kShortRows = SC_TILE_ROWS;          // 128
-// Longest segment one warp clusters on its own, in registers; the bit rows of longer ones come from the tile's Gram
-// matrix on the tensor core.  (A warp-private mma.sync path for 33..48 tokens was 16 % slower on lognormal chunks.)
-constexpr int kWarpSegMax = 32;
-constexpr int kNW = 8;                            // 32-bit words per (full) adjacency row
-constexpr int kKvBytes = kMaxRows * kRowBytes;    // 65536: short = K | V, long = one tensor
-constexpr int kVOff = kShortRows * kRowBytes;     // 32768
 constexpr int kHalfShort = kShortRows * kHalfRow; // 16384: distance between the column halves of a short tile
 constexpr int kHalfLong = kMaxRows * kHalfRow;    // 32768: ... of a long one
-constexpr int kCntOff = kKvBytes;                 // uint32[256] per seed row: what pool_clusters needs, then the member count
-constexpr int kAdjOff = kCntOff + kMaxRows * 4;
-constexpr int kAdjWords = 32 * (8 + 7 + 6 + 5 + 4 + 3 + 2 + 1);   // rows of block k keep words k..7
-constexpr int kNormOff = kAdjOff + kAdjWords * 4; // float[512]: norms (64 per warp, or one per row); later uint16 seed row per cluster
-constexpr int kRowNormOff = kNormOff + kWarps * 64 * 4; // float[256]: norms of the rows of long segments (from the tensor core's Gram diagonal)
-constexpr int kSegsOff = kRowNormOff + kMaxRows * 4; // 2 x int16[132]: segment starts (this tile, next tile)
-constexpr int kSegsStride = 132;
-constexpr int kMiscOff = kSegsOff + 2 * kSegsStride * 2;   // uint32 seedmask[8]; int geo[2][8]; int misc[4]
-constexpr int kBarOff = kMiscOff + 32 + 64 + 16 + 32 + 128 + 16 + 32;   // ... 8 spare words; uint8 multi[128]; tensor-memory slot, flag; uint32 membits[8]; three mbarriers
-constexpr int kSmemBytes = kBarOff + 24;
+constexpr int kVOff = 2 * kHalfShort;             // short: K | V, long = one tensor
+constexpr int kBitOff = 2 * kHalfLong;            // uint32[256][8]: earlier-neighbour bits of a long tile's rows
+constexpr int kNormOff = kBitOff;                 // float[128]: norms of a short tile's rows (no bits are stored for it)
+constexpr int kLongNormOff = kBitOff + kMaxRows * 32;        // float[256]
+// behind the norms, once the bits are in registers:
+constexpr int kRankOff = kBitOff + 1024;                     // uint8[256]: cluster of each token, see rank_slot
+constexpr int kCntOff = kRankOff + kMaxRows;                 // int32[256]: tokens of each cluster
+constexpr int kSeedOff = kCntOff + kMaxRows * 4;             // uint8[256]: the cluster's seed
+constexpr int kEndOff = kSeedOff + kMaxRows;                 // uint16[256]: end of the seed's segment
+constexpr int kMiscOff = kLongNormOff + kMaxRows * 4;        // seeds[8], members[8]; starts[2][4]; geo[2][8]; base, P, tmem slot, flags
+constexpr int kBarOff = kMiscOff + 64 + 32 + 64 + 32;
+constexpr int kSmemBytes = kBarOff + 64;
 constexpr int kTmemCols = 128;                    // one 128 x 128 fp32 accumulator per block (three blocks per SM: 384 of 512 columns)
 constexpr int kBlocksPerSm = 3;
-static_assert(kBarOff % 8 == 0, "mbarrier alignment");
+static_assert(kEndOff + kMaxRows * 2 <= kLongNormOff && kRankOff % 16 == 0 && kMiscOff % 16 == 0 && kBarOff % 8 == 0, "alignment");
 static_assert(kSmemBytes <= 76800, "three blocks per SM need <= 75 KB each");
 
-enum Mode { kCountOnly = 0, kWriteWithCounts = 1, kLookBack = 2 };
-enum Geo { gB = 0, gH = 1, gT = 2, gNseg = 3, gRow0 = 4, gR = 5, gLast = 6, gLayer = 7 };
+enum Mode { kCountOnly = 0, kLookBack = 1 };
+enum Geo { gB = 0, gH = 1, gT = 2, gNseg = 3, gRow0 = 4, gR = 5, gLast = 6, gLayer = 7 };   // gT = -1: no work left
 
-// cnts[seed row] while the cluster waits to be pooled: kPending | first row of its segment | (one past its last
-// row) << 9, the latter 0 for a segment of up to 32 tokens, whose member mask is one segment-relative word
-constexpr uint32_t kPending = 1u << 31;
 constexpr uint32_t kFlagAggregate = 1u << 30, kFlagPrefix = 2u << 30, kValueMask = (1u << 30) - 1;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // every wait gives up after 2 s
 constexpr int kPollGroups = 2;                               // the look-back reads 64 predecessors per poll (4 and 8 measured slower, 1 slower on short chunks)
 constexpr int kCtlWords = 64;                                // ticket, done counter, padding
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ unsigned long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t));
-    return t;
-}
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0u;
-}
-// Bounded wait for a phase of an mbarrier; false if it gave up.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
-    const unsigned long long t0 = global_ns();
-    for (;;) {
-#pragma unroll 1
-        for (int i = 0; i < 256; ++i)
-            if (mbar_try_wait(bar, parity)) return true;
-        if (global_ns() - t0 > kWaitLimitNs) return false;
-    }
-}
 // One TMA box: 32 rows x 64 columns of a [B, Hkv, n, 128] tensor, 128-byte swizzled, no multicast.
 __device__ __forceinline__ void tma_box(uint32_t dst, const CUtensorMap* map, int col, int row, int h, int b, uint32_t bar) {
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];\n"
                  ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(col), "r"(row), "r"(h), "r"(b), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void fence_async_proxy() { asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory"); }
-// Byte offset, inside one column half of a staged tensor, of 16-byte chunk `chunk` (0..7) of row
+// Byte offset, inside one column half of the staged keys, of 16-byte chunk `chunk` (0..7) of row
 // `row`: rows are 128 bytes apart and the chunk index is XORed with the row's low three bits (the
 // TMA 128-byte swizzle), which makes ldmatrix over eight consecutive rows conflict free.
 __device__ __forceinline__ uint32_t tile_addr(int row, int chunk) { return row * kHalfRow + ((chunk ^ (row & 7)) << 4); }
-__device__ __forceinline__ void compute_warps_sync() {   // the eight compute warps, not the service warp
-    asm volatile("bar.sync 1, 256;\n" ::: "memory");
-}
-__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
-}
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                  : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
@@ -158,25 +117,24 @@ __device__ __forceinline__ uint32_t ld_volatile(const uint32_t* p) {
     asm volatile("ld.volatile.global.u32 %0, [%1];\n" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
-// Word offset of adjacency word (row i, word i>>5) in the triangular store; word w >= i>>5 of the
-// same row follows at + (w - (i>>5)).
-__device__ __forceinline__ int adj_row(int i) {
-    const int k = i >> 5;
-    return 256 * k - 16 * k * (k - 1) + (i & 31) * (kNW - k);
-}
-
-// 16 consecutive fp32 columns of this thread's tensor-memory lane.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+// The four compute warps meet ...
+__device__ __forceinline__ void team_sync() { asm volatile("barrier.cta.sync 1, 128;\n" ::: "memory"); }
+// ... and learn whether any of them says so.
+__device__ __forceinline__ bool team_any(bool mine) {
+    uint32_t out;
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
+        "{\n"
+        ".reg .pred p, r;\n"
+        "setp.ne.u32 p, %1, 0;\n"
+        "barrier.cta.red.or.pred r, 1, 128, p;\n"
+        "selp.u32 %0, 1, 0, r;\n"
+        "}\n"
+        : "=r"(out) : "r"(mine ? 1u : 0u) : "memory");
+    return out != 0u;
 }
 
-// One 128 x 128 block of K.K^T of the staged keys: rows of 128-row block mb against rows of block nb (column
-// halves `hs` bytes apart, 128-byte-swizzled rows: what the TMA boxes wrote is the K-major layout tcgen05.mma
-// reads).  One thread issues the eight instructions; the mbarrier gets one arrival when they are complete.
+// One 128 x 128 block of K.K^T of the staged keys: rows of 128-row block mb against rows of block nb (column halves `hs` bytes
+// apart).  One thread issues the eight instructions; the mbarrier gets one arrival when they are complete.
 __device__ __forceinline__ void umma_gram_block(uint32_t kbase, int hs, int mb, int nb, uint32_t tmem, uint32_t bar) {
     constexpr uint32_t idesc = umma::instr_desc_bf16(128, 128, false, false);
 #pragma unroll
@@ -188,408 +146,343 @@ __device__ __forceinline__ void umma_gram_block(uint32_t kbase, int hs, int mb, 
     umma::mma_commit(bar);
 }
 
-// The diagonal of a diagonal block = squared norms: thread (quarter q, lane) of the four reading warps owns tile
-// row mb*128 + 32q + lane and finds its element in the 32 columns its warp's rows share.
-__device__ __forceinline__ void umma_norms(uint32_t tmem, int mb, int q, int lane, float* norm) {
+// Bits over 32 columns: bit c = (thr_c - G_c < 0), thr_c = norm_c * tni.  The sign of each difference is shifted in
+// behind the others, from the last column to the first; a difference of zero (Sim == tau) and one that is not a
+// number give no bit.
+__device__ __forceinline__ uint32_t sim_word(const uint32_t (&g)[32], const float* norm_c, float tni) {
+    uint32_t w = 0u;
+    const float4* nc = reinterpret_cast<const float4*>(norm_c);
+#pragma unroll
+    for (int k4 = 7; k4 >= 0; --k4) {
+        const float4 nv = nc[k4];
+        const float n4[4] = {nv.x, nv.y, nv.z, nv.w};
+#pragma unroll
+        for (int k = 3; k >= 0; --k)
+            w = __funnelshift_l(__float_as_uint(fmaf(n4[k], tni, -__uint_as_float(g[k4 * 4 + k]))), w, 1);
+    }
+    return w;
+}
+// A negative threshold: a zero-norm key has Sim = 0 > tau.
+__device__ __forceinline__ uint32_t sim_word_neg(const uint32_t (&g)[32], const float* norm_c, float tni) {
+    uint32_t w = 0u;
+#pragma unroll
+    for (int k = 0; k < 32; ++k) {
+        const float thr = norm_c[k] * tni;
+        w |= (__uint_as_float(g[k]) > thr || thr == 0.f ? 1u : 0u) << k;
+    }
+    return w;
+}
+
+// Algorithm 1 for the tile, given each row's earlier-neighbour words (rows tid + 128 r, r < NR, tile word warp + 4 r), and what
+// the pooling needs: every token's cluster, and every cluster's size, seed and end of segment.  `end`: end of the rows'
+// segments.  Returns the number of clusters.  All compute threads call it.
+__device__ __forceinline__ int rank_slot(int i) {   // where a token's cluster number is kept: the four a lane needs for one mma
+    return (i & ~15) | ((i & 6) << 1) | ((i & 8) >> 2) | (i & 1);   // fragment (2t, 2t+1, 2t+8, 2t+9 of sixteen) form one word
+}
+template <int NR>
+__device__ __forceinline__ int settle_rows(const uint32_t (&e)[NR][4 * NR], const bool (&act)[NR], const int (&end)[NR], unsigned char* smem,
+                                           int warp, int lane, int32_t* as, int row0, uint32_t* publish, int* sh_p) {
+    constexpr int NW = 4 * NR;
+    uint32_t* seeds = reinterpret_cast<uint32_t*>(smem + kMiscOff);
+    uint32_t* members = seeds + 8;
+    int* cnt = reinterpret_cast<int*>(smem + kCntOff);
+    bool open[NR], is_seed[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) { open[r] = act[r]; is_seed[r] = false; cnt[(warp + 4 * r) * 32 + lane] = 0; }
+    uint32_t sd[NW], mb[NW];   // all lanes hold the same words
+    bool more;
+    // round 0 needs no words: a row without earlier neighbours is a seed
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        uint32_t any = 0u;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) any |= e[r][w];
+        if (act[r] && any == 0u) { is_seed[r] = true; open[r] = false; }
+        const uint32_t ns = __ballot_sync(kFull, is_seed[r]);
+        if (lane == 0) { seeds[warp + 4 * r] = ns; members[warp + 4 * r] = 0u; }
+    }
+    team_sync();
+    for (;;) {   // the lowest open row is decided every round
+#pragma unroll
+        for (int w = 0; w < NW; w += 4) {
+            const uint4 a = *reinterpret_cast<const uint4*>(seeds + w), b = *reinterpret_cast<const uint4*>(members + w);
+            sd[w] = a.x; sd[w + 1] = a.y; sd[w + 2] = a.z; sd[w + 3] = a.w;
+            mb[w] = b.x; mb[w + 1] = b.y; mb[w + 2] = b.z; mb[w + 3] = b.w;
+        }
+        more = false;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            uint32_t near_seed = 0u, not_member = 0u;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) { near_seed |= e[r][w] & sd[w]; not_member |= e[r][w] & ~mb[w]; }
+            const bool to_member = open[r] && near_seed != 0u;
+            const bool to_seed = open[r] && near_seed == 0u && not_member == 0u;
+            if (to_member || to_seed) open[r] = false;
+            if (to_seed) is_seed[r] = true;
+            const uint32_t nm = __ballot_sync(kFull, to_member), ns = __ballot_sync(kFull, to_seed);
+            if (lane == 0) {   // only this warp writes its words
+                if (nm) members[warp + 4 * r] |= nm;
+                if (ns) seeds[warp + 4 * r] |= ns;
+            }
+            more |= open[r];
+        }
+        if (!team_any(more)) break;
+    }
+#pragma unroll
+    for (int w = 0; w < NW; w += 4) {
+        const uint4 a = *reinterpret_cast<const uint4*>(seeds + w);
+        sd[w] = a.x; sd[w + 1] = a.y; sd[w + 2] = a.z; sd[w + 3] = a.w;
+    }
+    int P = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) P += __popc(sd[w]);
+    if (threadIdx.x == 0) {
+        *sh_p = P;
+        if (publish) atomicExch(publish, kFlagAggregate | (uint32_t)P);
+    }
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+        // a member joins the earliest seed among its earlier neighbours; a cluster's number is the rank of its seed
+        const int i = (warp + 4 * r) * 32 + lane;
+        int s = i, before = 0, rank = 0;
+        bool found = false;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const uint32_t own = is_seed[r] && w == warp + 4 * r ? 1u << lane : 0u;
+            const uint32_t m = is_seed[r] ? own : e[r][w] & sd[w];
+            if (!found && m != 0u) {
+                const int bit = __ffs(m) - 1;
+                s = w * 32 + bit;
+                rank = before + __popc(sd[w] & ((1u << bit) - 1u));
+                found = true;
+            }
+            before += __popc(sd[w]);
+        }
+        (smem + kRankOff)[rank_slot(i)] = act[r] ? (uint8_t)rank : (uint8_t)255;   // past the tile's end: no cluster
+        if (act[r]) {
+            atomicAdd(&cnt[rank], 1);
+            if (is_seed[r]) {
+                (smem + kSeedOff)[rank] = (uint8_t)i;
+                reinterpret_cast<uint16_t*>(smem + kEndOff)[rank] = (uint16_t)end[r];
+            }
+            if (as) as[i] = row0 + s;
+        }
+    }
+    team_sync();
+    return P;
+}
+
+// The diagonal of a diagonal block = squared norms: thread (warp q, lane) owns row 32 q + lane of the block.  `g` holds the
+// 32 columns of the warp's own rows; this lane's element is picked by the bits of the lane number.
+__device__ __forceinline__ float diagonal(const uint32_t (&g)[32], int lane) {
+    uint32_t t[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) t[k] = (lane & 16) ? g[k + 16] : g[k];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t[k] = (lane & 8) ? t[k + 8] : t[k];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) t[k] = (lane & 4) ? t[k + 4] : t[k];
+    t[0] = (lane & 2) ? t[2] : t[0]; t[1] = (lane & 2) ? t[3] : t[1];
+    return __uint_as_float((lane & 1) ? t[1] : t[0]);
+}
+
+// Steps 1 and 2 for a tile of up to 128 rows, thread i = row i (the product of its keys is complete).  `starts`: bit words of the
+// rows that start a segment.
+__device__ __forceinline__ int settle_short_tile(unsigned char* smem, const uint32_t* starts, int R, uint32_t tmem, uint32_t phase_u, float tau,
+                                                 bool wait_failed, bool& failed, int32_t* as, int row0, uint32_t* publish, int* sh_p) {
+    float* norm = reinterpret_cast<float*>(smem + kNormOff);
+    const int i = threadIdx.x, lane = i & 31, q = i >> 5;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    float v = 0.f;
-#pragma unroll
-    for (int c = 0; c < 2; ++c) {
-        uint32_t g[16];
-        tmem_ld16(lane_addr + q * 32 + c * 16, g);
-        umma::tmem_ld_wait();
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-            if (lane == c * 16 + k) v = __uint_as_float(g[k]);
-    }
-    norm[mb * 128 + q * 32 + lane] = sqrtf(v);
-}
-
-// Reads this thread's row i = 128 mb + 32 q + lane of the block in tensor memory and returns, as four words over
-// the block's columns 128 nb .. 128 nb + 127, which EARLIER tokens of i's own segment [a_i, ...) are similar to it:
-// bit c of the result = Sim(c, i) > tau for a_i <= c < i, decided as G > |k_c| (tau |k_i|) -- the earlier token's
-// norm first, the product the short-segment path forms for the same pair.  Only the chunks of sixteen columns
-// that can hold a column below the warp's rows are read (`chunks`), and no word before the first (`w_lo`) that
-// holds a token of a segment one of the warp's rows is in (both uniform over the warp).
-template <bool kNegTau>
-__device__ __forceinline__ void umma_earlier(uint32_t tmem, int nb, int q, int i, int a_i, float tau, const float* norm,
-                                             int w_lo, int chunks, uint32_t (&words)[4]) {
-    const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    const float tni = tau * norm[i];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {   // 32 columns = one word at a time
-        uint32_t w = 0u;
-        if (c >= w_lo && 2 * c < chunks) {   // a word that holds an earlier token of some row's segment
-            uint32_t g[32];
-            umma::tmem_ld32(lane_addr + c * 32, g);
-            umma::tmem_ld_wait();
-            const float4* nc = reinterpret_cast<const float4*>(norm + nb * 128 + c * 32);
-#pragma unroll
-            for (int k4 = 0; k4 < 8; ++k4) {
-                const float4 nv = nc[k4];
-                const float thr[4] = {nv.x * tni, nv.y * tni, nv.z * tni, nv.w * tni};
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    bool hit = __uint_as_float(g[k4 * 4 + k]) > thr[k];
-                    if (kNegTau) hit = hit || (thr[k] == 0.f);   // a zero-norm key has Sim = 0 > tau
-                    w |= (hit ? 1u : 0u) << (k4 * 4 + k);
-                }
-            }
-        }
-        words[c] = w & bits_between(a_i, i, nb * 4 + c);
-    }
-}
-
-// One round of Algorithm 1's decisions for the 32 tokens a warp owns (tile word `word`, token 32 word + lane),
-// on each token's earlier-neighbour words `e`: a token with an earlier neighbour that is a seed is a member; a
-// token whose earlier neighbours are all members is a seed.  Both facts are final once true, so reading words
-// that other warps are updating is harmless.  `open` = not yet decided (false for tokens outside long segments);
-// the warp's new seeds and members go to the shared words with one atomic each.
-__device__ __forceinline__ void decide_round(const uint32_t (&e)[8], int word, int lane, bool& open, bool& is_seed,
-                                             volatile uint32_t* seeds, volatile uint32_t* members) {
-    // all lanes read the same sixteen words (broadcast), no branch per word
-    uint32_t sd[8], mb[8];
-#pragma unroll
-    for (int w = 0; w < 8; ++w) { sd[w] = seeds[w]; mb[w] = members[w]; }
-    uint32_t near_seed = 0u, not_member = 0u;
-#pragma unroll
-    for (int w = 0; w < 8; ++w) { near_seed |= e[w] & sd[w]; not_member |= e[w] & ~mb[w]; }
-    const bool to_member = open && near_seed != 0u;
-    const bool to_seed = open && near_seed == 0u && not_member == 0u;
-    if (to_member || to_seed) open = false;
-    if (to_seed) is_seed = true;
-    const uint32_t nm = __ballot_sync(kFull, to_member), ns = __ballot_sync(kFull, to_seed);
-    if (lane == 0) {
-        if (nm) atomicOr(const_cast<uint32_t*>(members) + word, nm);
-        if (ns) atomicOr(const_cast<uint32_t*>(seeds) + word, ns);
-    }
-}
-
-// After the rounds: a member joins the earliest seed among its earlier neighbours, as Algorithm 1 would have it.
-// The lanes of a warp that name the same seed are that cluster's members in the warp's word: one of them writes
-// the word into the seed's row of the triangular store (the seed's member mask, tile positions; the seed itself
-// is in it).  Words of the row that get no member were cleared beforehand.
-__device__ __forceinline__ void settle_round(const uint32_t (&e)[8], int word, int lane, bool active, bool is_seed,
-                                             int a_i, int e_i, const volatile uint32_t* seeds, uint32_t* adj,
-                                             uint32_t* cnts, int32_t* as, int row0) {
-    const int i = word * 32 + lane;
-    int s = active ? i : -1 - lane;   // inactive lanes: keys of their own
-    if (active && !is_seed) {
-#pragma unroll
-        for (int w = 7; w >= 0; --w) {
-            const uint32_t m = e[w] & seeds[w];
-            if (m) s = w * 32 + __ffs(m) - 1;
-        }
-    }
-    const uint32_t group = __match_any_sync(kFull, s);
-    if (!active) return;
-    if (is_seed) cnts[i] = kPending | (uint32_t)a_i | ((uint32_t)e_i << 9);
-    if ((int)(__ffs(group) - 1) == lane) adj[adj_row(s) + word - (s >> 5)] = group;
-    if (as) as[i] = row0 + s;
-}
-
-// `threads` threads of the block (whole warps) meet at barrier 2 ...
-__device__ __forceinline__ void warps_sync(int threads) { asm volatile("barrier.cta.sync 2, %0;\n" ::"r"(threads) : "memory"); }
-// ... and learn whether any of them still has work.
-__device__ __forceinline__ bool warps_any(bool mine, int threads) {
-    uint32_t out;
-    asm volatile(
-        "{\n"
-        ".reg .pred p, r;\n"
-        "setp.ne.u32 p, %1, 0;\n"
-        "barrier.cta.red.or.pred r, 2, %2, p;\n"
-        "selp.u32 %0, 1, 0, r;\n"
-        "}\n"
-        : "=r"(out) : "r"(mine ? 1u : 0u), "r"(threads) : "memory");
-    return out != 0u;
-}
-
-// Step 2 for one tile: Algorithm 1 for the rows of segments of more than kWarpSegMax tokens (all threads of the
-// block call it; a wait for the tensor core that gave up is left in the tile's failure flag).  The Gram matrix comes
-// from the tensor core, 128 x 128 at a time into tensor memory: one block for a tile of up to 128 tokens, else the
-// two diagonal blocks -- they give the norms -- and the lower one.  Compute thread tid settles tile row tid: warps
-// 0..3 read the accumulator rows of block 0, warps 4..7 those of block 1 (a warp reaches the tensor-memory lanes of
-// its quarter, warp % 4), and keep which earlier tokens of its segment each row is similar to; Algorithm 1 is then
-// settled for all those rows at once in decision rounds.  `words` has a bit for every 32-row word of the tile that
-// a long segment touches: in a tile of up to 128 rows only those warps stay, the others (and the service warp, once
-// it has issued the product) leave at once for the short segments and the next ticket.  Kept out of line: its
-// registers are not the main loop's.
-__device__ __noinline__ void settle_long_segments(unsigned char* smem, int hs, const int16_t* segs, int nseg, int R,
-                                                  uint32_t words, uint32_t tmem, uint32_t phase_u, float tau,
-                                                  int32_t* as, int row0) {
-    uint32_t* cnts = reinterpret_cast<uint32_t*>(smem + kCntOff);
-    uint32_t* adj = reinterpret_cast<uint32_t*>(smem + kAdjOff);
-    float* norm = reinterpret_cast<float*>(smem + kRowNormOff);
-    uint32_t* seedmask = reinterpret_cast<uint32_t*>(smem + kMiscOff);
-    volatile int* umma_failed = reinterpret_cast<volatile int*>(smem + kMiscOff + 276);
-    uint32_t* membits = reinterpret_cast<uint32_t*>(smem + kMiscOff + 288);
-    const uint32_t sbase = smem_u32(smem), bar_u = sbase + kBarOff + 16;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, q = warp & 3;
-    const bool service = warp == kWarps;
-    const bool long_tile = R > kShortRows;
-    if (!long_tile) {
-        if (service) {
-            if (lane == 0) {
-                umma::fence_after_sync();
-                umma_gram_block(sbase, hs, 0, 0, tmem, bar_u);
-            }
-            return;
-        }
-        if (!((words >> warp) & 1u)) return;
-    }
-    const int team = long_tile ? kWarps * 32 : 32 * __popc(words & 0xffu);   // threads that meet at barrier 2
-    // the segment [beg, end) this thread's row is in: the last start that is not beyond the row
-    int beg = tid, end = tid;
-    if (tid < R) {
-        int lo = 0, hi = nseg;   // segs[lo] <= tid < segs[hi]
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if ((int)segs[mid] <= tid) lo = mid; else hi = mid;
-        }
-        beg = segs[lo]; end = segs[hi];
-    }
-    const bool act = end - beg > kWarpSegMax;   // rows of shorter segments take no part
-    uint32_t ern[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};   // earlier neighbours of the row, tile words
-    if (!long_tile) {
-        if (!mbar_wait(bar_u, phase_u)) *umma_failed = 1;   // carry on (the barriers below must be met); the tile is dropped later
-        umma::fence_after_sync();
-        umma_norms(tmem, 0, q, lane, norm);
-        warps_sync(team);   // the norms of every row of a long segment are in place
-        uint32_t w4[4];
-        const int w_lo = __reduce_min_sync(kFull, act ? beg >> 5 : kNW);   // first word any of the warp's rows needs
-        if (tau < 0.f) umma_earlier<true>(tmem, 0, q, tid, beg, tau, norm, w_lo, 2 * q + 2, w4);
-        else umma_earlier<false>(tmem, 0, q, tid, beg, tau, norm, w_lo, 2 * q + 2, w4);
-        ern[0] = w4[0]; ern[1] = w4[1]; ern[2] = w4[2]; ern[3] = w4[3];
-        umma::fence_before_sync();
-    } else {
-        for (int ps = 0; ps < 3; ++ps) {   // (0,0); (1,1), (1,0)
-            const int mb = ps == 0 ? 0 : 1, nb = ps == 1 ? 1 : 0;
-            const bool reader = !service && (warp >> 2) == mb;
-            if (service && lane == 0) {
-                umma::fence_after_sync();
-                umma_gram_block(sbase, hs, mb, nb, tmem, bar_u);
-            }
-            if (reader) {
-                if (!mbar_wait(bar_u, phase_u)) *umma_failed = 1;
-                umma::fence_after_sync();
-                if (mb == nb) umma_norms(tmem, mb, q, lane, norm);
-            }
-            phase_u ^= 1u;
-            __syncthreads();   // the norms are in place
-            if (reader) {
-                const int chunks = mb == nb ? 2 * q + 2 : 8;   // a diagonal block: columns below the warp's rows
-                uint32_t w4[4];
-                if (tau < 0.f) umma_earlier<true>(tmem, nb, q, tid, beg, tau, norm, 0, chunks, w4);
-                else umma_earlier<false>(tmem, nb, q, tid, beg, tau, norm, 0, chunks, w4);
-                if (nb == 0) { ern[0] = w4[0]; ern[1] = w4[1]; ern[2] = w4[2]; ern[3] = w4[3]; }
-                else { ern[4] = w4[0]; ern[5] = w4[1]; ern[6] = w4[2]; ern[7] = w4[3]; }
-                umma::fence_before_sync();
-            }
-            if (ps < 2) __syncthreads();   // the accumulator may be overwritten
-        }
-        if (service) return;
-    }
-    // the row's place in the triangular store will hold the member mask if the row is a seed
-    if (act) for (int ww = warp; ww <= (end - 1) >> 5; ++ww) adj[adj_row(tid) + ww - warp] = 0u;
-    bool open = act, is_seed = false;
-    do {
-        decide_round(ern, warp, lane, open, is_seed, seedmask, membits);
-    } while (warps_any(open, team));   // the lowest open token is decided every round
-    settle_round(ern, warp, lane, act, is_seed, beg, end, seedmask, adj, cnts, as, row0);
-}
-
-// Eq. 3 building blocks.  A lane owns eight consecutive columns (one 16-byte chunk) of the K row
-// (lanes 0-15) or of the V row (lanes 16-31); `lane_base` is its tensor and column half, c7 its
-// chunk inside the half.  Sums are fp32, in token order.
-// s0 += low bf16 of v, s1 += high bf16 of v: the mixed-precision add takes the bf16 operand as it is (exact
-// widening, one fp32 rounding of the sum -- what unpacking by hand and adding gives, in half the instructions).
-__device__ __forceinline__ void add_pair(uint32_t v, float& s0, float& s1) {
-    asm("{\n.reg .b16 lo, hi;\nmov.b32 {lo, hi}, %2;\nadd.rn.f32.bf16 %0, lo, %0;\nadd.rn.f32.bf16 %1, hi, %1;\n}\n"
-        : "+f"(s0), "+f"(s1) : "r"(v));
-}
-__device__ __forceinline__ void add_chunk(const uint4& v, float (&s)[8]) {
-    add_pair(v.x, s[0], s[1]);
-    add_pair(v.y, s[2], s[3]);
-    add_pair(v.z, s[4], s[5]);
-    add_pair(v.w, s[6], s[7]);
-}
-// Adds the rows first + j for every set bit j of mem, in order; two loads are kept in flight (the
-// filler of an odd count is a row of zeros, which leaves the sums as they are).
-__device__ __forceinline__ void rows_add(const unsigned char* lane_base, int first, uint32_t mem, int c7, float (&s)[8]) {
-    while (mem) {
-        const int j0 = __ffs(mem) - 1;
-        mem &= mem - 1;
-        const uint4 v0 = *reinterpret_cast<const uint4*>(lane_base + tile_addr(first + j0, c7));
-        uint4 v1 = make_uint4(0u, 0u, 0u, 0u);
-        if (mem) {
-            const int j1 = __ffs(mem) - 1;
-            mem &= mem - 1;
-            v1 = *reinterpret_cast<const uint4*>(lane_base + tile_addr(first + j1, c7));
-        }
-        add_chunk(v0, s);
-        add_chunk(v1, s);
-    }
-}
-__device__ __forceinline__ void row_put_mean(unsigned char* lane_base, int row, int c7, const float (&s)[8], float inv) {
-    __nv_bfloat162 a = __floats2bfloat162_rn(s[0] * inv, s[1] * inv), b = __floats2bfloat162_rn(s[2] * inv, s[3] * inv);
-    __nv_bfloat162 c = __floats2bfloat162_rn(s[4] * inv, s[5] * inv), d = __floats2bfloat162_rn(s[6] * inv, s[7] * inv);
-    uint4 v;
-    v.x = *reinterpret_cast<uint32_t*>(&a); v.y = *reinterpret_cast<uint32_t*>(&b);
-    v.z = *reinterpret_cast<uint32_t*>(&c); v.w = *reinterpret_cast<uint32_t*>(&d);
-    *reinterpret_cast<uint4*>(lane_base + tile_addr(row, c7)) = v;
-}
-
-// Eq. 2 + Algorithm 1 for one segment of 2..32 tokens, by one warp, in registers.
-// Rows [a, a + l) of the staged keys.  The upper triangle of the segment's own Gram matrix comes
-// from mma tiles laid over the segment's rows (16-row tiles down, 8-column tiles across, only
-// those that reach above the diagonal); lane 4g + t ends up owning row g + 8t with its adjacency
-// bits (later tokens only) in one word, and the greedy pass is a handful of word operations and
-// one shuffle per seed.  Results: seed bits into the tile's seedmask; for pool_clusters each seed's
-// member mask (bit j = token a + j) in the first word of its adjacency row and a note in cnts;
-// optionally the seed of every token.
-template <bool kNegTau>
-__device__ __forceinline__ void gsc_short_segment(uint32_t kbase, int hs, int a, int l, float tau, float* nrm /*[32], this warp's*/,
-                                                  uint32_t* seedmask, uint32_t* adj, uint32_t* cnts, int32_t* as, int row0,
-                                                  int lane) {
-    const int g = lane >> 2, tig = lane & 3;
-    const int nnt = (l + 7) >> 3;          // 8-column tiles that hold tokens: 1..4
-    const bool two_mt = l > 16;
-    float acc[2][4][4];
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) acc[mt][nt][0] = acc[mt][nt][1] = acc[mt][nt][2] = acc[mt][nt][3] = 0.f;
+    // the segment [beg, end) of the row: the nearest start at or before it, and the next one
+    int beg = 0, end = R;
     {
-        const int j = lane >> 3, r8 = lane & 7;
-        const uint32_t a_base = kbase + tile_addr(a + r8 + ((j & 1) << 3), j >> 1);
-        const uint32_t b_base = kbase + tile_addr(a + r8 + ((j >> 1) << 3), j & 1);
-#pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {
-            uint32_t a0[4], a1[4], b0[4], b1[4];
-            const uint32_t a_addr = (a_base ^ ((ks & 3) << 5)) + (ks >> 2) * hs;
-            const uint32_t b_addr = (b_base ^ ((ks & 3) << 5)) + (ks >> 2) * hs;
-            ldmatrix_x4(a_addr, a0[0], a0[1], a0[2], a0[3]);
-            ldmatrix_x4(b_addr, b0[0], b0[1], b0[2], b0[3]);
-            mma_bf16(acc[0][0], a0[0], a0[1], a0[2], a0[3], b0[0], b0[1]);
-            if (nnt > 1) mma_bf16(acc[0][1], a0[0], a0[1], a0[2], a0[3], b0[2], b0[3]);
-            if (two_mt) {
-                ldmatrix_x4(a_addr + 16 * kHalfRow, a1[0], a1[1], a1[2], a1[3]);
-                ldmatrix_x4(b_addr + 16 * kHalfRow, b1[0], b1[1], b1[2], b1[3]);
-                mma_bf16(acc[0][2], a0[0], a0[1], a0[2], a0[3], b1[0], b1[1]);
-                mma_bf16(acc[1][2], a1[0], a1[1], a1[2], a1[3], b1[0], b1[1]);
-                if (nnt > 3) {
-                    mma_bf16(acc[0][3], a0[0], a0[1], a0[2], a0[3], b1[2], b1[3]);
-                    mma_bf16(acc[1][3], a1[0], a1[1], a1[2], a1[3], b1[2], b1[3]);
-                }
-            }
-        }
+        uint32_t m = starts[q] & (0xffffffffu >> (31 - lane));
+        int w = q;
+        while (m == 0u && w > 0) m = starts[--w];
+        if (m) beg = w * 32 + 31 - __clz(m);
+        m = lane == 31 ? 0u : starts[q] & (0xfffffffeu << lane);
+        w = q;
+        while (m == 0u && w < 3) m = starts[++w];
+        if (m) end = min(w * 32 + __ffs(m) - 1, R);
     }
-    // norms from the diagonal
-    if ((g >> 1) == tig) {
-        const int e = g & 1;
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh)
-                nrm[mt * 16 + hh * 8 + g] = sqrtf(e ? acc[mt][2 * mt + hh][hh * 2 + 1] : acc[mt][2 * mt + hh][hh * 2]);
-    }
+    wait_failed = wait_failed || !umma::mbar_wait(smem_u32(smem) + kBarOff + 16, phase_u);
     __syncwarp();
-    float tn[4][2];
+    umma::fence_after_sync();
+    uint32_t g[32];
+    umma::tmem_ld32(lane_addr + q * 32, g);   // the columns of the warp's own rows
+    umma::tmem_ld_wait();
+    norm[i] = sqrtf(diagonal(g, lane));
+    const bool act[1] = {i < R};
+    if (team_any(wait_failed)) { failed = true; return 0; }   // (the norms are in place)
+    const float tni = tau * norm[i];
+    const int w_lo = __reduce_min_sync(kFull, beg >> 5);   // first word any of the warp's rows needs
+    uint32_t e[1][4];
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const float2 nn = *reinterpret_cast<const float2*>(nrm + nt * 8 + 2 * tig);
-        tn[nt][0] = tau * nn.x;
-        tn[nt][1] = tau * nn.y;
-    }
-    uint32_t wrow[2][2];
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int hh = 0; hh < 2; ++hh) {
-            uint32_t w = 0;
-            if (mt == 0 || two_mt) {
-                const float ni = nrm[mt * 16 + hh * 8 + g];
-#pragma unroll
-                for (int nt = 0; nt < 4; ++nt) {
-                    if (nt < 2 * mt + hh) continue;   // columns before the row's own
-                    if (nt < nnt) {
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const float thr = ni * tn[nt][e];
-                            bool hit = acc[mt][nt][hh * 2 + e] > thr;
-                            if (kNegTau) hit = hit || (thr == 0.f);   // a zero-norm key has Sim = 0 > tau
-                            if (hit) w |= 1u << (nt * 8 + e);
-                        }
-                    }
-                }
-                w <<= 2 * tig;
-                w |= __shfl_xor_sync(kFull, w, 1);
-                w |= __shfl_xor_sync(kFull, w, 2);
+    for (int c = 3; c >= 0; --c) {
+        uint32_t w = 0u;
+        if (c >= w_lo && c <= q) {
+            if (c != q) {
+                umma::tmem_ld32(lane_addr + c * 32, g);
+                umma::tmem_ld_wait();
             }
-            wrow[mt][hh] = w;
+            w = tau < 0.f ? sim_word_neg(g, norm + c * 32, tni) : sim_word(g, norm + c * 32, tni);
+            w &= bits_between(beg, i, c);
         }
-    __syncwarp();   // the norms are spent: the next segment of this warp may overwrite them
-    // lane 4g + t owns token g + 8t
-    const int own = g + 8 * tig;
-    const uint32_t lowmask = l >= 32 ? 0xffffffffu : ((1u << l) - 1u);
-    uint32_t mine = (tig & 2) ? ((tig & 1) ? wrow[1][1] : wrow[1][0]) : ((tig & 1) ? wrow[0][1] : wrow[0][0]);
-    mine &= (0xfffffffeu << own) & lowmask;   // later tokens of the segment only
-    // Algorithm 1
-    uint32_t U = lowmask, seeds = 0u, mymem = 0u;
-    int seed_of = 0;
-    while (U) {
-        const int i = __ffs(U) - 1;                      // lowest unassigned token: a seed
-        const int src = ((i & 7) << 2) | (i >> 3);
-        const uint32_t mem = (__shfl_sync(kFull, mine, src) & U) | (1u << i);
-        U &= ~mem;
-        if ((mem >> own) & 1u) seed_of = i;
-        if (lane == src) mymem = mem;
-        seeds |= 1u << i;
+        e[0][c] = w;
     }
-    // hand the result to the tile
-    const int sh = a & 31, w0 = a >> 5;
-    if (lane == 0) {
-        atomicOr(&seedmask[w0], seeds << sh);
-        if (sh != 0 && (seeds >> (32 - sh)) != 0u) atomicOr(&seedmask[w0 + 1], seeds >> (32 - sh));
-    }
-    if (mymem != 0u) {
-        adj[adj_row(a + own)] = mymem;
-        cnts[a + own] = kPending | (uint32_t)a;
-    }
-    if (as != nullptr && own < l) as[a + own] = row0 + a + seed_of;
+    umma::fence_before_sync();
+    const int ends[1] = {end};
+    return settle_rows<1>(e, act, ends, smem, q, lane, as, row0, publish, sh_p);
 }
 
-// Eq. 3 for the tile's P clusters (seedrow[c] = seed row of cluster c), dealt to the compute warps in turn.  Every token belongs to
-// exactly one cluster, so a cluster's mean can overwrite its seed's staged row once its members are
-// summed (fp32, token order); a cluster of one is left as it is.  cnts[seed row] ends up holding the
-// member count.  `lanes` is 32 when K and V are both staged, 16 when only K is.
-__device__ __forceinline__ void pool_clusters(unsigned char* lane_base, const uint16_t* seedrow, int P, const uint32_t* adj,
-                                              uint32_t* cnts, int warp, int lane, int lanes) {
-    const int c7 = lane & 7;
-    {
-        for (int c = warp; c < P; c += kWarps) {
-            const int i = seedrow[c];
-            const uint32_t info = cnts[i];
-            if (!(info & kPending)) continue;   // a one-token segment: settled when the tile was staged
-            const int a = info & 511, e = (info >> 9) & 511;
-            float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            int cnt;
-            if (e == 0) {   // up to 32 tokens: one word, relative to the segment
-                uint32_t mem = adj[adj_row(i)];
-                cnt = __popc(mem);
-                if (cnt > 1 && lane < lanes) rows_add(lane_base, a, mem, c7, sum);
-            } else {        // longer: the row's words, at tile positions
-                const uint32_t* row = adj + adj_row(i) - (i >> 5);
-                cnt = 0;
-                for (int ww = i >> 5; ww <= (e - 1) >> 5; ++ww) {
-                    const uint32_t mem = row[ww];
-                    cnt += __popc(mem);
-                    if (lane < lanes) rows_add(lane_base, ww * 32, mem, c7, sum);
+// Steps 1 and 2 for a tile of more than 128 rows (one segment): three products, the two diagonal ones first (they give the
+// norms), each read before the next overwrites it; thread tid settles rows tid and tid + 128.
+__device__ __noinline__ int settle_long_tile(unsigned char* smem, int R, uint32_t tmem, uint32_t phase_u, float tau, bool wait_failed,
+                                             bool* failed, int32_t* as, int row0, uint32_t* publish, int* sh_p) {
+    float* norm = reinterpret_cast<float*>(smem + kLongNormOff);
+    const uint32_t sbase = smem_u32(smem), bar_u = sbase + kBarOff + 16;
+    const int tid = threadIdx.x, lane = tid & 31, q = tid >> 5;
+    const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
+    uint32_t e[2][8], g[32];
+#pragma unroll
+    for (int w = 0; w < 8; ++w) e[0][w] = e[1][w] = 0u;
+#pragma unroll
+    for (int ps = 0; ps < 3; ++ps) {   // blocks (0, 0); (1, 1); (1, 0)
+        const int mb = ps == 0 ? 0 : 1, nb = ps == 1 ? 1 : 0, i = mb * 128 + tid;
+        if (team_any(wait_failed)) { *failed = true; return 0; }   // (the product before has been read)
+        if (tid == 0) {
+            umma::fence_after_sync();
+            umma_gram_block(sbase, kHalfLong, mb, nb, tmem, bar_u);
+        }
+        __syncwarp();
+        wait_failed = !umma::mbar_wait(bar_u, phase_u);
+        phase_u ^= 1u;
+        __syncwarp();
+        umma::fence_after_sync();
+        if (mb == nb) {
+            umma::tmem_ld32(lane_addr + q * 32, g);
+            umma::tmem_ld_wait();
+            norm[i] = sqrtf(diagonal(g, lane));
+            if (team_any(wait_failed)) { *failed = true; return 0; }   // (the norms are in place)
+        }
+        const float tni = tau * norm[i];
+#pragma unroll
+        for (int c = 3; c >= 0; --c) {
+            if (mb == nb && c > q) continue;   // columns past the warp's rows
+            if (mb != nb || c != q) {
+                umma::tmem_ld32(lane_addr + c * 32, g);
+                umma::tmem_ld_wait();
+            }
+            const float* nc = norm + nb * 128 + c * 32;
+            const uint32_t w = tau < 0.f ? sim_word_neg(g, nc, tni) : sim_word(g, nc, tni);
+            e[mb][nb * 4 + c] = i < R ? w & bits_between(0, i, nb * 4 + c) : 0u;
+        }
+        umma::fence_before_sync();
+    }
+    if (team_any(wait_failed)) { *failed = true; return 0; }
+    const bool act[2] = {true, tid + 128 < R};
+    const int ends[2] = {R, R};
+    return settle_rows<2>(e, act, ends, smem, q, lane, as, row0, publish, sh_p);
+}
+
+// Step 3 for sixteen clusters whose sums are not all finite: each lane one column of the warp's quarter, member by member.
+__device__ __noinline__ void pool_by_members(const unsigned char* tensor, int hs, const unsigned char* smem, int m, int P, int t_lo, int t_hi,
+                                             __nv_bfloat16* dst, int room, int warp, int lane) {
+    const int* cnt = reinterpret_cast<const int*>(smem + kCntOff);
+    const int col = warp * 32 + lane;
+    for (int c = 16 * m; c < min(16 * m + 16, P); ++c) {
+        if (cnt[c] <= 1 || c >= room) continue;
+        float sum = 0.f;
+        for (int i = t_lo; i < t_hi; ++i)
+            if ((smem + kRankOff)[rank_slot(i)] == c)
+                sum += __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(tensor + (col >> 6) * hs + tile_addr(i, (col & 63) >> 3) + (col & 7) * 2));
+        dst[(size_t)c * kD + col] = __float2bfloat16_rn(sum * __frcp_rn((float)cnt[c]));
+    }
+}
+
+// Step 3 for the NT tensors staged at smem, smem + kVOff (column halves hs bytes apart): this warp's 32 columns of every cluster
+// of more than one token, and the one-token clusters that are its turn.  dst[]: the tile's first core (row 0 of 128
+// columns); `room`: cores that fit.
+template <int NT>
+__device__ __forceinline__ void pool_tile(unsigned char* smem, int hs, int P, __nv_bfloat16* dst_k, __nv_bfloat16* dst_v, int room,
+                                          int warp, int lane) {
+    const int g = lane >> 2, tig = lane & 3;
+    const uint32_t sbase = smem_u32(smem);
+    const int* cnt = reinterpret_cast<const int*>(smem + kCntOff);
+    const unsigned char* seedrow = smem + kSeedOff;
+    const uint16_t* seg_end = reinterpret_cast<const uint16_t*>(smem + kEndOff);
+    // ldmatrix.trans: matrix j of four holds tokens 8 (j & 1) .. + 7, columns 8 (j >> 1) .. + 7 of a 16 x 16 block
+    const int j = lane >> 3, r8 = lane & 7;
+    const uint32_t b_row = sbase + (warp >> 1) * hs + ((j & 1) * 8 + r8) * kHalfRow;
+    const uint32_t off0 = (uint32_t)((((warp & 1) * 4 + (j >> 1)) ^ r8) << 4), off1 = (uint32_t)((((warp & 1) * 4 + 2 + (j >> 1)) ^ r8) << 4);
+    for (int m = 0; m * 16 < P; ++m) {
+        const int k_lo = seedrow[16 * m] >> 4, k_hi = (seg_end[min(16 * m + 15, P - 1)] + 15) >> 4;
+        float acc[NT][4][4];
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt) acc[t][nt][0] = acc[t][nt][1] = acc[t][nt][2] = acc[t][nt][3] = 0.f;
+        const uint32_t c0 = (uint32_t)(16 * m + g) * 0x01010101u, c1 = c0 + 0x08080808u;
+#pragma unroll 2
+        for (int kk = k_lo; kk < k_hi; ++kk) {
+            // M's fragment: rows g and g + 8 of the sixteen clusters, tokens 2 tig, +1, +8, +9 of the sixteen
+            const uint32_t ranks = *reinterpret_cast<const uint32_t*>(smem + kRankOff + kk * 16 + 4 * tig);
+            const uint32_t m0 = __vcmpeq4(ranks, c0), m1 = __vcmpeq4(ranks, c1);
+            const uint32_t a0 = __byte_perm(m0, 0u, 0x1100) & 0x3f803f80u, a1 = __byte_perm(m1, 0u, 0x1100) & 0x3f803f80u;
+            const uint32_t a2 = __byte_perm(m0, 0u, 0x3322) & 0x3f803f80u, a3 = __byte_perm(m1, 0u, 0x3322) & 0x3f803f80u;
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                const uint32_t row = b_row + t * kVOff + kk * 16 * kHalfRow;
+                uint32_t b0, b1, b2, b3;
+                ldmatrix_x4_trans(row + off0, b0, b1, b2, b3);
+                mma_bf16(acc[t][0], a0, a1, a2, a3, b0, b1);
+                mma_bf16(acc[t][1], a0, a1, a2, a3, b2, b3);
+                ldmatrix_x4_trans(row + off1, b0, b1, b2, b3);
+                mma_bf16(acc[t][2], a0, a1, a2, a3, b0, b1);
+                mma_bf16(acc[t][3], a0, a1, a2, a3, b2, b3);
+            }
+        }
+        float check = 0.f;   // stays zero as long as every sum is finite
+#pragma unroll
+        for (int t = 0; t < NT; ++t)
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) check = fmaf(acc[t][nt][x], 0.f, check);
+        if (__any_sync(kFull, !(check == 0.f))) {
+            const int t_lo = k_lo * 16, t_hi = seg_end[min(16 * m + 15, P - 1)];
+            pool_by_members(smem, hs, smem, m, P, t_lo, t_hi, dst_k, room, warp, lane);
+            if (NT > 1) pool_by_members(smem + kVOff, hs, smem, m, P, t_lo, t_hi, dst_v, room, warp, lane);
+        } else {
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+                const int c = 16 * m + 8 * hh + g;
+                const int n = c < P ? cnt[c] : 0;
+                if (n > 1 && c < room) {
+                    const float inv = __frcp_rn((float)n);
+                    const size_t o = (size_t)c * kD + warp * 32 + 2 * tig;
+#pragma unroll
+                    for (int t = 0; t < NT; ++t)
+#pragma unroll
+                        for (int nt = 0; nt < 4; ++nt) {
+                            const __nv_bfloat162 v = __floats2bfloat162_rn(acc[t][nt][2 * hh] * inv, acc[t][nt][2 * hh + 1] * inv);
+                            *reinterpret_cast<__nv_bfloat162*>((t ? dst_v : dst_k) + o + nt * 8) = v;
+                        }
                 }
             }
-            __syncwarp();
-            if (lane == 0) cnts[i] = (uint32_t)cnt;
-            if (cnt > 1 && lane < lanes) row_put_mean(lane_base, i, c7, sum, 1.0f / (float)cnt);
+        }
+    }
+    // clusters of one token: bit for bit, sixteen lanes a row
+    const int t = lane >> 4, chunk = lane & 15;
+    for (int c0 = 0; c0 < P; c0 += 32) {
+        const bool single = c0 + lane < P && c0 + lane < room && cnt[c0 + lane] == 1;
+        uint32_t todo = __ballot_sync(kFull, single) & (0x11111111u << warp);
+        while (todo) {
+            const int c = c0 + __ffs(todo) - 1;
+            todo &= todo - 1;
+            if (t < NT)
+                *reinterpret_cast<uint4*>((t ? dst_v : dst_k) + (size_t)c * kD + chunk * 8) =
+                    *reinterpret_cast<const uint4*>(smem + t * kVOff + (chunk >> 3) * hs + tile_addr(seedrow[c], chunk & 7));
         }
     }
 }
@@ -616,17 +509,14 @@ struct Params {
     LayerRefs layer[NL];
 };
 
-
-
-// The service warp draws the next ticket, turns it into a tile (sequence, head, tile index, rows) and
-// copies the tile's segment starts into shared memory.  Tickets go round the (sequence, head) pairs:
-// ticket w is tile w / (B*Hkv) of pair w % (B*Hkv), so consecutive tiles of one head are B*Hkv
-// tickets apart and a tile's predecessor has usually published its cluster count (and often its
-// prefix) by the time the tile looks back.  A pair with fewer tiles skips its surplus tickets.
+// The service warp draws the next ticket, turns it into a tile (layer, sequence, head, tile index, rows) and marks the rows
+// that start a segment.  Tickets go round the (layer, sequence, head) units: ticket w is tile w / units of unit
+// w % units, so a tile's predecessor has usually published its cluster count (and often its prefix) by the time
+// the tile looks back.  A unit with fewer tiles skips its surplus tickets.
 // geo[gT] = -1 when no work is left (max_nt = most tiles any sequence has).
 template <int NL>
-__device__ __forceinline__ void fetch_tile(const Params<NL>& p, int lane, int max_nt, int* geo, int16_t* segs) {
-    const int pairs = p.B * p.Hkv, units = pairs * p.L;   // (layer, sequence, head) units take the tickets in turn
+__device__ __forceinline__ void fetch_tile(const Params<NL>& p, int lane, int max_nt, int* geo, uint32_t* starts) {
+    const int pairs = p.B * p.Hkv, units = pairs * p.L;
     int b, h, t, nt, ly;
     for (;;) {
         int w = 0;
@@ -635,6 +525,7 @@ __device__ __forceinline__ void fetch_tile(const Params<NL>& p, int lane, int ma
         t = w / units;
         if (t >= max_nt) {
             if (lane == 0) geo[gT] = -1;
+            __syncwarp();
             return;
         }
         const int unit = w - t * units;
@@ -649,79 +540,91 @@ __device__ __forceinline__ void fetch_tile(const Params<NL>& p, int lane, int ma
     const int s_begin = ts[t], s_end = ts[t + 1];
     const int nseg = max(min(s_end - s_begin, kShortRows), 1);
     const int g_row0 = p.seg_off[s_begin];
-    for (int i = lane; i <= nseg; i += 32) segs[i] = (int16_t)min(p.seg_off[s_begin + i] - g_row0, kMaxRows);
-    const int R = min(p.seg_off[s_begin + nseg] - g_row0, kMaxRows);
+    const int R = max(min(p.seg_off[s_begin + nseg] - g_row0, kMaxRows), 1);
+    if (lane < 4) starts[lane] = 0u;
+    __syncwarp();
+    if (R <= kShortRows)
+        for (int i = lane; i < nseg; i += 32) {
+            const int a = min(p.seg_off[s_begin + i] - g_row0, kShortRows - 1);
+            atomicOr(&starts[a >> 5], 1u << (a & 31));
+        }
     if (lane == 0) {
         geo[gB] = b; geo[gH] = h; geo[gT] = t; geo[gNseg] = nseg; geo[gRow0] = g_row0 - b * p.n; geo[gR] = R;
         geo[gLast] = (t == nt - 1);
         geo[gLayer] = ly;
     }
+    __syncwarp();
 }
 
-// Stages rows [row0, row0 + R) of head (b, h) of one tensor with TMA: one box of 32 rows x 64 columns
-// per lane (R <= 256 needs at most 16 boxes for both column halves), the halves `hs` bytes apart at
-// `dst`.  Rows past R inside the last box are the cache's next rows, or zeros past the end of the
-// sequence; no one reads them.
-__device__ __forceinline__ void stage_rows(uint32_t dst, int hs, const CUtensorMap* map, int row0, int R, int h, int b,
-                                           uint32_t bar, int lane) {
-    const int nb = (R + kBoxRows - 1) / kBoxRows;
-    if (lane == 0) mbar_expect_tx(bar, (uint32_t)(2 * nb * kBoxBytes));
+// Stages the rows of a tile of one tensor with TMA: one box of 32 rows x 64 columns per lane (R <= 256 needs at most 16 boxes for
+// both column halves), the halves `hs` bytes apart at `dst`.  Rows past R inside the last box are the cache's next rows,
+// or zeros past the end of the sequence; no cluster holds them.
+__device__ __forceinline__ void stage_rows(uint32_t dst, int hs, const CUtensorMap* map, const int* geo, uint32_t bar, int lane) {
+    const int nb = (geo[gR] + kBoxRows - 1) / kBoxRows;
+    if (lane == 0) umma::mbar_expect_tx(bar, (uint32_t)(2 * nb * kBoxBytes));
     __syncwarp();
     if (lane < 2 * nb) {
         const int half = lane >= nb, i = lane - half * nb;
-        tma_box(dst + half * hs + i * kBoxBytes, map, half * 64, row0 + i * kBoxRows, h, b, bar);
+        tma_box(dst + half * hs + i * kBoxBytes, map, half * 64, geo[gRow0] + i * kBoxRows, geo[gH], geo[gB], bar);
     }
 }
 
-// The same for the second tensor of a tile longer than SC_TILE_ROWS (V staged where K was): one
-// segment [a, e), seeds in seedmask, member masks in the seeds' adjacency rows, counts already known.
-__device__ __forceinline__ void merge_long_segment(unsigned char* lane_base, int a, int e, const uint32_t* seedmask,
-                                                   const uint32_t* adj, int warp, int lane, int lanes) {
-    const int c7 = lane & 7, w_end = (e - 1) >> 5;
-    int turn = 0;
-    for (int w = a >> 5; w <= w_end; ++w) {
-        uint32_t sb = seedmask[w] & bits_between(a, e, w);
-        while (sb) {
-            const int i = w * 32 + __ffs(sb) - 1;
-            sb &= sb - 1;
-            if ((turn++ & (kWarps - 1)) != warp) continue;
-            const uint32_t* row = adj + adj_row(i) - (i >> 5);
-            float sum[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-            int cnt = 0;
-            for (int ww = i >> 5; ww <= w_end; ++ww) {
-                const uint32_t mem = row[ww];
-                cnt += __popc(mem);
-                if (lane < lanes) rows_add(lane_base, ww * 32, mem, c7, sum);
-            }
-            if (cnt > 1 && lane < lanes) row_put_mean(lane_base, i, c7, sum, 1.0f / (float)cnt);
+// Look-back by one warp: clusters of tiles 0 .. t - 1 of a head (their counts may still be on their way).
+// Reads kPollGroups x 32 status words at a time, nearest first, until one that holds a full prefix.
+__device__ __forceinline__ int look_back(const uint32_t* stt, int t, int lane, int32_t* status) {
+    int upto = t, sum = 0;   // tiles [0, upto) still to be accounted for
+    bool done = false;
+    unsigned long long t0 = 0;
+    while (upto > 0 && !done) {
+        uint32_t v[kPollGroups];
+#pragma unroll
+        for (int j = 0; j < kPollGroups; ++j) {
+            const int k = upto - 1 - lane - 32 * j;
+            v[j] = (k >= 0) ? ld_volatile(&stt[k]) : kFlagPrefix;   // before tile 0: prefix 0
+        }
+        bool stalled = false, progressed = false;
+#pragma unroll
+        for (int j = 0; j < kPollGroups; ++j) {
+            if (done || stalled) continue;
+            const uint32_t ready = __ballot_sync(kFull, (v[j] >> 30) != 0u);
+            const uint32_t pref = __ballot_sync(kFull, (v[j] >> 30) == 2u);
+            // usable run: lanes 0..m-1 all ready, stopping at the first that holds a full prefix
+            const int first_unready = (ready == kFull) ? 32 : __ffs(~ready) - 1;
+            const int first_pref = pref ? __ffs(pref) - 1 : 32;
+            const int take = min(first_unready, first_pref + 1);
+            sum += warp_sum_i((lane < take) ? (int)(v[j] & kValueMask) : 0);
+            if (first_pref < first_unready) { done = true; continue; }   // reached an inclusive prefix
+            upto -= take;
+            progressed |= take > 0;
+            stalled = take < 32;
+        }
+        if (!done && !progressed) {
+            const unsigned long long now = __shfl_sync(kFull, umma::global_ns(), 0);   // one clock for the warp
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > kWaitLimitNs) { set_status(status, SC_ERR_TIMEOUT); return 0; }
+            __nanosleep(64);
         }
     }
+    return sum;
 }
 
 template <int kMode, int NL>
-__global__ void __launch_bounds__(kThreads, 3) compress_fused_kernel(const __grid_constant__ Params<NL> p) {
+__global__ void __launch_bounds__(kThreads, kBlocksPerSm) compress_fused_kernel(const __grid_constant__ Params<NL> p) {
     extern __shared__ __align__(1024) unsigned char smem[];   // the swizzle pattern repeats every 1024 bytes
-    uint32_t* cnts = reinterpret_cast<uint32_t*>(smem + kCntOff);
-    uint32_t* adj = reinterpret_cast<uint32_t*>(smem + kAdjOff);
-    float* norm = reinterpret_cast<float*>(smem + kNormOff);
-    uint16_t* seedrow = reinterpret_cast<uint16_t*>(smem + kNormOff);   // reuses the norms once they are spent
-    int16_t* segs_buf = reinterpret_cast<int16_t*>(smem + kSegsOff);
-    uint32_t* seedmask = reinterpret_cast<uint32_t*>(smem + kMiscOff);
-    int* geo_buf = reinterpret_cast<int*>(smem + kMiscOff + 32);        // [2][8]
-    int* misc = reinterpret_cast<int*>(smem + kMiscOff + 96);           // [0] output offset of the tile, [1] last block,
-                                                                        // [2] 32-row blocks that a segment of > 32 tokens touches,
-                                                                        // [3] number of segments of more than one token
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kMiscOff + 272);
-    volatile int* umma_failed = reinterpret_cast<volatile int*>(smem + kMiscOff + 276);   // a wait for the tensor core gave up
-    int* claim = reinterpret_cast<int*>(smem + kMiscOff + 112);         // next entry of multi[] to be worked on
-    uint8_t* multi = smem + kMiscOff + 144;                             // [128] the segments of more than one token
-    uint32_t* membits = reinterpret_cast<uint32_t*>(smem + kMiscOff + 288);     // [8] tokens of long segments known to be members
+    uint32_t* starts_buf = reinterpret_cast<uint32_t*>(smem + kMiscOff + 64);   // [2][4] rows that start a segment
+    int* geo_buf = reinterpret_cast<int*>(smem + kMiscOff + 96);                // [2][8]
+    volatile int* sh_base = reinterpret_cast<volatile int*>(smem + kMiscOff + 160);   // first core of the tile
+    int* sh_p = reinterpret_cast<int*>(smem + kMiscOff + 164);                        // its clusters
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kMiscOff + 168);
+    int* last_block = reinterpret_cast<int*>(smem + kMiscOff + 172);
     const uint32_t sbase = smem_u32(smem);
-    const uint32_t bar_k = sbase + kBarOff, bar_v = bar_k + 8, bar_u = bar_k + 16;
+    // keys landed; values landed; product done; offset known; count known; buffer free; (long tile) keys spent
+    const uint32_t bar_k = sbase + kBarOff, bar_v = bar_k + 8, bar_u = bar_k + 16, bar_base = bar_k + 24, bar_p = bar_k + 32,
+                   bar_free = bar_k + 40, bar_half = bar_k + 48;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool service = warp == kWarps;   // the ninth warp
-    int max_nt = 0;                        // most tiles any sequence has (service warp)
+    const bool service = warp == kWarps;   // the fifth warp
+    int max_nt = 0;                        // most tiles any sequence has
 
     if (p.skip != nullptr && *p.skip != 0) return;   // uniform over the grid: nothing touched, nothing to clean
     const float tau = p.tau_dev != nullptr ? *p.tau_dev : p.tau;
@@ -729,256 +632,154 @@ __global__ void __launch_bounds__(kThreads, 3) compress_fused_kernel(const __gri
     // serialization (a no-op otherwise); this kernel waits for its predecessor only at its very end.
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     if (tid == 0) {
-        mbar_init(bar_k, 1);
-        mbar_init(bar_v, 1);
-        mbar_init(bar_u, 1);
-        *umma_failed = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        umma::mbar_init(bar_k, 1);
+        umma::mbar_init(bar_v, 1);
+        umma::mbar_init(bar_u, 1);
+        umma::mbar_init(bar_base, 1);
+        umma::mbar_init(bar_p, 1);
+        umma::mbar_init(bar_free, kWarps);
+        umma::mbar_init(bar_half, kWarps);
+        umma::mbar_fence_init();
         if ((sbase & 1023u) != 0u) set_status(p.status, SC_ERR_CUDA);   // the swizzled addressing assumes this
     }
-    fence_async_proxy();
-    uint32_t phase_k = 0, phase_v = 0, phase_u = 0;
-    bool failed = false;
-    // Tensor memory for the Gram blocks of long segments: allocated once per (persistent) block by the service warp,
+    umma::fence_async_proxy();
+    // Tensor memory for the product of a tile's keys: allocated once per (persistent) block by the service warp,
     // which then gives up the permit (a block may not allocate again after that, so it is not done per tile).
-    if (warp == kWarps) umma::tmem_alloc(sbase + kMiscOff + 272, kTmemCols);
+    if (service) umma::tmem_alloc(sbase + kMiscOff + 168, kTmemCols);
     umma::fence_before_sync();
-
-    if (service) {
-        for (int b = lane; b < p.B; b += 32) max_nt = max(max_nt, min(p.seq_tile_cnt[b], p.n_tile_cap));
-        max_nt = warp_max_i(max_nt);
-        fetch_tile(p, lane, max_nt, geo_buf, segs_buf);
-    }
-    if (tid == kNW) { misc[2] = misc[3] = 0; *claim = 0; }
-    if (tid >= 32 && tid < 32 + kNW) { seedmask[tid - 32] = 0u; membits[tid - 32] = 0u; }
+    for (int b = lane; b < p.B; b += 32) max_nt = max(max_nt, min(p.seq_tile_cnt[b], p.n_tile_cap));
+    max_nt = warp_max_i(max_nt);
     __syncthreads();
     umma::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    bool failed = false;
 
-    int buf = 0;
-    for (;;) {
-        const int* geo = geo_buf + buf * 8;
-        const int16_t* segs = segs_buf + buf * kSegsStride;
-        const int t = geo[gT];
-        if (t < 0) break;
-        const int b = geo[gB], h = geo[gH], nseg = geo[gNseg], row0 = geo[gRow0], R = geo[gR];
-        const int bh = b * p.Hkv + h;
-        const LayerRefs& lr = p.layer[NL == 1 ? 0 : geo[gLayer]];
-        const int unit = (NL == 1 ? 0 : geo[gLayer]) * p.B * p.Hkv + bh;   // index of this (layer, sequence, head)
-        const bool long_tile = R > kShortRows;
-        const bool two_tensors = (kMode != kCountOnly) && !long_tile;   // V staged beside K
-        const int hs = long_tile ? kHalfLong : kHalfShort;
-
-        // ---- 1. stage the rows (service warp, TMA); prefetch ahead ----
-        if (service) {
-            stage_rows(sbase, hs, &lr.map_k, row0, R, h, b, bar_k, lane);
-            if (two_tensors) stage_rows(sbase + kVOff, hs, &lr.map_v, row0, R, h, b, bar_v, lane);
-        }
-        // end of the segment each row is in (0 past the tile)
-        // also: one-token segments (delimiters, lone tokens) are clusters of their own -- no key needed;
-        // the others are listed for the warps
-        int32_t* as = lr.assign ? lr.assign + (size_t)bh * p.n + row0 : nullptr;
-        if (nseg == 1 && R > 1) {
-            if (tid == 0) { multi[0] = 0; misc[3] = 1; if (R > kWarpSegMax) misc[2] = (int)((1u << ((R + 31) >> 5)) - 1u); }
-        } else {
-            for (int s = tid; s < nseg; s += kThreads) {
-                const int a = segs[s], e = segs[s + 1];
-                if (e - a == 1) {
-                    cnts[a] = 1u;
-                    atomicOr(&seedmask[a >> 5], 1u << (a & 31));
-                    if (as) as[a] = row0 + a;
-                    continue;
-                }
-                multi[atomicAdd(&misc[3], 1)] = (uint8_t)s;
-                if (e - a > kWarpSegMax)   // the tile takes the tensor-core step: which 32-row words it concerns
-                    for (int k = a >> 5; k <= (e - 1) >> 5; ++k) atomicOr(&misc[2], 1 << k);
+    if (service) {
+        fetch_tile(p, lane, max_nt, geo_buf, starts_buf);
+        uint32_t n_half = 0;
+        for (uint32_t it = 0;; ++it) {
+            const int* geo = geo_buf + (it & 1) * 8;
+            // the buffer is free: the compute warps are through with the tile before
+            if (it > 0 && !umma::mbar_wait(bar_free, (it - 1) & 1)) { failed = true; break; }
+            if (geo[gT] < 0) {
+                if (lane == 0) umma::mbar_arrive(bar_k);
+                break;
             }
-        }
-        failed = !mbar_wait(bar_k, phase_k);   // K has landed
-        phase_k ^= 1u;
-        if (two_tensors && !failed) {
-            failed = !mbar_wait(bar_v, phase_v);   // and V
-            phase_v ^= 1u;
-        }
-        if (__syncthreads_or(failed)) { failed = true; break; }
-
-        // ---- 2. segments of more than kWarpSegMax tokens: the tile's Gram matrix on the tensor core, 128 x 128 at a
-        //         time into tensor memory (one block for a tile of up to 128 tokens, else the two diagonal blocks --
-        //         they give the norms -- and the lower one).  Four warps read it, one row per thread, and keep which
-        //         earlier tokens of its segment each row is similar to; Algorithm 1 is then settled for all those rows
-        //         at once in decision rounds (the sequential pass visits one seed at a time) ----
-        if (misc[2] != 0) {
-            settle_long_segments(smem, hs, segs, nseg, R, (uint32_t)misc[2], tmem, phase_u, tau, as, row0);
-            phase_u ^= 1u;   // one or three blocks
-        }
-
-        // ---- 3. the service warp draws the block's next ticket; compute warps: Algorithm 1 for the segments of up
-        //         to 32 tokens, one warp each, in registers ----
-        unsigned char* lane_base = smem + (lane >> 4) * kVOff + ((lane >> 3) & 1) * hs;   // see rows_add
-        if (service) {
-            fetch_tile(p, lane, max_nt, geo_buf + (buf ^ 1) * 8, segs_buf + (buf ^ 1) * kSegsStride);
-        } else {
-            const int nmulti = misc[3];
-            for (;;) {   // whichever warp is free takes the next segment
-                int k = 0;
-                if (lane == 0) k = atomicAdd(claim, 1);
-                k = __shfl_sync(kFull, k, 0);
-                if (k >= nmulti) break;
-                const int s = multi[k];
-                const int a = segs[s], e = segs[s + 1];
-                if (e - a > kWarpSegMax) continue;   // settled above
-                if (tau < 0.f) gsc_short_segment<true>(sbase, hs, a, e - a, tau, norm + warp * 64, seedmask, adj, cnts, as, row0, lane);
-                else gsc_short_segment<false>(sbase, hs, a, e - a, tau, norm + warp * 64, seedmask, adj, cnts, as, row0, lane);
-            }
-        }
-        __syncthreads();
-        if (*umma_failed) { failed = true; break; }   // a wait for the tensor core gave up in step 2 (known to all by now)
-
-        // ---- 4. cluster count of the tile, published at once.  Service warp: output offset of the tile
-        //         (look-back).  Compute warps: the seed row of every cluster, and Eq. 3 ----
-        int P = 0;
-#pragma unroll
-        for (int w = 0; w < kNW; ++w) P += __popc(seedmask[w]);
-        uint32_t* stt = p.tile_state + (size_t)unit * p.n_tile_cap;
-        if (kMode == kCountOnly) {
-            if (tid == 0) {
-                if (p.count_into_len) atomicAdd(&lr.core_len[bh], P);
-                else stt[t] = (uint32_t)P;
-            }
-        } else {
-            if (!service) {
-                if (tid < R) {
-                    const uint32_t wbits = seedmask[tid >> 5];
-                    if ((wbits >> (tid & 31)) & 1u) {
-                        int rank = __popc(wbits & ((1u << (tid & 31)) - 1u));
-                        for (int w = 0; w < (tid >> 5); ++w) rank += __popc(seedmask[w]);
-                        seedrow[rank] = (uint16_t)tid;
-                    }
-                }
-                compute_warps_sync();   // the table of seed rows is complete
-                pool_clusters(lane_base, seedrow, P, adj, cnts, warp, lane, long_tile ? 16 : 32);
-            } else {
-                if (kMode == kLookBack && lane == 0)
-                    atomicExch(&stt[t], (t == 0 ? kFlagPrefix : kFlagAggregate) | (uint32_t)P);
-                int base = 0;
-                if (kMode == kWriteWithCounts) {
-                    for (int k = lane; k < t; k += 32) base += (int)stt[k];
-                    base = warp_sum_i(base);
-                } else {
-                    // look back over the predecessors, nearest first: one poll reads kPollGroups x 32 status
-                    // words (the loads overlap), then they are consumed 32 at a time
-                    int upto = t;      // tiles [0, upto) still to be accounted for
-                    bool gave_up = false, done = false;
-                    unsigned long long t0 = 0;
-                    while (upto > 0 && !done) {
-                        uint32_t v[kPollGroups];
-#pragma unroll
-                        for (int j = 0; j < kPollGroups; ++j) {
-                            const int k = upto - 1 - lane - 32 * j;
-                            v[j] = (k >= 0) ? ld_volatile(&stt[k]) : kFlagPrefix;   // before tile 0: prefix 0
-                        }
-                        bool stalled = false, progressed = false;
-#pragma unroll
-                        for (int j = 0; j < kPollGroups; ++j) {
-                            if (done || stalled) continue;
-                            const uint32_t ready = __ballot_sync(kFull, (v[j] >> 30) != 0u);
-                            const uint32_t pref = __ballot_sync(kFull, (v[j] >> 30) == 2u);
-                            // usable run: lanes 0..m-1 all ready, stopping at the first that holds a full prefix
-                            const int first_unready = (ready == kFull) ? 32 : __ffs(~ready) - 1;
-                            const int first_pref = pref ? __ffs(pref) - 1 : 32;
-                            const int take = min(first_unready, first_pref + 1);
-                            const int contrib = (lane < take) ? (int)(v[j] & kValueMask) : 0;
-                            base += warp_sum_i(contrib);
-                            if (first_pref < first_unready) { done = true; continue; }   // reached an inclusive prefix
-                            upto -= take;
-                            progressed |= take > 0;
-                            stalled = take < 32;
-                        }
-                        if (!done && !progressed) {
-                            if (t0 == 0) t0 = global_ns();
-                            else if (global_ns() - t0 > kWaitLimitNs) { gave_up = true; break; }
-                            __nanosleep(64);
-                        }
-                    }
-                    if (gave_up) { set_status(p.status, SC_ERR_TIMEOUT); base = 0; }
-                    if (lane == 0 && t > 0) atomicExch(&stt[t], kFlagPrefix | (uint32_t)(base + P));
-                }
+            const LayerRefs& lr = p.layer[NL == 1 ? 0 : geo[gLayer]];
+            const bool long_tile = geo[gR] > kShortRows;
+            stage_rows(sbase, long_tile ? kHalfLong : kHalfShort, &lr.map_k, geo, bar_k, lane);
+            if (kMode != kCountOnly && !long_tile) stage_rows(sbase + kVOff, kHalfShort, &lr.map_v, geo, bar_v, lane);
+            if (kMode != kCountOnly) {
+                const int bh = geo[gB] * p.Hkv + geo[gH];
+                uint32_t* stt = p.tile_state + (size_t)((NL == 1 ? 0 : geo[gLayer]) * p.B * p.Hkv + bh) * p.n_tile_cap;
+                const int base = look_back(stt, geo[gT], lane, p.status);
                 if (lane == 0) {
-                    misc[0] = base;
+                    *sh_base = base;
+                    umma::mbar_arrive(bar_base);
+                }
+                if (!umma::mbar_wait(bar_p, it & 1)) { failed = true; break; }
+                if (lane == 0) {
+                    const int upto = base + *sh_p;
+                    atomicExch(&stt[geo[gT]], kFlagPrefix | (uint32_t)upto);
                     if (geo[gLast]) {
-                        lr.core_len[bh] = base + P;
-                        if (base + P > p.cap) set_status(p.status, SC_ERR_CAPACITY);
+                        lr.core_len[bh] = upto;
+                        if (upto > p.cap) set_status(p.status, SC_ERR_CAPACITY);
                     }
                 }
-            }
-            __syncthreads();
-
-            // ---- compact, coalesced stores of the cores: cluster `row` of the tile sits in its seed's staged row ----
-            const int base = misc[0];
-            const size_t obase = (size_t)bh * p.cap;
-            for (int idx = tid; idx < P * 16; idx += kThreads) {
-                const int row = idx >> 4, c = idx & 15;
-                if (base + row < p.cap) {
-                    const size_t o = (obase + base + row) * kD + c * 8;
-                    const unsigned char* src = smem + (c >> 3) * hs + tile_addr(seedrow[row], c & 7);
-                    *reinterpret_cast<uint4*>(lr.core_k + o) = *reinterpret_cast<const uint4*>(src);
-                    if (!long_tile) *reinterpret_cast<uint4*>(lr.core_v + o) = *reinterpret_cast<const uint4*>(src + kVOff);
+                if (long_tile) {   // V takes the place of K
+                    if (!umma::mbar_wait(bar_half, n_half & 1)) { failed = true; break; }
+                    ++n_half;
+                    stage_rows(sbase, kHalfLong, &lr.map_v, geo, bar_v, lane);
                 }
             }
-            for (int row = tid; row < P; row += kThreads)
-                if (base + row < p.cap)
-                    lr.count[obase + base + row] = (int32_t)cnts[seedrow[row]];
-
-            // ---- a tile longer than SC_TILE_ROWS: V takes the place of K and is pooled with the same masks ----
-            if (long_tile) {
-                fence_async_proxy();   // the copies below overwrite what ordinary accesses read and wrote
-                __syncthreads();
-                if (service) stage_rows(sbase, hs, &lr.map_v, row0, R, h, b, bar_v, lane);
-                failed = !mbar_wait(bar_v, phase_v);
-                phase_v ^= 1u;
-                if (__syncthreads_or(failed)) { failed = true; break; }
-                if (!service) merge_long_segment(lane_base, 0, R, seedmask, adj, warp, lane, 16);
-                __syncthreads();
-                for (int idx = tid; idx < P * 16; idx += kThreads) {
-                    const int row = idx >> 4, c = idx & 15;
-                    if (base + row < p.cap)
-                        *reinterpret_cast<uint4*>(lr.core_v + (obase + base + row) * kD + c * 8) =
-                            *reinterpret_cast<const uint4*>(smem + (c >> 3) * hs + tile_addr(seedrow[row], c & 7));
-                }
-            }
+            // drawn now, not earlier: a tile drawn by a block that is still waiting would hold up its successors
+            fetch_tile(p, lane, max_nt, geo_buf + ((it & 1) ^ 1) * 8, starts_buf + ((it & 1) ^ 1) * 4);
         }
-            if (tid == kNW) { misc[2] = misc[3] = 0; *claim = 0; }
-        if (tid >= 32 && tid < 32 + kNW) { seedmask[tid - 32] = 0u; membits[tid - 32] = 0u; }
-        fence_async_proxy();   // the next tile's copies overwrite what ordinary accesses read and wrote
-        __syncthreads();
-        buf ^= 1;
+    } else {
+        uint32_t phase_u = 0;
+        bool bad = false;   // a wait of this warp gave up
+        for (uint32_t it = 0;; ++it) {
+            const int* geo = geo_buf + (it & 1) * 8;
+            const uint32_t par = it & 1;
+            bad = !umma::mbar_wait(bar_k, par) || bad;   // the keys have landed (or there is no more work)
+            if (!bad && geo[gT] < 0) break;
+            const int R = bad ? 1 : geo[gR], row0 = geo[gRow0], bh = geo[gB] * p.Hkv + geo[gH], ly = NL == 1 || bad ? 0 : geo[gLayer];
+            const LayerRefs& lr = p.layer[ly];
+            int32_t* as = (lr.assign && !p.count_into_len) ? lr.assign + (size_t)bh * p.n + row0 : nullptr;
+            uint32_t* publish = kMode == kCountOnly && p.count_into_len
+                                    ? nullptr : p.tile_state + (size_t)(ly * p.B * p.Hkv + bh) * p.n_tile_cap + geo[gT];
+            const bool long_tile = R > kShortRows;
+            int P;
+            if (!long_tile) {
+                if (tid == 0 && !bad) {
+                    umma::fence_after_sync();
+                    umma_gram_block(sbase, kHalfShort, 0, 0, tmem, bar_u);
+                }
+                __syncwarp();
+                P = settle_short_tile(smem, starts_buf + par * 4, R, tmem, phase_u, tau, bad, failed, as, row0, publish, sh_p);
+                phase_u ^= 1u;
+            } else {
+                P = settle_long_tile(smem, R, tmem, phase_u, tau, bad, &failed, as, row0, publish, sh_p);
+                phase_u ^= 1u;   // three products
+            }
+            if (failed) break;
+            if (kMode == kCountOnly) {
+                if (tid == 0 && p.count_into_len) atomicAdd(&lr.core_len[bh], P);
+            } else {
+                if (tid == 0) umma::mbar_arrive(bar_p);
+                bad = !umma::mbar_wait(bar_base, par) || bad;
+                if (!long_tile) bad = !umma::mbar_wait(bar_v, par) || bad;
+                __syncwarp();
+                const int base = *sh_base, room = bad ? 0 : p.cap - base;   // a wait that gave up: nothing is stored
+                const size_t first = (size_t)bh * p.cap + base;
+                for (int c = tid; c < P && c < room; c += kTeam) lr.count[first + c] = reinterpret_cast<const int*>(smem + kCntOff)[c];
+                if (!long_tile) {
+                    pool_tile<2>(smem, kHalfShort, P, lr.core_k + first * kD, lr.core_v + first * kD, room, warp, lane);
+                } else {
+                    pool_tile<1>(smem, kHalfLong, P, lr.core_k + first * kD, nullptr, room, warp, lane);
+                    umma::fence_async_proxy();   // the values' copies overwrite what ordinary accesses read
+                    __syncwarp();
+                    if (lane == 0) umma::mbar_arrive(bar_half);
+                    bad = !umma::mbar_wait(bar_v, par) || bad;
+                    __syncwarp();
+                    pool_tile<1>(smem, kHalfLong, P, lr.core_v + first * kD, nullptr, bad ? 0 : room, warp, lane);
+                }
+            }
+            umma::fence_async_proxy();   // the next tile's copies overwrite what ordinary accesses read
+            __syncwarp();
+            if (lane == 0) umma::mbar_arrive(bar_free);
+        }
+        failed = failed || bad;
     }
 
     // ---- exit: the last block to finish leaves the workspace zeroed for the next call ----
     if (failed) {   // a wait gave up: report it, and give copies that may still be in flight one more bounded
                     // wait (either parity: whichever phase is open) before the block's shared memory goes away
-        if (tid == 0) set_status(p.status, SC_ERR_TIMEOUT);
-        mbar_wait(bar_k, phase_k ^ 1u);
-        mbar_wait(bar_v, phase_v ^ 1u);
-        mbar_wait(bar_v, phase_v);
+        set_status(p.status, SC_ERR_TIMEOUT);
+        for (uint32_t ph = 0; ph < 2; ++ph) {
+            umma::mbar_wait(bar_k, ph);
+            umma::mbar_wait(bar_v, ph);
+            umma::mbar_wait(bar_u, ph);
+        }
     }
     umma::fence_before_sync();
     __syncthreads();
-    if (warp == kWarps) umma::tmem_dealloc(tmem, kTmemCols);
+    if (service) umma::tmem_dealloc(tmem, kTmemCols);
     // Under an overlapped launch a block does not finish before the kernel enqueued ahead of this one has
     // completed, so completion is transitive along a run of overlapped launches (a no-op otherwise).
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     if (tid == 0) {
         __threadfence();
         const int done = atomicAdd(&p.ctl[1], 1);
-        misc[1] = (done == (int)gridDim.x - 1);
+        *last_block = (done == (int)gridDim.x - 1);
     }
     __syncthreads();
-    if (misc[1]) {
+    if (*last_block) {
         __threadfence();
-        if (kMode != kCountOnly) {
-            const size_t words = (size_t)p.L * p.B * p.Hkv * p.n_tile_cap;
-            for (size_t i = tid; i < words; i += kThreads) p.tile_state[i] = 0u;
+        if (kMode != kCountOnly) {   // the words of tiles that exist
+            const int units = p.L * p.B * p.Hkv;
+            for (int u = warp; u < units; u += kWarps + 1)
+                for (int i = lane; i < max_nt; i += 32) p.tile_state[(size_t)u * p.n_tile_cap + i] = 0u;
         }
         if (tid == 0) { p.ctl[0] = 0; p.ctl[1] = 0; }
     }
@@ -1044,7 +845,6 @@ int resident_blocks() {
     dev &= 63;
     if (grid_of[dev] == 0) {
         cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kCountOnly, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
-        cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kWriteWithCounts, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
         cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kLookBack, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
         cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kLookBack, cf::kMaxLayers>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
         // Blocks per SM by construction: launch bounds (registers), 75 KB of shared memory and 128 of the 512
@@ -1093,7 +893,7 @@ cudaError_t launch_compress_fused(const CompressArgs& a, cudaStream_t st) {
         cf::Params<1> pc = p;
         pc.layer[0].assign = nullptr;
         cf::compress_fused_kernel<cf::kCountOnly, 1><<<grid, cf::kThreads, cf::kSmemBytes, st>>>(pc);
-        cf::compress_fused_kernel<cf::kWriteWithCounts, 1><<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
+        cf::compress_fused_kernel<cf::kLookBack, 1><<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
         note_launches(2);
     } else {
         // With SC_FLAG_OVERLAP_PREV the kernel may start while the one enqueued before it on the stream is
@@ -1143,4 +943,3 @@ size_t compress_fused_layers_ws_bytes(int32_t L, int32_t B, int32_t Hkv, int32_t
 }
 
 }  // namespace sc
-
