@@ -2,16 +2,20 @@
 // three kernels per layer -- GSC per segment, prefix sum of cluster counts per (b, head),
 // mean-pool merge per segment.  CUDA-core arithmetic in fp32; serves SC_F32 and is the
 // cross-check of the fused bf16 path.
+// One warp per segment; bounded by the latency of its loads, so several rows are in flight at a time: eight in the
+// similarities (eight lanes per row, four columns per load), four in the merge, whose members come
+// from bit masks of the segment's assignments.  8 heads x 8K tokens of fp32: GSC 101 -> 45 us, merge 83 -> 36 us (50 us
+// with K and V in one warp) against one row at a time.
 #include "common.cuh"
 
 namespace sc {
 
 constexpr int kGenWarps = 8;
-constexpr int kMaxPerLane = 8;  // d <= 256
 
-// Algorithm 1 for one segment per warp.  Keys are read straight from global memory; the seed
-// row is held in registers and each candidate row is dotted against it across the warp.
-template <typename T>
+// Algorithm 1 for one segment per warp.  Rows are read straight from global memory, eight at a time: lanes 8r .. 8r + 7
+// form the product of row r (of four) with the seed's row, which they hold in registers.  NC: the most 32-column pieces
+// a row has (4 or 8).
+template <typename T, int NC>
 __global__ void __launch_bounds__(kGenWarps * 32)
 gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d,
             const int32_t* __restrict__ seg_off, const int32_t* __restrict__ n_seg_p, int seg_stride,
@@ -20,57 +24,74 @@ gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d
     __shared__ float norms[kGenWarps][SC_MAX_CHUNK_LEN];
     if (skip != nullptr && *skip != 0) return;
     const float tau = tau_dev != nullptr ? *tau_dev : tau_host;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane & 7, rsub = lane >> 3;
     const int n_seg = min(*n_seg_p, seg_stride);
     const int64_t items = (int64_t)n_seg * Hkv;
-    const int per = d / 32 + ((d % 32) ? 1 : 0);
     for (int64_t it = (int64_t)blockIdx.x * kGenWarps + w; it < items; it += (int64_t)gridDim.x * kGenWarps) {
         const int s = (int)(it % n_seg), h = (int)(it / n_seg);
         const int a = seg_off[s], e = seg_off[s + 1];
         const int b = a / n, r = a - b * n, l = min(e - a, SC_MAX_CHUNK_LEN);
-        const T* Kb = K + b * st.b + h * st.h;
-        int32_t* as = assign + ((int64_t)b * Hkv + h) * n;
-        // norms
-        for (int i = 0; i < l; ++i) {
-            const T* row = Kb + (int64_t)(r + i) * st.n;
+        const T* Kb = K + b * st.b + h * st.h + (int64_t)r * st.n + sub * 4;   // this lane's first columns of the segment's first row
+        int32_t* as = assign + ((int64_t)b * Hkv + h) * n + r;
+        // sum over the row's columns of x.y, x = row j (skipped where !on), the same in the row's eight lanes
+        auto load_row = [&](int j, bool on, float4 (&v)[NC]) {
+            const T* row = Kb + (int64_t)j * st.n;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) v[c] = on && (c * 8 + sub) * 4 < d ? load4(row + c * 32) : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        auto dot = [&](const float4 (&x)[NC], const float4 (&y)[NC]) {
             float acc = 0.f;
-            for (int c = lane; c < d; c += 32) { float x = Elem<T>::load(row + c); acc = fmaf(x, x, acc); }
-            acc = warp_sum(acc);
-            if (lane == 0) norms[w][i] = sqrtf(acc);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc = fmaf(x[c].x, y[c].x, fmaf(x[c].y, y[c].y, fmaf(x[c].z, y[c].z, fmaf(x[c].w, y[c].w, acc))));
+            return acc;
+        };
+        for (int j0 = 0; j0 < l; j0 += 8) {
+            float4 v0[NC], v1[NC];
+            load_row(j0 + rsub, j0 + rsub < l, v0);
+            load_row(j0 + 4 + rsub, j0 + 4 + rsub < l, v1);
+            float d0 = dot(v0, v0), d1 = dot(v1, v1);
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) { d0 += __shfl_xor_sync(kFull, d0, o); d1 += __shfl_xor_sync(kFull, d1, o); }
+            if (sub == 0) {
+                if (j0 + rsub < l) norms[w][j0 + rsub] = sqrtf(d0);
+                if (j0 + 4 + rsub < l) norms[w][j0 + 4 + rsub] = sqrtf(d1);
+            }
         }
         __syncwarp();
         unsigned word = 0;  // lane c holds the assigned bits of tokens 32c .. 32c+31
         int p = 0;
         for (int i = 0; i < l; ++i) {
-            unsigned wi = __shfl_sync(kFull, word, i >> 5);
+            const unsigned wi = __shfl_sync(kFull, word, i >> 5);
             if ((wi >> (i & 31)) & 1u) continue;
             ++p;
             if (lane == (i >> 5)) word |= 1u << (i & 31);
-            if (lane == 0) as[r + i] = r + i;
-            float seed[kMaxPerLane];
-            const T* srow = Kb + (int64_t)(r + i) * st.n;
-#pragma unroll
-            for (int u = 0; u < kMaxPerLane; ++u) {
-                int c = lane + 32 * u;
-                seed[u] = (u < per && c < d) ? Elem<T>::load(srow + c) : 0.f;
-            }
+            if (lane == 0) as[i] = r + i;
+            if (i + 1 >= l) break;
+            float4 seed[NC];
+            load_row(i, true, seed);
             const float ni = norms[w][i];
-            for (int j = i + 1; j < l; ++j) {
-                unsigned wj = __shfl_sync(kFull, word, j >> 5);
-                if ((wj >> (j & 31)) & 1u) continue;
-                const T* row = Kb + (int64_t)(r + j) * st.n;
-                float acc = 0.f;
+            for (int j0 = (i + 1) & ~7; j0 < l; j0 += 8) {   // eight tokens of one word
+                const unsigned open = (~__shfl_sync(kFull, word, j0 >> 5)) >> (j0 & 31);
+                const bool on0 = j0 + rsub > i && j0 + rsub < l && ((open >> rsub) & 1u);
+                const bool on1 = j0 + 4 + rsub > i && j0 + 4 + rsub < l && ((open >> (4 + rsub)) & 1u);
+                if (!__any_sync(kFull, on0 || on1)) continue;
+                float4 v0[NC], v1[NC];
+                load_row(j0 + rsub, on0, v0);
+                load_row(j0 + 4 + rsub, on1, v1);
+                float d0 = dot(seed, v0), d1 = dot(seed, v1);
 #pragma unroll
-                for (int u = 0; u < kMaxPerLane; ++u) {
-                    int c = lane + 32 * u;
-                    if (u < per && c < d) acc = fmaf(seed[u], Elem<T>::load(row + c), acc);
-                }
-                acc = warp_sum(acc);
-                const float nj = norms[w][j];
-                const float sim = (ni == 0.f || nj == 0.f) ? 0.f : acc / (ni * nj);
-                if (sim > tau) {
-                    if (lane == (j >> 5)) word |= 1u << (j & 31);
-                    if (lane == 0) as[r + j] = r + i;
+                for (int o = 1; o < 8; o <<= 1) { d0 += __shfl_xor_sync(kFull, d0, o); d1 += __shfl_xor_sync(kFull, d1, o); }
+                const float n0 = on0 ? norms[w][j0 + rsub] : 0.f, n1 = on1 ? norms[w][j0 + 4 + rsub] : 0.f;
+                const float s0 = (ni == 0.f || n0 == 0.f) ? 0.f : d0 / (ni * n0);
+                const float s1 = (ni == 0.f || n1 == 0.f) ? 0.f : d1 / (ni * n1);
+                const bool hit0 = on0 && s0 > tau, hit1 = on1 && s1 > tau;
+                const unsigned b0 = __ballot_sync(kFull, hit0) & 0x01010101u, b1 = __ballot_sync(kFull, hit1) & 0x01010101u;
+                const unsigned hits = ((b0 | (b0 >> 7) | (b0 >> 14) | (b0 >> 21)) & 15u) |
+                                      (((b1 | (b1 >> 7) | (b1 >> 14) | (b1 >> 21)) & 15u) << 4);
+                if (lane == (j0 >> 5)) word |= hits << (j0 & 31);
+                if (sub == 0) {
+                    if (hit0) as[j0 + rsub] = r + i;
+                    if (hit1) as[j0 + 4 + rsub] = r + i;
                 }
             }
         }
@@ -86,6 +107,7 @@ scan_generic(int Hkv, const int32_t* __restrict__ seq_seg_off, int seg_stride,
              int32_t* __restrict__ core_len, int cap, int32_t* status, const int32_t* __restrict__ skip,
              int count_only) {
     __shared__ int wt[8];
+    wait_for_previous();
     if (skip != nullptr && *skip != 0) return;
     const int b = blockIdx.x / Hkv, h = blockIdx.x % Hkv;
     const int s0 = min(seq_seg_off[b], seg_stride), s1 = min(seq_seg_off[b + 1], seg_stride);
@@ -109,55 +131,79 @@ scan_generic(int Hkv, const int32_t* __restrict__ seq_seg_off, int seg_stride,
     }
 }
 
-// Eq. 3 for one segment per warp: fp32 sums in token order, one divide, one rounding.
-template <typename T>
+// Eq. 3 for one segment of K or of V per warp: fp32 sums in token order, one divide, one rounding.  A lane owns four
+// columns (eight where d > 128); a cluster's members come from ballots over the segment's assignments, four rows
+// requested together.
+template <typename T, int kPer>
 __global__ void __launch_bounds__(kGenWarps * 32)
 merge_generic(const T* __restrict__ K, const T* __restrict__ V, sc_strides st, int B, int Hkv, int n, int d,
               const int32_t* __restrict__ seg_off, const int32_t* __restrict__ n_seg_p, int seg_stride,
               const int32_t* __restrict__ assign, const int32_t* __restrict__ seg_core_off,
               T* __restrict__ core_k, T* __restrict__ core_v, int32_t* __restrict__ count, int cap) {
+    constexpr int kWords = SC_MAX_CHUNK_LEN / 32;
+    wait_for_previous();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int n_seg = min(*n_seg_p, seg_stride);
-    const int64_t items = (int64_t)n_seg * Hkv;
+    const int64_t items = 2 * (int64_t)n_seg * Hkv;
     for (int64_t it = (int64_t)blockIdx.x * kGenWarps + w; it < items; it += (int64_t)gridDim.x * kGenWarps) {
-        const int s = (int)(it % n_seg), h = (int)(it / n_seg);
+        const bool is_v = it & 1;
+        const int s = (int)((it >> 1) % n_seg), h = (int)((it >> 1) / n_seg);
         const int a = seg_off[s], e = seg_off[s + 1];
-        const int b = a / n, r = a - b * n, l = min(e - a, SC_MAX_CHUNK_LEN);
-        const T* Kb = K + b * st.b + h * st.h;
-        const T* Vb = V + b * st.b + h * st.h;
-        const int32_t* as = assign + ((int64_t)b * Hkv + h) * n;
+        const int b = a / n, r = a - b * n, l = min(e - a, SC_MAX_CHUNK_LEN), nw = (l + 31) >> 5;
+        const T* rows = (is_v ? V : K) + b * st.b + h * st.h + (int64_t)r * st.n + lane * 4;
+        const int32_t* as = assign + ((int64_t)b * Hkv + h) * n + r;
         int row = seg_core_off[(int64_t)h * seg_stride + s];
         const int64_t obase = ((int64_t)b * Hkv + h) * cap;
-        for (int i = 0; i < l; ++i) {
-            if (as[r + i] != r + i) continue;
-            float sk[kMaxPerLane], sv[kMaxPerLane];
+        T* cores = (is_v ? core_v : core_k) + obase * d + lane * 4;
+        int mine[kWords];   // seed (relative) of tokens 32 k + lane
 #pragma unroll
-            for (int u = 0; u < kMaxPerLane; ++u) sk[u] = sv[u] = 0.f;
-            int cnt = 0;
-            for (int j = i; j < l; ++j) {
-                if (as[r + j] != r + i) continue;
-                ++cnt;
-                const T* kr = Kb + (int64_t)(r + j) * st.n;
-                const T* vr = Vb + (int64_t)(r + j) * st.n;
+        for (int k = 0; k < kWords; ++k) mine[k] = 32 * k + lane < l ? as[32 * k + lane] - r : -1;
+        for (int ws = 0; ws < nw; ++ws) {
+            int own = -1;
 #pragma unroll
-                for (int u = 0; u < kMaxPerLane; ++u) {
-                    int c = lane + 32 * u;
-                    if (c < d) { sk[u] += Elem<T>::load(kr + c); sv[u] += Elem<T>::load(vr + c); }
-                }
-            }
-            if (row < cap) {
-                const float fc = (float)cnt;
+            for (int k = 0; k < kWords; ++k) if (k == ws) own = mine[k];
+            unsigned seeds = __ballot_sync(kFull, own == 32 * ws + lane);
+            while (seeds) {
+                const int i = 32 * ws + __ffs(seeds) - 1;
+                seeds &= seeds - 1;
+                float4 sum[kPer];
 #pragma unroll
-                for (int u = 0; u < kMaxPerLane; ++u) {
-                    int c = lane + 32 * u;
-                    if (c < d) {
-                        Elem<T>::store(core_k + (obase + row) * d + c, sk[u] / fc);
-                        Elem<T>::store(core_v + (obase + row) * d + c, sv[u] / fc);
+                for (int u = 0; u < kPer; ++u) sum[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                int cnt = 0;
+#pragma unroll
+                for (int k = 0; k < kWords; ++k) {
+                    if (k < ws || k >= nw) continue;
+                    unsigned mem = __ballot_sync(kFull, mine[k] == i);
+                    cnt += __popc(mem);
+                    while (mem) {   // four members at a time
+                        int j[4];
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) { j[x] = mem ? 32 * k + __ffs(mem) - 1 : -1; mem &= mem - 1; }
+#pragma unroll
+                        for (int u = 0; u < kPer; ++u) {
+                            float4 v[4];
+#pragma unroll
+                            for (int x = 0; x < 4; ++x)
+                                v[x] = j[x] >= 0 && (u * 32 + lane) * 4 < d ? load4(rows + (int64_t)j[x] * st.n + u * 128)
+                                                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) { sum[u].x += v[x].x; sum[u].y += v[x].y; sum[u].z += v[x].z; sum[u].w += v[x].w; }
+                        }
                     }
                 }
-                if (lane == 0) count[obase + row] = cnt;
+                if (row < cap) {
+                    const float fc = (float)cnt;
+#pragma unroll
+                    for (int u = 0; u < kPer; ++u) {
+                        if ((u * 32 + lane) * 4 >= d) continue;
+                        const float4 v = cnt == 1 ? load4(rows + (int64_t)i * st.n + u * 128)   // as it is
+                                                  : make_float4(sum[u].x / fc, sum[u].y / fc, sum[u].z / fc, sum[u].w / fc);
+                        store4(cores + (int64_t)row * d + u * 128, v);
+                    }
+                    if (lane == 0 && !is_v) count[obase + row] = cnt;
+                }
+                ++row;
             }
-            ++row;
         }
     }
 }
@@ -179,17 +225,22 @@ static cudaError_t run(const CompressArgs& a, cudaStream_t st) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int grid = sms * 8;
-    gsc_generic<T><<<grid, kGenWarps * 32, 0, st>>>((const T*)a.K, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off, a.n_seg,
-                                                    seg_stride, a.tau, a.tau_dev, a.skip, assign, seg_p);
-    scan_generic<<<a.B * a.Hkv, 256, 0, st>>>(a.Hkv, a.seq_seg_off, seg_stride, seg_p, seg_core_off, a.core_len,
-                                              a.cap, a.status, a.skip, a.count_only);
+    auto gsc = a.d <= 128 ? gsc_generic<T, 4> : gsc_generic<T, 8>;
+    gsc<<<grid, kGenWarps * 32, 0, st>>>((const T*)a.K, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off, a.n_seg, seg_stride, a.tau, a.tau_dev,
+                                         a.skip, assign, seg_p);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    e = launch_after_previous(scan_generic, dim3(a.B * a.Hkv), 256, st, a.Hkv, a.seq_seg_off, seg_stride, (const int32_t*)seg_p,
+                              seg_core_off, a.core_len, a.cap, a.status, a.skip, a.count_only);
+    if (e != cudaSuccess) return e;
     if (a.count_only) {   // budget search: per-head cluster counts only
         note_launches(2);
-        return cudaGetLastError();
+        return cudaSuccess;
     }
-    merge_generic<T><<<grid, kGenWarps * 32, 0, st>>>((const T*)a.K, (const T*)a.V, a.st, a.B, a.Hkv, a.n, a.d,
-                                                      a.seg_off, a.n_seg, seg_stride, assign, seg_core_off,
-                                                      (T*)a.core_k, (T*)a.core_v, a.count, a.cap);
+    e = launch_after_previous(a.d <= 128 ? merge_generic<T, 1> : merge_generic<T, 2>, dim3(grid), kGenWarps * 32, st, (const T*)a.K,
+                              (const T*)a.V, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off, a.n_seg, seg_stride, (const int32_t*)assign,
+                              (const int32_t*)seg_core_off, (T*)a.core_k, (T*)a.core_v, a.count, a.cap);
+    if (e != cudaSuccess) return e;
     note_launches(3);
     return cudaGetLastError();
 }
