@@ -1,11 +1,15 @@
 // sc_chunk: delimiter-bounded chunking (Sec. 2.2, Eq. 1) as a segmented boundary scan.
 //
 // Per sequence position p: isd[p] = token id in the delimiter set.  A non-delimiter run starts
-// at p when p == 0 or isd[p-1]; run_start(p) is the running maximum of those positions, and p
+// at p when p == 0 or isd[p-1]; run_start(p) is the last such position at or before p, and p
 // opens a segment iff isd[p] or (p - run_start(p)) % max_chunk_len == 0.  Segment offsets are
-// the compacted positions of those flags.  Four small kernels over 2048-token tiles (no
-// inter-block waiting), then one block per sequence packs consecutive segments into the
-// <= SC_TILE_ROWS-token work tiles sc_compress consumes.
+// the compacted positions of those flags.
+// Two kernels.  chunk_flags: one block per 2048 tokens; it finds the run it starts in by looking back for the last
+// delimiter before it (256 tokens at a time: nearly always one look), writes the flags as bits and counts them.
+// chunk_write_pack: one block per sequence turns flags into offsets and packs consecutive segments into the
+// <= SC_TILE_ROWS-token work tiles sc_compress consumes.  The second is launched while the first drains.
+// What bounds it: launches and dependent round trips, not bytes.  Five kernels before (carry, count, scan, write, pack, with
+// token ids read four times and the tile chain walked one tile at a time): MEASURED.
 #include "common.cuh"
 
 namespace sc {
@@ -13,7 +17,9 @@ namespace sc {
 constexpr int kChunkThreads = 256;
 constexpr int kChunkPer = 8;
 constexpr int kChunkTile = kChunkThreads * kChunkPer;  // 2048 tokens per block
-constexpr int kPackWindow = 4096;
+constexpr int kPackThreads = 1024;
+constexpr int kPackWindow = 4096;                      // segments packed at a time
+constexpr int kPackJump = 8;                           // tiles per step of the chain walk
 
 struct DelimSet {
     int32_t id[SC_MAX_DELIMS];
@@ -26,228 +32,198 @@ __device__ __forceinline__ bool in_set(int32_t tok, const DelimSet& D) {
     return hit;
 }
 
-// Block-wide inclusive scan of one int per thread (sum or max), 256 threads.
-template <bool kMax>
-__device__ __forceinline__ int block_scan(int v, int* warp_tot /*[8]*/, int* block_total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    int s = kMax ? warp_scan_max(v, lane) : warp_scan_add(v, lane);
-    if (lane == 31) warp_tot[w] = s;
+// Maximum of one int per thread over the block, 256 threads.
+__device__ __forceinline__ int block_max(int v, int* wt /*[8]*/) {
+    v = warp_max_i(v);
+    if ((threadIdx.x & 31) == 0) wt[threadIdx.x >> 5] = v;
     __syncthreads();
-    int carry = kMax ? -1 : 0, tot = kMax ? -1 : 0;
-    for (int i = 0; i < kChunkThreads / 32; ++i) {
-        int t = warp_tot[i];
-        if (i < w) carry = kMax ? max(carry, t) : carry + t;
-        tot = kMax ? max(tot, t) : tot + t;
-    }
-    __syncthreads();
-    *block_total = tot;
-    return kMax ? max(s, carry) : s + carry;
-}
-
-// Loads this thread's 8 consecutive tokens and the one before them; returns delimiter bits
-// (bit i = token i is a delimiter, bit 8 = the token before is one / sequence start marker).
-__device__ __forceinline__ void load_flags(const int32_t* ids, int n, int p0, const DelimSet& D,
-                                           unsigned& isd_bits, bool& prev_isd) {
-    isd_bits = 0;
+    int r = wt[0];
 #pragma unroll
-    for (int i = 0; i < kChunkPer; ++i) {
-        int p = p0 + i;
-        if (p < n && in_set(ids[p], D)) isd_bits |= 1u << i;
-    }
-    prev_isd = (p0 > 0 && p0 - 1 < n) ? in_set(ids[p0 - 1], D) : false;
-}
-
-// Kernel 1: last run-start position inside each tile (-1 if none).
-__global__ void __launch_bounds__(kChunkThreads)
-chunk_tile_last(const int32_t* __restrict__ token_ids, int n, int tps, DelimSet D, int32_t* __restrict__ tile_last) {
-    const int b = blockIdx.x / tps, tile = blockIdx.x % tps;
-    const int32_t* ids = token_ids + (int64_t)b * n;
-    const int p0 = tile * kChunkTile + threadIdx.x * kChunkPer;
-    unsigned isd; bool prev;
-    load_flags(ids, n, p0, D, isd, prev);
-    int last = -1;
-#pragma unroll
-    for (int i = 0; i < kChunkPer; ++i) {
-        int p = p0 + i;
-        bool pv = (i == 0) ? prev : ((isd >> (i - 1)) & 1u);
-        if (p < n && (p == 0 || pv)) last = p;
-    }
-    __shared__ int wt[kChunkThreads / 32];
-    int tot;
-    block_scan<true>(last, wt, &tot);
-    if (threadIdx.x == 0) tile_last[blockIdx.x] = tot;
-}
-
-// Segment-start flags of this thread's 8 tokens, given the run start carried into the tile.
-__device__ __forceinline__ unsigned start_flags(int n, int p0, unsigned isd, bool prev, int carry_in,
-                                                int max_len, int* wt) {
-    // thread-local inclusive max of run-start candidates, then block scan of the thread maxima
-    int cand[kChunkPer];
-    int tmax = -1;
-#pragma unroll
-    for (int i = 0; i < kChunkPer; ++i) {
-        int p = p0 + i;
-        bool pv = (i == 0) ? prev : ((isd >> (i - 1)) & 1u);
-        cand[i] = (p < n && (p == 0 || pv)) ? p : -1;
-        tmax = max(tmax, cand[i]);
-    }
-    int tot;
-    int incl = block_scan<true>(tmax, wt, &tot);
-    // exclusive value for this thread = max over earlier threads and the carry
-    int excl = __shfl_up_sync(kFull, incl, 1);
-    if ((threadIdx.x & 31) == 0) excl = -1;
-    __shared__ int warp_excl[kChunkThreads / 32];
-    if ((threadIdx.x & 31) == 31) warp_excl[threadIdx.x >> 5] = incl;
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0 && threadIdx.x > 0) excl = warp_excl[(threadIdx.x >> 5) - 1];
-    __syncthreads();
-    int run = max(excl, carry_in);
-    unsigned flags = 0;
-#pragma unroll
-    for (int i = 0; i < kChunkPer; ++i) {
-        int p = p0 + i;
-        run = max(run, cand[i]);
-        if (p < n) {
-            bool d = (isd >> i) & 1u;
-            if (d || ((p - run) % max_len) == 0) flags |= 1u << i;
-        }
-    }
-    return flags;
-}
-
-__device__ __forceinline__ int carry_into_tile(const int32_t* tile_last, int b, int tps, int tile) {
-    // run start carried in from the earlier tiles of the same sequence (tps is small: n / 2048)
-    int c = -1;
-    for (int t = threadIdx.x; t < tile; t += kChunkThreads) c = max(c, tile_last[b * tps + t]);
-    __shared__ int wt2[kChunkThreads / 32];
-    c = warp_max_i(c);
-    if ((threadIdx.x & 31) == 0) wt2[threadIdx.x >> 5] = c;
-    __syncthreads();
-    int r = -1;
-    for (int i = 0; i < kChunkThreads / 32; ++i) r = max(r, wt2[i]);
+    for (int i = 1; i < kChunkThreads / 32; ++i) r = max(r, wt[i]);
     __syncthreads();
     return r;
 }
 
-// Kernel 2: number of segment starts per tile.
+// Kernel 1: segment-start flags of 2048 tokens (a byte per thread, bit i = token i of its eight) and their number.
 __global__ void __launch_bounds__(kChunkThreads)
-chunk_tile_count(const int32_t* __restrict__ token_ids, int n, int tps, DelimSet D, int max_len,
-                 const int32_t* __restrict__ tile_last, int32_t* __restrict__ tile_cnt) {
-    const int b = blockIdx.x / tps, tile = blockIdx.x % tps;
+chunk_flags(const int32_t* __restrict__ token_ids, int n, int tps, DelimSet D, int max_len, uint8_t* __restrict__ flags,
+            int32_t* __restrict__ tile_cnt) {
+    __shared__ int wt[kChunkThreads / 32];
+    const int b = blockIdx.x / tps, tile = blockIdx.x % tps, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int32_t* ids = token_ids + (int64_t)b * n;
-    const int p0 = tile * kChunkTile + threadIdx.x * kChunkPer;
-    __shared__ int wt[kChunkThreads / 32];
-    unsigned isd; bool prev;
-    load_flags(ids, n, p0, D, isd, prev);
-    int carry = carry_into_tile(tile_last, b, tps, tile);
-    unsigned flags = start_flags(n, p0, isd, prev, carry, max_len, wt);
-    int tot;
-    block_scan<false>(__popc(flags), wt, &tot);
-    if (threadIdx.x == 0) tile_cnt[blockIdx.x] = tot;
-}
-
-// Kernel 3: one block scans the tile counts -> tile bases, n_seg, seq_seg_off.
-__global__ void __launch_bounds__(kChunkThreads)
-chunk_scan_tiles(int B, int n, int tps, const int32_t* __restrict__ tile_cnt, int32_t* __restrict__ tile_base,
-                 int32_t* __restrict__ seq_seg_off, int32_t* __restrict__ n_seg, int32_t* __restrict__ seg_off,
-                 int n_seg_cap, int32_t* status) {
-    __shared__ int wt[kChunkThreads / 32];
-    const int total_tiles = B * tps;
+    const int tile0 = tile * kChunkTile, p0 = tile0 + threadIdx.x * kChunkPer;
+    int32_t tok[kChunkPer];
+    if (p0 + kChunkPer <= n && (reinterpret_cast<uintptr_t>(ids + p0) & 15u) == 0) {
+        const int4 x = *reinterpret_cast<const int4*>(ids + p0), y = *reinterpret_cast<const int4*>(ids + p0 + 4);
+        tok[0] = x.x; tok[1] = x.y; tok[2] = x.z; tok[3] = x.w; tok[4] = y.x; tok[5] = y.y; tok[6] = y.z; tok[7] = y.w;
+    } else {
+#pragma unroll
+        for (int i = 0; i < kChunkPer; ++i) tok[i] = p0 + i < n ? ids[p0 + i] : 0;
+    }
+    const int32_t prev_tok = p0 > 0 && p0 - 1 < n ? ids[p0 - 1] : 0;
+    // start of the run that reaches into the tile: behind the last delimiter before it
     int carry = 0;
-    for (int base = 0; base < total_tiles; base += kChunkThreads) {
-        int i = base + threadIdx.x;
-        int v = (i < total_tiles) ? tile_cnt[i] : 0;
-        int tot;
-        int incl = block_scan<false>(v, wt, &tot);
-        if (i < total_tiles) {
-            int excl = carry + incl - v;
-            tile_base[i] = excl;
-            if (i % tps == 0) seq_seg_off[i / tps] = excl;
+    if (D.n > 0) {
+        for (int back = tile0 - 1; back >= 0; back -= kChunkThreads) {
+            const int p = back - (int)threadIdx.x;
+            const int found = block_max(p >= 0 && in_set(ids[p], D) ? p + 1 : 0, wt);
+            if (found > 0) { carry = found; break; }
         }
-        carry += tot;
     }
-    if (threadIdx.x == 0) {
-        seq_seg_off[B] = carry;
-        *n_seg = carry;
-        if (carry > n_seg_cap) set_status(status, SC_ERR_CAPACITY);
-        else seg_off[carry] = B * n;
-    }
-}
-
-// Kernel 4: write the compacted segment offsets.
-__global__ void __launch_bounds__(kChunkThreads)
-chunk_write(const int32_t* __restrict__ token_ids, int n, int tps, DelimSet D, int max_len,
-            const int32_t* __restrict__ tile_last, const int32_t* __restrict__ tile_base,
-            int32_t* __restrict__ seg_off, int n_seg_cap) {
-    const int b = blockIdx.x / tps, tile = blockIdx.x % tps;
-    const int32_t* ids = token_ids + (int64_t)b * n;
-    const int p0 = tile * kChunkTile + threadIdx.x * kChunkPer;
-    __shared__ int wt[kChunkThreads / 32];
-    unsigned isd; bool prev;
-    load_flags(ids, n, p0, D, isd, prev);
-    int carry = carry_into_tile(tile_last, b, tps, tile);
-    unsigned flags = start_flags(n, p0, isd, prev, carry, max_len, wt);
-    int cnt = __popc(flags), tot;
-    int incl = block_scan<false>(cnt, wt, &tot);
-    int rank = tile_base[blockIdx.x] + incl - cnt;
+    unsigned isd = 0u;
+#pragma unroll
+    for (int i = 0; i < kChunkPer; ++i)
+        if (p0 + i < n && in_set(tok[i], D)) isd |= 1u << i;
+    // run starts among this thread's tokens; the last one carries over to the threads behind it
+    unsigned starts = (isd << 1) & 0xffu;
+    if (p0 == 0 || (p0 < n && in_set(prev_tok, D))) starts |= 1u;
+    int last = starts ? p0 + 31 - __clz(starts) : -1;
+    int incl = warp_scan_max(last, lane);
+    if (lane == 31) wt[w] = incl;
+    __syncthreads();
+    int run = __shfl_up_sync(kFull, incl, 1);
+    if (lane == 0) run = -1;
+    run = max(run, carry);
+    for (int i = 0; i < w; ++i) run = max(run, wt[i]);
+    unsigned f = 0u;
 #pragma unroll
     for (int i = 0; i < kChunkPer; ++i) {
-        if ((flags >> i) & 1u) {
-            if (rank < n_seg_cap) seg_off[rank] = b * n + p0 + i;
-            ++rank;
-        }
+        const int p = p0 + i;
+        if ((starts >> i) & 1u) run = p;
+        const int off = p - run;
+        if (p < n && (((isd >> i) & 1u) || off == 0 || (off >= max_len && off % max_len == 0))) f |= 1u << i;
+    }
+    flags[(size_t)blockIdx.x * kChunkThreads + threadIdx.x] = (uint8_t)f;
+    __syncthreads();   // wt is read above
+    const int c = warp_sum_i(__popc(f));
+    if (lane == 0) wt[w] = c;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+#pragma unroll
+        for (int i = 0; i < kChunkThreads / 32; ++i) t += wt[i];
+        tile_cnt[blockIdx.x] = t;
     }
 }
 
-// Kernel 5: one block per sequence packs consecutive segments into work tiles: as many whole
-// segments as fit in SC_TILE_ROWS tokens, or one longer segment alone.  The chain tile -> next tile is
-// sequential, but where a tile that starts at segment s ends does not depend on the chain: the
-// sequence's offsets are staged through shared memory in windows, every thread finds the end of the
-// tile that would start at its segments (a binary search over the monotone offsets), and one thread then
-// walks the chain with a single shared-memory lookup per tile.
-__global__ void __launch_bounds__(kChunkThreads)
-chunk_pack_tiles(const int32_t* __restrict__ seg_off, const int32_t* __restrict__ seq_seg_off, int n_seg_cap,
-                 int32_t* __restrict__ tile_seg, int n_tile_cap, int32_t* __restrict__ seq_tile_cnt,
-                 int32_t* status) {
+// Inclusive scan of one int per thread over 1024 threads; *total = the sum.
+__device__ __forceinline__ int block_scan(int v, int* wt /*[32]*/, int* total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int s = warp_scan_add(v, lane);
+    if (lane == 31) wt[w] = s;
+    __syncthreads();
+    const int t = warp_scan_add(wt[lane], lane);   // every warp scans the 32 totals
+    *total = __shfl_sync(kFull, t, 31);
+    const int before = __shfl_sync(kFull, t, max(w - 1, 0));
+    __syncthreads();
+    return s + (w > 0 ? before : 0);
+}
+
+// Kernel 2: one block per sequence.  Offsets from the flags; then the work tiles: as many whole segments as fit in
+// SC_TILE_ROWS tokens, or one longer segment alone.  The chain tile -> next tile is sequential, but where a tile that
+// starts at segment s ends does not depend on the chain: for a window of segments in shared memory every thread finds
+// the end of the tile that would start at its segments (a binary search over the monotone offsets), the table is
+// composed with itself three times, one thread walks the chain eight tiles per lookup, and the tiles between are
+// filled in by all.
+__global__ void __launch_bounds__(kPackThreads)
+chunk_write_pack(const uint8_t* __restrict__ flags, const int32_t* __restrict__ tile_cnt, int B, int n, int tps,
+                 int32_t* __restrict__ seg_off, int n_seg_cap, int32_t* __restrict__ seq_seg_off, int32_t* __restrict__ n_seg,
+                 int32_t* __restrict__ tile_seg, int n_tile_cap, int32_t* __restrict__ seq_tile_cnt, int32_t* status) {
     __shared__ int buf[kPackWindow + 1];
-    __shared__ int nxt[kPackWindow];       // window index of the segment the next tile starts at
-    __shared__ int sh_cur, sh_nt;
-    const int b = blockIdx.x;
-    const int s0 = seq_seg_off[b];
-    const int s1 = min(seq_seg_off[b + 1], n_seg_cap);  // clamped when sc_chunk overflowed
+    __shared__ uint16_t nxt[kPackWindow + 1], ja[kPackWindow + 1], jb[kPackWindow + 1];   // next tile's segment; jumps
+    __shared__ uint16_t chain[kPackWindow / kPackJump + 2];
+    __shared__ int wt[32];
+    __shared__ int sh_cur, sh_nodes, sh_steps;
+    const int b = blockIdx.x, tid = threadIdx.x;
+    wait_for_previous();
+    // segments of the sequences before this one, and of this one
+    int before = 0, own = 0, s0, cnt_b;
+    for (int i = tid; i < b * tps; i += kPackThreads) before += tile_cnt[i];
+    for (int i = tid; i < tps; i += kPackThreads) own += tile_cnt[b * tps + i];
+    block_scan(before, wt, &s0);
+    block_scan(own, wt, &cnt_b);
+    if (tid == 0) {
+        seq_seg_off[b] = s0;
+        if (b == B - 1) {
+            const int total = s0 + cnt_b;
+            seq_seg_off[B] = total;
+            *n_seg = total;
+            if (total > n_seg_cap) set_status(status, SC_ERR_CAPACITY);
+            else seg_off[total] = B * n;
+        }
+    }
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(flags + (size_t)b * tps * kChunkThreads);
+    const int n_words = (n + 31) >> 5;
+    int done = 0;   // segments written
+    for (int w0 = 0; w0 < n_words; w0 += kPackThreads) {
+        const int wi = w0 + tid;
+        uint32_t f = wi < n_words ? words[wi] : 0u;
+        int total;
+        int rank = done + block_scan(__popc(f), wt, &total) - __popc(f);
+        while (f) {
+            const int off = b * n + wi * 32 + __ffs(f) - 1;
+            f &= f - 1;
+            if (s0 + rank < n_seg_cap) seg_off[s0 + rank] = off;
+            if (rank <= kPackWindow) buf[rank] = off;   // the first window of the packing
+            ++rank;
+        }
+        done += total;
+    }
+    __syncthreads();
+    const int s1 = min(s0 + cnt_b, n_seg_cap);   // clamped when the offsets overflowed
     int32_t* out = tile_seg + (int64_t)b * (n_tile_cap + 1);
     int cur = s0, nt = 0;
     while (cur < s1) {
-        const int ws = cur;
-        const int cnt = min(kPackWindow, s1 - ws);
-        for (int i = threadIdx.x; i <= cnt; i += kChunkThreads) buf[i] = seg_off[ws + i];
+        const int ws = cur, cnt = min(kPackWindow, s1 - ws);
+        const bool last_window = ws + cnt == s1;
+        if (ws != s0) for (int i = tid; i < cnt; i += kPackThreads) buf[i] = seg_off[ws + i];
+        if (tid == 0 && (ws != s0 || ws + cnt == s0 + cnt_b)) buf[cnt] = last_window ? (b + 1) * n : seg_off[ws + cnt];
         __syncthreads();
-        for (int i = threadIdx.x; i < cnt; i += kChunkThreads) {
-            // largest e in (i, cnt] with buf[e] - buf[i] <= SC_TILE_ROWS, or i + 1 for a segment longer than a tile
-            const int limit = buf[i] + SC_TILE_ROWS;
-            int lo = i + 1, hi = min(cnt, i + SC_TILE_ROWS);   // a segment holds at least one token
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (buf[mid] <= limit) lo = mid; else hi = mid - 1;
+        // a tile's end is known for sure only if SC_TILE_ROWS + 1 offsets behind its start are in the window
+        const int lim = last_window ? cnt : cnt - SC_TILE_ROWS;
+        for (int i = tid; i <= cnt; i += kPackThreads) {
+            int lo = i;   // not known (or the end): the chain stops here
+            if (i < lim) {
+                // largest e in (i, cnt] with buf[e] - buf[i] <= SC_TILE_ROWS, or i + 1 for a segment longer than a tile
+                const int limit = buf[i] + SC_TILE_ROWS;
+                int hi = min(cnt, i + SC_TILE_ROWS);   // a segment holds at least one token
+                lo = i + 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi + 1) >> 1;
+                    if (buf[mid] <= limit) lo = mid; else hi = mid - 1;
+                }
             }
-            nxt[i] = lo;
+            nxt[i] = (uint16_t)lo;
         }
         __syncthreads();
-        if (threadIdx.x == 0) {
-            // a tile's end is known for sure only if SC_TILE_ROWS + 1 offsets behind its start are in the window
-            const bool last_window = (ws + cnt == s1);
-            while (cur < s1 && (last_window || cur - ws + SC_TILE_ROWS + 1 <= cnt)) {
-                if (nt < n_tile_cap) out[nt] = cur;
-                ++nt;
-                cur = ws + nxt[cur - ws];
-            }
-            sh_cur = cur; sh_nt = nt;
+        for (int i = tid; i <= cnt; i += kPackThreads) ja[i] = nxt[nxt[i]];
+        __syncthreads();
+        for (int i = tid; i <= cnt; i += kPackThreads) jb[i] = ja[ja[i]];
+        __syncthreads();
+        for (int i = tid; i <= cnt; i += kPackThreads) ja[i] = jb[jb[i]];
+        __syncthreads();
+        if (tid == 0) {
+            int x = 0, k = 0;
+            while (x < lim) { chain[k++] = (uint16_t)x; x = ja[x]; }
+            sh_cur = ws + x; sh_nodes = k;
         }
         __syncthreads();
-        cur = sh_cur; nt = sh_nt;
+        const int nodes = sh_nodes;
+        int steps = 0;
+        for (int k = tid; k < nodes; k += kPackThreads) {   // (at most one node per thread: a step passes kPackJump segments)
+            int x = chain[k];
+            for (steps = 0; steps < kPackJump && x < lim; ++steps) {
+                const int t = nt + k * kPackJump + steps;
+                if (t < n_tile_cap) out[t] = ws + x;
+                x = nxt[x];
+            }
+            if (k == nodes - 1) sh_steps = steps;
+        }
+        cur = sh_cur;
         __syncthreads();
+        nt += (nodes - 1) * kPackJump + sh_steps;
     }
-    if (threadIdx.x == 0) {
+    if (tid == 0) {
         out[min(nt, n_tile_cap)] = s1;
         seq_tile_cnt[b] = nt;
         if (nt > n_tile_cap) set_status(status, SC_ERR_CAPACITY);
@@ -255,29 +231,24 @@ chunk_pack_tiles(const int32_t* __restrict__ seg_off, const int32_t* __restrict_
 }
 
 size_t chunk_ws_bytes(int32_t B, int32_t n) {
-    int tps = div_up(n, kChunkTile);
-    return sizeof(int32_t) * 3 * (size_t)B * tps + 64;
+    const size_t tiles = (size_t)B * div_up(n, kChunkTile);
+    return tiles * (kChunkThreads + sizeof(int32_t)) + 64;
 }
 
 cudaError_t launch_chunk(const ChunkArgs& a, cudaStream_t st) {
     const int tps = div_up(a.n, kChunkTile);
     const int tiles = a.B * tps;
-    int32_t* tile_last = a.ws;
-    int32_t* tile_cnt = a.ws + tiles;
-    int32_t* tile_base = a.ws + 2 * tiles;
+    int32_t* tile_cnt = a.ws;
+    uint8_t* flags = reinterpret_cast<uint8_t*>(a.ws + (tiles + 15) / 16 * 16);   // (64 spare bytes cover the padding)
     DelimSet D;
     D.n = a.n_delim;
     for (int i = 0; i < SC_MAX_DELIMS; ++i) D.id[i] = (i < a.n_delim) ? a.delim[i] : 0;
-    chunk_tile_last<<<tiles, kChunkThreads, 0, st>>>(a.token_ids, a.n, tps, D, tile_last);
-    chunk_tile_count<<<tiles, kChunkThreads, 0, st>>>(a.token_ids, a.n, tps, D, a.max_chunk_len, tile_last, tile_cnt);
-    chunk_scan_tiles<<<1, kChunkThreads, 0, st>>>(a.B, a.n, tps, tile_cnt, tile_base, a.seq_seg_off, a.n_seg,
-                                                  a.seg_off, a.n_seg_cap, a.status);
-    chunk_write<<<tiles, kChunkThreads, 0, st>>>(a.token_ids, a.n, tps, D, a.max_chunk_len, tile_last, tile_base,
-                                                 a.seg_off, a.n_seg_cap);
-    chunk_pack_tiles<<<a.B, kChunkThreads, 0, st>>>(a.seg_off, a.seq_seg_off, a.n_seg_cap, a.tile_seg,
-                                                    a.n_tile_cap, a.seq_tile_cnt, a.status);
-    note_launches(5);
-    return cudaGetLastError();
+    chunk_flags<<<tiles, kChunkThreads, 0, st>>>(a.token_ids, a.n, tps, D, a.max_chunk_len, flags, tile_cnt);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    note_launches(2);
+    return launch_after_previous(chunk_write_pack, dim3(a.B), kPackThreads, st, (const uint8_t*)flags, (const int32_t*)tile_cnt, a.B, a.n, tps,
+                                 a.seg_off, a.n_seg_cap, a.seq_seg_off, a.n_seg, a.tile_seg, a.n_tile_cap, a.seq_tile_cnt, a.status);
 }
 
 }  // namespace sc
