@@ -117,20 +117,45 @@ def lib() -> ctypes.CDLL:
     return _lib
 
 
+_native_module = None
+
+
+def _native():
+    """The CPython entry to the library for the calls made per layer or per token (csrc/native_calls.c)."""
+    global _native_module
+    if _native_module is None:
+        lib()   # raises if nothing was built
+        try:
+            from . import _native_calls
+        except ImportError as e:
+            raise RuntimeError(f"_native_calls.so is missing or does not load ({e}): run "
+                               "`python -m paper_2603_14303_b200.build`") from e
+        _native_module = _native_calls
+    return _native_module
+
+
 def _ptr(t):
     return None if t is None else t.data_ptr()
 
 
+# The raw stream handle, without building a torch.cuda.Stream object per call (0.1 us against 2).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(t: torch.Tensor):
+    if _raw_stream is not None:
+        return _raw_stream(t.get_device())
     return torch.cuda.current_stream(t.device).cuda_stream
 
 
+_DTYPES = {torch.bfloat16: SC_BF16, torch.float32: SC_F32}
+
+
 def _dt(t: torch.Tensor) -> int:
-    if t.dtype == torch.bfloat16:
-        return SC_BF16
-    if t.dtype == torch.float32:
-        return SC_F32
-    raise TypeError(f"unsupported dtype {t.dtype}")
+    dt = _DTYPES.get(t.dtype)
+    if dt is None:
+        raise TypeError(f"unsupported dtype {t.dtype}")
+    return dt
 
 
 def _check(where: str, code: int):
@@ -142,6 +167,10 @@ def _need_cuda(*ts):
     for t in ts:
         if t is not None and not t.is_cuda:
             raise ValueError("device tensors required")
+
+
+def _bytes(t: torch.Tensor) -> int:
+    return t.numel() * t.element_size()
 
 
 def launch_counter() -> int:
@@ -164,12 +193,10 @@ def sc_chunk(token_ids, delim_ids, max_chunk_len, seg_off, seq_seg_off, n_seg, t
     _need_cuda(token_ids, seg_off, seq_seg_off, n_seg, tile_seg, seq_tile_cnt, workspace)
     B, n = token_ids.shape
     assert token_ids.dtype == torch.int32 and token_ids.is_contiguous()
-    dl = (_i32 * max(len(delim_ids), 1))(*[int(x) for x in delim_ids])
     n_tile_cap = tile_seg.shape[1] - 1 if tile_seg.dim() == 2 else tile_seg.numel() // max(B, 1) - 1
-    code = lib().sc_chunk(_ptr(token_ids), B, n, dl, len(delim_ids), max_chunk_len, _ptr(seg_off),
-                          seg_off.numel() - 1, _ptr(seq_seg_off), _ptr(n_seg), _ptr(tile_seg), n_tile_cap,
-                          _ptr(seq_tile_cnt), _ptr(workspace), workspace.numel() * workspace.element_size(),
-                          _ptr(status), _stream(seg_off))
+    code = _native().chunk(token_ids.data_ptr(), B, n, delim_ids, max_chunk_len, seg_off.data_ptr(), seg_off.numel() - 1,
+                           seq_seg_off.data_ptr(), n_seg.data_ptr(), tile_seg.data_ptr(), n_tile_cap, seq_tile_cnt.data_ptr(),
+                           workspace.data_ptr(), _bytes(workspace), _ptr(status), _stream(seg_off))
     _check("sc_chunk", code)
 
 
@@ -180,14 +207,12 @@ def sc_compress(K, V, plan: "ChunkPlan", tau, core_k, core_v, count, core_len, a
     B, Hkv, n, d = K.shape
     assert V.shape == K.shape and V.stride() == K.stride() and V.dtype == K.dtype and K.stride(3) == 1
     assert core_k.is_contiguous() and core_v.is_contiguous() and count.is_contiguous()
-    cap = core_k.shape[2]
-    prm = _GscParams(float(tau), int(plan.max_chunk_len), int(flags))
-    st = _Strides(K.stride(0), K.stride(1), K.stride(2))
-    code = lib().sc_compress(_ptr(K), _ptr(V), st, _dt(K), B, Hkv, n, d, _ptr(plan.seg_off), _ptr(plan.seq_seg_off),
-                             _ptr(plan.n_seg), _ptr(plan.tile_seg), _ptr(plan.seq_tile_cnt), plan.n_tile_cap,
-                             ctypes.byref(prm), _ptr(core_k), _ptr(core_v), _ptr(count), cap, _ptr(core_len),
-                             _ptr(assign), _ptr(workspace), workspace.numel() * workspace.element_size(),
-                             _ptr(status), _stream(K))
+    sb, sh, sn, _ = K.stride()
+    code = _native().compress(K.data_ptr(), V.data_ptr(), sb, sh, sn, _dt(K), B, Hkv, n, d, plan.seg_off.data_ptr(),
+                              plan.seq_seg_off.data_ptr(), plan.n_seg.data_ptr(), plan.tile_seg.data_ptr(),
+                              plan.seq_tile_cnt.data_ptr(), plan.n_tile_cap, float(tau), int(plan.max_chunk_len), int(flags),
+                              core_k.data_ptr(), core_v.data_ptr(), count.data_ptr(), core_k.shape[2], core_len.data_ptr(),
+                              _ptr(assign), workspace.data_ptr(), _bytes(workspace), (_ptr(status), _stream(K)))
     _check("sc_compress", code)
 
 
@@ -203,18 +228,22 @@ def sc_compress_layers(Ks, Vs, plan: "ChunkPlan", tau, outs, workspace, status=N
     K0 = Ks[0]
     B, Hkv, n, d = K0.shape
     cap = outs[0].core_k.shape[2]
-    rows = (_CompressLayer * L)()
-    for l in range(L):
-        K, V, o = Ks[l], Vs[l], outs[l]
-        _need_cuda(K, V, o.core_k, o.core_v, o.count, o.core_len, o.assign)
-        assert K.shape == K0.shape and V.shape == K0.shape and K.stride() == K0.stride() and V.stride() == K0.stride()
-        assert K.dtype == K0.dtype and V.dtype == K0.dtype and K.stride(3) == 1 and o.core_k.shape[2] == cap
-        assert o.core_k.is_contiguous() and o.core_v.is_contiguous() and o.count.is_contiguous()
-        rows[l] = _CompressLayer(_ptr(K), _ptr(V), _ptr(o.core_k), _ptr(o.core_v), _ptr(o.count), _ptr(o.core_len),
-                                 _ptr(o.assign))
+    shape, strides, dtype = K0.shape, K0.stride(), K0.dtype
+    assert strides[3] == 1
+    rows = (ctypes.c_uint64 * (7 * L))()   # L rows of seven pointers, as sc_compress_layer lays them out
+    at = 0
+    for K, V, o in zip(Ks, Vs, outs):
+        ck, cv, assign = o.core_k, o.core_v, o.assign
+        _need_cuda(K, V, ck, cv, o.count, o.core_len, assign)
+        assert K.shape == shape and V.shape == shape and K.stride() == strides and V.stride() == strides
+        assert K.dtype == dtype and V.dtype == dtype and ck.shape[2] == cap
+        assert ck.is_contiguous() and cv.is_contiguous() and o.count.is_contiguous()
+        rows[at:at + 7] = (K.data_ptr(), V.data_ptr(), ck.data_ptr(), cv.data_ptr(), o.count.data_ptr(), o.core_len.data_ptr(),
+                           0 if assign is None else assign.data_ptr())
+        at += 7
     prm = _GscParams(float(tau), int(plan.max_chunk_len), int(flags))
     st = _Strides(K0.stride(0), K0.stride(1), K0.stride(2))
-    code = lib().sc_compress_layers(rows, L, st, _dt(K0), B, Hkv, n, d, _ptr(plan.seg_off), _ptr(plan.seq_seg_off),
+    code = lib().sc_compress_layers(ctypes.cast(rows, ctypes.POINTER(_CompressLayer)), L, st, _dt(K0), B, Hkv, n, d, _ptr(plan.seg_off), _ptr(plan.seq_seg_off),
                                     _ptr(plan.n_seg), _ptr(plan.tile_seg), _ptr(plan.seq_tile_cnt), plan.n_tile_cap,
                                     ctypes.byref(prm), cap, _ptr(workspace),
                                     workspace.numel() * workspace.element_size(), _ptr(status), _stream(K0))
@@ -263,9 +292,9 @@ def sc_decode_attn(q, core_k, core_v, count, core_len, out, workspace, scale=0.0
     B, Hq, d = q.shape
     _, Hkv, cap, _ = core_k.shape
     assert q.is_contiguous() and out.is_contiguous() and core_k.is_contiguous() and core_v.is_contiguous()
-    code = lib().sc_decode_attn(_ptr(q), _dt(q), B, Hq, Hkv, d, _ptr(core_k), _ptr(core_v), _ptr(count), cap,
-                                _ptr(core_len), float(scale), int(flags), _ptr(out), _ptr(workspace),
-                                workspace.numel() * workspace.element_size(), _ptr(status), _stream(q))
+    code = _native().decode_attn(q.data_ptr(), _dt(q), B, Hq, Hkv, d, core_k.data_ptr(), core_v.data_ptr(), _ptr(count), cap,
+                                 core_len.data_ptr(), float(scale), int(flags), out.data_ptr(), workspace.data_ptr(),
+                                 _bytes(workspace), _ptr(status), _stream(q))
     _check("sc_decode_attn", code)
 
 
@@ -276,8 +305,8 @@ def sc_prefill_attn(q, core_k, core_v, count, core_len, out, scale=0.0, status=N
     _, Hkv, cap, _ = core_k.shape
     assert q.is_contiguous() and out.is_contiguous() and core_k.is_contiguous() and core_v.is_contiguous()
     assert out.shape == q.shape and out.dtype == q.dtype
-    code = lib().sc_prefill_attn(_ptr(q), _dt(q), B, Hq, Hkv, m, d, _ptr(core_k), _ptr(core_v), _ptr(count), cap,
-                                 _ptr(core_len), float(scale), int(flags), _ptr(out), _ptr(status), _stream(q))
+    code = _native().prefill_attn(q.data_ptr(), _dt(q), B, Hq, Hkv, m, d, core_k.data_ptr(), core_v.data_ptr(), _ptr(count), cap,
+                                  core_len.data_ptr(), float(scale), int(flags), out.data_ptr(), _ptr(status), _stream(q))
     _check("sc_prefill_attn", code)
 
 
@@ -306,10 +335,9 @@ def sc_append(k_new, v_new, token_ids, delim_ids, max_chunk_len, tau, core_k, co
     cap = core_k.shape[2]
     assert k_new.is_contiguous() and v_new.is_contiguous() and core_k.is_contiguous() and core_v.is_contiguous()
     assert core_k.shape == (B, Hkv, cap, d) and token_ids.dtype == torch.int32 and token_ids.numel() == B
-    delims = (_i32 * max(len(delim_ids), 1))(*[int(x) for x in delim_ids])
-    code = lib().sc_append(_ptr(k_new), _ptr(v_new), _dt(k_new), B, Hkv, d, _ptr(token_ids), delims, len(delim_ids),
-                           int(max_chunk_len), float(tau), _ptr(core_k), _ptr(core_v), _ptr(count), cap,
-                           _ptr(core_len), _ptr(tail_len), _ptr(attn_len), _ptr(status), _stream(k_new))
+    code = _native().append(k_new.data_ptr(), v_new.data_ptr(), _dt(k_new), B, Hkv, d, token_ids.data_ptr(), delim_ids,
+                            int(max_chunk_len), float(tau), core_k.data_ptr(), core_v.data_ptr(), count.data_ptr(), cap,
+                            core_len.data_ptr(), tail_len.data_ptr(), attn_len.data_ptr(), _ptr(status), _stream(k_new))
     _check("sc_append", code)
 
 
@@ -328,10 +356,8 @@ def sc_append_layers(table, k_new0, token_ids, delim_ids, max_chunk_len, tau, ca
     _need_cuda(table, k_new0, token_ids, status)
     B, Hkv, d = k_new0.shape
     assert table.dtype == torch.int64 and table.dim() == 2 and table.shape[1] == 8 and table.is_contiguous()
-    delims = (_i32 * max(len(delim_ids), 1))(*[int(x) for x in delim_ids])
-    code = lib().sc_append_layers(_ptr(table), table.shape[0], _dt(k_new0), B, Hkv, d, _ptr(token_ids), delims,
-                                  len(delim_ids), int(max_chunk_len), float(tau), int(cap), _ptr(status),
-                                  _stream(k_new0))
+    code = _native().append_layers(table.data_ptr(), table.shape[0], _dt(k_new0), B, Hkv, d, token_ids.data_ptr(), delim_ids,
+                                   int(max_chunk_len), float(tau), int(cap), _ptr(status), _stream(k_new0))
     _check("sc_append_layers", code)
 
 
@@ -372,14 +398,14 @@ def check_status(status: torch.Tensor, where: str = "device status"):
 
 def chunk(token_ids: torch.Tensor, delim_ids, max_chunk_len: int = SC_MAX_CHUNK_LEN) -> ChunkPlan:
     """Allocate worst-case outputs and run sc_chunk.  Does not synchronise."""
-    dev = token_ids.device
     B, n = token_ids.shape
-    n_seg_cap, n_tile_cap = chunk_bounds(B, n)
-    i32 = dict(dtype=torch.int32, device=dev)
-    plan = ChunkPlan(B, n, max_chunk_len, torch.empty(n_seg_cap + 1, **i32), torch.empty(B + 1, **i32),
-                     torch.empty(1, **i32), torch.empty((B, n_tile_cap + 1), **i32), torch.empty(max(B, 1), **i32),
-                     n_tile_cap, torch.zeros(1, **i32))
-    ws = torch.empty(lib().sc_chunk_workspace_bytes(B, n), dtype=torch.uint8, device=dev)
+    code, n_seg_cap, n_tile_cap, ws_bytes = _native().chunk_sizes(B, n)
+    _check("sc_chunk_bounds", code)
+    new = token_ids.new_empty   # int32 on the same device, as the raw call asks
+    i32 = torch.int32
+    plan = ChunkPlan(B, n, max_chunk_len, new(n_seg_cap + 1, dtype=i32), new(B + 1, dtype=i32), new(1, dtype=i32),
+                     new((B, n_tile_cap + 1), dtype=i32), new(max(B, 1), dtype=i32), n_tile_cap, token_ids.new_zeros(1, dtype=i32))
+    ws = new(ws_bytes, dtype=torch.uint8)
     sc_chunk(token_ids, delim_ids, max_chunk_len, plan.seg_off, plan.seq_seg_off, plan.n_seg, plan.tile_seg,
              plan.seq_tile_cnt, ws, plan.status)
     return plan
