@@ -17,7 +17,7 @@
 //      of cliques take two.  A member joins the earliest seed among its earlier neighbours.  The tile's cluster count is
 //      published at once; every token's cluster number (rank of its seed) goes to shared memory.
 //   3. Eq. 3: the members' sum of a cluster is a row of M V, M the 0/1 matrix clusters x tokens; M's fragments are made
-//      from the cluster numbers, K and V come transposed from their staged rows (ldmatrix.trans), mma.m16n8k16 adds up in
+//      from the cluster numbers (kept as bf16: comparing two of them gives the 1.0 or 0.0 the product wants), K and V come transposed from their staged rows (ldmatrix.trans), mma.m16n8k16 adds up in
 //      fp32 (products with 1 and 0 are exact).  Sixteen clusters at a time, over the tokens from their first seed to the
 //      end of their last segment only; each warp takes a quarter of the columns.  Sums are scaled by 1/|S|, rounded once
 //      and stored.  Clusters of one token are copied bit for bit; a sum that is not finite (0 * inf would reach other
@@ -31,7 +31,10 @@
 // the product, 1245 us / 475 us (single-token chains of shared loads are longer than the products); keys and values
 // released and pooled separately so that the next keys load earlier, +13 %; L2 prefetch of the next tile, +5 %; only
 // clusters of more than one token in the product, +5 %; a second service warp (96 registers a thread), worse throughout.
-// Long tiles by mma.sync blocks instead of tcgen05: 16 x 16K +8 %.
+// Long tiles by mma.sync blocks instead of tcgen05: 16 x 16K +8 %.  Masks, segment bounds and seeds without branches per lane,
+// and the code for negative thresholds in instances of its own: 16 x 16K 633 -> 612 us, chunks of 128 tokens 738 -> 589 us (a
+// settled long tile 19 K -> 12 K cycles); one step out of line or not moves a workload by up to 5 % either way.
+// mbarrier waits with a suspend-time hint, tickets staggered between heads: no change.
 //
 // Offsets: a prefix sum over the tiles of each head by decoupled look-back over per-tile status words; tickets are handed
 // out in order, so every predecessor is held by a running block and the bounded wait cannot starve.  A block draws its
@@ -67,8 +70,8 @@ constexpr int kBitOff = 2 * kHalfLong;            // uint32[256][8]: earlier-nei
 constexpr int kNormOff = kBitOff;                 // float[128]: norms of a short tile's rows (no bits are stored for it)
 constexpr int kLongNormOff = kBitOff + kMaxRows * 32;        // float[256]
 // behind the norms, once the bits are in registers:
-constexpr int kRankOff = kBitOff + 1024;                     // uint8[256]: cluster of each token, see rank_slot
-constexpr int kCntOff = kRankOff + kMaxRows;                 // int32[256]: tokens of each cluster
+constexpr int kRankOff = kBitOff + 1024;                     // bf16[256]: cluster of each token (whole numbers to 256 are exact), see rank_slot
+constexpr int kCntOff = kRankOff + kMaxRows * 2;                 // int32[256]: tokens of each cluster
 constexpr int kSeedOff = kCntOff + kMaxRows * 4;             // uint8[256]: the cluster's seed
 constexpr int kEndOff = kSeedOff + kMaxRows;                 // uint16[256]: end of the seed's segment
 constexpr int kMiscOff = kLongNormOff + kMaxRows * 4;        // seeds[8], members[8]; starts[2][4]; geo[2][8]; base, P, tmem slot, flags
@@ -107,10 +110,11 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ uint32_t bits_between(int lo, int hi, int word) {   // bits [lo, hi) that fall in `word`
-    lo = max(lo, word * 32); hi = min(hi, word * 32 + 32);
-    if (hi <= lo) return 0u;
-    return (0xffffffffu >> (32 - (hi - lo))) << (lo - word * 32);
+// Bits of word `word` at or above position `lo` (any position of the tile); no branch.
+__device__ __forceinline__ uint32_t bits_from(int lo, int word) {
+    uint32_t m;
+    asm("shl.b32 %0, %1, %2;\n" : "=r"(m) : "r"(0xffffffffu), "r"(max(lo - word * 32, 0)));   // (shl gives 0 for 32 and more)
+    return m;
 }
 __device__ __forceinline__ uint32_t ld_volatile(const uint32_t* p) {
     uint32_t v;
@@ -177,7 +181,7 @@ __device__ __forceinline__ uint32_t sim_word_neg(const uint32_t (&g)[32], const 
 // the pooling needs: every token's cluster, and every cluster's size, seed and end of segment.  `end`: end of the rows'
 // segments.  Returns the number of clusters.  All compute threads call it.
 __device__ __forceinline__ int rank_slot(int i) {   // where a token's cluster number is kept: the four a lane needs for one mma
-    return (i & ~15) | ((i & 6) << 1) | ((i & 8) >> 2) | (i & 1);   // fragment (2t, 2t+1, 2t+8, 2t+9 of sixteen) form one word
+    return (i & ~15) | ((i & 6) << 1) | ((i & 8) >> 2) | (i & 1);   // fragment (2t, 2t+1, 2t+8, 2t+9 of sixteen) are together
 }
 template <int NR>
 __device__ __forceinline__ int settle_rows(const uint32_t (&e)[NR][4 * NR], const bool (&act)[NR], const int (&end)[NR], unsigned char* smem,
@@ -244,21 +248,17 @@ __device__ __forceinline__ int settle_rows(const uint32_t (&e)[NR][4 * NR], cons
     for (int r = 0; r < NR; ++r) {
         // a member joins the earliest seed among its earlier neighbours; a cluster's number is the rank of its seed
         const int i = (warp + 4 * r) * 32 + lane;
-        int s = i, before = 0, rank = 0;
-        bool found = false;
+        uint32_t m = 0u, in = 0u;   // the word that holds the seed: candidates, all seeds of the word
+        int at = 0, before = 0, upto = 0;
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
-            const uint32_t own = is_seed[r] && w == warp + 4 * r ? 1u << lane : 0u;
-            const uint32_t m = is_seed[r] ? own : e[r][w] & sd[w];
-            if (!found && m != 0u) {
-                const int bit = __ffs(m) - 1;
-                s = w * 32 + bit;
-                rank = before + __popc(sd[w] & ((1u << bit) - 1u));
-                found = true;
-            }
+            const uint32_t mw = is_seed[r] ? (w == warp + 4 * r ? 1u << lane : 0u) : e[r][w] & sd[w];
+            const bool take = m == 0u && mw != 0u;
+            m = take ? mw : m; in = take ? sd[w] : in; at = take ? w * 32 : at; upto = take ? before : upto;
             before += __popc(sd[w]);
         }
-        (smem + kRankOff)[rank_slot(i)] = act[r] ? (uint8_t)rank : (uint8_t)255;   // past the tile's end: no cluster
+        const int bit = __ffs(m) - 1, s = at + bit, rank = upto + __popc(in & ((1u << (bit & 31)) - 1u));
+        reinterpret_cast<__nv_bfloat16*>(smem + kRankOff)[rank_slot(i)] = __int2bfloat16_rn(act[r] ? rank : -1);   // -1: past the tile's end, no cluster
         if (act[r]) {
             atomicAdd(&cnt[rank], 1);
             if (is_seed[r]) {
@@ -288,22 +288,28 @@ __device__ __forceinline__ float diagonal(const uint32_t (&g)[32], int lane) {
 
 // Steps 1 and 2 for a tile of up to 128 rows, thread i = row i (the product of its keys is complete).  `starts`: bit words of the
 // rows that start a segment.
-__device__ __forceinline__ int settle_short_tile(unsigned char* smem, const uint32_t* starts, int R, uint32_t tmem, uint32_t phase_u, float tau,
-                                                 bool wait_failed, bool& failed, int32_t* as, int row0, uint32_t* publish, int* sh_p) {
+template <bool kAnyTau>
+__device__ __noinline__ int settle_short_tile(unsigned char* smem, const uint32_t* starts, int R, uint32_t tmem, uint32_t phase_u, float tau,
+                                                 bool wait_failed, int32_t* as, int row0, uint32_t* publish, int* sh_p) {
     float* norm = reinterpret_cast<float*>(smem + kNormOff);
     const int i = threadIdx.x, lane = i & 31, q = i >> 5;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
     // the segment [beg, end) of the row: the nearest start at or before it, and the next one
-    int beg = 0, end = R;
+    int beg, end;
     {
-        uint32_t m = starts[q] & (0xffffffffu >> (31 - lane));
-        int w = q;
-        while (m == 0u && w > 0) m = starts[--w];
-        if (m) beg = w * 32 + 31 - __clz(m);
-        m = lane == 31 ? 0u : starts[q] & (0xfffffffeu << lane);
-        w = q;
-        while (m == 0u && w < 3) m = starts[++w];
-        if (m) end = min(w * 32 + __ffs(m) - 1, R);
+        const uint4 sv = *reinterpret_cast<const uint4*>(starts);
+        const uint32_t st[4] = {sv.x, sv.y, sv.z, sv.w};
+        int last = 0, next = R;       // outside the warp's word
+        uint32_t own = 0u;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) {
+            if (w == q) own = st[w];
+            if (w < q && st[w] != 0u) last = w * 32 + 31 - __clz(st[w]);
+            if (3 - w > q && st[3 - w] != 0u) next = (3 - w) * 32 + __ffs(st[3 - w]) - 1;
+        }
+        const uint32_t upto = own & (0xffffffffu >> (31 - lane)), later = own & ~(0xffffffffu >> (31 - lane));
+        beg = upto ? q * 32 + 31 - __clz(upto) : last;
+        end = min(later ? q * 32 + __ffs(later) - 1 : next, R);
     }
     wait_failed = wait_failed || !umma::mbar_wait(smem_u32(smem) + kBarOff + 16, phase_u);
     __syncwarp();
@@ -313,7 +319,7 @@ __device__ __forceinline__ int settle_short_tile(unsigned char* smem, const uint
     umma::tmem_ld_wait();
     norm[i] = sqrtf(diagonal(g, lane));
     const bool act[1] = {i < R};
-    if (team_any(wait_failed)) { failed = true; return 0; }   // (the norms are in place)
+    if (team_any(wait_failed)) return -1;   // (the norms are in place)
     const float tni = tau * norm[i];
     const int w_lo = __reduce_min_sync(kFull, beg >> 5);   // first word any of the warp's rows needs
     uint32_t e[1][4];
@@ -325,8 +331,9 @@ __device__ __forceinline__ int settle_short_tile(unsigned char* smem, const uint
                 umma::tmem_ld32(lane_addr + c * 32, g);
                 umma::tmem_ld_wait();
             }
-            w = tau < 0.f ? sim_word_neg(g, norm + c * 32, tni) : sim_word(g, norm + c * 32, tni);
-            w &= bits_between(beg, i, c);
+            w = kAnyTau && tau < 0.f ? sim_word_neg(g, norm + c * 32, tni) : sim_word(g, norm + c * 32, tni);
+            w &= bits_from(beg, c);
+            if (c == q) w &= (1u << lane) - 1u;   // earlier rows only
         }
         e[0][c] = w;
     }
@@ -337,8 +344,9 @@ __device__ __forceinline__ int settle_short_tile(unsigned char* smem, const uint
 
 // Steps 1 and 2 for a tile of more than 128 rows (one segment): three products, the two diagonal ones first (they give the
 // norms), each read before the next overwrites it; thread tid settles rows tid and tid + 128.
+template <bool kAnyTau>
 __device__ __noinline__ int settle_long_tile(unsigned char* smem, int R, uint32_t tmem, uint32_t phase_u, float tau, bool wait_failed,
-                                             bool* failed, int32_t* as, int row0, uint32_t* publish, int* sh_p) {
+                                             int32_t* as, int row0, uint32_t* publish, int* sh_p) {
     float* norm = reinterpret_cast<float*>(smem + kLongNormOff);
     const uint32_t sbase = smem_u32(smem), bar_u = sbase + kBarOff + 16;
     const int tid = threadIdx.x, lane = tid & 31, q = tid >> 5;
@@ -349,7 +357,7 @@ __device__ __noinline__ int settle_long_tile(unsigned char* smem, int R, uint32_
 #pragma unroll
     for (int ps = 0; ps < 3; ++ps) {   // blocks (0, 0); (1, 1); (1, 0)
         const int mb = ps == 0 ? 0 : 1, nb = ps == 1 ? 1 : 0, i = mb * 128 + tid;
-        if (team_any(wait_failed)) { *failed = true; return 0; }   // (the product before has been read)
+        if (team_any(wait_failed)) return -1;   // (the product before has been read)
         if (tid == 0) {
             umma::fence_after_sync();
             umma_gram_block(sbase, kHalfLong, mb, nb, tmem, bar_u);
@@ -363,7 +371,7 @@ __device__ __noinline__ int settle_long_tile(unsigned char* smem, int R, uint32_
             umma::tmem_ld32(lane_addr + q * 32, g);
             umma::tmem_ld_wait();
             norm[i] = sqrtf(diagonal(g, lane));
-            if (team_any(wait_failed)) { *failed = true; return 0; }   // (the norms are in place)
+            if (team_any(wait_failed)) return -1;   // (the norms are in place)
         }
         const float tni = tau * norm[i];
 #pragma unroll
@@ -374,12 +382,12 @@ __device__ __noinline__ int settle_long_tile(unsigned char* smem, int R, uint32_
                 umma::tmem_ld_wait();
             }
             const float* nc = norm + nb * 128 + c * 32;
-            const uint32_t w = tau < 0.f ? sim_word_neg(g, nc, tni) : sim_word(g, nc, tni);
-            e[mb][nb * 4 + c] = i < R ? w & bits_between(0, i, nb * 4 + c) : 0u;
+            const uint32_t w = kAnyTau && tau < 0.f ? sim_word_neg(g, nc, tni) : sim_word(g, nc, tni);
+            e[mb][nb * 4 + c] = i >= R ? 0u : (mb == nb && c == q) ? w & ((1u << lane) - 1u) : w;   // earlier rows only
         }
         umma::fence_before_sync();
     }
-    if (team_any(wait_failed)) { *failed = true; return 0; }
+    if (team_any(wait_failed)) return -1;
     const bool act[2] = {true, tid + 128 < R};
     const int ends[2] = {R, R};
     return settle_rows<2>(e, act, ends, smem, q, lane, as, row0, publish, sh_p);
@@ -394,10 +402,16 @@ __device__ __noinline__ void pool_by_members(const unsigned char* tensor, int hs
         if (cnt[c] <= 1 || c >= room) continue;
         float sum = 0.f;
         for (int i = t_lo; i < t_hi; ++i)
-            if ((smem + kRankOff)[rank_slot(i)] == c)
+            if ((int)__bfloat162float(reinterpret_cast<const __nv_bfloat16*>(smem + kRankOff)[rank_slot(i)]) == c)
                 sum += __bfloat162float(*reinterpret_cast<const __nv_bfloat16*>(tensor + (col >> 6) * hs + tile_addr(i, (col & 63) >> 3) + (col & 7) * 2));
         dst[(size_t)c * kD + col] = __float2bfloat16_rn(sum * __frcp_rn((float)cnt[c]));
     }
+}
+
+// 1 where the halves are equal, else 0 (one instruction: the result is the operand the product wants).
+__device__ __forceinline__ uint32_t same_as(__nv_bfloat162 a, __nv_bfloat162 b) {
+    const __nv_bfloat162 r = __heq2(a, b);
+    return *reinterpret_cast<const uint32_t*>(&r);
 }
 
 // Step 3 for the NT tensors staged at smem, smem + kVOff (column halves hs bytes apart): this warp's 32 columns of every cluster
@@ -422,14 +436,13 @@ __device__ __forceinline__ void pool_tile(unsigned char* smem, int hs, int P, __
         for (int t = 0; t < NT; ++t)
 #pragma unroll
             for (int nt = 0; nt < 4; ++nt) acc[t][nt][0] = acc[t][nt][1] = acc[t][nt][2] = acc[t][nt][3] = 0.f;
-        const uint32_t c0 = (uint32_t)(16 * m + g) * 0x01010101u, c1 = c0 + 0x08080808u;
+        const __nv_bfloat162 c0 = __bfloat162bfloat162(__int2bfloat16_rn(16 * m + g)), c1 = __bfloat162bfloat162(__int2bfloat16_rn(16 * m + 8 + g));
 #pragma unroll 2
         for (int kk = k_lo; kk < k_hi; ++kk) {
             // M's fragment: rows g and g + 8 of the sixteen clusters, tokens 2 tig, +1, +8, +9 of the sixteen
-            const uint32_t ranks = *reinterpret_cast<const uint32_t*>(smem + kRankOff + kk * 16 + 4 * tig);
-            const uint32_t m0 = __vcmpeq4(ranks, c0), m1 = __vcmpeq4(ranks, c1);
-            const uint32_t a0 = __byte_perm(m0, 0u, 0x1100) & 0x3f803f80u, a1 = __byte_perm(m1, 0u, 0x1100) & 0x3f803f80u;
-            const uint32_t a2 = __byte_perm(m0, 0u, 0x3322) & 0x3f803f80u, a3 = __byte_perm(m1, 0u, 0x3322) & 0x3f803f80u;
+            const uint2 ranks = *reinterpret_cast<const uint2*>(smem + kRankOff + kk * 32 + 8 * tig);
+            const __nv_bfloat162 r01 = *reinterpret_cast<const __nv_bfloat162*>(&ranks.x), r89 = *reinterpret_cast<const __nv_bfloat162*>(&ranks.y);
+            const uint32_t a0 = same_as(r01, c0), a1 = same_as(r01, c1), a2 = same_as(r89, c0), a3 = same_as(r89, c1);
 #pragma unroll
             for (int t = 0; t < NT; ++t) {
                 const uint32_t row = b_row + t * kVOff + kk * 16 * kHalfRow;
@@ -608,7 +621,8 @@ __device__ __forceinline__ int look_back(const uint32_t* stt, int t, int lane, i
     return sum;
 }
 
-template <int kMode, int NL>
+// kAnyTau: the threshold may be negative (the code for it costs the other case registers).
+template <int kMode, int NL, bool kAnyTau>
 __global__ void __launch_bounds__(kThreads, kBlocksPerSm) compress_fused_kernel(const __grid_constant__ Params<NL> p) {
     extern __shared__ __align__(1024) unsigned char smem[];   // the swizzle pattern repeats every 1024 bytes
     uint32_t* starts_buf = reinterpret_cast<uint32_t*>(smem + kMiscOff + 64);   // [2][4] rows that start a segment
@@ -716,13 +730,13 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) compress_fused_kernel(
                     umma_gram_block(sbase, kHalfShort, 0, 0, tmem, bar_u);
                 }
                 __syncwarp();
-                P = settle_short_tile(smem, starts_buf + par * 4, R, tmem, phase_u, tau, bad, failed, as, row0, publish, sh_p);
+                P = settle_short_tile<kAnyTau>(smem, starts_buf + par * 4, R, tmem, phase_u, tau, bad, as, row0, publish, sh_p);
                 phase_u ^= 1u;
             } else {
-                P = settle_long_tile(smem, R, tmem, phase_u, tau, bad, &failed, as, row0, publish, sh_p);
+                P = settle_long_tile<kAnyTau>(smem, R, tmem, phase_u, tau, bad, as, row0, publish, sh_p);
                 phase_u ^= 1u;   // three products
             }
-            if (failed) break;
+            if (P < 0) { failed = true; break; }   // a wait for the product gave up
             if (kMode == kCountOnly) {
                 if (tid == 0 && p.count_into_len) atomicAdd(&lr.core_len[bh], P);
             } else {
@@ -844,9 +858,12 @@ int resident_blocks() {
     cudaGetDevice(&dev);
     dev &= 63;
     if (grid_of[dev] == 0) {
-        cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kCountOnly, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
-        cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kLookBack, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
-        cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kLookBack, cf::kMaxLayers>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
+        cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kCountOnly, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
+        cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kCountOnly, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
+        cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kLookBack, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
+        cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kLookBack, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
+        cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kLookBack, cf::kMaxLayers, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
+        cudaFuncSetAttribute(cf::compress_fused_kernel<cf::kLookBack, cf::kMaxLayers, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, cf::kSmemBytes);
         // Blocks per SM by construction: launch bounds (registers), 75 KB of shared memory and 128 of the 512
         // tensor-memory columns each.  (The occupancy query answers 1 for a kernel that allocates tensor memory.)
         // Launching more blocks than are resident would be harmless: a block draws its first ticket when it starts.
@@ -886,14 +903,17 @@ cudaError_t launch_compress_fused(const CompressArgs& a, cudaStream_t st) {
     // no more blocks than there can be tiles
     const int64_t max_tiles = (int64_t)a.B * a.Hkv * a.n_tile_cap;
     const int grid = (int)(max_tiles < resident ? max_tiles : resident);
+    const bool any_tau = a.tau < 0.f;   // (of a search: its lowest threshold)
+    const auto count = any_tau ? cf::compress_fused_kernel<cf::kCountOnly, 1, true> : cf::compress_fused_kernel<cf::kCountOnly, 1, false>;
+    const auto full = any_tau ? cf::compress_fused_kernel<cf::kLookBack, 1, true> : cf::compress_fused_kernel<cf::kLookBack, 1, false>;
     if (a.count_only) {   // budget search: per-head cluster counts only
-        cf::compress_fused_kernel<cf::kCountOnly, 1><<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
+        count<<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
         note_launches(1);
     } else if (a.flags & SC_FLAG_TWO_PASS) {
         cf::Params<1> pc = p;
         pc.layer[0].assign = nullptr;
-        cf::compress_fused_kernel<cf::kCountOnly, 1><<<grid, cf::kThreads, cf::kSmemBytes, st>>>(pc);
-        cf::compress_fused_kernel<cf::kLookBack, 1><<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
+        count<<<grid, cf::kThreads, cf::kSmemBytes, st>>>(pc);
+        full<<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
         note_launches(2);
     } else {
         // With SC_FLAG_OVERLAP_PREV the kernel may start while the one enqueued before it on the stream is
@@ -910,7 +930,7 @@ cudaError_t launch_compress_fused(const CompressArgs& a, cudaStream_t st) {
         cfg.attrs = attr;
         cfg.numAttrs = (a.flags & SC_FLAG_OVERLAP_PREV) ? 1 : 0;
         note_launches(1);
-        return cudaLaunchKernelEx(&cfg, cf::compress_fused_kernel<cf::kLookBack, 1>, p);
+        return cudaLaunchKernelEx(&cfg, full, p);
     }
     return cudaGetLastError();
 }
@@ -932,7 +952,8 @@ cudaError_t launch_compress_fused_layers(const CompressArgs& a, const sc_compres
     for (int l = L; l < cf::kMaxLayers; ++l) p.layer[l] = p.layer[0];
     const int64_t max_tiles = (int64_t)L * a.B * a.Hkv * a.n_tile_cap;
     const int grid = (int)(max_tiles < resident ? max_tiles : resident);
-    cf::compress_fused_kernel<cf::kLookBack, cf::kMaxLayers><<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
+    const auto full = a.tau < 0.f ? cf::compress_fused_kernel<cf::kLookBack, cf::kMaxLayers, true> : cf::compress_fused_kernel<cf::kLookBack, cf::kMaxLayers, false>;
+    full<<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
     note_launches(1);
     return cudaGetLastError();
 }
