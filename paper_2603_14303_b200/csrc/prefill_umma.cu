@@ -21,9 +21,20 @@
 // of a head are split over the CTAs of a thread-block cluster: each walks its share of the key tiles, leaves its
 // unnormalised (m, l, O) in its own shared memory, and after a cluster barrier every CTA folds a slice of the
 // query rows out of all members' shared memory (distributed shared memory) and writes that slice of the output.
+// What bounds it: the softmax of a tile (its arithmetic on packed pairs, one exponential per score) with the weighted sum
+// issued twice for the bf16 pair behind it.  4 layers x 512 causal queries per head over 8.5 K cores: 538 -> 489 us when the
+// tile's counts were requested a tile ahead (480 cycles per tile), one barrier per tile instead of two, the scores were
+// read from tensor memory once and two scores went through each fma and add (one at a time: 523 us).  Tried: the two
+// groups of four warps on alternate tiles with a row per thread and an accumulator each, 569 us.
+// Cluster width: as many CTAs per query tile as let every cluster of the launch be resident at once (asked of the
+// occupancy query: on this GPU 15 clusters of 8 or 9, 11 of 10, 7 of 11 to 16); powers of two up to 8 before.  8 queries per
+// head, 8 KV heads: 10 instead of 8 CTAs, 29 -> 24 us per layer with the above; 16 clusters: 7 instead of 8 (which took
+// two waves), 64 queries per head 190 -> 132 us for 4 layers.
 // Every wait is bounded; a wait that gives up is reported through the status word.
 // A CUDA-core kernel (one warp per query) serves other dtypes and head sizes.
 #include <cooperative_groups.h>
+
+#include <mutex>
 
 #include "common.cuh"
 #include "umma.cuh"
@@ -45,7 +56,7 @@ constexpr int kStages = 3;                    // K/V ring
 constexpr int kSmQ = 0, kSmK = kTile, kSmV = (1 + kStages) * kTile, kSmLc = (1 + 2 * kStages) * kTile, kSmMx = kSmLc + 2 * kT * 4,
               kSmBar = kSmMx + 2 * kT * 4;
 constexpr int kSmemBytes = kSmBar + 256;
-constexpr int kMaxSplit = 8;                  // portable cluster size
+constexpr int kMaxSplit = 16;                 // CTAs that share one query tile: a cluster (more than 8 needs the non-portable opt-in)
 constexpr float kMaxSlack = 8.f;              // log2 units a score may exceed the running maximum before it is raised
 static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
 
@@ -97,8 +108,25 @@ __device__ __forceinline__ void remainders(uint32_t ph, float w0, float w1, floa
         "fma.rn.f32.bf16 %0, lo, m1, %3;\nfma.rn.f32.bf16 %1, hi, m1, %4;\n}\n"
         : "=f"(r0), "=f"(r1) : "r"(ph), "f"(w0), "f"(w1));
 }
-__device__ __forceinline__ float bf_lo(uint32_t v) { return __uint_as_float(v << 16); }
-__device__ __forceinline__ float bf_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
+
+__device__ __forceinline__ float max3(float a, float b, float c) {
+    float y;
+    asm("max.f32 %0, %1, %2, %3;\n" : "=f"(y) : "f"(a), "f"(b), "f"(c));
+    return y;
+}
+// Two fp32 operations per instruction.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 y;
+    asm("{\n.reg .b64 a, b, c, y;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nmov.b64 c, {%6, %7};\nfma.rn.f32x2 y, a, b, c;\nmov.b64 {%0, %1}, y;\n}\n"
+        : "=f"(y.x), "=f"(y.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return y;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 y;
+    asm("{\n.reg .b64 a, b, y;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nadd.rn.f32x2 y, a, b;\nmov.b64 {%0, %1}, y;\n}\n"
+        : "=f"(y.x), "=f"(y.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return y;
+}
 
 __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_constant__ Params p) {
     extern __shared__ __align__(1024) unsigned char smem[];   // the swizzle pattern repeats every 1024 bytes
@@ -118,7 +146,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         return;
     }
     float* lc_s = reinterpret_cast<float*>(smem + kSmLc);     // [2][128] log2(count) of the tile's keys
-    float* mx_s = reinterpret_cast<float*>(smem + kSmMx);     // [2][128] each half's row maximum (at the end the row sums)
+    __nv_bfloat16* mx_s = reinterpret_cast<__nv_bfloat16*>(smem + kSmMx);   // [2][2][128] each half's row maximum, rounded up
+    float* ls_s = reinterpret_cast<float*>(smem + kSmMx);     // [2][128] at the end: each half's row sum
     int* lcm_s = reinterpret_cast<int*>(smem + kSmBar + 128);  // [2][4] largest log2(count) of a tile, per writing warp (float bits)
     const uint32_t bar0 = sbase + kSmBar;
     const uint32_t q_full = bar0, kv_full0 = bar0 + 8, kv_empty0 = bar0 + 32, s_full0 = bar0 + 56, p_full0 = bar0 + 72,
@@ -226,18 +255,53 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         const int32_t* cnt = p.count ? p.count + (size_t)bh * p.cap : nullptr;
         float m_run = -INFINITY, l_run = 0.f;                 // l_run: this thread's keys only
         bool failed = false;
+        const bool idle = qt * kT + q * 32 >= rows_total;     // none of the warp's rows exists: it only keeps step
+        const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
+        // log2(count) of a tile's keys, one key per thread of the first four warps.  The counts of the next tile are requested
+        // a tile ahead and published behind this tile's barrier, when nobody reads that buffer any more.
+        auto count_of = [&](int t) { const int j = (t_lo + t) * kT + r; return cnt != nullptr && t < nt && j < len ? cnt[j] : 1; };
+        auto publish_counts = [&](int t, int c) {
+            const float lc = lg2((float)max(c, 1));
+            lc_s[(t & 1) * kT + r] = lc;
+            const int top = __reduce_max_sync(kFull, __float_as_int(lc));   // lc >= 0: the bits order like the values
+            if (lane == 0) lcm_s[(t & 1) * 4 + q] = top;
+        };
+        if (wg == 0) publish_counts(0, count_of(0));
         for (int t = 0; t < nt; ++t) {
             const int s = t & 1, st = t % kStages, j0 = (t_lo + t) * kT, jw = j0 + wg * 64;   // jw: first key of this thread's half
-            if (wg == 0) {
-                const float lc = (cnt != nullptr && j0 + r < len) ? lg2((float)max(cnt[j0 + r], 1)) : 0.f;
-                lc_s[s * kT + r] = lc;
-                const int top = __reduce_max_sync(kFull, __float_as_int(lc));   // lc >= 0: the bits order like the values
-                if (lane == 0) lcm_s[s * 4 + q] = top;
-            }
+            const int next_count = wg == 0 ? count_of(t + 1) : 1;
             if (!mbar_wait(s_full0 + 8 * s, (t >> 1) & 1)) { *sh_fail = 1; *sh_fail_sm = 1; }
             fence_after_sync();
-            asm volatile("bar.sync 1, 256;\n" ::: "memory");   // the eight softmax warps: log2(count) is in place
-            if (*sh_fail_sm) { failed = true; break; }
+            // pass 1: the row's largest raw product in this tile (each thread its half, then the two are exchanged).  That times
+            // the scale plus the tile's largest log2(count) bounds the row's largest score: any reference at or above the
+            // true maximum serves the softmax, and this one is at most log2 of the largest count above it.  (A scale that
+            // is not positive takes the smallest product.)
+            uint32_t g[64];
+            const bool all_seen = __all_sync(kFull, jw + 64 <= vis);   // no key of this half is masked for any row of the warp
+            float mx = -INFINITY;
+            if (!idle) {
+                tmem_ld32(lane_addr + kColS + s * kT + wg * 64, *reinterpret_cast<uint32_t(*)[32]>(&g[0]));
+                tmem_ld32(lane_addr + kColS + s * kT + wg * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&g[32]));
+                tmem_ld_wait();
+                if (!(p.scale_log2 > 0.f)) {
+#pragma unroll
+                    for (int k = 0; k < 64; ++k)
+                        if (jw + k < vis) mx = fmaxf(mx, -__uint_as_float(g[k]));
+                } else if (all_seen) {
+                    float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                    for (int k = 0; k < 64; k += 8)
+#pragma unroll
+                        for (int x = 0; x < 4; ++x) m4[x] = max3(m4[x], __uint_as_float(g[k + x]), __uint_as_float(g[k + 4 + x]));
+                    mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 64; ++k)
+                        if (jw + k < vis) mx = fmaxf(mx, __uint_as_float(g[k]));
+                }
+            }
+            const __nv_bfloat16 mx_up = __float2bfloat16_ru(mx);   // (a bound as well; both threads of the row use the rounded values)
+            mx_s[(s * 2 + wg) * kT + r] = mx_up;
             // Rows of the stage past the head's end hold whatever lies behind the cores (0 * NaN would poison
             // the second product): this row's threads clear its V row.  K rows need nothing, their scores are masked.
             if (j0 + r >= len) {
@@ -245,103 +309,73 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
                 for (int u = 0; u < 8; ++u)
                     *reinterpret_cast<uint4*>(smem + kSmV + st * kTile + wg * kHalf + r * 128 + u * 16) = make_uint4(0u, 0u, 0u, 0u);
             }
-            // pass 1: a bound on the row's largest score in this tile (each thread its half, then the two are
-            // exchanged): the largest raw product times the scale plus the tile's largest log2(count).  Any reference
-            // at or above the true maximum serves the softmax; this one is at most log2 of the largest count above it,
-            // and costs one instruction per score.  (A scale that is not positive takes the exact form.)
-            float mx = -INFINITY;
-            const bool all_seen = __all_sync(kFull, jw + 64 <= vis);   // no key of this half is masked for any row of the warp
-            const bool exact = !(p.scale_log2 > 0.f);
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t g[32];
-                tmem_ld32(lane_addr + kColS + s * kT + wg * 64 + c * 32, g);
-                tmem_ld_wait();
-                if (exact) {
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) {
-                        const float x = fmaf(__uint_as_float(g[k]), p.scale_log2, lc_s[s * kT + wg * 64 + c * 32 + k]);
-                        if (jw + c * 32 + k < vis) mx = fmaxf(mx, x);
-                    }
-                } else if (all_seen) {
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) mx = fmaxf(mx, __uint_as_float(g[k]));
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 32; ++k)
-                        if (jw + c * 32 + k < vis) mx = fmaxf(mx, __uint_as_float(g[k]));
+            asm volatile("bar.sync 2, 256;\n" ::: "memory");   // both halves' maxima and this tile's log2(count) are in place
+            if (*sh_fail_sm) { failed = true; break; }
+            if (wg == 0 && t + 1 < nt) publish_counts(t + 1, next_count);
+            if (!idle) {
+                mx = fmaxf(__bfloat162float(mx_up), __bfloat162float(mx_s[(s * 2 + (wg ^ 1)) * kT + r]));
+                if (mx != -INFINITY) {
+                    const int top = max(max(lcm_s[s * 4], lcm_s[s * 4 + 1]), max(lcm_s[s * 4 + 2], lcm_s[s * 4 + 3]));
+                    mx = fmaf(mx, fabsf(p.scale_log2), __int_as_float(top));
                 }
-            }
-            if (!exact && mx != -INFINITY) {
-                const int top = max(max(lcm_s[s * 4], lcm_s[s * 4 + 1]), max(lcm_s[s * 4 + 2], lcm_s[s * 4 + 3]));
-                mx = fmaf(mx, p.scale_log2, __int_as_float(top));
-            }
-            mx_s[wg * kT + r] = mx;
-            asm volatile("bar.sync 2, 256;\n" ::: "memory");   // both halves' maxima are in place
-            mx = fmaxf(mx, mx_s[(wg ^ 1) * kT + r]);
-            const bool raise = mx > m_run + kMaxSlack;      // also the first finite score (m_run = -inf); same in both threads
-            if (__any_sync(kFull, raise)) {
-                const float f = raise ? ex2(m_run - mx) : 1.f;   // 0 when nothing had been seen
-                // the accumulator may be touched only between two weighted sums: the previous one must be complete
-                // (this tile's cannot start before this warp has handed in its weights)
-                if (t > 0 && !mbar_wait(pv_done0 + 8 * ((t - 1) & 1), ((t - 1) >> 1) & 1)) { *sh_fail = 1; *sh_fail_sm = 1; }
-                fence_after_sync();
-                if (t > 0) {
+                const bool raise = mx > m_run + kMaxSlack;      // also the first finite score (m_run = -inf); same in both threads
+                if (__any_sync(kFull, raise)) {
+                    const float f = raise ? ex2(m_run - mx) : 1.f;   // 0 when nothing had been seen
+                    // the accumulator may be touched only between two weighted sums: the previous one must be complete
+                    // (this tile's cannot start before this warp has handed in its weights)
+                    if (t > 0 && !mbar_wait(pv_done0 + 8 * ((t - 1) & 1), ((t - 1) >> 1) & 1)) { *sh_fail = 1; *sh_fail_sm = 1; }
+                    fence_after_sync();
+                    if (t > 0) {
 #pragma unroll
-                    for (int c = 0; c < 2; ++c) {
-                        uint32_t o[32];
-                        tmem_ld32(lane_addr + kColO + wg * 64 + c * 32, o);
-                        tmem_ld_wait();
+                        for (int c = 0; c < 2; ++c) {
+                            uint32_t o[32];
+                            tmem_ld32(lane_addr + kColO + wg * 64 + c * 32, o);
+                            tmem_ld_wait();
 #pragma unroll
-                        for (int k = 0; k < 32; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * f);
-                        tmem_st32(lane_addr + kColO + wg * 64 + c * 32, o);
+                            for (int k = 0; k < 32; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * f);
+                            tmem_st32(lane_addr + kColO + wg * 64 + c * 32, o);
+                        }
+                        tmem_st_wait();
                     }
-                    tmem_st_wait();
+                    l_run *= f;
+                    if (raise) m_run = mx;
                 }
-                l_run *= f;
-                if (raise) m_run = mx;
-            }
-            // pass 2: weights, as bf16 pairs (leading part + remainder), back into the score buffer's columns
-            const float mref = m_run == -INFINITY ? 0.f : m_run;
-            // (the row sum takes the weights before the split: the pair carries sixteen bits of each, the difference
-            // is below 2^-17 of the sum)
+                // pass 2: weights, as bf16 pairs (leading part + remainder), back into the score buffer's columns: the 32 score
+                // columns of a chunk become 16 columns of packed leading parts and 16 of remainders
+                const float mref = m_run == -INFINITY ? 0.f : m_run;
+                const float2 nref2 = make_float2(-mref, -mref);
+                // (the row sum takes the weights before the split: the pair carries sixteen bits of each, the difference
+                // is below 2^-17 of the sum)
+                float2 l2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t g[32];
-                tmem_ld32(lane_addr + kColS + s * kT + wg * 64 + c * 32, g);
-                tmem_ld_wait();
-                uint32_t hi[16], lo[16];
-                if (all_seen) {   // no key of this half is masked for any row of the warp
+                for (int c = 0; c < 2; ++c) {
+                    uint32_t hi[16], lo[16];
 #pragma unroll
-                    for (int k = 0; k < 32; k += 2) {
-                        const float x0 = fmaf(__uint_as_float(g[k]), p.scale_log2, lc_s[s * kT + wg * 64 + c * 32 + k]);
-                        const float x1 = fmaf(__uint_as_float(g[k + 1]), p.scale_log2, lc_s[s * kT + wg * 64 + c * 32 + k + 1]);
-                        const float w0 = ex2(x0 - mref), w1 = ex2(x1 - mref);
-                        const uint32_t ph = pack2(w0, w1);
-                        float r0, r1;
-                        remainders(ph, w0, w1, r0, r1);
-                        l_run += w0 + w1;
-                        hi[k >> 1] = ph; lo[k >> 1] = pack2(r0, r1);
+                    for (int k = 0; k < 32; k += 4) {
+                        const float4 lc = *reinterpret_cast<const float4*>(lc_s + s * kT + wg * 64 + c * 32 + k);
+                        const uint32_t* gk = g + c * 32 + k;
+                        const float2 x0 = add2(fma2(make_float2(__uint_as_float(gk[0]), __uint_as_float(gk[1])), scale2, make_float2(lc.x, lc.y)), nref2);
+                        const float2 x1 = add2(fma2(make_float2(__uint_as_float(gk[2]), __uint_as_float(gk[3])), scale2, make_float2(lc.z, lc.w)), nref2);
+                        float2 w0 = make_float2(ex2(x0.x), ex2(x0.y)), w1 = make_float2(ex2(x1.x), ex2(x1.y));
+                        if (!all_seen) {
+                            const int j = jw + c * 32 + k;
+                            w0.x = j < vis ? w0.x : 0.f; w0.y = j + 1 < vis ? w0.y : 0.f;
+                            w1.x = j + 2 < vis ? w1.x : 0.f; w1.y = j + 3 < vis ? w1.y : 0.f;
+                        }
+                        l2[0] = add2(l2[0], w0); l2[1] = add2(l2[1], w1);
+                        const uint32_t p0 = pack2(w0.x, w0.y), p1 = pack2(w1.x, w1.y);
+                        float r0, r1, r2, r3;
+                        remainders(p0, w0.x, w0.y, r0, r1);
+                        remainders(p1, w1.x, w1.y, r2, r3);
+                        hi[k >> 1] = p0; hi[(k >> 1) + 1] = p1;
+                        lo[k >> 1] = pack2(r0, r1); lo[(k >> 1) + 1] = pack2(r2, r3);
                     }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 32; k += 2) {
-                        const float x0 = fmaf(__uint_as_float(g[k]), p.scale_log2, lc_s[s * kT + wg * 64 + c * 32 + k]);
-                        const float x1 = fmaf(__uint_as_float(g[k + 1]), p.scale_log2, lc_s[s * kT + wg * 64 + c * 32 + k + 1]);
-                        const float w0 = (jw + c * 32 + k < vis) ? ex2(x0 - mref) : 0.f;
-                        const float w1 = (jw + c * 32 + k + 1 < vis) ? ex2(x1 - mref) : 0.f;
-                        const uint32_t ph = pack2(w0, w1);
-                        float r0, r1;
-                        remainders(ph, w0, w1, r0, r1);
-                        l_run += w0 + w1;
-                        hi[k >> 1] = ph; lo[k >> 1] = pack2(r0, r1);
-                    }
+                    tmem_st16(lane_addr + kColS + s * kT + wg * 64 + c * 32, hi);
+                    tmem_st16(lane_addr + kColS + s * kT + wg * 64 + c * 32 + 16, lo);
                 }
-                // the 32 score columns just read become 16 columns of packed leading parts and 16 of remainders
-                tmem_st16(lane_addr + kColS + s * kT + wg * 64 + c * 32, hi);
-                tmem_st16(lane_addr + kColS + s * kT + wg * 64 + c * 32 + 16, lo);
+                l_run += (l2[0].x + l2[0].y) + (l2[1].x + l2[1].y);
+                tmem_st_wait();
             }
-            tmem_st_wait();
             fence_before_sync();      // this thread's accesses to tensor memory
             fence_async_proxy();      // a cleared V row, for the tensor core's reads
             __syncwarp();
@@ -353,9 +387,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             fence_after_sync();
         }
         asm volatile("bar.sync 2, 256;\n" ::: "memory");   // nobody still reads the last tile's maxima
-        mx_s[wg * kT + r] = l_run;
+        ls_s[wg * kT + r] = l_run;
         asm volatile("bar.sync 1, 256;\n" ::: "memory");
-        const float l_row = l_run + mx_s[(wg ^ 1) * kT + r];
+        const float l_row = l_run + ls_s[(wg ^ 1) * kT + r];
         if (n_split == 1) {
             __nv_bfloat16* orow = p.out + (size_t)(q_row0 + r) * 128 + wg * 64;
             const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
@@ -409,43 +443,43 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         fence_before_sync();
         cluster.sync();   // every member's partial is in its shared memory
         if (warp >= 2) {
-            // this CTA folds query rows [split * R, (split + 1) * R) of the tile, R = 128 / n_split: one thread per
-            // (row, four output columns), reading that piece of every member's partial
+            // this CTA folds query rows [split * R, (split + 1) * R) of the tile, R = 128 / n_split rounded up: one thread per
+            // (row, four output columns), reading that piece of every member's partial, four members at a time
             const float* part_o = reinterpret_cast<const float*>(smem + kSmK);
             const float* part_ml = reinterpret_cast<const float*>(smem + kSmV);
-            const int R = kT / n_split;
+            const int R = (kT + n_split - 1) / n_split, r_end = min(min((split + 1) * R, kT), rows_total - qt * kT);
             for (int it = tid - 64; it < R * 32; it += 256) {
                 const int r = split * R + (it >> 5), c4 = it & 31;
-                float mv[kMaxSplit], lv[kMaxSplit];
-                float4 ov[kMaxSplit];
-#pragma unroll
-                for (int j = 0; j < kMaxSplit; ++j) {
-                    const int src = j < n_split ? j : 0;
-                    const float* ml = cluster.map_shared_rank(part_ml, src);
-                    const float* po = cluster.map_shared_rank(part_o, src);
-                    mv[j] = j < n_split ? ml[r] : -INFINITY;
-                    lv[j] = j < n_split ? ml[kT + r] : 0.f;
-                    ov[j] = j < n_split ? *reinterpret_cast<const float4*>(po + r * 128 + ((c4 ^ (r & 31)) << 2)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                }
-                float gm = mv[0];
-#pragma unroll
-                for (int j = 1; j < kMaxSplit; ++j) gm = fmaxf(gm, mv[j]);
+                if (r >= r_end) break;
+                float gm = -INFINITY;
+                for (int j = 0; j < n_split; ++j) gm = fmaxf(gm, cluster.map_shared_rank(part_ml, j)[r]);
                 float lsum = 0.f;
                 float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int j0 = 0; j0 < n_split; j0 += 4) {
+                    float mv[4], lv[4];
+                    float4 ov[4];
 #pragma unroll
-                for (int j = 0; j < kMaxSplit; ++j) {
-                    const float w = (mv[j] == -INFINITY) ? 0.f : ex2(mv[j] - gm);
-                    lsum = fmaf(w, lv[j], lsum);
-                    acc.x = fmaf(w, ov[j].x, acc.x); acc.y = fmaf(w, ov[j].y, acc.y);
-                    acc.z = fmaf(w, ov[j].z, acc.z); acc.w = fmaf(w, ov[j].w, acc.w);
+                    for (int j = 0; j < 4; ++j) {
+                        const bool on = j0 + j < n_split;
+                        const float* ml = cluster.map_shared_rank(part_ml, on ? j0 + j : 0);
+                        const float* po = cluster.map_shared_rank(part_o, on ? j0 + j : 0);
+                        mv[j] = on ? ml[r] : -INFINITY;
+                        lv[j] = on ? ml[kT + r] : 0.f;
+                        ov[j] = on ? *reinterpret_cast<const float4*>(po + r * 128 + ((c4 ^ (r & 31)) << 2)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float w = (mv[j] == -INFINITY) ? 0.f : ex2(mv[j] - gm);
+                        lsum = fmaf(w, lv[j], lsum);
+                        acc.x = fmaf(w, ov[j].x, acc.x); acc.y = fmaf(w, ov[j].y, acc.y);
+                        acc.z = fmaf(w, ov[j].z, acc.z); acc.w = fmaf(w, ov[j].w, acc.w);
+                    }
                 }
-                if (qt * kT + r < rows_total) {
-                    const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
-                    uint2 v;
-                    v.x = pack2(acc.x * inv, acc.y * inv);
-                    v.y = pack2(acc.z * inv, acc.w * inv);
-                    *reinterpret_cast<uint2*>(p.out + (size_t)(q_row0 + r) * 128 + c4 * 4) = v;
-                }
+                const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
+                uint2 v;
+                v.x = pack2(acc.x * inv, acc.y * inv);
+                v.y = pack2(acc.z * inv, acc.w * inv);
+                *reinterpret_cast<uint2*>(p.out + (size_t)(q_row0 + r) * 128 + c4 * 4) = v;
             }
         }
         cluster.sync();   // every member's shared memory has been read: they may leave
@@ -528,18 +562,17 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
     const long long q_rows = (long long)a.B * a.Hq * a.m, c_rows = (long long)a.B * a.Hkv * a.cap;
     if (a.dt == SC_BF16 && a.d == 128 && !(a.flags & SC_FLAG_GENERIC) && a.cap > 0 && q_rows < 0x7fffffff &&
         c_rows < 0x7fffffff && a.Hkv <= 65535 && a.B <= 65535) {
-        // per device: the opt-in to large dynamic shared memory, the SM count, and the largest cluster of these
-        // one-per-SM CTAs that can be scheduled
-        static int sms_of[64] = {0}, cmax_of[64] = {0};
+        // per device: the opt-ins, and how many clusters of each size (one CTA per SM) can be resident at once
+        static int fit_of[64][kMaxSplit + 1] = {{0}};
+        static std::once_flag once_of[64];
         int dev = 0;
         cudaGetDevice(&dev);
         dev &= 63;
-        if (sms_of[dev] == 0) {
+        int* fit = fit_of[dev];
+        std::call_once(once_of[dev], [&] {
             cudaFuncSetAttribute(prefill_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-            int v = 0;
-            cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-            int cmax = 1;
-            for (int c = kMaxSplit; c > 1; c >>= 1) {
+            const bool wide = cudaFuncSetAttribute(prefill_umma_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+            for (int c = 2; c <= (wide ? kMaxSplit : 8); ++c) {
                 cudaLaunchConfig_t probe = {};
                 probe.gridDim = dim3(c, 1, 1);
                 probe.blockDim = dim3(kThreads);
@@ -550,26 +583,23 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
                 probe.attrs = pa;
                 probe.numAttrs = 1;
                 int n_clusters = 0;
-                if (cudaOccupancyMaxActiveClusters(&n_clusters, prefill_umma_kernel, &probe) == cudaSuccess && n_clusters > 0) {
-                    cmax = c;
-                    break;
-                }
+                if (cudaOccupancyMaxActiveClusters(&n_clusters, prefill_umma_kernel, &probe) == cudaSuccess) fit[c] = n_clusters;
             }
-            (void)cudaGetLastError();   // a refused probe is not an error of this call
-            cmax_of[dev] = cmax;
-            sms_of[dev] = v < 1 ? 1 : v;
-        }
+            (void)cudaGetLastError();   // a refused opt-in or probe is not an error of this call
+        });
         Params p;
         p.count = a.count; p.core_len = a.core_len; p.out = (__nv_bfloat16*)a.out;
         p.Hq = a.Hq; p.Hkv = a.Hkv; p.m = a.m; p.cap = a.cap; p.causal = causal; p.scale_log2 = scale_log2; p.status = a.status;
         if (make_map_bf16_rows(&p.map_q, a.q, 0, 0, 128, 1, 1, q_rows, kT) &&
             make_map_bf16_rows(&p.map_k, a.core_k, 0, 0, 128, 1, 1, c_rows, kT) &&
             make_map_bf16_rows(&p.map_v, a.core_v, 0, 0, 128, 1, 1, c_rows, kT)) {
-            // Few query tiles (short chunks, speculative decoding): split the keys over a cluster, as many ways as
-            // fill the GPU, but leave every CTA at least two key tiles of the capacity.
+            // Few query tiles (short chunks, speculative decoding): split the keys over a cluster, as wide as all clusters of the
+            // launch fit at once, but leave every CTA at least four key tiles of the capacity (heads are usually half full).
             const long long ctas = (long long)((G * a.m + kT - 1) / kT) * a.Hkv * a.B;
+            const int key_tiles = (a.cap + kT - 1) / kT;
             int n_split = 1;
-            while (n_split * 2 <= cmax_of[dev] && ctas * n_split * 2 <= sms_of[dev] && (a.cap + kT - 1) / kT >= n_split * 4) n_split *= 2;
+            for (int c = 2; c <= kMaxSplit; ++c)
+                if (ctas <= fit[c] && key_tiles >= c * 4) n_split = c;
             p.n_split = n_split;
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)((G * a.m + kT - 1) / kT) * n_split, a.Hkv, a.B);
