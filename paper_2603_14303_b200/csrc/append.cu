@@ -154,6 +154,7 @@ __device__ __forceinline__ void append_block(const AppendArgs& a, const LayerPtr
 
 template <typename T>
 __global__ void __launch_bounds__(kAppendThreads) append_kernel(const AppendArgs a) {
+    in_stream_order();
     LayerPtrs p;
     p.k_new = a.k_new; p.v_new = a.v_new; p.core_k = a.core_k; p.core_v = a.core_v; p.count = a.count;
     p.core_len = a.core_len; p.tail_len = a.tail_len; p.attn_len = a.attn_len;
@@ -163,6 +164,7 @@ __global__ void __launch_bounds__(kAppendThreads) append_kernel(const AppendArgs
 // Every layer of one generated token in one launch: blockIdx.y picks the layer's row of the table.
 template <typename T>
 __global__ void __launch_bounds__(kAppendThreads) append_layers_kernel(const AppendArgs a, const sc_append_layer* __restrict__ table) {
+    in_stream_order();
     const sc_append_layer t = table[blockIdx.y];
     LayerPtrs p;
     p.k_new = t.k_new; p.v_new = t.v_new; p.core_k = t.core_k; p.core_v = t.core_v; p.count = t.count;
@@ -176,19 +178,15 @@ cudaError_t launch_append_layers(const AppendArgs& a, const sc_append_layer* tab
     const int blocks = a.B * a.Hkv;
     if (blocks == 0 || L == 0) return cudaSuccess;
     const dim3 grid(blocks, L);
-    if (a.dt == SC_BF16) append_layers_kernel<__nv_bfloat16><<<grid, kAppendThreads, 0, st>>>(a, table);
-    else append_layers_kernel<float><<<grid, kAppendThreads, 0, st>>>(a, table);
     note_launches(1);
-    return cudaGetLastError();
+    return launch_in_order(a.dt == SC_BF16 ? append_layers_kernel<__nv_bfloat16> : append_layers_kernel<float>, grid, kAppendThreads, 0, st, a, table);
 }
 
 cudaError_t launch_append(const AppendArgs& a, cudaStream_t st) {
     const int blocks = a.B * a.Hkv;
     if (blocks == 0) return cudaSuccess;
-    if (a.dt == SC_BF16) append_kernel<__nv_bfloat16><<<blocks, kAppendThreads, 0, st>>>(a);
-    else append_kernel<float><<<blocks, kAppendThreads, 0, st>>>(a);
     note_launches(1);
-    return cudaGetLastError();
+    return launch_in_order(a.dt == SC_BF16 ? append_kernel<__nv_bfloat16> : append_kernel<float>, dim3(blocks), kAppendThreads, 0, st, a);
 }
 
 }  // namespace sc

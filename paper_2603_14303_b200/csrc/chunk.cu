@@ -7,7 +7,7 @@
 // Two kernels.  chunk_flags: one block per 2048 tokens; it finds the run it starts in by looking back for the last
 // delimiter before it (256 tokens at a time: nearly always one look), writes the flags as bits and counts them.
 // chunk_write_pack: one block per sequence turns flags into offsets and packs consecutive segments into the
-// <= SC_TILE_ROWS-token work tiles sc_compress consumes.  The second is launched while the first drains.
+// <= SC_TILE_ROWS-token work tiles sc_compress consumes.
 // What bounds it: launches and dependent round trips, not bytes.  Five kernels before (carry, count, scan, write, pack, with
 // token ids read four times and the tile chain walked one tile at a time) took 17.8 us for 2048 tokens, 40 us for 32K,
 // 30 us for 16 x 16K; these take 8.2, 11.7 and 10.5 us (back to back in a CUDA graph).
@@ -50,6 +50,7 @@ __global__ void __launch_bounds__(kChunkThreads)
 chunk_flags(const int32_t* __restrict__ token_ids, int n, int tps, DelimSet D, int max_len, uint8_t* __restrict__ flags,
             int32_t* __restrict__ tile_cnt) {
     __shared__ int wt[kChunkThreads / 32];
+    in_stream_order();
     const int b = blockIdx.x / tps, tile = blockIdx.x % tps, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int32_t* ids = token_ids + (int64_t)b * n;
     const int tile0 = tile * kChunkTile, p0 = tile0 + threadIdx.x * kChunkPer;
@@ -136,7 +137,7 @@ chunk_write_pack(const uint8_t* __restrict__ flags, const int32_t* __restrict__ 
     __shared__ int wt[32];
     __shared__ int sh_cur, sh_nodes, sh_steps;
     const int b = blockIdx.x, tid = threadIdx.x;
-    wait_for_previous();
+    in_stream_order();
     // segments of the sequences before this one, and of this one
     int before = 0, own = 0, s0, cnt_b;
     for (int i = tid; i < b * tps; i += kPackThreads) before += tile_cnt[i];
@@ -244,11 +245,10 @@ cudaError_t launch_chunk(const ChunkArgs& a, cudaStream_t st) {
     DelimSet D;
     D.n = a.n_delim;
     for (int i = 0; i < SC_MAX_DELIMS; ++i) D.id[i] = (i < a.n_delim) ? a.delim[i] : 0;
-    chunk_flags<<<tiles, kChunkThreads, 0, st>>>(a.token_ids, a.n, tps, D, a.max_chunk_len, flags, tile_cnt);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_in_order(chunk_flags, dim3(tiles), kChunkThreads, 0, st, a.token_ids, a.n, tps, D, a.max_chunk_len, flags, tile_cnt);
     if (e != cudaSuccess) return e;
     note_launches(2);
-    return launch_after_previous(chunk_write_pack, dim3(a.B), kPackThreads, st, (const uint8_t*)flags, (const int32_t*)tile_cnt, a.B, a.n, tps,
+    return launch_in_order(chunk_write_pack, dim3(a.B), kPackThreads, 0, st, (const uint8_t*)flags, (const int32_t*)tile_cnt, a.B, a.n, tps,
                                  a.seg_off, a.n_seg_cap, a.seq_seg_off, a.n_seg, a.tile_seg, a.n_tile_cap, a.seq_tile_cnt, a.status);
 }
 

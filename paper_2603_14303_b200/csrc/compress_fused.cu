@@ -518,6 +518,7 @@ struct Params {
     int32_t* status;
     const float* tau_dev;    // threshold in device memory (budget search), or null: use tau
     const int32_t* skip;     // device flag: nonzero = this launch has nothing to do (budget search), or null
+    int overlap;             // SC_FLAG_OVERLAP_PREV
     int count_into_len;      // kCountOnly: add the tile's cluster count to core_len instead of recording it per tile
     LayerRefs layer[NL];
 };
@@ -640,11 +641,12 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) compress_fused_kernel(
     const bool service = warp == kWarps;   // the fifth warp
     int max_nt = 0;                        // most tiles any sequence has
 
+    // An ordinary launch waits here for the kernel before it; under an overlapped one the next kernel may start beside this one,
+    // and this one waits for its predecessor only at its very end.
+    if (!p.overlap) in_stream_order();
+    else asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     if (p.skip != nullptr && *p.skip != 0) return;   // uniform over the grid: nothing touched, nothing to clean
     const float tau = p.tau_dev != nullptr ? *p.tau_dev : p.tau;
-    // Let the next kernel of the stream start beside this one if it was launched with programmatic stream
-    // serialization (a no-op otherwise); this kernel waits for its predecessor only at its very end.
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     if (tid == 0) {
         umma::mbar_init(bar_k, 1);
         umma::mbar_init(bar_v, 1);
@@ -880,6 +882,7 @@ void fill_common(cf::Params<NL>& p, const CompressArgs& a, int L) {
     p.seg_off = a.seg_off; p.tile_seg = a.tile_seg; p.seq_tile_cnt = a.seq_tile_cnt; p.n_tile_cap = a.n_tile_cap;
     p.tau = a.tau; p.cap = a.cap;
     p.tau_dev = a.tau_dev; p.skip = a.skip; p.count_into_len = a.count_only ? 1 : 0;
+    p.overlap = 0;
     p.ctl = (int32_t*)a.ws;
     p.tile_state = (uint32_t*)a.ws + cf::kCtlWords;
     p.status = a.status;
@@ -907,32 +910,22 @@ cudaError_t launch_compress_fused(const CompressArgs& a, cudaStream_t st) {
     const auto count = any_tau ? cf::compress_fused_kernel<cf::kCountOnly, 1, true> : cf::compress_fused_kernel<cf::kCountOnly, 1, false>;
     const auto full = any_tau ? cf::compress_fused_kernel<cf::kLookBack, 1, true> : cf::compress_fused_kernel<cf::kLookBack, 1, false>;
     if (a.count_only) {   // budget search: per-head cluster counts only
-        count<<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
         note_launches(1);
+        return launch_in_order(count, dim3(grid), cf::kThreads, cf::kSmemBytes, st, p);
     } else if (a.flags & SC_FLAG_TWO_PASS) {
         cf::Params<1> pc = p;
         pc.layer[0].assign = nullptr;
-        count<<<grid, cf::kThreads, cf::kSmemBytes, st>>>(pc);
-        full<<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
         note_launches(2);
+        const cudaError_t e = launch_in_order(count, dim3(grid), cf::kThreads, cf::kSmemBytes, st, pc);
+        return e != cudaSuccess ? e : launch_in_order(full, dim3(grid), cf::kThreads, cf::kSmemBytes, st, p);
     } else {
         // With SC_FLAG_OVERLAP_PREV the kernel may start while the one enqueued before it on the stream is
         // still draining (the caller has promised they share nothing either writes): the tail of one
         // layer's persistent blocks then overlaps the start of the next layer's.
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(grid);
-        cfg.blockDim = dim3(cf::kThreads);
-        cfg.dynamicSmemBytes = cf::kSmemBytes;
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = (a.flags & SC_FLAG_OVERLAP_PREV) ? 1 : 0;
+        p.overlap = (a.flags & SC_FLAG_OVERLAP_PREV) ? 1 : 0;
         note_launches(1);
-        return cudaLaunchKernelEx(&cfg, full, p);
+        return launch_in_order(full, dim3(grid), cf::kThreads, cf::kSmemBytes, st, p);
     }
-    return cudaGetLastError();
 }
 
 // Several layers in one launch (sc_compress_layers): the (layer, sequence, head) units take the tickets in turn,
@@ -953,9 +946,8 @@ cudaError_t launch_compress_fused_layers(const CompressArgs& a, const sc_compres
     const int64_t max_tiles = (int64_t)L * a.B * a.Hkv * a.n_tile_cap;
     const int grid = (int)(max_tiles < resident ? max_tiles : resident);
     const auto full = a.tau < 0.f ? cf::compress_fused_kernel<cf::kLookBack, cf::kMaxLayers, true> : cf::compress_fused_kernel<cf::kLookBack, cf::kMaxLayers, false>;
-    full<<<grid, cf::kThreads, cf::kSmemBytes, st>>>(p);
     note_launches(1);
-    return cudaGetLastError();
+    return launch_in_order(full, dim3(grid), cf::kThreads, cf::kSmemBytes, st, p);
 }
 
 size_t compress_fused_layers_ws_bytes(int32_t L, int32_t B, int32_t Hkv, int32_t n) {

@@ -22,6 +22,7 @@ gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d
             float tau_host, const float* __restrict__ tau_dev, const int32_t* __restrict__ skip,
             int32_t* __restrict__ assign, int32_t* __restrict__ seg_p) {
     __shared__ float norms[kGenWarps][SC_MAX_CHUNK_LEN];
+    in_stream_order();
     if (skip != nullptr && *skip != 0) return;
     const float tau = tau_dev != nullptr ? *tau_dev : tau_host;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane & 7, rsub = lane >> 3;
@@ -107,7 +108,7 @@ scan_generic(int Hkv, const int32_t* __restrict__ seq_seg_off, int seg_stride,
              int32_t* __restrict__ core_len, int cap, int32_t* status, const int32_t* __restrict__ skip,
              int count_only) {
     __shared__ int wt[8];
-    wait_for_previous();
+    in_stream_order();
     if (skip != nullptr && *skip != 0) return;
     const int b = blockIdx.x / Hkv, h = blockIdx.x % Hkv;
     const int s0 = min(seq_seg_off[b], seg_stride), s1 = min(seq_seg_off[b + 1], seg_stride);
@@ -141,7 +142,7 @@ merge_generic(const T* __restrict__ K, const T* __restrict__ V, sc_strides st, i
               const int32_t* __restrict__ assign, const int32_t* __restrict__ seg_core_off,
               T* __restrict__ core_k, T* __restrict__ core_v, int32_t* __restrict__ count, int cap) {
     constexpr int kWords = SC_MAX_CHUNK_LEN / 32;
-    wait_for_previous();
+    in_stream_order();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int n_seg = min(*n_seg_p, seg_stride);
     const int64_t items = 2 * (int64_t)n_seg * Hkv;
@@ -226,18 +227,17 @@ static cudaError_t run(const CompressArgs& a, cudaStream_t st) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int grid = sms * 8;
     auto gsc = a.d <= 128 ? gsc_generic<T, 4> : gsc_generic<T, 8>;
-    gsc<<<grid, kGenWarps * 32, 0, st>>>((const T*)a.K, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off, a.n_seg, seg_stride, a.tau, a.tau_dev,
-                                         a.skip, assign, seg_p);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_in_order(gsc, dim3(grid), kGenWarps * 32, 0, st, (const T*)a.K, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off,
+                                    a.n_seg, seg_stride, a.tau, a.tau_dev, a.skip, assign, seg_p);
     if (e != cudaSuccess) return e;
-    e = launch_after_previous(scan_generic, dim3(a.B * a.Hkv), 256, st, a.Hkv, a.seq_seg_off, seg_stride, (const int32_t*)seg_p,
+    e = launch_in_order(scan_generic, dim3(a.B * a.Hkv), 256, 0, st, a.Hkv, a.seq_seg_off, seg_stride, (const int32_t*)seg_p,
                               seg_core_off, a.core_len, a.cap, a.status, a.skip, a.count_only);
     if (e != cudaSuccess) return e;
     if (a.count_only) {   // budget search: per-head cluster counts only
         note_launches(2);
         return cudaSuccess;
     }
-    e = launch_after_previous(a.d <= 128 ? merge_generic<T, 1> : merge_generic<T, 2>, dim3(grid), kGenWarps * 32, st, (const T*)a.K,
+    e = launch_in_order(a.d <= 128 ? merge_generic<T, 1> : merge_generic<T, 2>, dim3(grid), kGenWarps * 32, 0, st, (const T*)a.K,
                               (const T*)a.V, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off, a.n_seg, seg_stride, (const int32_t*)assign,
                               (const int32_t*)seg_core_off, (T*)a.core_k, (T*)a.core_v, a.count, a.cap);
     if (e != cudaSuccess) return e;

@@ -30,6 +30,7 @@ decode_generic(const T* __restrict__ q, int Hq, int Hkv, int d, const T* __restr
     __shared__ __align__(16) float so[kDecWarps][kDecHeads][kDecMaxD];   // the warps' sums
     __shared__ float sm[kDecWarps][kDecHeads], sl[kDecWarps][kDecHeads];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane & 7, rsub = lane >> 3;
+    in_stream_order();
     const int G = Hq / Hkv, groups = (G + kDecHeads - 1) / kDecHeads;
     // blockIdx.x = ((b * Hkv + h) * groups + group) * n_split + split
     const int split = blockIdx.x % n_split, hg = (blockIdx.x / n_split) % (Hkv * groups), b = blockIdx.x / n_split / (Hkv * groups);
@@ -163,7 +164,7 @@ combine_generic(int64_t heads, int d, int n_split, const float* __restrict__ par
     __shared__ float sw[kDecWarps][64];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t hd = (int64_t)blockIdx.x * kDecWarps + w;
-    wait_for_previous();
+    in_stream_order();
     if (hd >= heads) return;
     const float* pr = part + hd * n_split * (d + 2);
     float2 ml[2];   // (m, l) of splits lane, lane + 32
@@ -214,16 +215,12 @@ static cudaError_t run(const DecodeArgs& a, cudaStream_t st) {
     const int64_t blocks = (int64_t)n_split * a.Hkv * groups * a.B;
     if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
     const unsigned grid = (unsigned)blocks;
-    if (a.d <= 128)
-        decode_generic<T, 4><<<grid, kDecWarps * 32, 0, st>>>((const T*)a.q, a.Hq, a.Hkv, a.d, (const T*)a.core_k, (const T*)a.core_v,
-                                                              a.count, a.cap, a.core_len, scale, n_split, (float*)a.ws);
-    else
-        decode_generic<T, 8><<<grid, kDecWarps * 32, 0, st>>>((const T*)a.q, a.Hq, a.Hkv, a.d, (const T*)a.core_k, (const T*)a.core_v,
-                                                              a.count, a.cap, a.core_len, scale, n_split, (float*)a.ws);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_in_order(a.d <= 128 ? decode_generic<T, 4> : decode_generic<T, 8>, dim3(grid), kDecWarps * 32, 0, st,
+                                    (const T*)a.q, a.Hq, a.Hkv, a.d, (const T*)a.core_k, (const T*)a.core_v, a.count, a.cap,
+                                    a.core_len, scale, n_split, (float*)a.ws);
     if (e != cudaSuccess) return e;
     const int64_t heads = (int64_t)a.B * a.Hq;
-    e = launch_after_previous(combine_generic<T>, dim3(div_up(heads, kDecWarps)), kDecWarps * 32, st, heads, a.d, n_split,
+    e = launch_in_order(combine_generic<T>, dim3(div_up(heads, kDecWarps)), kDecWarps * 32, 0, st, heads, a.d, n_split,
                               (const float*)a.ws, (T*)a.out);
     if (e != cudaSuccess) return e;
     note_launches(2);

@@ -33,6 +33,8 @@ namespace dm {
 
 namespace cg = cooperative_groups;
 
+enum LaunchMode { kOrdinary = 0, kOverlapped = 1, kChained = 2 };
+
 constexpr int kWarps = 4;
 constexpr int kStages = 3;
 constexpr int kTile = 16;                       // rows per warp tile
@@ -201,7 +203,7 @@ __device__ __forceinline__ void ticket_and_merge(const float* __restrict__ part,
 __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm)
 decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __nv_bfloat16* __restrict__ core_k,
                   const __nv_bfloat16* __restrict__ core_v, const int32_t* __restrict__ count, int cap,
-                  const int32_t* __restrict__ core_len, float scale_log2, int n_split, int min_split, int rows_block, int q_from_prev,
+                  const int32_t* __restrict__ core_len, float scale_log2, int n_split, int min_split, int rows_block, int mode,
                   __nv_bfloat16* __restrict__ out, float* __restrict__ part, int32_t* __restrict__ tickets) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ float sh_m[kWarps][8];
@@ -213,11 +215,11 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const int G = Hq / Hkv;
     const int bh = b * Hkv + h;
-    // Let the next kernel of the stream start beside this one if it was launched with programmatic
-    // stream serialization (a no-op otherwise).  Whatever this block reads before its own
-    // griddepcontrol.wait below (core_len, cores, counts) must not be written by a kernel that may
-    // still be running then; that is the caller's promise when it asks for an overlapped launch.
-    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    // An ordinary launch waits here for the kernel before it.  Under an overlapped one the next kernel may start beside
+    // this one, and whatever this block reads before its own griddepcontrol.wait below (core_len, cores, counts) must not
+    // be written by a kernel that may still be running then; that is the caller's promise when it asks for one.
+    if (mode == kOrdinary) in_stream_order();
+    else asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int len = max(min(core_len[bh], cap), 0);
     const int tiles_total = (len + kTile - 1) / kTile;
     // The split count was chosen from the capacity; a head that is far from full is shared out among fewer blocks
@@ -273,7 +275,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     // Chained launch (SC_FLAG_OVERLAP_CHAIN): q is the preceding kernel's product.  The cores' first
     // tiles are on their way to shared memory and the rest of the block's share to L2; only now wait
     // for that kernel to complete (and its writes to be visible), then read q.
-    if (q_from_prev) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    if (mode == kChained) asm volatile("griddepcontrol.wait;\n" ::: "memory");
 
     // q^T as the B operand of every k-step: b0 = q[head g][16ks + 2tig, +1], b1 = same + 8
     uint32_t qb[8][2];
@@ -595,15 +597,15 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = (a.flags & (SC_FLAG_OVERLAP_PREV | SC_FLAG_OVERLAP_CHAIN)) ? 2 : 1;
-    const int q_from_prev = (a.flags & SC_FLAG_OVERLAP_CHAIN) ? 1 : 0;
+    cfg.numAttrs = 2;
+    const int mode = (a.flags & SC_FLAG_OVERLAP_CHAIN) ? dm::kChained : (a.flags & SC_FLAG_OVERLAP_PREV) ? dm::kOverlapped : dm::kOrdinary;
     // fewest blocks a head is shared out among, however short it is: three blocks per SM over the launch
     const int heads = a.B * a.Hkv;
     const int min_split = (3 * sms_of[dev] + heads - 1) / heads;
     note_launches(1);
     return cudaLaunchKernelEx(&cfg, dm::decode_mma_kernel, (const __nv_bfloat16*)a.q, a.Hq, a.Hkv,
                               (const __nv_bfloat16*)a.core_k, (const __nv_bfloat16*)a.core_v, a.count, a.cap,
-                              a.core_len, scale, plan.n_split, min_split, dm::rows_per_block(a.B, a.Hkv, a.cap), q_from_prev, (__nv_bfloat16*)a.out, part, tickets);
+                              a.core_len, scale, plan.n_split, min_split, dm::rows_per_block(a.B, a.Hkv, a.cap), mode, (__nv_bfloat16*)a.out, part, tickets);
 }
 
 }  // namespace sc

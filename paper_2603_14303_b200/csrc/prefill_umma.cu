@@ -134,17 +134,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     const int qt = blockIdx.x / n_split, h = blockIdx.y, b = blockIdx.z;
     const int G = p.Hq / p.Hkv, bh = b * p.Hkv + h;
     const int rows_total = G * p.m;                           // query rows of this (sequence, KV head)
-    const int len = max(min(p.core_len[bh], p.cap), 0);
-    const int nt_all = (len + kT - 1) / kT;                   // key tiles of the head
-    const int per_split = (nt_all + n_split - 1) / n_split;
-    const int t_lo = min(split * per_split, nt_all);          // this CTA's tiles: [t_lo, t_lo + nt)
-    const int nt = min(t_lo + per_split, nt_all) - t_lo;
-    const long long q_row0 = ((long long)b * p.Hq + (long long)h * G) * p.m + (long long)qt * kT;
     const uint32_t sbase = smem_u32(smem);
-    if ((sbase & 1023u) != 0u) {   // the swizzled addressing assumes this; uniform over the block
-        if (threadIdx.x == 0) set_status(p.status, SC_ERR_CUDA);
-        return;
-    }
     float* lc_s = reinterpret_cast<float*>(smem + kSmLc);     // [2][128] log2(count) of the tile's keys
     __nv_bfloat16* mx_s = reinterpret_cast<__nv_bfloat16*>(smem + kSmMx);   // [2][2][128] each half's row maximum, rounded up
     float* ls_s = reinterpret_cast<float*>(smem + kSmMx);     // [2][128] at the end: each half's row sum
@@ -178,6 +168,19 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     fence_after_sync();
     const uint32_t tmem = *tmem_slot;
 
+    in_stream_order();   // everything above needs nothing from the kernel before
+    const int len = max(min(p.core_len[bh], p.cap), 0);
+    const int nt_all = (len + kT - 1) / kT;                   // key tiles of the head
+    const int per_split = (nt_all + n_split - 1) / n_split;
+    const int t_lo = min(split * per_split, nt_all);          // this CTA's tiles: [t_lo, t_lo + nt)
+    const int nt = min(t_lo + per_split, nt_all) - t_lo;
+    const long long q_row0 = ((long long)b * p.Hq + (long long)h * G) * p.m + (long long)qt * kT;
+    if ((sbase & 1023u) != 0u) {   // the swizzled addressing assumes this; uniform over the block
+        if (tid == 0) set_status(p.status, SC_ERR_CUDA);
+        __syncthreads();
+        if (warp == 1) tmem_dealloc(tmem, kTmemCols);
+        return;
+    }
     if (warp == 0) {
         if (lane == 0 && nt > 0) {   // ---- TMA producer ----
             mbar_expect_tx(q_full, kTile);
@@ -506,6 +509,7 @@ __global__ void __launch_bounds__(128) prefill_generic_kernel(const T* __restric
                                                               const int32_t* __restrict__ count, int cap,
                                                               const int32_t* __restrict__ core_len, float scale_log2, int causal,
                                                               T* __restrict__ out) {
+    in_stream_order();
     const int lane = threadIdx.x & 31;
     const long long it = (long long)blockIdx.x * 4 + (threadIdx.x >> 5);
     if (it >= (long long)B * Hq * m) return;
@@ -606,25 +610,25 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
             cfg.blockDim = dim3(kThreads);
             cfg.dynamicSmemBytes = kSmemBytes;
             cfg.stream = st;
-            cudaLaunchAttribute attr[1];
+            cudaLaunchAttribute attr[2];
             attr[0].id = cudaLaunchAttributeClusterDimension;
             attr[0].val.clusterDim.x = n_split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+            attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[1].val.programmaticStreamSerializationAllowed = 1;
             cfg.attrs = attr;
-            cfg.numAttrs = 1;
+            cfg.numAttrs = 2;
             note_launches(1);
             return cudaLaunchKernelEx(&cfg, prefill_umma_kernel, p);
         }
     }
     const unsigned blocks = (unsigned)((q_rows + 3) / 4);
-    if (a.dt == SC_BF16)
-        prefill_generic_kernel<__nv_bfloat16><<<blocks, 128, 0, st>>>((const __nv_bfloat16*)a.q, a.B, a.Hq, a.Hkv, a.m, a.d,
-            (const __nv_bfloat16*)a.core_k, (const __nv_bfloat16*)a.core_v, a.count, a.cap, a.core_len, scale_log2, causal,
-            (__nv_bfloat16*)a.out);
-    else
-        prefill_generic_kernel<float><<<blocks, 128, 0, st>>>((const float*)a.q, a.B, a.Hq, a.Hkv, a.m, a.d, (const float*)a.core_k,
-            (const float*)a.core_v, a.count, a.cap, a.core_len, scale_log2, causal, (float*)a.out);
     note_launches(1);
-    return cudaGetLastError();
+    if (a.dt == SC_BF16)
+        return launch_in_order(prefill_generic_kernel<__nv_bfloat16>, dim3(blocks), 128, 0, st, (const __nv_bfloat16*)a.q, a.B, a.Hq, a.Hkv, a.m,
+                               a.d, (const __nv_bfloat16*)a.core_k, (const __nv_bfloat16*)a.core_v, a.count, a.cap, a.core_len, scale_log2,
+                               causal, (__nv_bfloat16*)a.out);
+    return launch_in_order(prefill_generic_kernel<float>, dim3(blocks), 128, 0, st, (const float*)a.q, a.B, a.Hq, a.Hkv, a.m, a.d,
+                           (const float*)a.core_k, (const float*)a.core_v, a.count, a.cap, a.core_len, scale_log2, causal, (float*)a.out);
 }
 
 }  // namespace sc
