@@ -10,13 +10,10 @@
 //     O^T[128 dims x 8 heads] += V_tile^T . P^T              (ldmatrix.trans, P^T via movmatrix,
 //                                                             as a bf16 pair: leading part + remainder)
 // Warps are merged in a fixed order through shared memory into one (m, l, O) partial per block.
-// When the launch is about one wave of blocks, the splits of a head form a thread-block cluster
-// and fold their partials through distributed shared memory, each block its own slice of the
-// output (no partial leaves the SMs); otherwise, or when a head needs several clusters, partials go
-// to global memory and the last block of a head to arrive (atomic ticket, no waiting) merges them.
-// In such a launch of several waves the split count comes from the capacity, which the host knows; how many of
-// those blocks a head really uses is settled by each block from the head's length (about 1024 rows a block, 768 in the largest launches, but
-// enough blocks over the launch to fill the GPU three times): the others take their ticket and leave.
+// The splits of a head form a thread-block cluster and fold their partials through distributed shared memory, each
+// block its own slice of the output (no partial leaves the SMs).  Where a head has several clusters, or blocks outside
+// clusters, partials go to global memory and the last one of a head to arrive (atomic ticket, no waiting) merges them.
+// How many splits: plan_for.
 // Every order is fixed, so results are bit-reproducible.
 //
 // Launch modes: ordinary; overlapped with the preceding kernel (programmatic stream
@@ -24,6 +21,8 @@
 // in addition q is read only after that wait (q is the preceding kernel's product) while the cores
 // were requested before it.
 #include <cooperative_groups.h>
+
+#include <mutex>
 
 #include "common.cuh"
 
@@ -46,14 +45,11 @@ constexpr int kWarpBytes = kStages * kStageBytes;
 constexpr int kSmemBytes = kWarps * kWarpBytes;
 constexpr int kPartStride = 8 * kD + 16;        // floats per (b, h, split): acc[8 heads][128], m[8], l[8]
 constexpr int kCtasPerSm = 2;                   // two kernels (consecutive layers) can be co-resident
-constexpr size_t kL2PrefetchBytes = 512 * 1024;  // per tensor and block
 constexpr float kMaxSlack = 8.f;                // log2 units a score may exceed the running maximum before it is raised
 constexpr int kMergeGroup = 16;                 // cluster partials folded per round by the merging block
 constexpr int kMaxCluster = 16;                 // blocks per cluster (more than 8 needs the non-portable opt-in)
-constexpr int kRowsPerBlock = 1024;              // rows a block should stream at least, where the head's length allows ...
-constexpr int kRowsPerBlockBig = 768;            // ... in a launch over kBigLaunchRows rows of capacity (more, shorter blocks keep HBM busier there)
-constexpr long long kBigLaunchRows = 1300000;
-constexpr int kCapRowsPerSplit = 1408;           // of capacity (heads are usually half full or less): about 700 rows a block
+constexpr int kCapRowsPerBlock = 1408;          // rows of capacity per block from which a head gets another cluster (heads are usually half full or less)
+constexpr int kMaxSlots = 160;                  // partials in global memory over the launch (at least one per head)
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -146,24 +142,23 @@ __device__ __forceinline__ void issue_tile(uint32_t stage, const __nv_bfloat16* 
 }
 
 // Several partials per head in global memory (one per cluster, or per block outside clusters): the last block
-// to arrive merges the first `n_parts` of them (the others belong to blocks that found no tiles).  All threads of
-// the block call it.  The cluster barrier / fence before the call orders this block's partial stores before its
+// to arrive merges the `n_parts` of them.  All threads of the block call it.  The cluster barrier / fence before the call orders this block's partial stores before its
 // ticket, whose release makes them visible to whoever reads the ticket with acquire (the last arrival); that
 // block's other threads are ordered behind its thread 0 by the barrier below and read the partials from L2.
 __device__ __forceinline__ void ticket_and_merge(const float* __restrict__ part, int32_t* __restrict__ tickets, int bh,
-                                                 int n_expected, int n_parts, int G, int Hq, int b, int h,
+                                                 int n_parts, int G, int Hq, int b, int h,
                                                  __nv_bfloat16* __restrict__ out, int* sh_last_p) {
     if (threadIdx.x == 0) {
         int t;
         asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;\n" : "=r"(t) : "l"(tickets + bh) : "memory");
-        *sh_last_p = (t == n_expected - 1);
+        *sh_last_p = (t == n_parts - 1);
         if (*sh_last_p) tickets[bh] = 0;   // leave the counter ready for the next call
     }
     __syncthreads();
     if (!*sh_last_p) return;
     // One thread per (head, four output columns); the partials are folded sixteen at a time, all of a
     // group's loads in flight together (one round trip to L2 per group).
-    const float* hp = part + (size_t)bh * n_expected * kPartStride;
+    const float* hp = part + (size_t)bh * n_parts * kPartStride;
     for (int e4 = threadIdx.x; e4 < G * (kD / 4); e4 += kWarps * 32) {
         const int hd = e4 / (kD / 4), d4 = (e4 % (kD / 4)) * 4;
         float gm = -INFINITY, lsum = 0.f;
@@ -203,7 +198,7 @@ __device__ __forceinline__ void ticket_and_merge(const float* __restrict__ part,
 __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm)
 decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __nv_bfloat16* __restrict__ core_k,
                   const __nv_bfloat16* __restrict__ core_v, const int32_t* __restrict__ count, int cap,
-                  const int32_t* __restrict__ core_len, float scale_log2, int n_split, int min_split, int rows_block, int mode,
+                  const int32_t* __restrict__ core_len, float scale_log2, int n_split, int mode,
                   __nv_bfloat16* __restrict__ out, float* __restrict__ part, int32_t* __restrict__ tickets) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ float sh_m[kWarps][8];
@@ -222,17 +217,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     else asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int len = max(min(core_len[bh], cap), 0);
     const int tiles_total = (len + kTile - 1) / kTile;
-    // The split count was chosen from the capacity; a head that is far from full is shared out among fewer blocks
-    // (about rows_block rows each: shorter blocks are mostly prologue and merge), the others find no tiles and
-    // hand in an empty partial.  Not inside a cluster, whose blocks are few and fold on chip.
-    int eff_split = n_split;
-    if (cg::this_cluster().num_blocks() == 1) eff_split = min(n_split, max(min_split, (len + rows_block - 1) / rows_block));
-    const int tiles_per_split = (tiles_total + eff_split - 1) / eff_split;
-    if (split >= eff_split) {   // a block without tiles: it only takes its ticket (and merges, if it is the last)
-        asm volatile("griddepcontrol.wait;\n" ::: "memory");   // no global write before the preceding kernel is complete
-        ticket_and_merge(part, tickets, bh, n_split, eff_split, G, Hq, b, h, out, &sh_last);
-        return;
-    }
+    const int tiles_per_split = (tiles_total + n_split - 1) / n_split;
     const int t0 = min(split * tiles_per_split, tiles_total);
     const int t1 = min(t0 + tiles_per_split, tiles_total);
     // this warp's tiles: t0 + warp, t0 + warp + kWarps, ...
@@ -242,21 +227,6 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     const __nv_bfloat16* vh = core_v + (size_t)bh * cap * kD;
     const int32_t* ch = count ? count + (size_t)bh * cap : nullptr;
     const uint32_t wbase = smem_u32(smem) + warp * kWarpBytes;
-
-    // Ask L2 for this block's whole share up front (bounded), so that under an overlapped launch
-    // the HBM reads run while the preceding kernel is still finishing.
-    if (threadIdx.x == 0 && t1 > t0) {
-        const int r0 = t0 * kTile, r1 = min(t1 * kTile, len);
-        size_t bytes = (size_t)(r1 - r0) * kRowBytes;
-        if (bytes > kL2PrefetchBytes) bytes = kL2PrefetchBytes;
-        const char* pk = reinterpret_cast<const char*>(kh + (size_t)r0 * kD);
-        const char* pv = reinterpret_cast<const char*>(vh + (size_t)r0 * kD);
-        for (size_t off = 0; off < bytes; off += 65536) {
-            const uint32_t sz = (uint32_t)min((size_t)65536, bytes - off);
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(pk + off), "r"(sz) : "memory");
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(pv + off), "r"(sz) : "memory");
-        }
-    }
 
     uint32_t soff[8];   // this lane's eight chunk places inside a K or V tile (see issue_tile)
 #pragma unroll
@@ -273,7 +243,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     }
 
     // Chained launch (SC_FLAG_OVERLAP_CHAIN): q is the preceding kernel's product.  The cores' first
-    // tiles are on their way to shared memory and the rest of the block's share to L2; only now wait
+    // tiles are on their way to shared memory; only now wait
     // for that kernel to complete (and its writes to be visible), then read q.
     if (mode == kChained) asm volatile("griddepcontrol.wait;\n" ::: "memory");
 
@@ -439,7 +409,6 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     const int n_clusters = n_split / csize, cidx = split / csize;   // clusters per head, this one's index
     float* my_part = part + ((size_t)bh * n_clusters + cidx) * kPartStride;
     const bool direct = n_clusters == 1;   // this cluster holds the whole head: its fold is the result
-    const int n_parts = csize == 1 ? eff_split : n_clusters;   // partials that hold something
     const int slice = (G * (kD / 4) + csize - 1) / csize;
     cluster.sync();
     // Nothing has been written to global memory so far (the block partials live in shared memory).  Under
@@ -486,48 +455,54 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     if (direct || crank != 0) return;
 
     // ---- several partials per head: the last block to arrive merges them ----
-    ticket_and_merge(part, tickets, bh, n_clusters, n_parts, G, Hq, b, h, out, &sh_last);
+    ticket_and_merge(part, tickets, bh, n_clusters, G, Hq, b, h, out, &sh_last);
 }
 
 // Block split of one head: how many blocks stream it, and how they are grouped into clusters.
 struct SplitPlan { int n_split, cluster; };
+// Largest number of clusters of c blocks (c = 2..16) that are resident at once, two blocks per SM: fit[c].
+struct Resident { int sms; int fit[kMaxCluster + 1]; };
 
-inline int splits_for(int B, int Hkv, int cap, int sms) {
-    const int heads = B * Hkv;
-    int s = sms / heads;   // one block per SM, so the next layer's blocks fit beside this one's
-    // ... unless that leaves a block thousands of rows to stream alone (many heads, long caches): then several
-    // waves of shorter blocks keep HBM busier (measured: 0.81 -> 1.06 of the copy peak at 128 heads x 8K rows)
-    const int by_len = (cap + kCapRowsPerSplit - 1) / kCapRowsPerSplit;
-    if (by_len > s) s = by_len;
-    const int max_by_rows = (cap + 4 * kTile - 1) / (4 * kTile);   // at least 64 rows per split
-    if (s > max_by_rows) s = max_by_rows;
-    if (s > 256) s = 256;
-    return s < 1 ? 1 : s;
+inline int head_slots(long long heads, int cap) {   // most partials a head can leave in global memory
+    const int by_rows = (cap + 63) / 64;
+    const int s = heads >= kMaxSlots ? 1 : (int)(kMaxSlots / heads);
+    return s < by_rows ? s : (by_rows < 1 ? 1 : by_rows);
 }
 
-// Splits are grouped into clusters whose blocks fold their partials through distributed shared memory
-// when the whole launch is about one wave of blocks (few heads: the latency of the merge is then a large
-// part of the launch).  One cluster per head (no partial ever leaves the SMs) whenever the wanted split count is within a
-// quarter of the largest cluster; otherwise as few equal clusters as cover it.
-inline int rows_per_block(int B, int Hkv, int cap) { return (long long)B * Hkv * cap >= kBigLaunchRows ? kRowsPerBlockBig : kRowsPerBlock; }
-
-inline SplitPlan plan_for(int B, int Hkv, int cap, int sms, int cmax) {
-    const int s0 = splits_for(B, Hkv, cap, sms);
-    if (s0 <= 1 || cmax <= 1) return {s0, 1};
-    // Several waves of blocks (many heads): a block that waits at a cluster barrier holds an SM slot the next
-    // wave wants, and the merge is a small part of such a launch; there every block is a cluster of its own,
-    // leaves its partial in global memory and goes (measured: clusters of 6 cost 7 % at 128 heads x 8K rows).
-    if ((long long)B * Hkv * s0 > 2LL * sms) {
-        // ... and the shares are cut finer (a head that is full streams kRowsPerBlock rows per block; how many of
-        // the blocks a shorter head uses is settled in the kernel, from its length)
-        const int rpb = rows_per_block(B, Hkv, cap);
-        const int fine = (cap + rpb - 1) / rpb;
-        const int s1 = fine > s0 ? fine : s0;
-        return {s1 > 256 ? 256 : s1, 1};
+// The rules and what they were measured against (us per layer, Llama-shaped heads of 128 columns, 2 x 148 block slots; the
+// plan before took splits from the capacity alone, up to 256 a head in several waves, and asked L2 for up to 1 MB per
+// block in advance -- which cost more than anything else, 10 to 30 % of every batched or long launch):
+//   - one cluster per head, as wide as lets the clusters of all heads be resident at once: 128 heads x 3.4 K rows, 2 blocks
+//     each, 51.6 -> 41.2; 56 heads x 6.3 K, 5, 43.7 -> 33.9; 32 x 6.3 K, 8, 31.9 -> 22.5; 24 x 12.6 K, 10, 45.7 -> 31.9; 16 x 25 K, 12,
+//     47.0 -> 36.0; 8 x 34 K, 16, 40.2 -> 27.8.  (13 fits 16 heads too and is 3 to 9 % slower than 12.)
+//   - fewer blocks for short capacities, whose time is the fold and the barrier: 8 heads x 0.5 K rows of 1 K capacity: 9 blocks
+//     4.5, 16 blocks 5.0; x 2.1 K of 4 K: 12 blocks 6.1, 16 blocks 6.6; from 8 K of capacity on 16.
+//   - several clusters per head where few heads would leave blocks with thousands of rows: 4 heads x 34 K rows, 3 x 16, 19.7 (one: 21;
+//     21.1 to 43.6 before); not below, the ticket and the merge cost 2: 4 heads x 8.5 K, one cluster 9.2, three 11.1.
+//   - more heads than any cluster width fits: one block per head (256 heads x 3.4 K rows: 82.1, split in two 83.2, 94.0 before).
+//   - a cache without counts is a raw one, whose heads are full and alike: one block per SM outside clusters keeps HBM
+//     busiest (32 heads x 64 K rows, 4 each, 157; 8 each in clusters 166; 192 before; 8 heads x 131 K: 83.5 against 116.9).
+inline SplitPlan plan_for(long long heads, int cap, bool raw, const Resident& res) {
+    const int by_rows = (cap + 4 * kTile - 1) / (4 * kTile);   // at least 64 rows per split
+    if (raw && cap >= 8192) {
+        int s = heads >= res.sms ? 1 : (int)(res.sms / heads);
+        const int slots = head_slots(heads, cap);
+        s = s < 16 ? s : 16 * (s / 16);
+        if (s > slots) s = slots;
+        return {s, s == 2 && heads <= res.fit[2] ? 2 : 1};
     }
-    if (s0 <= cmax + cmax / 4) { const int c = s0 < cmax ? s0 : cmax; return {c, c}; }
-    const int k = (s0 + cmax - 1) / cmax, c = s0 / k;
-    return {c * k, c};
+    int limit = 8 + cap / 1024;
+    if (limit > by_rows) limit = by_rows;
+    if (limit > kMaxCluster) limit = kMaxCluster;
+    int c = 1;
+    for (int w = 2; w <= limit; ++w)
+        if (w != 13 && heads <= res.fit[w]) c = w;
+    if (c < kMaxCluster) return {c, c};
+    int k = (cap + kMaxCluster * kCapRowsPerBlock - 1) / (kMaxCluster * kCapRowsPerBlock);   // clusters per head
+    if (k > res.fit[c] / heads) k = (int)(res.fit[c] / heads);
+    const int slots = head_slots(heads, cap);
+    if (k > slots) k = slots;
+    return {c * (k < 1 ? 1 : k), c};
 }
 
 }  // namespace dm
@@ -541,48 +516,42 @@ size_t decode_mma_counter_bytes(int32_t B, int32_t Hkv) { return sizeof(int32_t)
 
 size_t decode_mma_ws_bytes(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t cap) {
     (void)Hq; (void)d;
-    // tickets (one per (b, head), zero between calls) + partials for the largest split count
-    const int s = dm::plan_for(B, Hkv, cap, 256, dm::kMaxCluster).n_split;
-    const int s2 = dm::plan_for(B, Hkv, cap, 132, dm::kMaxCluster).n_split;
-    const int s3 = dm::plan_for(B, Hkv, cap, 132, 8).n_split;
-    int smax = s > s2 ? s : s2;
-    if (s3 > smax) smax = s3;
-    const int fine = (cap + dm::kRowsPerBlockBig - 1) / dm::kRowsPerBlockBig;   // the finest split of a launch of several waves
-    if (fine > smax) smax = fine > 256 ? 256 : fine;
+    // tickets (one per (b, head), zero between calls) + partials
     return 256 + decode_mma_counter_bytes(B, Hkv) +
-           sizeof(float) * (size_t)B * Hkv * smax * dm::kPartStride;
+           sizeof(float) * (size_t)B * Hkv * dm::head_slots((long long)B * Hkv, cap) * dm::kPartStride;
 }
 
 cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
-    // per device: SM count, the opt-in to large dynamic shared memory, and the largest cluster that can be scheduled
-    static int sms_of[64] = {0}, cmax_of[64] = {0};
+    // per device: SM count, the opt-ins, and how many clusters of each width can be resident at once
+    static dm::Resident res_of[64];
+    static std::once_flag once_of[64];
     int dev = 0;
     cudaGetDevice(&dev);
     dev &= 63;
-    if (sms_of[dev] == 0) {
+    dm::Resident& res = res_of[dev];
+    std::call_once(once_of[dev], [&res, dev] {
         int v = 0;
         cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        res.sms = v < 1 ? 1 : v;
         cudaFuncSetAttribute(dm::decode_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dm::kSmemBytes);
-        int cmax = 8;   // the portable cluster size
-        if (cudaFuncSetAttribute(dm::decode_mma_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        const bool wide = cudaFuncSetAttribute(dm::decode_mma_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        for (int c = 2; c <= dm::kMaxCluster; ++c) {
             cudaLaunchConfig_t probe = {};
-            probe.gridDim = dim3(dm::kMaxCluster, 1, 1);
+            probe.gridDim = dim3(c, 1, 1);
             probe.blockDim = dim3(dm::kWarps * 32);
             probe.dynamicSmemBytes = dm::kSmemBytes;
             cudaLaunchAttribute pa[1];
             pa[0].id = cudaLaunchAttributeClusterDimension;
-            pa[0].val.clusterDim.x = dm::kMaxCluster; pa[0].val.clusterDim.y = 1; pa[0].val.clusterDim.z = 1;
+            pa[0].val.clusterDim.x = c; pa[0].val.clusterDim.y = 1; pa[0].val.clusterDim.z = 1;
             probe.attrs = pa;
             probe.numAttrs = 1;
             int n_clusters = 0;
-            if (cudaOccupancyMaxActiveClusters(&n_clusters, dm::decode_mma_kernel, &probe) == cudaSuccess && n_clusters > 0)
-                cmax = dm::kMaxCluster;
+            res.fit[c] = 0;
+            if ((c <= 8 || wide) && cudaOccupancyMaxActiveClusters(&n_clusters, dm::decode_mma_kernel, &probe) == cudaSuccess) res.fit[c] = n_clusters;
         }
         (void)cudaGetLastError();   // a refused opt-in or probe is not an error of this call
-        cmax_of[dev] = cmax;
-        sms_of[dev] = v > 256 ? 256 : (v < 1 ? 1 : v);
-    }
-    const dm::SplitPlan plan = dm::plan_for(a.B, a.Hkv, a.cap, sms_of[dev], cmax_of[dev]);
+    });
+    const dm::SplitPlan plan = dm::plan_for((long long)a.B * a.Hkv, a.cap, a.count == nullptr, res);
     int32_t* tickets = (int32_t*)a.ws;
     float* part = (float*)((char*)a.ws + decode_mma_counter_bytes(a.B, a.Hkv));
     const float scale = (a.scale == 0.f ? 1.f / sqrtf((float)a.d) : a.scale) * 1.4426950408889634f;
@@ -599,13 +568,10 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     const int mode = (a.flags & SC_FLAG_OVERLAP_CHAIN) ? dm::kChained : (a.flags & SC_FLAG_OVERLAP_PREV) ? dm::kOverlapped : dm::kOrdinary;
-    // fewest blocks a head is shared out among, however short it is: three blocks per SM over the launch
-    const int heads = a.B * a.Hkv;
-    const int min_split = (3 * sms_of[dev] + heads - 1) / heads;
     note_launches(1);
     return cudaLaunchKernelEx(&cfg, dm::decode_mma_kernel, (const __nv_bfloat16*)a.q, a.Hq, a.Hkv,
                               (const __nv_bfloat16*)a.core_k, (const __nv_bfloat16*)a.core_v, a.count, a.cap,
-                              a.core_len, scale, plan.n_split, min_split, dm::rows_per_block(a.B, a.Hkv, a.cap), mode, (__nv_bfloat16*)a.out, part, tickets);
+                              a.core_len, scale, plan.n_split, mode, (__nv_bfloat16*)a.out, part, tickets);
 }
 
 }  // namespace sc
