@@ -18,7 +18,7 @@
 //      published at once; every token's cluster number (rank of its seed) goes to shared memory.
 //   3. Eq. 3: the members' sum of a cluster is a row of M V, M the 0/1 matrix clusters x tokens; M's fragments are made
 //      from the cluster numbers (kept as bf16: comparing two of them gives the 1.0 or 0.0 the product wants), K and V come transposed from their staged rows (ldmatrix.trans), mma.m16n8k16 adds up in
-//      fp32 (products with 1 and 0 are exact).  Sixteen clusters at a time, over the tokens from their first seed to the
+//      fp32 (products with 1 and 0 are exact).  Sixteen clusters of more than one token at a time, over the tokens from their first seed to the
 //      end of their last segment only; each warp takes a quarter of the columns.  Sums are scaled by 1/|S|, rounded once
 //      and stored.  Clusters of one token are copied bit for bit; a sum that is not finite (0 * inf would reach other
 //      clusters) sends the sixteen clusters to a loop over their members.
@@ -29,12 +29,12 @@
 // 7.4 K.  32 layers x 8 heads x 32K tokens in one launch: 1395 -> 1115 us (3.9 -> 4.8 TB/s); 16 sequences x 16K, lognormal
 // chunks, 8 heads, per layer: 500 -> 310 us.  Measured on the way: sums over member rows in cluster order instead of
 // the product, 1245 us / 475 us (single-token chains of shared loads are longer than the products); keys and values
-// released and pooled separately so that the next keys load earlier, +13 %; L2 prefetch of the next tile, +5 %; only
-// clusters of more than one token in the product, +5 %; a second service warp (96 registers a thread), worse throughout.
+// released and pooled separately so that the next keys load earlier, +13 %; L2 prefetch of the next tile, +5 %; a second
+// service warp (96 registers a thread), worse throughout.
 // Long tiles by mma.sync blocks instead of tcgen05: 16 x 16K +8 %.  Masks, segment bounds and seeds without branches per lane,
 // and the code for negative thresholds in instances of its own: 16 x 16K 633 -> 612 us, chunks of 128 tokens 738 -> 589 us (a
 // settled long tile 19 K -> 12 K cycles); one step out of line or not moves a workload by up to 5 % either way.
-// mbarrier waits with a suspend-time hint, tickets staggered between heads: no change.
+// Clusters of one token out of the product: chunks of 8 tokens -7 %, 16 x 16K -3 %, 32K -1 %.  mbarrier waits with a suspend-time hint, tickets staggered between heads: no change.
 //
 // Offsets: a prefix sum over the tiles of each head by decoupled look-back over per-tile status words; tickets are handed
 // out in order, so every predecessor is held by a running block and the bounded wait cannot starve.  A block draws its
@@ -73,7 +73,8 @@ constexpr int kLongNormOff = kBitOff + kMaxRows * 32;        // float[256]
 constexpr int kRankOff = kBitOff + 1024;                     // bf16[256]: cluster of each token (whole numbers to 256 are exact), see rank_slot
 constexpr int kCntOff = kRankOff + kMaxRows * 2;                 // int32[256]: tokens of each cluster
 constexpr int kSeedOff = kCntOff + kMaxRows * 4;             // uint8[256]: the cluster's seed
-constexpr int kEndOff = kSeedOff + kMaxRows;                 // uint16[256]: end of the seed's segment
+constexpr int kListOff = kSeedOff + kMaxRows;                // uint8[256]: the clusters of more than one token, in order
+constexpr int kEndOff = kListOff + kMaxRows;                 // uint16[256]: end of the seed's segment
 constexpr int kMiscOff = kLongNormOff + kMaxRows * 4;        // seeds[8], members[8]; starts[2][4]; geo[2][8]; base, P, tmem slot, flags
 constexpr int kBarOff = kMiscOff + 64 + 32 + 64 + 32;
 constexpr int kSmemBytes = kBarOff + 64;
@@ -394,11 +395,12 @@ __device__ __noinline__ int settle_long_tile(unsigned char* smem, int R, uint32_
 }
 
 // Step 3 for sixteen clusters whose sums are not all finite: each lane one column of the warp's quarter, member by member.
-__device__ __noinline__ void pool_by_members(const unsigned char* tensor, int hs, const unsigned char* smem, int m, int P, int t_lo, int t_hi,
+__device__ __noinline__ void pool_by_members(const unsigned char* tensor, int hs, const unsigned char* smem, bool listed, int m, int n_multi, int t_lo, int t_hi,
                                              __nv_bfloat16* dst, int room, int warp, int lane) {
     const int* cnt = reinterpret_cast<const int*>(smem + kCntOff);
     const int col = warp * 32 + lane;
-    for (int c = 16 * m; c < min(16 * m + 16, P); ++c) {
+    for (int x = 16 * m; x < min(16 * m + 16, n_multi); ++x) {
+        const int c = listed ? (smem + kListOff)[x] : x;
         if (cnt[c] <= 1 || c >= room) continue;
         float sum = 0.f;
         for (int i = t_lo; i < t_hi; ++i)
@@ -429,14 +431,26 @@ __device__ __forceinline__ void pool_tile(unsigned char* smem, int hs, int P, __
     const int j = lane >> 3, r8 = lane & 7;
     const uint32_t b_row = sbase + (warp >> 1) * hs + ((j & 1) * 8 + r8) * kHalfRow;
     const uint32_t off0 = (uint32_t)((((warp & 1) * 4 + (j >> 1)) ^ r8) << 4), off1 = (uint32_t)((((warp & 1) * 4 + 2 + (j >> 1)) ^ r8) << 4);
-    for (int m = 0; m * 16 < P; ++m) {
-        const int k_lo = seedrow[16 * m] >> 4, k_hi = (seg_end[min(16 * m + 15, P - 1)] + 15) >> 4;
+    // the clusters of more than one token, in order (every warp writes the same list)
+    unsigned char* list = smem + kListOff;
+    int n_multi = NT > 1 ? 0 : P;   // (a long tile has few clusters of one token: all its clusters take part)
+    for (int x0 = 0; NT > 1 && x0 < P; x0 += 32) {
+        const bool multi = x0 + lane < P && cnt[x0 + lane] > 1;
+        const uint32_t mm = __ballot_sync(kFull, multi);
+        if (multi) list[n_multi + __popc(mm & ((1u << lane) - 1u))] = (unsigned char)(x0 + lane);
+        n_multi += __popc(mm);
+    }
+    __syncwarp();
+    for (int m = 0; m * 16 < n_multi; ++m) {
+        const auto at = [&](int x) { x = min(x, n_multi - 1); return NT > 1 ? (int)list[x] : x; };   // (past the end: the last again)
+        const int la = at(16 * m + g), lb = at(16 * m + 8 + g);
+        const int k_lo = seedrow[at(16 * m)] >> 4, t_hi = seg_end[at(16 * m + 15)], k_hi = (t_hi + 15) >> 4;
         float acc[NT][4][4];
 #pragma unroll
         for (int t = 0; t < NT; ++t)
 #pragma unroll
             for (int nt = 0; nt < 4; ++nt) acc[t][nt][0] = acc[t][nt][1] = acc[t][nt][2] = acc[t][nt][3] = 0.f;
-        const __nv_bfloat162 c0 = __bfloat162bfloat162(__int2bfloat16_rn(16 * m + g)), c1 = __bfloat162bfloat162(__int2bfloat16_rn(16 * m + 8 + g));
+        const __nv_bfloat162 c0 = __bfloat162bfloat162(__int2bfloat16_rn(la)), c1 = __bfloat162bfloat162(__int2bfloat16_rn(lb));
 #pragma unroll 2
         for (int kk = k_lo; kk < k_hi; ++kk) {
             // M's fragment: rows g and g + 8 of the sixteen clusters, tokens 2 tig, +1, +8, +9 of the sixteen
@@ -463,14 +477,14 @@ __device__ __forceinline__ void pool_tile(unsigned char* smem, int hs, int P, __
 #pragma unroll
                 for (int x = 0; x < 4; ++x) check = fmaf(acc[t][nt][x], 0.f, check);
         if (__any_sync(kFull, !(check == 0.f))) {
-            const int t_lo = k_lo * 16, t_hi = seg_end[min(16 * m + 15, P - 1)];
-            pool_by_members(smem, hs, smem, m, P, t_lo, t_hi, dst_k, room, warp, lane);
-            if (NT > 1) pool_by_members(smem + kVOff, hs, smem, m, P, t_lo, t_hi, dst_v, room, warp, lane);
+            const int t_lo = k_lo * 16;
+            pool_by_members(smem, hs, smem, NT > 1, m, n_multi, t_lo, t_hi, dst_k, room, warp, lane);
+            if (NT > 1) pool_by_members(smem + kVOff, hs, smem, NT > 1, m, n_multi, t_lo, t_hi, dst_v, room, warp, lane);
         } else {
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
-                const int c = 16 * m + 8 * hh + g;
-                const int n = c < P ? cnt[c] : 0;
+                const int c = hh ? lb : la;
+                const int n = 16 * m + 8 * hh + g < n_multi ? cnt[c] : 0;
                 if (n > 1 && c < room) {
                     const float inv = __frcp_rn((float)n);
                     const size_t o = (size_t)c * kD + warp * 32 + 2 * tig;
