@@ -2,21 +2,84 @@
 // three kernels per layer -- GSC per segment, prefix sum of cluster counts per (b, head),
 // mean-pool merge per segment.  CUDA-core arithmetic in fp32; serves SC_F32 and is the
 // cross-check of the fused bf16 path.
-// One warp per segment; bounded by the latency of its loads, so several rows are in flight at a time: eight in the
-// similarities (eight lanes per row, four columns per load), four in the merge, whose members come
-// from bit masks of the segment's assignments.  8 heads x 8K tokens of fp32: GSC 101 -> 45 us, merge 83 -> 36 us (50 us
-// with K and V in one warp) against one row at a time.
+// One warp per segment; bounded by the latency of its loads, so all rows of a segment of up to 32 tokens are in flight at
+// once: clustering keeps them in registers for every seed, the merge adds them, eight at a time, to its clusters' sums in shared memory.
+// 8 heads x 8K tokens of fp32, chunks of 20 / 8 tokens (caches cold): clustering 43 / 34 us -> 29 / 20, merge 35 / 41 -> 30 / 31
+// against eight and four rows in flight, which longer segments, larger heads and segments of many clusters still
+// take (101 and 83 us with one row at a time).  Clustering: 128 registers of rows leave three blocks of four warps per SM; four blocks spill, +8 %.
+// The eight lanes of a row group share out the sums of their rows (seven shuffles and one division for eight rows; with
+// 24 and eight, 34 / 39 us).  Merge: the rows in registers and a sum over them per cluster, 35 / 52 us.
 #include "common.cuh"
 
 namespace sc {
 
-constexpr int kGenWarps = 8;
+constexpr int kGenWarps = 4;
+constexpr int kGenBlocks = 3;      // per SM (168 registers a thread): a short segment's rows are kept in registers
+constexpr int kShortSeg = 32;      // rows of a short segment (d <= 128)
+constexpr int kMergeSlots = 16;    // clusters of a short segment summed up in shared memory (8 KB per warp)
+constexpr int kMergeBlocks = 6;
 
-// Algorithm 1 for one segment per warp.  Rows are read straight from global memory, eight at a time: lanes 8r .. 8r + 7
+// Sums over the eight lanes of a row group: x[q] of every lane in, the sum for q = lane % R out (R = 8, 4, 2).
+template <int R>
+__device__ __forceinline__ float group_sums(float (&x)[R], int lane) {
+#pragma unroll
+    for (int o = 1; o < R; o <<= 1) {   // halve the number of sums a lane holds
+        const bool odd = lane & o;
+#pragma unroll
+        for (int q = 0; q < R / (2 * o); ++q) {
+            const float give = odd ? x[2 * q] : x[2 * q + 1], keep = odd ? x[2 * q + 1] : x[2 * q];
+            x[q] = keep + __shfl_xor_sync(kFull, give, o);
+        }
+    }
+#pragma unroll
+    for (int o = R; o < 8; o <<= 1) x[0] += __shfl_xor_sync(kFull, x[0], o);
+    return x[0];
+}
+
+// Algorithm 1 for a segment of at most 4 R rows: all of them are requested at once and stay in registers, R per group of
+// eight lanes; only the seeds' rows are read again.  A lane decides for row (its group) R + lane % R.  Same sums in the
+// same order as the loop for longer ones.
+template <int R, int NC, typename Load, typename Dot>
+__device__ __forceinline__ int short_segment(int l, float tau, int32_t* as, int r, int lane, const Load& load_row, const Dot& dot) {
+    const int row0 = (lane >> 3) * R;
+    float4 v[R][NC];
+    float x[R];
+#pragma unroll
+    for (int q = 0; q < R; ++q) load_row(row0 + q, row0 + q < l, v[q]);
+#pragma unroll
+    for (int q = 0; q < R; ++q) x[q] = dot(v[q], v[q]);
+    const float nj = sqrtf(group_sums<R>(x, lane));
+    unsigned open = 0xffffffffu >> (32 - l);
+    int p = 0, mine = 0;   // mine: seed of token `lane`
+    while (open) {
+        const int i = __ffs(open) - 1;
+        ++p;
+        open &= open - 1;
+        if (lane == i) mine = i;
+        if (!open) break;
+        float4 seed[NC];
+        load_row(i, true, seed);
+        const float ni = __shfl_sync(kFull, nj, (i / R) * 8 + i % R);
+#pragma unroll
+        for (int q = 0; q < R; ++q) x[q] = dot(seed, v[q]);
+        const float prod = group_sums<R>(x, lane);
+        const float sim = (ni == 0.f || nj == 0.f) ? 0.f : prod / (ni * nj);
+        unsigned hits = __ballot_sync(kFull, sim > tau);   // group g's rows in byte g
+        if (R == 4) hits = (hits & 15u) | ((hits >> 4) & 0xf0u) | ((hits >> 8) & 0xf00u) | ((hits >> 12) & 0xf000u);
+        if (R == 2) hits = (hits & 3u) | ((hits >> 6) & 12u) | ((hits >> 12) & 48u) | ((hits >> 18) & 192u);
+        hits &= open;
+        if ((hits >> lane) & 1u) mine = i;
+        open &= ~hits;
+    }
+    if (lane < l) as[lane] = r + mine;
+    return p;
+}
+
+// Algorithm 1 for one segment per warp.  Longer segments' rows are read straight from global memory, eight at a time: lanes 8r .. 8r + 7
 // form the product of row r (of four) with the seed's row, which they hold in registers.  NC: the most 32-column pieces
 // a row has (4 or 8).
 template <typename T, int NC>
-__global__ void __launch_bounds__(kGenWarps * 32)
+__global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks)
 gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d,
             const int32_t* __restrict__ seg_off, const int32_t* __restrict__ n_seg_p, int seg_stride,
             float tau_host, const float* __restrict__ tau_dev, const int32_t* __restrict__ skip,
@@ -27,8 +90,9 @@ gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d
     const float tau = tau_dev != nullptr ? *tau_dev : tau_host;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, sub = lane & 7, rsub = lane >> 3;
     const int n_seg = min(*n_seg_p, seg_stride);
-    const int64_t items = (int64_t)n_seg * Hkv;
-    for (int64_t it = (int64_t)blockIdx.x * kGenWarps + w; it < items; it += (int64_t)gridDim.x * kGenWarps) {
+    const int64_t items = (int64_t)n_seg * Hkv, warps = (int64_t)gridDim.x * kGenWarps;
+    // two segments in a row per warp and step: runs and the delimiters between them alternate
+    for (int64_t it = ((int64_t)blockIdx.x * kGenWarps + w) * 2; it < items; it += (it & 1) ? 2 * warps - 1 : 1) {
         const int s = (int)(it % n_seg), h = (int)(it / n_seg);
         const int a = seg_off[s], e = seg_off[s + 1];
         const int b = a / n, r = a - b * n, l = min(e - a, SC_MAX_CHUNK_LEN);
@@ -46,6 +110,19 @@ gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d
             for (int c = 0; c < NC; ++c) acc = fmaf(x[c].x, y[c].x, fmaf(x[c].y, y[c].y, fmaf(x[c].z, y[c].z, fmaf(x[c].w, y[c].w, acc))));
             return acc;
         };
+        if (l == 1) {
+            if (lane == 0) { as[0] = r; seg_p[(int64_t)h * seg_stride + s] = 1; }
+            continue;
+        }
+        if constexpr (NC == 4) {
+            if (l <= kShortSeg) {
+                const int p = l <= 8 ? short_segment<2, NC>(l, tau, as, r, lane, load_row, dot)
+                              : l <= 16 ? short_segment<4, NC>(l, tau, as, r, lane, load_row, dot)
+                                        : short_segment<8, NC>(l, tau, as, r, lane, load_row, dot);
+                if (lane == 0) seg_p[(int64_t)h * seg_stride + s] = p;
+                continue;
+            }
+        }
         for (int j0 = 0; j0 < l; j0 += 8) {
             float4 v0[NC], v1[NC];
             load_row(j0 + rsub, j0 + rsub < l, v0);
@@ -133,22 +210,24 @@ scan_generic(int Hkv, const int32_t* __restrict__ seq_seg_off, int seg_stride,
 }
 
 // Eq. 3 for one segment of K or of V per warp: fp32 sums in token order, one divide, one rounding.  A lane owns four
-// columns (eight where d > 128); a cluster's members come from ballots over the segment's assignments, four rows
-// requested together.
+// columns (eight where d > 128).  Beyond 32 tokens, 16 clusters (8 KB of sums per warp, six blocks per SM) or 128
+// columns a cluster's members come from ballots over the segment's assignments, four rows requested together.
 template <typename T, int kPer>
-__global__ void __launch_bounds__(kGenWarps * 32)
+__global__ void __launch_bounds__(kGenWarps * 32, kMergeBlocks)
 merge_generic(const T* __restrict__ K, const T* __restrict__ V, sc_strides st, int B, int Hkv, int n, int d,
               const int32_t* __restrict__ seg_off, const int32_t* __restrict__ n_seg_p, int seg_stride,
               const int32_t* __restrict__ assign, const int32_t* __restrict__ seg_core_off,
               T* __restrict__ core_k, T* __restrict__ core_v, int32_t* __restrict__ count, int cap) {
     constexpr int kWords = SC_MAX_CHUNK_LEN / 32;
+    __shared__ __align__(16) float4 sums[kGenWarps][kPer == 1 ? kMergeSlots : 1][32];
     in_stream_order();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int n_seg = min(*n_seg_p, seg_stride);
-    const int64_t items = 2 * (int64_t)n_seg * Hkv;
-    for (int64_t it = (int64_t)blockIdx.x * kGenWarps + w; it < items; it += (int64_t)gridDim.x * kGenWarps) {
-        const bool is_v = it & 1;
-        const int s = (int)((it >> 1) % n_seg), h = (int)((it >> 1) / n_seg);
+    const int64_t segs = (int64_t)n_seg * Hkv, warps = (int64_t)gridDim.x * kGenWarps / 2;   // per tensor
+    const int64_t me = (int64_t)blockIdx.x * kGenWarps + w;
+    const bool is_v = me & 1;
+    for (int64_t it = (me >> 1) * 2; it < segs; it += (it & 1) ? 2 * warps - 1 : 1) {   // two segments in a row, as above
+        const int s = (int)(it % n_seg), h = (int)(it / n_seg);
         const int a = seg_off[s], e = seg_off[s + 1];
         const int b = a / n, r = a - b * n, l = min(e - a, SC_MAX_CHUNK_LEN), nw = (l + 31) >> 5;
         const T* rows = (is_v ? V : K) + b * st.b + h * st.h + (int64_t)r * st.n + lane * 4;
@@ -156,6 +235,44 @@ merge_generic(const T* __restrict__ K, const T* __restrict__ V, sc_strides st, i
         int row = seg_core_off[(int64_t)h * seg_stride + s];
         const int64_t obase = ((int64_t)b * Hkv + h) * cap;
         T* cores = (is_v ? core_v : core_k) + obase * d + lane * 4;
+        if constexpr (kPer == 1) {
+            const int own = lane < l ? as[lane] - r : -1;
+            const unsigned seeds = __ballot_sync(kFull, own == lane);
+            if (l <= kShortSeg && __popc(seeds) <= kMergeSlots) {
+                // rows in token order, eight requested together, each added to its cluster's sum in shared memory (a lane
+                // touches its own four columns only); a cluster's first row starts the sum
+                const bool on = lane * 4 < d;
+                const int rank = __popc(seeds & ((1u << (own & 31)) - 1u));
+                for (int j0 = 0; j0 < l; j0 += 8) {
+                    float4 v[8];
+#pragma unroll
+                    for (int x = 0; x < 8; ++x) v[x] = on && j0 + x < l ? load4(rows + (int64_t)(j0 + x) * st.n) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int x = 0; x < 8; ++x) {
+                        if (j0 + x >= l) break;
+                        float4* to = &sums[w][__shfl_sync(kFull, rank, j0 + x)][lane];
+                        if (!((seeds >> (j0 + x)) & 1u)) {
+                            const float4 t = *to;
+                            v[x].x += t.x; v[x].y += t.y; v[x].z += t.z; v[x].w += t.w;
+                        }
+                        *to = v[x];
+                    }
+                }
+                int c = 0;
+                for (unsigned todo = seeds; todo; todo &= todo - 1, ++c, ++row) {
+                    const int cnt = __popc(__ballot_sync(kFull, own == __ffs(todo) - 1));
+                    if (row >= cap) break;
+                    float4 v = sums[w][c][lane];
+                    if (cnt > 1) {
+                        const float fc = (float)cnt;
+                        v = make_float4(v.x / fc, v.y / fc, v.z / fc, v.w / fc);
+                    }
+                    if (on) store4(cores + (int64_t)row * d, v);
+                    if (lane == 0 && !is_v) count[obase + row] = cnt;
+                }
+                continue;
+            }
+        }
         int mine[kWords];   // seed (relative) of tokens 32 k + lane
 #pragma unroll
         for (int k = 0; k < kWords; ++k) mine[k] = 32 * k + lane < l ? as[32 * k + lane] - r : -1;
@@ -225,7 +342,7 @@ static cudaError_t run(const CompressArgs& a, cudaStream_t st) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int grid = sms * 8;
+    const int grid = sms * 16;
     auto gsc = a.d <= 128 ? gsc_generic<T, 4> : gsc_generic<T, 8>;
     cudaError_t e = launch_in_order(gsc, dim3(grid), kGenWarps * 32, 0, st, (const T*)a.K, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off,
                                     a.n_seg, seg_stride, a.tau, a.tau_dev, a.skip, assign, seg_p);

@@ -1,10 +1,11 @@
 // Generic decode path for Eq. 4 (any dtype, d <= 256 multiple of 8).  One block serves one (sequence, KV head, split of
 // its cores, up to four of its query heads); its four warps take 32-row tiles in turn: eight lanes per row form the
-// scores (so four rows, eight requested ahead, are in flight per warp), one lane per row takes part in the online softmax in
-// fp32, and for the weighted sum a lane owns four columns of every row.  A second kernel combines the splits in order.
+// scores (four rows at a time, sixteen requested ahead), one lane per row takes part in the online softmax in
+// fp32, and for the weighted sum a lane owns four columns of every row, sixteen rows requested together.  A second kernel combines the splits in order.
 // Serves SC_F32 and cross-checks the tensor-core bf16 kernel.
 // Bounded by the latency of its loads: 2162 cores x 8 heads of fp32, 16 splits: 217 + 18 us when a warp served one query
-// head row by row (each row a dependent chain of load, five shuffles and two exponentials), 37 + 7 us like this.
+// head row by row (each row a dependent chain of load, five shuffles and two exponentials), 19 + 7 us like this (37 + 7 with
+// eight rows requested at a time).
 #include "common.cuh"
 
 namespace sc {
@@ -56,7 +57,7 @@ decode_generic(const T* __restrict__ q, int Hq, int Hkv, int d, const T* __restr
         const int nr = min(32, t1 - tb);
         // ln s, in base-2 units (a valid row has count >= 1)
         const float lc = count != nullptr && lane < nr ? log2f((float)max(count[cbase + tb + lane], 1)) : 0.f;
-#pragma unroll 2
+#pragma unroll (16 / NC)
         for (int it = 0; it < 8; ++it) {   // four rows at a time
             const int r = it * 4 + rsub;
             const T* kr = core_k + (cbase + tb + min(r, nr - 1)) * d;
@@ -107,12 +108,12 @@ decode_generic(const T* __restrict__ q, int Hq, int Hkv, int d, const T* __restr
             const int col = (u * 32 + lane) * 4;
             if (col >= d) continue;
             const T* vc = core_v + (cbase + tb) * d + col;
-            for (int r0 = 0; r0 < nr; r0 += 8) {   // eight rows requested together
-                float4 vv[8];
+            for (int r0 = 0; r0 < nr; r0 += 16) {   // sixteen rows requested together
+                float4 vv[16];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) vv[j] = r0 + j < nr ? load4(vc + (size_t)(r0 + j) * d) : make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int j = 0; j < 16; ++j) vv[j] = r0 + j < nr ? load4(vc + (size_t)(r0 + j) * d) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
+                for (int j = 0; j < 16; ++j) {
                     const float4 pv = sp[w][r0 + j];
                     const float pg[kDecHeads] = {pv.x, pv.y, pv.z, pv.w};
 #pragma unroll
