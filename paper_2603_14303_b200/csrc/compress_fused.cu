@@ -17,24 +17,29 @@
 //      of cliques take two.  A member joins the earliest seed among its earlier neighbours.  The tile's cluster count is
 //      published at once; every token's cluster number (rank of its seed) goes to shared memory.
 //   3. Eq. 3: the members' sum of a cluster is a row of M V, M the 0/1 matrix clusters x tokens; M's fragments are made
-//      from the cluster numbers (kept as bf16: comparing two of them gives the 1.0 or 0.0 the product wants), K and V come transposed from their staged rows (ldmatrix.trans), mma.m16n8k16 adds up in
-//      fp32 (products with 1 and 0 are exact).  Sixteen clusters of more than one token at a time, over the tokens from their first seed to the
-//      end of their last segment only; each warp takes a quarter of the columns.  Sums are scaled by 1/|S|, rounded once
-//      and stored.  Clusters of one token are copied bit for bit; a sum that is not finite (0 * inf would reach other
+//      from the cluster numbers (kept as bf16: comparing two of them gives the 1.0 or 0.0 the product wants), K and V come
+//      transposed from their staged rows (ldmatrix.trans), mma.m16n8k16 adds up in fp32 (products with 1 and 0 are exact).
+//      Sixteen clusters of more than one token at a time, over the tokens from their first seed to the end of their last
+//      segment only; each warp takes a quarter of the columns.  Sums are scaled by 1/|S|, rounded once and stored.  Clusters of one token are copied bit for bit; a sum that is not finite (0 * inf would reach other
 //      clusters) sends the sixteen clusters to a loop over their members.
 //
-// What bounds it: the length of a tile's chain of steps with three 64 KB tiles in flight per SM (issue slots a quarter
-// used).  The kernel before this one clustered every segment with one warp's mma.sync tiles and greedy pass and added up
-// member rows on the CUDA cores, nine warps and five block barriers a tile, 13 K warp instructions per 128 tokens; here
-// 7.4 K.  32 layers x 8 heads x 32K tokens in one launch: 1395 -> 1115 us (3.9 -> 4.8 TB/s); 16 sequences x 16K, lognormal
-// chunks, 8 heads, per layer: 500 -> 310 us.  Measured on the way: sums over member rows in cluster order instead of
-// the product, 1245 us / 475 us (single-token chains of shared loads are longer than the products); keys and values
-// released and pooled separately so that the next keys load earlier, +13 %; L2 prefetch of the next tile, +5 %; a second
-// service warp (96 registers a thread), worse throughout.
-// Long tiles by mma.sync blocks instead of tcgen05: 16 x 16K +8 %.  Masks, segment bounds and seeds without branches per lane,
-// and the code for negative thresholds in instances of its own: 16 x 16K 633 -> 612 us, chunks of 128 tokens 738 -> 589 us (a
-// settled long tile 19 K -> 12 K cycles); one step out of line or not moves a workload by up to 5 % either way.
-// Clusters of one token out of the product: chunks of 8 tokens -7 %, 16 x 16K -3 %, 32K -1 %.  mbarrier waits with a suspend-time hint, tickets staggered between heads: no change.
+// What bounds it: one launch over 32 layers x 8 heads x 32K tokens takes 1105 us on resident inputs (4.9 TB/s); copies
+// of the kernel with steps left out take 707 us (loads only), 834 (loads, steps 1 and 2) and 1025 (all but the
+// stores of the means), so step 3's shared-memory traffic and arithmetic are the largest part above the loads, then the stores.
+// A tile of 129..256 tokens spends 12 K cycles on step 2 and holds up the look-back of the tiles behind it.
+// The kernel before this one clustered every segment with one warp's mma.sync tiles and greedy pass and added up member
+// rows on the CUDA cores, nine warps and five block barriers a tile, 13 K warp instructions per 128 tokens (7.4 K here):
+// 1395 us; 16 sequences x 16K, lognormal chunks, 8 heads, per layer 500 us, 300 here; 4 x 64K in chunks of 128 with
+// sc_chunk 794 and 578.
+// Of that: masks, segment bounds and seeds without branches per lane, and the code for negative thresholds in instances
+// of its own, 16 x 16K 633 -> 612 us for two layers, chunks of 128 tokens 738 -> 589 (a settled long tile 19 K -> 12 K cycles);
+// clusters of one token out of the product, chunks of 8 tokens -7 %, 16 x 16K -3 %, 32K -1 %.
+// Measured and not taken: sums over member rows in cluster order instead of the product, 1245 us; keys and values released
+// and pooled separately so that the next keys load earlier, +13 %; L2 prefetch of the next tile, +5 %; a second service
+// warp (96 registers a thread), worse throughout; eight pooling warps (72 registers), +1 %; means written to their seeds'
+// staged rows and copied out in 16-byte pieces, +3 %, and +5 % with the offset awaited only before the copy; products of
+// long tiles by mma.sync, 16 x 16K +8 %; mbarrier waits with a suspend-time hint and tickets staggered between heads, no
+// change.  One step out of line or not moves a workload by up to 5 % either way.
 //
 // Offsets: a prefix sum over the tiles of each head by decoupled look-back over per-tile status words; tickets are handed
 // out in order, so every predecessor is held by a running block and the bounded wait cannot starve.  A block draws its
