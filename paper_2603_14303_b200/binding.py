@@ -401,13 +401,14 @@ def chunk(token_ids: torch.Tensor, delim_ids, max_chunk_len: int = SC_MAX_CHUNK_
     B, n = token_ids.shape
     code, n_seg_cap, n_tile_cap, ws_bytes = _native().chunk_sizes(B, n)
     _check("sc_chunk_bounds", code)
-    new = token_ids.new_empty   # int32 on the same device, as the raw call asks
-    i32 = torch.int32
-    plan = ChunkPlan(B, n, max_chunk_len, new(n_seg_cap + 1, dtype=i32), new(B + 1, dtype=i32), new(1, dtype=i32),
-                     new((B, n_tile_cap + 1), dtype=i32), new(max(B, 1), dtype=i32), n_tile_cap, token_ids.new_zeros(1, dtype=i32))
-    ws = new(ws_bytes, dtype=torch.uint8)
-    sc_chunk(token_ids, delim_ids, max_chunk_len, plan.seg_off, plan.seq_seg_off, plan.n_seg, plan.tile_seg,
-             plan.seq_tile_cnt, ws, plan.status)
+    # one zeroed int32 array for everything (23 us on the host; 27 with an allocation each); the workspace leads, a multiple
+    # of 256 bytes long
+    sizes = ((ws_bytes + 255) // 256 * 64, n_seg_cap + 1, B * (n_tile_cap + 1), B + 1, max(B, 1), 1, 1)
+    ws, seg_off, tile_seg, seq_seg_off, seq_tile_cnt, n_seg, status = \
+        token_ids.new_zeros(sum(sizes), dtype=torch.int32).split_with_sizes(sizes)
+    plan = ChunkPlan(B, n, max_chunk_len, seg_off, seq_seg_off, n_seg, tile_seg.view(B, n_tile_cap + 1), seq_tile_cnt, n_tile_cap,
+                     status)
+    sc_chunk(token_ids, delim_ids, max_chunk_len, seg_off, seq_seg_off, n_seg, plan.tile_seg, seq_tile_cnt, ws, status)
     return plan
 
 
