@@ -28,7 +28,7 @@
 // stores of the means), so step 3's shared-memory traffic and arithmetic are the largest part above the loads, then the stores.
 // A tile of 129..256 tokens spends 12 K cycles on step 2 and holds up the look-back of the tiles behind it.
 // The kernel before this one clustered every segment with one warp's mma.sync tiles and greedy pass and added up member
-// rows on the CUDA cores, nine warps and five block barriers a tile, 13 K warp instructions per 128 tokens (7.4 K here):
+// rows on the CUDA cores, nine warps and five block barriers a tile, 13 K warp instructions per 128 tokens (6.5 K here):
 // 1395 us; 16 sequences x 16K, lognormal chunks, 8 heads, per layer 500 us, 300 here; 4 x 64K in chunks of 128 with
 // sc_chunk 794 and 578.
 // Of that: masks, segment bounds and seeds without branches per lane, and the code for negative thresholds in instances
