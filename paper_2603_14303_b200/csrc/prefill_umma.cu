@@ -28,7 +28,7 @@
 // groups of four warps on alternate tiles with a row per thread and an accumulator each, 569 us.
 // Cluster width: as many CTAs per query tile as let every cluster of the launch be resident at once (asked of the
 // occupancy query: on this GPU 15 clusters of 8 or 9, 11 of 10, 7 of 11 to 16); powers of two up to 8 before.  8 queries per
-// head, 8 KV heads: 10 instead of 8 CTAs, 29 -> 24 us per layer with the above; 16 clusters: 7 instead of 8 (which took
+// head, 8 KV heads: 10 instead of 8 CTAs, 29 -> 24 us per layer with the above (four replicas of the rows, see kRep: 19); 16 clusters: 7 instead of 8 (which took
 // two waves), 64 queries per head 190 -> 132 us for 4 layers.
 // Every wait is bounded; a wait that gives up is reported through the status word.
 // A CUDA-core kernel (one warp per query) serves other dtypes and head sizes.
@@ -82,6 +82,18 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32
           "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
         : "memory");
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&r)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n"
+                 ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]) : "memory");
+}
 __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
@@ -128,6 +140,10 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
     return y;
 }
 
+// kRep: how often the query rows stand in the tile's 128 lanes.  Up to 32 (64) rows they do so four times (twice), and each
+// replica takes a quarter (half) of every key tile -- its weights of the other keys are zero --, so that all eight softmax warps work
+// and a thread has 16 (32) scores a tile instead of 64; the replicas are folded at the end like the CTAs of a split.
+template <int kRep>
 __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_constant__ Params p) {
     extern __shared__ __align__(1024) unsigned char smem[];   // the swizzle pattern repeats every 1024 bytes
     const int n_split = p.n_split, split = blockIdx.x % n_split;   // the CTAs of a cluster are consecutive in x
@@ -184,8 +200,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     if (warp == 0) {
         if (lane == 0 && nt > 0) {   // ---- TMA producer ----
             mbar_expect_tx(q_full, kTile);
-            tma_load_4d(sbase + kSmQ, &p.map_q, 0, (int)q_row0, 0, 0, q_full);
-            tma_load_4d(sbase + kSmQ + kHalf, &p.map_q, 64, (int)q_row0, 0, 0, q_full);
+            for (int c = 0; c < kRep; ++c) {   // (boxes of 128 / kRep rows)
+                tma_load_4d(sbase + kSmQ + c * (kHalf / kRep), &p.map_q, 0, (int)q_row0, 0, 0, q_full);
+                tma_load_4d(sbase + kSmQ + kHalf + c * (kHalf / kRep), &p.map_q, 64, (int)q_row0, 0, 0, q_full);
+            }
             const int row_base = bh * p.cap + t_lo * kT;
             for (int t = 0; t < nt; ++t) {
                 const int s = t % kStages;
@@ -250,7 +268,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         // ---- softmax: two threads per query row (= tensor-memory lane), each owning 64 of a tile's 128 keys
         //      and 64 of the accumulator's 128 columns; warps 2-5 take the first halves, warps 6-9 the second ----
         const int q = warp & 3, r = q * 32 + lane, wg = (warp - 2) >> 2;
-        const int row = qt * kT + r;                          // row among the G*m of this head group
+        constexpr int kRows = kT / kRep, kKeys = 64 / kRep;   // rows of a replica; keys of a tile per thread
+        const int col0 = (r / kRows) * kRows + wg * kKeys;    // the first of them (a replica has as many keys as rows)
+        const int row = qt * kT + r % kRows;                  // row among the G*m of this head group
         const bool row_ok = row < rows_total;
         const int qi = row % p.m;                             // which of the m queries
         const int vis = p.causal ? len - (p.m - 1 - qi) : len;   // keys this row sees: [0, vis)
@@ -258,7 +278,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         const int32_t* cnt = p.count ? p.count + (size_t)bh * p.cap : nullptr;
         float m_run = -INFINITY, l_run = 0.f;                 // l_run: this thread's keys only
         bool failed = false;
-        const bool idle = qt * kT + q * 32 >= rows_total;     // none of the warp's rows exists: it only keeps step
+        const bool idle = qt * kT + (q * 32) % kRows >= rows_total;     // none of the warp's rows exists: it only keeps step
         const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
         // log2(count) of a tile's keys, one key per thread of the first four warps.  The counts of the next tile are requested
         // a tile ahead and published behind this tile's barrier, when nobody reads that buffer any more.
@@ -271,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         };
         if (wg == 0) publish_counts(0, count_of(0));
         for (int t = 0; t < nt; ++t) {
-            const int s = t & 1, st = t % kStages, j0 = (t_lo + t) * kT, jw = j0 + wg * 64;   // jw: first key of this thread's half
+            const int s = t & 1, st = t % kStages, j0 = (t_lo + t) * kT, jw = j0 + col0;   // jw: first key of this thread
             const int next_count = wg == 0 ? count_of(t + 1) : 1;
             if (!mbar_wait(s_full0 + 8 * s, (t >> 1) & 1)) { *sh_fail = 1; *sh_fail_sm = 1; }
             fence_after_sync();
@@ -279,27 +299,31 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             // the scale plus the tile's largest log2(count) bounds the row's largest score: any reference at or above the
             // true maximum serves the softmax, and this one is at most log2 of the largest count above it.  (A scale that
             // is not positive takes the smallest product.)
-            uint32_t g[64];
-            const bool all_seen = __all_sync(kFull, jw + 64 <= vis);   // no key of this half is masked for any row of the warp
+            uint32_t g[kKeys];
+            const bool all_seen = __all_sync(kFull, jw + kKeys <= vis);   // none of these keys is masked for any row of the warp
             float mx = -INFINITY;
             if (!idle) {
-                tmem_ld32(lane_addr + kColS + s * kT + wg * 64, *reinterpret_cast<uint32_t(*)[32]>(&g[0]));
-                tmem_ld32(lane_addr + kColS + s * kT + wg * 64 + 32, *reinterpret_cast<uint32_t(*)[32]>(&g[32]));
+                if constexpr (kRep == 4) {
+                    tmem_ld16(lane_addr + kColS + s * kT + col0, g);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < kKeys; k += 32) tmem_ld32(lane_addr + kColS + s * kT + col0 + k, *reinterpret_cast<uint32_t(*)[32]>(&g[k]));
+                }
                 tmem_ld_wait();
                 if (!(p.scale_log2 > 0.f)) {
 #pragma unroll
-                    for (int k = 0; k < 64; ++k)
+                    for (int k = 0; k < kKeys; ++k)
                         if (jw + k < vis) mx = fmaxf(mx, -__uint_as_float(g[k]));
                 } else if (all_seen) {
                     float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-                    for (int k = 0; k < 64; k += 8)
+                    for (int k = 0; k < kKeys; k += 8)
 #pragma unroll
                         for (int x = 0; x < 4; ++x) m4[x] = max3(m4[x], __uint_as_float(g[k + x]), __uint_as_float(g[k + 4 + x]));
                     mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
                 } else {
 #pragma unroll
-                    for (int k = 0; k < 64; ++k)
+                    for (int k = 0; k < kKeys; ++k)
                         if (jw + k < vis) mx = fmaxf(mx, __uint_as_float(g[k]));
                 }
             }
@@ -316,6 +340,11 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             if (*sh_fail_sm) { failed = true; break; }
             if (wg == 0 && t + 1 < nt) publish_counts(t + 1, next_count);
             if (!idle) {
+                if (kRep > 1) {   // the weights of the other replicas' keys
+                    const uint32_t zero[16] = {0u};
+#pragma unroll
+                    for (int c = kRows; c < kT; c += 32) tmem_st16(lane_addr + kColS + s * kT + (((r / kRows) * kRows + c) & (kT - 1)) + wg * 16, zero);
+                }
                 mx = fmaxf(__bfloat162float(mx_up), __bfloat162float(mx_s[(s * 2 + (wg ^ 1)) * kT + r]));
                 if (mx != -INFINITY) {
                     const int top = max(max(lcm_s[s * 4], lcm_s[s * 4 + 1]), max(lcm_s[s * 4 + 2], lcm_s[s * 4 + 3]));
@@ -351,11 +380,12 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
                 // is below 2^-17 of the sum)
                 float2 l2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    uint32_t hi[16], lo[16];
+                for (int c = 0; c < (kRep == 1 ? 2 : 1); ++c) {
+                    constexpr int kChunk = kRep == 4 ? 16 : 32;
+                    uint32_t hi[kChunk / 2], lo[kChunk / 2];
 #pragma unroll
-                    for (int k = 0; k < 32; k += 4) {
-                        const float4 lc = *reinterpret_cast<const float4*>(lc_s + s * kT + wg * 64 + c * 32 + k);
+                    for (int k = 0; k < kChunk; k += 4) {
+                        const float4 lc = *reinterpret_cast<const float4*>(lc_s + s * kT + col0 + c * 32 + k);
                         const uint32_t* gk = g + c * 32 + k;
                         const float2 x0 = add2(fma2(make_float2(__uint_as_float(gk[0]), __uint_as_float(gk[1])), scale2, make_float2(lc.x, lc.y)), nref2);
                         const float2 x1 = add2(fma2(make_float2(__uint_as_float(gk[2]), __uint_as_float(gk[3])), scale2, make_float2(lc.z, lc.w)), nref2);
@@ -373,8 +403,13 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
                         hi[k >> 1] = p0; hi[(k >> 1) + 1] = p1;
                         lo[k >> 1] = pack2(r0, r1); lo[(k >> 1) + 1] = pack2(r2, r3);
                     }
-                    tmem_st16(lane_addr + kColS + s * kT + wg * 64 + c * 32, hi);
-                    tmem_st16(lane_addr + kColS + s * kT + wg * 64 + c * 32 + 16, lo);
+                    if constexpr (kRep == 4) {   // two threads share a chunk of 32 columns
+                        tmem_st8(lane_addr + kColS + s * kT + q * 32 + wg * 8, hi);
+                        tmem_st8(lane_addr + kColS + s * kT + q * 32 + 16 + wg * 8, lo);
+                    } else {
+                        tmem_st16(lane_addr + kColS + s * kT + col0 + c * 32, hi);
+                        tmem_st16(lane_addr + kColS + s * kT + col0 + c * 32 + 16, lo);
+                    }
                 }
                 l_run += (l2[0].x + l2[0].y) + (l2[1].x + l2[1].y);
                 tmem_st_wait();
@@ -393,7 +428,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         ls_s[wg * kT + r] = l_run;
         asm volatile("bar.sync 1, 256;\n" ::: "memory");
         const float l_row = l_run + ls_s[(wg ^ 1) * kT + r];
-        if (n_split == 1) {
+        if (kRep == 1 && n_split == 1) {
             __nv_bfloat16* orow = p.out + (size_t)(q_row0 + r) * 128 + wg * 64;
             const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
 #pragma unroll
@@ -421,7 +456,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         } else {
             // this CTA's share of the keys: unnormalised O, m and l into its own shared memory (the K ring is spent)
             float* part_o = reinterpret_cast<float*>(smem + kSmK);      // [128 rows][32 float4], float4 index ^ (row & 31)
-            float* part_ml = reinterpret_cast<float*>(smem + kSmV);     // [128] m, [128] l
+            float* part_ml = reinterpret_cast<float*>(smem + kSmV);     // [128] m, [128] l; the folded replicas' [128] m, [128] l
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 uint32_t o[32];
@@ -439,9 +474,29 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
                 }
             }
             if (wg == 0) { part_ml[r] = (nt > 0 && !failed) ? m_run : -INFINITY; part_ml[kT + r] = (nt > 0 && !failed) ? l_row : 0.f; }
+            if (kRep > 1) {   // the replicas of a row into the first, one thread per (row, four output columns)
+                asm volatile("bar.sync 1, 256;\n" ::: "memory");
+                for (int it = tid - 64; it < kRows * 32; it += 256) {
+                    const int fr = it >> 5, c4 = it & 31;
+                    float gm = -INFINITY, lsum = 0.f;
+                    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                    for (int j = 0; j < kRep; ++j) gm = fmaxf(gm, part_ml[fr + kRows * j]);
+#pragma unroll
+                    for (int j = 0; j < kRep; ++j) {
+                        const float mj = part_ml[fr + kRows * j], w = mj == -INFINITY ? 0.f : ex2(mj - gm);
+                        const float4 o = *reinterpret_cast<const float4*>(part_o + (fr + kRows * j) * 128 + ((c4 ^ (fr & 31)) << 2));
+                        lsum = fmaf(w, part_ml[kT + fr + kRows * j], lsum);
+                        acc.x = fmaf(w, o.x, acc.x); acc.y = fmaf(w, o.y, acc.y);
+                        acc.z = fmaf(w, o.z, acc.z); acc.w = fmaf(w, o.w, acc.w);
+                    }
+                    *reinterpret_cast<float4*>(part_o + fr * 128 + ((c4 ^ (fr & 31)) << 2)) = acc;   // (read by this thread only)
+                    if (c4 == 0) { part_ml[2 * kT + fr] = gm; part_ml[3 * kT + fr] = lsum; }
+                }
+            }
         }
     }
-    if (n_split > 1) {
+    if (kRep > 1 || n_split > 1) {
         cg::cluster_group cluster = cg::this_cluster();
         fence_before_sync();
         cluster.sync();   // every member's partial is in its shared memory
@@ -449,8 +504,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             // this CTA folds query rows [split * R, (split + 1) * R) of the tile, R = 128 / n_split rounded up: one thread per
             // (row, four output columns), reading that piece of every member's partial, four members at a time
             const float* part_o = reinterpret_cast<const float*>(smem + kSmK);
-            const float* part_ml = reinterpret_cast<const float*>(smem + kSmV);
-            const int R = (kT + n_split - 1) / n_split, r_end = min(min((split + 1) * R, kT), rows_total - qt * kT);
+            const float* part_ml = reinterpret_cast<const float*>(smem + kSmV) + (kRep > 1 ? 2 * kT : 0);
+            constexpr int kRows = kT / kRep;
+            const int R = (kRows + n_split - 1) / n_split, r_end = min(min((split + 1) * R, kRows), rows_total - qt * kT);
             for (int it = tid - 64; it < R * 32; it += 256) {
                 const int r = split * R + (it >> 5), c4 = it & 31;
                 if (r >= r_end) break;
@@ -574,8 +630,11 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
         dev &= 63;
         int* fit = fit_of[dev];
         std::call_once(once_of[dev], [&] {
-            cudaFuncSetAttribute(prefill_umma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-            const bool wide = cudaFuncSetAttribute(prefill_umma_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+            bool wide = true;
+            for (auto kernel : {prefill_umma_kernel<1>, prefill_umma_kernel<2>, prefill_umma_kernel<4>}) {
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+                wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess && wide;
+            }
             for (int c = 2; c <= (wide ? kMaxSplit : 8); ++c) {
                 cudaLaunchConfig_t probe = {};
                 probe.gridDim = dim3(c, 1, 1);
@@ -587,14 +646,18 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
                 probe.attrs = pa;
                 probe.numAttrs = 1;
                 int n_clusters = 0;
-                if (cudaOccupancyMaxActiveClusters(&n_clusters, prefill_umma_kernel, &probe) == cudaSuccess) fit[c] = n_clusters;
+                if (cudaOccupancyMaxActiveClusters(&n_clusters, prefill_umma_kernel<1>, &probe) == cudaSuccess) fit[c] = n_clusters;
             }
             (void)cudaGetLastError();   // a refused opt-in or probe is not an error of this call
         });
         Params p;
         p.count = a.count; p.core_len = a.core_len; p.out = (__nv_bfloat16*)a.out;
         p.Hq = a.Hq; p.Hkv = a.Hkv; p.m = a.m; p.cap = a.cap; p.causal = causal; p.scale_log2 = scale_log2; p.status = a.status;
-        if (make_map_bf16_rows(&p.map_q, a.q, 0, 0, 128, 1, 1, q_rows, kT) &&
+        // Replicas: the tile's chain of steps is the time of a launch with few rows, and most of it is a thread's scores.  8 layers of
+        // 8 tokens verified and accepted (32 rows): 214 us with one, 180 with four; of 9 tokens (36 rows) 220 with one, 190 with
+        // two; of 16 (64 rows) 247 and 219.
+        const int rep = G * a.m <= 32 ? 4 : G * a.m <= 64 ? 2 : 1;
+        if (make_map_bf16_rows(&p.map_q, a.q, 0, 0, 128, 1, 1, q_rows, kT / rep) &&
             make_map_bf16_rows(&p.map_k, a.core_k, 0, 0, 128, 1, 1, c_rows, kT) &&
             make_map_bf16_rows(&p.map_v, a.core_v, 0, 0, 128, 1, 1, c_rows, kT)) {
             // Few query tiles (short chunks, speculative decoding): split the keys over a cluster, as wide as all clusters of the
@@ -618,7 +681,7 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
             cfg.attrs = attr;
             cfg.numAttrs = 2;
             note_launches(1);
-            return cudaLaunchKernelEx(&cfg, prefill_umma_kernel, p);
+            return cudaLaunchKernelEx(&cfg, rep == 4 ? prefill_umma_kernel<4> : rep == 2 ? prefill_umma_kernel<2> : prefill_umma_kernel<1>, p);
         }
     }
     const unsigned blocks = (unsigned)((q_rows + 3) / 4);
