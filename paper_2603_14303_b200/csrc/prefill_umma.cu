@@ -152,7 +152,6 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     const int rows_total = G * p.m;                           // query rows of this (sequence, KV head)
     const uint32_t sbase = smem_u32(smem);
     float* lc_s = reinterpret_cast<float*>(smem + kSmLc);     // [2][128] log2(count) of the tile's keys
-    __nv_bfloat16* mx_s = reinterpret_cast<__nv_bfloat16*>(smem + kSmMx);   // [2][2][128] each half's row maximum, rounded up
     float* ls_s = reinterpret_cast<float*>(smem + kSmMx);     // [2][128] at the end: each half's row sum
     int* lcm_s = reinterpret_cast<int*>(smem + kSmBar + 128);  // [2][4] largest log2(count) of a tile, per writing warp (float bits)
     const uint32_t bar0 = sbase + kSmBar;
@@ -327,8 +326,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
                         if (jw + k < vis) mx = fmaxf(mx, __uint_as_float(g[k]));
                 }
             }
-            const __nv_bfloat16 mx_up = __float2bfloat16_ru(mx);   // (a bound as well; both threads of the row use the rounded values)
-            mx_s[(s * 2 + wg) * kT + r] = mx_up;
+            // The halves' maxima [2][128] go where the tile's keys were: their product is complete, and the stage is filled again
+            // only after every warp has handed in this tile's weights (behind the proxy fence below).
+            float* mx_s = reinterpret_cast<float*>(smem + kSmK + st * kTile);
+            mx_s[wg * kT + r] = mx;
             // Rows of the stage past the head's end hold whatever lies behind the cores (0 * NaN would poison
             // the second product): this row's threads clear its V row.  K rows need nothing, their scores are masked.
             if (j0 + r >= len) {
@@ -345,7 +346,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
 #pragma unroll
                     for (int c = kRows; c < kT; c += 32) tmem_st16(lane_addr + kColS + s * kT + (((r / kRows) * kRows + c) & (kT - 1)) + wg * 16, zero);
                 }
-                mx = fmaxf(__bfloat162float(mx_up), __bfloat162float(mx_s[(s * 2 + (wg ^ 1)) * kT + r]));
+                mx = fmaxf(mx, mx_s[(wg ^ 1) * kT + r]);
                 if (mx != -INFINITY) {
                     const int top = max(max(lcm_s[s * 4], lcm_s[s * 4 + 1]), max(lcm_s[s * 4 + 2], lcm_s[s * 4 + 3]));
                     mx = fmaf(mx, fabsf(p.scale_log2), __int_as_float(top));
@@ -415,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
                 tmem_st_wait();
             }
             fence_before_sync();      // this thread's accesses to tensor memory
-            fence_async_proxy();      // a cleared V row, for the tensor core's reads
+            fence_async_proxy();      // a cleared V row, for the tensor core's reads; the maxima, for the copies to come
             __syncwarp();
             if (lane == 0) mbar_arrive(p_full0 + 8 * s);
         }
