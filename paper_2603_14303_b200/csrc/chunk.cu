@@ -4,13 +4,16 @@
 // at p when p == 0 or isd[p-1]; run_start(p) is the last such position at or before p, and p
 // opens a segment iff isd[p] or (p - run_start(p)) % max_chunk_len == 0.  Segment offsets are
 // the compacted positions of those flags.
-// Two kernels.  chunk_flags: one block per 2048 tokens; it finds the run it starts in by looking back for the last
-// delimiter before it (256 tokens at a time: nearly always one look), writes the flags as bits and counts them.
+// Two kernels.  chunk_flags: one block per 2048 tokens (per several such tiles where a sequence has more than kMaxSpans of
+// them); it finds the run it starts in by looking back for the last delimiter before it, writes the flags as bits and
+// counts them.  The first look is at 256 tokens and finds one in ordinary text; further looks take 16 K tokens each, and no
+// more than kMaxSpans blocks of a sequence look back, so that text without delimiters costs time proportional to its length.
 // chunk_write_pack: one block per sequence turns flags into offsets and packs consecutive segments into the
 // <= SC_TILE_ROWS-token work tiles sc_compress consumes.
 // What bounds it: launches and dependent round trips, not bytes.  Five kernels before (carry, count, scan, write, pack, with
 // token ids read four times and the tile chain walked one tile at a time) took 17.8 us for 2048 tokens, 40 us for 32K,
-// 30 us for 16 x 16K; these take 8.2, 11.7 and 10.5 us (back to back in a CUDA graph).
+// 30 us for 16 x 16K; these take 8.2, 12.1 and 10.5 us (back to back in a CUDA graph).  Without a delimiter in the text: 14 us for
+// 32K, 31 for 128K, 196 for 1M (226 with delimiters); 55, 204 and 1877 when every look took 256 tokens.
 #include "common.cuh"
 
 namespace sc {
@@ -18,6 +21,8 @@ namespace sc {
 constexpr int kChunkThreads = 256;
 constexpr int kChunkPer = 8;
 constexpr int kChunkTile = kChunkThreads * kChunkPer;  // 2048 tokens per block
+constexpr int kMaxSpans = 128;                         // blocks of a sequence (each may look back to its start)
+constexpr int kLookUnroll = 32, kLookRounds = 2;       // tokens per thread of a further look: 64
 constexpr int kPackThreads = 1024;
 constexpr int kPackWindow = 4096;                      // segments packed at a time
 constexpr int kPackJump = 8;                           // tiles per step of the chain walk
@@ -45,66 +50,98 @@ __device__ __forceinline__ int block_max(int v, int* wt /*[8]*/) {
     return r;
 }
 
-// Kernel 1: segment-start flags of 2048 tokens (a byte per thread, bit i = token i of its eight) and their number.
+// Last delimiter among tokens [lo, hi), as its position + 1, or 0; all threads of the block get the answer.
+__device__ __noinline__ int last_delimiter(const int32_t* ids, int lo, int hi, const DelimSet& D, int* wt) {
+    int last = 0;
+    for (int p0 = lo + threadIdx.x; p0 < hi; p0 += kLookUnroll * kChunkThreads) {
+        int32_t tok[kLookUnroll];   // requested together
+#pragma unroll
+        for (int i = 0; i < kLookUnroll; ++i) tok[i] = ids[min(p0 + i * kChunkThreads, hi - 1)];
+        unsigned hits = 0u;
+        for (int k = 0; k < D.n; ++k) {   // (one delimiter against all: the other way round each comparison waits for its own fetch of the id)
+            const int32_t id = D.id[k];
+#pragma unroll
+            for (int i = 0; i < kLookUnroll; ++i) hits |= (tok[i] == id ? 1u : 0u) << i;
+        }
+        if (hits) last = min(p0 + (31 - __clz(hits)) * kChunkThreads, hi - 1) + 1;
+    }
+    return block_max(last, wt);
+}
+
+// Kernel 1: segment-start flags of `span` tiles of 2048 tokens (a byte per thread and tile, bit i = token i of its eight)
+// and their number per tile.  kOne: span is 1 (the loop costs 0.4 us of 12).
+template <bool kOne>
 __global__ void __launch_bounds__(kChunkThreads)
-chunk_flags(const int32_t* __restrict__ token_ids, int n, int tps, DelimSet D, int max_len, uint8_t* __restrict__ flags,
+chunk_flags(const int32_t* __restrict__ token_ids, int n, int tps, int span, const __grid_constant__ DelimSet D, int max_len, uint8_t* __restrict__ flags,
             int32_t* __restrict__ tile_cnt) {
     __shared__ int wt[kChunkThreads / 32];
     in_stream_order();
-    const int b = blockIdx.x / tps, tile = blockIdx.x % tps, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (kOne) span = 1;
+    const int spans = kOne ? tps : (tps + span - 1) / span;
+    const int b = blockIdx.x / spans, first = (blockIdx.x - b * spans) * span, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int32_t* ids = token_ids + (int64_t)b * n;
-    const int tile0 = tile * kChunkTile, p0 = tile0 + threadIdx.x * kChunkPer;
-    int32_t tok[kChunkPer];
-    if (p0 + kChunkPer <= n && (reinterpret_cast<uintptr_t>(ids + p0) & 15u) == 0) {
-        const int4 x = *reinterpret_cast<const int4*>(ids + p0), y = *reinterpret_cast<const int4*>(ids + p0 + 4);
-        tok[0] = x.x; tok[1] = x.y; tok[2] = x.z; tok[3] = x.w; tok[4] = y.x; tok[5] = y.y; tok[6] = y.z; tok[7] = y.w;
-    } else {
-#pragma unroll
-        for (int i = 0; i < kChunkPer; ++i) tok[i] = p0 + i < n ? ids[p0 + i] : 0;
-    }
-    const int32_t prev_tok = p0 > 0 && p0 - 1 < n ? ids[p0 - 1] : 0;
-    // start of the run that reaches into the tile: behind the last delimiter before it
+    // start of the run that reaches into the first tile: behind the last delimiter before it
     int carry = 0;
-    if (D.n > 0) {
-        for (int back = tile0 - 1; back >= 0; back -= kChunkThreads) {
-            const int p = back - (int)threadIdx.x;
-            const int found = block_max(p >= 0 && in_set(ids[p], D) ? p + 1 : 0, wt);
-            if (found > 0) { carry = found; break; }
+    if (D.n > 0 && first > 0) {
+        int hi = first * kChunkTile;
+        const int p = hi - 1 - (int)threadIdx.x;
+        carry = block_max(in_set(ids[p], D) ? p + 1 : 0, wt);
+        hi -= kChunkThreads;
+        while (carry == 0 && hi > 0) {
+            const int lo = max(hi - kLookUnroll * kLookRounds * kChunkThreads, 0);
+            carry = last_delimiter(ids, lo, hi, D, wt);
+            hi = lo;
         }
     }
-    unsigned isd = 0u;
+    for (int tile = first; kOne ? tile == first : tile < min(first + span, tps); ++tile) {
+        const int p0 = tile * kChunkTile + threadIdx.x * kChunkPer;
+        int32_t tok[kChunkPer];
+        if (p0 + kChunkPer <= n && (reinterpret_cast<uintptr_t>(ids + p0) & 15u) == 0) {
+            const int4 x = *reinterpret_cast<const int4*>(ids + p0), y = *reinterpret_cast<const int4*>(ids + p0 + 4);
+            tok[0] = x.x; tok[1] = x.y; tok[2] = x.z; tok[3] = x.w; tok[4] = y.x; tok[5] = y.y; tok[6] = y.z; tok[7] = y.w;
+        } else {
 #pragma unroll
-    for (int i = 0; i < kChunkPer; ++i)
-        if (p0 + i < n && in_set(tok[i], D)) isd |= 1u << i;
-    // run starts among this thread's tokens; the last one carries over to the threads behind it
-    unsigned starts = (isd << 1) & 0xffu;
-    if (p0 == 0 || (p0 < n && in_set(prev_tok, D))) starts |= 1u;
-    int last = starts ? p0 + 31 - __clz(starts) : -1;
-    int incl = warp_scan_max(last, lane);
-    if (lane == 31) wt[w] = incl;
-    __syncthreads();
-    int run = __shfl_up_sync(kFull, incl, 1);
-    if (lane == 0) run = -1;
-    run = max(run, carry);
-    for (int i = 0; i < w; ++i) run = max(run, wt[i]);
-    unsigned f = 0u;
+            for (int i = 0; i < kChunkPer; ++i) tok[i] = p0 + i < n ? ids[p0 + i] : 0;
+        }
+        const int32_t prev_tok = p0 > 0 && p0 - 1 < n ? ids[p0 - 1] : 0;
+        unsigned isd = 0u;
 #pragma unroll
-    for (int i = 0; i < kChunkPer; ++i) {
-        const int p = p0 + i;
-        if ((starts >> i) & 1u) run = p;
-        const int off = p - run;
-        if (p < n && (((isd >> i) & 1u) || off == 0 || (off >= max_len && off % max_len == 0))) f |= 1u << i;
-    }
-    flags[(size_t)blockIdx.x * kChunkThreads + threadIdx.x] = (uint8_t)f;
-    __syncthreads();   // wt is read above
-    const int c = warp_sum_i(__popc(f));
-    if (lane == 0) wt[w] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int t = 0;
+        for (int i = 0; i < kChunkPer; ++i)
+            if (p0 + i < n && in_set(tok[i], D)) isd |= 1u << i;
+        // run starts among this thread's tokens; the last one carries over to the threads behind it
+        unsigned starts = (isd << 1) & 0xffu;
+        if (p0 == 0 || (p0 < n && in_set(prev_tok, D))) starts |= 1u;
+        int last = starts ? p0 + 31 - __clz(starts) : -1;
+        int incl = warp_scan_max(last, lane);
+        if (lane == 31) wt[w] = incl;
+        __syncthreads();
+        int run = __shfl_up_sync(kFull, incl, 1);
+        if (lane == 0) run = -1;
+        run = max(run, carry);
+        for (int i = 0; i < (kOne ? w : kChunkThreads / 32); ++i) {
+            if (kOne || i < w) run = max(run, wt[i]);
+            carry = max(carry, wt[i]);   // for the next tile
+        }
+        unsigned f = 0u;
 #pragma unroll
-        for (int i = 0; i < kChunkThreads / 32; ++i) t += wt[i];
-        tile_cnt[blockIdx.x] = t;
+        for (int i = 0; i < kChunkPer; ++i) {
+            const int p = p0 + i;
+            if ((starts >> i) & 1u) run = p;
+            const int off = p - run;
+            if (p < n && (((isd >> i) & 1u) || off == 0 || (off >= max_len && off % max_len == 0))) f |= 1u << i;
+        }
+        flags[((size_t)b * tps + tile) * kChunkThreads + threadIdx.x] = (uint8_t)f;
+        __syncthreads();   // wt is read above
+        const int c = warp_sum_i(__popc(f));
+        if (lane == 0) wt[w] = c;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            int t = 0;
+#pragma unroll
+            for (int i = 0; i < kChunkThreads / 32; ++i) t += wt[i];
+            tile_cnt[b * tps + tile] = t;
+        }
+        if (!kOne) __syncthreads();   // wt is written again
     }
 }
 
@@ -245,7 +282,8 @@ cudaError_t launch_chunk(const ChunkArgs& a, cudaStream_t st) {
     DelimSet D;
     D.n = a.n_delim;
     for (int i = 0; i < SC_MAX_DELIMS; ++i) D.id[i] = (i < a.n_delim) ? a.delim[i] : 0;
-    cudaError_t e = launch_in_order(chunk_flags, dim3(tiles), kChunkThreads, 0, st, a.token_ids, a.n, tps, D, a.max_chunk_len, flags, tile_cnt);
+    const int span = div_up(tps, kMaxSpans), spans = div_up(tps, span);
+    cudaError_t e = launch_in_order(span == 1 ? chunk_flags<true> : chunk_flags<false>, dim3(a.B * spans), kChunkThreads, 0, st, a.token_ids, a.n, tps, span, D, a.max_chunk_len, flags, tile_cnt);
     if (e != cudaSuccess) return e;
     note_launches(2);
     return launch_in_order(chunk_write_pack, dim3(a.B), kPackThreads, 0, st, (const uint8_t*)flags, (const int32_t*)tile_cnt, a.B, a.n, tps,
