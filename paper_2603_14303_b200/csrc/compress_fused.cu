@@ -660,12 +660,11 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) compress_fused_kernel(
     const bool service = warp == kWarps;   // the fifth warp
     int max_nt = 0;                        // most tiles any sequence has
 
-    // An ordinary launch waits here for the kernel before it; under an overlapped one the next kernel may start beside this one,
-    // and this one waits for its predecessor only at its very end.
-    if (!p.overlap) in_stream_order();
-    else asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    // An ordinary launch waits here for the kernel before it; an overlapped one waits for its predecessor only at its very end.
+    if (!p.overlap) asm volatile("griddepcontrol.wait;\n" ::: "memory");
     if (p.skip != nullptr && *p.skip != 0) return;   // uniform over the grid: nothing touched, nothing to clean
-    const float tau = p.tau_dev != nullptr ? *p.tau_dev : p.tau;
+    // (+ 0: a threshold of -0.0 becomes +0.0; its sign would reach the differences of sim_word)
+    const float tau = (p.tau_dev != nullptr ? *p.tau_dev : p.tau) + 0.f;
     if (tid == 0) {
         umma::mbar_init(bar_k, 1);
         umma::mbar_init(bar_v, 1);
