@@ -235,6 +235,14 @@ merge_generic(const T* __restrict__ K, const T* __restrict__ V, sc_strides st, i
         int row = seg_core_off[(int64_t)h * seg_stride + s];
         const int64_t obase = ((int64_t)b * Hkv + h) * cap;
         T* cores = (is_v ? core_v : core_k) + obase * d + lane * 4;
+        if (l == 1) {   // as it is (delimiters, and whatever stands between two of them)
+            if (row >= cap) continue;
+#pragma unroll
+            for (int u = 0; u < kPer; ++u)
+                if ((u * 32 + lane) * 4 < d) store4(cores + (int64_t)row * d + u * 128, load4(rows + u * 128));
+            if (lane == 0 && !is_v) count[obase + row] = 1;
+            continue;
+        }
         if constexpr (kPer == 1) {
             const int own = lane < l ? as[lane] - r : -1;
             const unsigned seeds = __ballot_sync(kFull, own == lane);
