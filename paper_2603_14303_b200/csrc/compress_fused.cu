@@ -686,6 +686,9 @@ __global__ void __launch_bounds__(kThreads, kBlocksPerSm) compress_fused_kernel(
     __syncthreads();
     umma::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    // The next kernel may be set up (under an overlapped launch of it: run) beside this one from here on, and not earlier: a block of
+    // it that took the tensor memory first would keep this block waiting for it, while itself waiting for this kernel.
+    asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     bool failed = false;
 
     if (service) {
