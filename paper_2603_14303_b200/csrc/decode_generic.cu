@@ -216,16 +216,18 @@ static cudaError_t run(const DecodeArgs& a, cudaStream_t st) {
     const int64_t blocks = (int64_t)n_split * a.Hkv * groups * a.B;
     if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
     const unsigned grid = (unsigned)blocks;
+    // partials are read and written in pairs of floats; a workspace need only be aligned to one (256 spare bytes cover the step)
+    float* part = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(a.ws) + 7) & ~(uintptr_t)7);
     cudaError_t e = launch_in_order(a.d <= 128 ? decode_generic<T, 4> : decode_generic<T, 8>, dim3(grid), kDecWarps * 32, 0, st,
                                     (const T*)a.q, a.Hq, a.Hkv, a.d, (const T*)a.core_k, (const T*)a.core_v, a.count, a.cap,
-                                    a.core_len, scale, n_split, (float*)a.ws);
+                                    a.core_len, scale, n_split, part);
     if (e != cudaSuccess) return e;
     const int64_t heads = (int64_t)a.B * a.Hq;
     e = launch_in_order(combine_generic<T>, dim3(div_up(heads, kDecWarps)), kDecWarps * 32, 0, st, heads, a.d, n_split,
-                              (const float*)a.ws, (T*)a.out);
+                              (const float*)part, (T*)a.out);
     if (e != cudaSuccess) return e;
     note_launches(2);
-    return cudaGetLastError();
+    return cudaSuccess;
 }
 
 cudaError_t launch_decode_generic(const DecodeArgs& a, cudaStream_t st) {

@@ -1,0 +1,30 @@
+"""The float32 calls: a decode workspace that starts on any float."""
+import pytest
+import torch
+
+from helpers import TOL, assert_close_vectors, to_f64
+from paper_2603_14303_b200 import binding
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _layer(cap=1500, H=2, d=40):
+    g = torch.Generator().manual_seed(cap)
+    k, v = torch.randn((1, H, cap, d), generator=g), torch.randn((1, H, cap, d), generator=g)
+    y = binding.CompressedLayer(k.to(DEV), v.to(DEV), torch.ones((1, H, cap), dtype=torch.int32, device=DEV),
+                                torch.full((1, H), cap, dtype=torch.int32, device=DEV))
+    q = torch.randn((1, 2 * H, d), generator=g)
+    x = torch.einsum("hgd,htd->hgt", q.view(H, 2, d).double(), k[0].double()) / d ** 0.5
+    return q.to(DEV), y, torch.einsum("hgt,htd->hgd", torch.softmax(x, -1), v[0].double()).reshape(1, 2 * H, d).numpy()
+
+
+@pytest.mark.parametrize("shift", [0, 4, 8, 12])
+def test_decode_workspace_on_any_float(shift):
+    q, y, ref = _layer()
+    need = binding.lib().sc_decode_workspace_bytes(1, 4, 2, 40, 1500)
+    whole = torch.zeros(need + 64, dtype=torch.uint8, device=DEV)
+    whole[shift + need:] = 77
+    got = binding.decode_attn(q, y, workspace=whole[shift:shift + need])
+    assert_close_vectors(to_f64(got), ref, TOL[torch.float32], f"workspace shifted by {shift}")
+    assert bool((whole[shift + need:] == 77).all()) and bool((whole[:shift] == 0).all())
