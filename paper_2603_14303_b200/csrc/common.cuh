@@ -89,6 +89,11 @@ __device__ __forceinline__ void in_stream_order() {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
 }
+// A refused launch is reported by the call that made it: taken out of the runtime's record, where the next call would find it.
+inline cudaError_t own_error(cudaError_t e) {
+    if (e != cudaSuccess) (void)cudaGetLastError();
+    return e;
+}
 template <typename... P, typename... A>
 inline cudaError_t launch_in_order(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchConfig_t cfg = {};
@@ -101,7 +106,7 @@ inline cudaError_t launch_in_order(void (*kernel)(P...), dim3 grid, int threads,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    return own_error(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
 }
 
 inline int div_up(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }

@@ -569,9 +569,9 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
     cfg.numAttrs = 2;
     const int mode = (a.flags & SC_FLAG_OVERLAP_CHAIN) ? dm::kChained : (a.flags & SC_FLAG_OVERLAP_PREV) ? dm::kOverlapped : dm::kOrdinary;
     note_launches(1);
-    return cudaLaunchKernelEx(&cfg, dm::decode_mma_kernel, (const __nv_bfloat16*)a.q, a.Hq, a.Hkv,
-                              (const __nv_bfloat16*)a.core_k, (const __nv_bfloat16*)a.core_v, a.count, a.cap,
-                              a.core_len, scale, plan.n_split, mode, (__nv_bfloat16*)a.out, part, tickets);
+    return own_error(cudaLaunchKernelEx(&cfg, dm::decode_mma_kernel, (const __nv_bfloat16*)a.q, a.Hq, a.Hkv,
+                                        (const __nv_bfloat16*)a.core_k, (const __nv_bfloat16*)a.core_v, a.count, a.cap,
+                                        a.core_len, scale, plan.n_split, mode, (__nv_bfloat16*)a.out, part, tickets));
 }
 
 }  // namespace sc

@@ -682,7 +682,7 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
             cfg.attrs = attr;
             cfg.numAttrs = 2;
             note_launches(1);
-            return cudaLaunchKernelEx(&cfg, rep == 4 ? prefill_umma_kernel<4> : rep == 2 ? prefill_umma_kernel<2> : prefill_umma_kernel<1>, p);
+            return own_error(cudaLaunchKernelEx(&cfg, rep == 4 ? prefill_umma_kernel<4> : rep == 2 ? prefill_umma_kernel<2> : prefill_umma_kernel<1>, p));
         }
     }
     const unsigned blocks = (unsigned)((q_rows + 3) / 4);

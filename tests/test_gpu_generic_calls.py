@@ -1,4 +1,7 @@
-"""The float32 calls: a decode workspace that starts on any float."""
+"""The float32 calls: a decode workspace that starts on any float, and a launch that the runtime refuses, which is an error of
+its own call only."""
+import ctypes
+
 import pytest
 import torch
 
@@ -28,3 +31,12 @@ def test_decode_workspace_on_any_float(shift):
     got = binding.decode_attn(q, y, workspace=whole[shift:shift + need])
     assert_close_vectors(to_f64(got), ref, TOL[torch.float32], f"workspace shifted by {shift}")
     assert bool((whole[shift + need:] == 77).all()) and bool((whole[:shift] == 0).all())
+
+
+def test_a_refused_launch_is_not_an_error_of_the_next_call():
+    q, y, ref = _layer()
+    none = ctypes.c_void_p(q.data_ptr())
+    # 2^33 queries are 2^31 blocks of four, one more than a grid can have: the runtime refuses the launch, nothing runs
+    code = binding.lib().sc_prefill_attn(none, binding.SC_F32, 1 << 20, 1 << 13, 1 << 13, 1, 40, none, none, None, 8, none, 0.0, 0, none, None, None)
+    assert code == binding.SC_ERR_CUDA
+    assert_close_vectors(to_f64(binding.decode_attn(q, y)), ref, TOL[torch.float32], "decode")
