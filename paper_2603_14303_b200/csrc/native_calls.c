@@ -7,8 +7,9 @@
 #include "semanticache.h"
 
 static void* ptr(PyObject* o) { return o == Py_None ? NULL : (void*)PyLong_AsUnsignedLongLong(o); }
-static int32_t i32(PyObject* o) { return (int32_t)PyLong_AsLong(o); }
-static uint32_t u32(PyObject* o) { return (uint32_t)PyLong_AsUnsignedLong(o); }
+/* integers modulo 2^32: what ctypes' c_int32 and c_uint32 take */
+static uint32_t u32(PyObject* o) { return (uint32_t)PyLong_AsUnsignedLongMask(o); }
+static int32_t i32(PyObject* o) { return (int32_t)u32(o); }
 static size_t sz(PyObject* o) { return (size_t)PyLong_AsUnsignedLongLong(o); }
 static float f32(PyObject* o) { return (float)PyFloat_AsDouble(o); }
 
@@ -17,8 +18,10 @@ static int arity(Py_ssize_t n, Py_ssize_t want, const char* name) {
     PyErr_Format(PyExc_TypeError, "%s takes %zd arguments, got %zd", name, want, n);
     return 0;
 }
-/* a sequence of token ids; its length, or -1 with an exception set.  One too many is kept: the library refuses the count. */
+/* anything that has a length and can be iterated, its items made ints; the length, or -1 with an exception set.  One too many
+ * is kept: the library refuses the count. */
 static int32_t ids_of(PyObject* seq, int32_t* out) {
+    if (PyObject_Size(seq) < 0) return -1;
     PyObject* fast = PySequence_Fast(seq, "delim_ids must be a sequence");
     if (!fast) return -1;
     const Py_ssize_t n = PySequence_Fast_GET_SIZE(fast);
