@@ -35,6 +35,7 @@
 #include <cooperative_groups.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "umma.cuh"
@@ -503,44 +504,54 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         cluster.sync();   // every member's partial is in its shared memory
         if (warp >= 2) {
             // this CTA folds query rows [split * R, (split + 1) * R) of the tile, R = 128 / n_split rounded up: one thread per
-            // (row, four output columns), reading that piece of every member's partial, four members at a time
+            // (row, four output columns), reading that piece of every member's partial, four or eight members at a time
             const float* part_o = reinterpret_cast<const float*>(smem + kSmK);
             const float* part_ml = reinterpret_cast<const float*>(smem + kSmV) + (kRep > 1 ? 2 * kT : 0);
             constexpr int kRows = kT / kRep;
             const int R = (kRows + n_split - 1) / n_split, r_end = min(min((split + 1) * R, kRows), rows_total - qt * kT);
-            for (int it = tid - 64; it < R * 32; it += 256) {
-                const int r = split * R + (it >> 5), c4 = it & 31;
-                if (r >= r_end) break;
-                float gm = -INFINITY;
-                for (int j = 0; j < n_split; ++j) gm = fmaxf(gm, cluster.map_shared_rank(part_ml, j)[r]);
-                float lsum = 0.f;
-                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int j0 = 0; j0 < n_split; j0 += 4) {
-                    float mv[4], lv[4];
-                    float4 ov[4];
+            const auto fold_rows = [&](auto width) {   // `width` partials at a time
+                constexpr int kFold = decltype(width)::value;
+                for (int it = tid - 64; it < R * 32; it += 256) {
+                    const int r = split * R + (it >> 5), c4 = it & 31;
+                    if (r >= r_end) break;
+                    float gm = -INFINITY, lsum = 0.f;
+                    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int j0 = 0; j0 < n_split; j0 += kFold) {
+                        float mv[kFold], lv[kFold];
+                        float4 ov[kFold];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool on = j0 + j < n_split;
-                        const float* ml = cluster.map_shared_rank(part_ml, on ? j0 + j : 0);
-                        const float* po = cluster.map_shared_rank(part_o, on ? j0 + j : 0);
-                        mv[j] = on ? ml[r] : -INFINITY;
-                        lv[j] = on ? ml[kT + r] : 0.f;
-                        ov[j] = on ? *reinterpret_cast<const float4*>(po + r * 128 + ((c4 ^ (r & 31)) << 2)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
+                        for (int j = 0; j < kFold; ++j) {   // requested together
+                            const bool on = j0 + j < n_split;
+                            const float* ml = cluster.map_shared_rank(part_ml, on ? j0 + j : 0);
+                            const float* po = cluster.map_shared_rank(part_o, on ? j0 + j : 0);
+                            mv[j] = on ? ml[r] : -INFINITY;
+                            lv[j] = on ? ml[kT + r] : 0.f;
+                            ov[j] = on ? *reinterpret_cast<const float4*>(po + r * 128 + ((c4 ^ (r & 31)) << 2)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+                        float top = gm;
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float w = (mv[j] == -INFINITY) ? 0.f : ex2(mv[j] - gm);
-                        lsum = fmaf(w, lv[j], lsum);
-                        acc.x = fmaf(w, ov[j].x, acc.x); acc.y = fmaf(w, ov[j].y, acc.y);
-                        acc.z = fmaf(w, ov[j].z, acc.z); acc.w = fmaf(w, ov[j].w, acc.w);
+                        for (int j = 0; j < kFold; ++j) top = fmaxf(top, mv[j]);
+                        if (top == -INFINITY) continue;   // nothing but empty shares so far
+                        const float f = gm == -INFINITY ? 0.f : ex2(gm - top);
+                        lsum *= f; acc.x *= f; acc.y *= f; acc.z *= f; acc.w *= f;
+                        gm = top;
+#pragma unroll
+                        for (int j = 0; j < kFold; ++j) {
+                            const float w = (mv[j] == -INFINITY) ? 0.f : ex2(mv[j] - gm);
+                            lsum = fmaf(w, lv[j], lsum);
+                            acc.x = fmaf(w, ov[j].x, acc.x); acc.y = fmaf(w, ov[j].y, acc.y);
+                            acc.z = fmaf(w, ov[j].z, acc.z); acc.w = fmaf(w, ov[j].w, acc.w);
+                        }
                     }
+                    const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
+                    uint2 v;
+                    v.x = pack2(acc.x * inv, acc.y * inv);
+                    v.y = pack2(acc.z * inv, acc.w * inv);
+                    *reinterpret_cast<uint2*>(p.out + (size_t)(q_row0 + r) * 128 + c4 * 4) = v;
                 }
-                const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
-                uint2 v;
-                v.x = pack2(acc.x * inv, acc.y * inv);
-                v.y = pack2(acc.z * inv, acc.w * inv);
-                *reinterpret_cast<uint2*>(p.out + (size_t)(q_row0 + r) * 128 + c4 * 4) = v;
-            }
+            };
+            if (n_split <= 4) fold_rows(std::integral_constant<int, 4>());
+            else fold_rows(std::integral_constant<int, 8>());
         }
         cluster.sync();   // every member's shared memory has been read: they may leave
     }
@@ -661,13 +672,17 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
         if (make_map_bf16_rows(&p.map_q, a.q, 0, 0, 128, 1, 1, q_rows, kT / rep) &&
             make_map_bf16_rows(&p.map_k, a.core_k, 0, 0, 128, 1, 1, c_rows, kT) &&
             make_map_bf16_rows(&p.map_v, a.core_v, 0, 0, 128, 1, 1, c_rows, kT)) {
-            // Few query tiles (short chunks, speculative decoding): split the keys over a cluster, as wide as all clusters of the
-            // launch fit at once, but leave every CTA at least four key tiles of the capacity (heads are usually half full).
+            // Few query tiles (short chunks, speculative decoding): the keys are split over a cluster.  Of the widths whose clusters
+            // all fit at once, the narrowest that leaves a CTA the fewest key tiles of a head that fills half the capacity (as
+            // compressed heads do or less): a wider one has the same tiles to walk and more partials to fold.  8 heads x 4 K
+            // rows of 8 K, 128 query rows: 8 CTAs 16.6 us, 10 CTAs 17.5; 8 K rows of 16 K: 23.5 and 23.1; 500 rows of 1 K: 4 CTAs 10.6,
+            // 2 CTAs 14.6.  Fewer than four are not worth their fold (3 us with two) for less than eight tiles, unless the
+            // rows stand in the tile more than once and the fold is short.
             const long long ctas = (long long)((G * a.m + kT - 1) / kT) * a.Hkv * a.B;
-            const int key_tiles = (a.cap + kT - 1) / kT;
+            const int half_tiles = ((a.cap + kT - 1) / kT + 1) / 2;
             int n_split = 1;
-            for (int c = 2; c <= kMaxSplit; ++c)
-                if (ctas <= fit[c] && key_tiles >= c * 4) n_split = c;
+            for (int c = rep == 1 && half_tiles < 8 ? 4 : 2; c <= kMaxSplit; ++c)
+                if (ctas <= fit[c] && (half_tiles + c - 1) / c < (half_tiles + n_split - 1) / n_split) n_split = c;
             p.n_split = n_split;
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)((G * a.m + kT - 1) / kT) * n_split, a.Hkv, a.B);
