@@ -50,6 +50,7 @@ constexpr int kMergeGroup = 16;                 // cluster partials folded per r
 constexpr int kMaxCluster = 16;                 // blocks per cluster (more than 8 needs the non-portable opt-in)
 constexpr int kCapRowsPerBlock = 1408;          // rows of capacity per block from which a head gets another cluster (heads are usually half full or less)
 constexpr int kMaxSlots = 160;                  // partials in global memory over the launch (at least one per head)
+constexpr int kMaxTickets = 512;                // heads of a launch whose blocks may meet through global memory
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -468,6 +469,13 @@ inline int head_slots(long long heads, int cap) {   // most partials a head can 
     const int s = heads >= kMaxSlots ? 1 : (int)(kMaxSlots / heads);
     return s < by_rows ? s : (by_rows < 1 ? 1 : by_rows);
 }
+// Partials a launch can leave.  It grows with the number of heads and with the capacity, so that a workspace for the largest batch
+// serves every smaller one (more than kMaxTickets heads have one cluster each and leave none).
+inline size_t all_slots(long long heads, int cap) {
+    const long long by_rows = cap < 64 ? 1 : (cap + 63) / 64, split = heads * by_rows;
+    const long long several = split < kMaxSlots ? split : kMaxSlots, own = heads < kMaxTickets ? heads : kMaxTickets;
+    return (size_t)(several > own ? several : own);
+}
 
 // The rules and what they were measured against (us per layer, Llama-shaped heads of 128 columns, 2 x 148 block slots; the
 // plan before took splits from the capacity alone, up to 256 a head in several waves, and asked L2 for up to 1 MB per
@@ -511,14 +519,14 @@ bool decode_mma_supported(const DecodeArgs& a) {
     return a.dt == SC_BF16 && a.d == dm::kD && (a.Hq / a.Hkv) <= 8 && a.cap > 0 && a.Hkv <= 65535 && a.B <= 65535;
 }
 
-// Bytes at the front of the workspace that hold the arrival counters (zero between calls).
-size_t decode_mma_counter_bytes(int32_t B, int32_t Hkv) { return sizeof(int32_t) * (((size_t)B * Hkv + 63) / 64 * 64); }
+// Bytes at the front of the workspace that hold the arrival counters (zero between calls): the same for every shape, so that
+// no call's partials lie where another one's counters are.
+size_t decode_mma_counter_bytes() { return sizeof(int32_t) * dm::kMaxTickets; }
 
 size_t decode_mma_ws_bytes(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t cap) {
     (void)Hq; (void)d;
     // tickets (one per (b, head), zero between calls) + partials
-    return 256 + decode_mma_counter_bytes(B, Hkv) +
-           sizeof(float) * (size_t)B * Hkv * dm::head_slots((long long)B * Hkv, cap) * dm::kPartStride;
+    return 256 + decode_mma_counter_bytes() + sizeof(float) * dm::all_slots((long long)B * Hkv, cap) * dm::kPartStride;
 }
 
 cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
@@ -553,7 +561,7 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
     });
     const dm::SplitPlan plan = dm::plan_for((long long)a.B * a.Hkv, a.cap, a.count == nullptr, res);
     int32_t* tickets = (int32_t*)a.ws;
-    float* part = (float*)((char*)a.ws + decode_mma_counter_bytes(a.B, a.Hkv));
+    float* part = (float*)((char*)a.ws + decode_mma_counter_bytes());
     const float scale = (a.scale == 0.f ? 1.f / sqrtf((float)a.d) : a.scale) * 1.4426950408889634f;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(plan.n_split, a.Hkv, a.B);

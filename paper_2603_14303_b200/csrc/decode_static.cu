@@ -44,7 +44,7 @@ cudaError_t static_scratch(void** out) {
 
 namespace sc {
 bool decode_mma_supported(const DecodeArgs& a);
-size_t decode_mma_counter_bytes(int32_t B, int32_t Hkv);
+size_t decode_mma_counter_bytes();
 }  // namespace sc
 
 extern "C" sc_status sc_decode_attn_static(const void* q, sc_dtype dt, int32_t B, int32_t Hq, int32_t Hkv,
@@ -71,7 +71,7 @@ extern "C" sc_status sc_decode_attn_static(const void* q, sc_dtype dt, int32_t B
     sc::DecodeArgs probe = {};
     probe.dt = dt; probe.B = B; probe.Hq = Hq; probe.Hkv = Hkv; probe.d = d; probe.cap = cap;
     if (!(flags & SC_FLAG_GENERIC) && sc::decode_mma_supported(probe)) {
-        if (cudaMemsetAsync(scratch, 0, sc::decode_mma_counter_bytes(B, Hkv), (cudaStream_t)stream) != cudaSuccess)
+        if (cudaMemsetAsync(scratch, 0, sc::decode_mma_counter_bytes(), (cudaStream_t)stream) != cudaSuccess)
             return SC_ERR_CUDA;
     }
     return sc_decode_attn(q, dt, B, Hq, Hkv, d, core_k, core_v, count, cap, core_len, scale, flags, out, scratch,
