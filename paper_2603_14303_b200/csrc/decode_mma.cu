@@ -13,7 +13,8 @@
 // The splits of a head form a thread-block cluster and fold their partials through distributed shared memory, each
 // block its own slice of the output (no partial leaves the SMs).  Where a head has several clusters, or blocks outside
 // clusters, partials go to global memory and the last one of a head to arrive (atomic ticket, no waiting) merges them.
-// How many splits: plan_for.
+// How many splits: plan_for.  In a batch the blocks that the plan gives a head are one unit; a head much longer than the mean
+// of the launch gets more units (plan_units), so that a long sequence among short ones is not streamed by a few blocks.
 // Every order is fixed, so results are bit-reproducible.
 //
 // Launch modes: ordinary; overlapped with the preceding kernel (programmatic stream
@@ -49,7 +50,7 @@ constexpr float kMaxSlack = 8.f;                // log2 units a score may exceed
 constexpr int kMergeGroup = 16;                 // cluster partials folded per round by the merging block
 constexpr int kMaxCluster = 16;                 // blocks per cluster (more than 8 needs the non-portable opt-in)
 constexpr int kCapRowsPerBlock = 1408;          // rows of capacity per block from which a head gets another cluster (heads are usually half full or less)
-constexpr int kMaxSlots = 160;                  // partials in global memory over the launch (at least one per head)
+constexpr int kMaxSlots = 160;                  // partials in global memory over the launch's own units (at least one per head)
 constexpr int kMaxTickets = 512;                // heads of a launch whose blocks may meet through global memory
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -143,12 +144,13 @@ __device__ __forceinline__ void issue_tile(uint32_t stage, const __nv_bfloat16* 
 }
 
 // Several partials per head in global memory (one per cluster, or per block outside clusters): the last block
-// to arrive merges the `n_parts` of them.  All threads of the block call it.  The cluster barrier / fence before the call orders this block's partial stores before its
+// to arrive merges the `n_parts` of them: the first `n_first` lie in the slots from `first` on, the others from `more` on.  All threads of the block call
+// it.  The cluster barrier / fence before the call orders this block's partial stores before its
 // ticket, whose release makes them visible to whoever reads the ticket with acquire (the last arrival); that
 // block's other threads are ordered behind its thread 0 by the barrier below and read the partials from L2.
-__device__ __forceinline__ void ticket_and_merge(const float* __restrict__ part, int32_t* __restrict__ tickets, int bh,
-                                                 int n_parts, int G, int Hq, int b, int h,
-                                                 __nv_bfloat16* __restrict__ out, int* sh_last_p) {
+template <bool kSpares>
+__device__ __forceinline__ void ticket_and_merge(const float* __restrict__ part, int first, int more, int n_first, int n_parts, int32_t* __restrict__ tickets,
+                                                 int bh, int G, __nv_bfloat16* __restrict__ out, int* sh_last_p) {
     if (threadIdx.x == 0) {
         int t;
         asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;\n" : "=r"(t) : "l"(tickets + bh) : "memory");
@@ -159,7 +161,6 @@ __device__ __forceinline__ void ticket_and_merge(const float* __restrict__ part,
     if (!*sh_last_p) return;
     // One thread per (head, four output columns); the partials are folded sixteen at a time, all of a
     // group's loads in flight together (one round trip to L2 per group).
-    const float* hp = part + (size_t)bh * n_parts * kPartStride;
     for (int e4 = threadIdx.x; e4 < G * (kD / 4); e4 += kWarps * 32) {
         const int hd = e4 / (kD / 4), d4 = (e4 % (kD / 4)) * 4;
         float gm = -INFINITY, lsum = 0.f;
@@ -170,7 +171,8 @@ __device__ __forceinline__ void ticket_and_merge(const float* __restrict__ part,
 #pragma unroll
             for (int j = 0; j < kMergeGroup; ++j) {
                 const bool ok = s0 + j < n_parts;
-                const float* sp = hp + (size_t)(ok ? s0 + j : 0) * kPartStride;
+                const int s = ok ? s0 + j : 0, slot = s + (!kSpares || s < n_first ? first : more - n_first);
+                const float* sp = part + (size_t)slot * kPartStride;
                 mv[j] = ok ? __ldcg(sp + 8 * kD + hd) : -INFINITY;
                 lv[j] = ok ? __ldcg(sp + 8 * kD + 8 + hd) : 0.f;
                 ov[j] = ok ? __ldcg(reinterpret_cast<const float4*>(sp + hd * kD + d4)) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -192,14 +194,51 @@ __device__ __forceinline__ void ticket_and_merge(const float* __restrict__ part,
             }
         }
         const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
-        store_out4(out + ((size_t)b * Hq + (size_t)h * G + hd) * kD + d4, acc, inv);
+        store_out4(out + ((size_t)bh * G + hd) * kD + d4, acc, inv);
     }
 }
 
+// Units of a batched launch.  Every head has its own; a head of more than one and a half times the mean number of tiles gets as
+// many more, from a pool of as many spare units as there are heads, as brings its units nearest to the mean.  Worked out by
+// every warp from the lengths alone (one round trip for all of them, beside the block's own): head `want` has units
+// 1 + extra, its extra units are numbers [begin, begin + extra) of the pool.  For a spare unit (`spare` >= 0) `want` is found
+// first: the head that unit belongs to, or -1.  16 sequences x 8 heads, one of 32 K rows among 1 K: 134 us with equal
+// shares, 72 with shares cut by capacity and used as a head's length warranted, 43 like this.
+struct Units { int head, extra, begin; };
+__device__ __forceinline__ Units plan_units(const int32_t* __restrict__ core_len, int heads, int cap, int want, int spare, int lane) {
+    auto tiles_of = [&](int i) { return i < heads ? (max(min(core_len[i], cap), 0) + kTile - 1) / kTile : 0; };
+    int sum = 0;
+#pragma unroll 4
+    for (int i = lane; i < heads; i += 32) sum += tiles_of(i);
+    sum = max(__reduce_add_sync(kFull, sum), 1);
+    // units nearest to tiles * heads / sum, at least one
+    auto extra_of = [&](int i) {
+        const long long x2 = 2ll * tiles_of(i) * heads;
+        return x2 < 3ll * sum ? 0 : (int)((x2 + sum) / (2ll * sum)) - 1;
+    };
+    Units u = {want, want >= 0 ? extra_of(want) : 0, 0};
+    if (want >= 0 && u.extra == 0) return u;
+    int before = 0;
+    for (int i0 = 0; i0 < heads; i0 += 32) {
+        const int mine = extra_of(i0 + lane), upto = before + warp_scan_add(mine, lane);
+        const unsigned here = __ballot_sync(kFull, want >= 0 ? i0 + lane == want : (mine > 0 && spare < upto));
+        if (here) {
+            const int src = __ffs(here) - 1;
+            u.head = i0 + src;
+            u.extra = __shfl_sync(kFull, mine, src);
+            u.begin = __shfl_sync(kFull, upto, src) - u.extra;
+            return u;
+        }
+        before = __shfl_sync(kFull, upto, 31);
+    }
+    return u;
+}
+
+template <bool kSpares>   // the launch has spare units (the code for them costs the others 0.2 us)
 __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm)
 decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __nv_bfloat16* __restrict__ core_k,
                   const __nv_bfloat16* __restrict__ core_v, const int32_t* __restrict__ count, int cap,
-                  const int32_t* __restrict__ core_len, float scale_log2, int n_split, int mode,
+                  const int32_t* __restrict__ core_len, float scale_log2, int B, int mode,
                   __nv_bfloat16* __restrict__ out, float* __restrict__ part, int32_t* __restrict__ tickets) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ float sh_m[kWarps][8];
@@ -208,14 +247,25 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, tig = lane & 3;
-    const int split = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const int G = Hq / Hkv;
-    const int bh = b * Hkv + h;
     // An ordinary launch waits here for the kernel before it.  Under an overlapped one the next kernel may start beside
     // this one, and whatever this block reads before its own griddepcontrol.wait below (core_len, cores, counts) must not
     // be written by a kernel that may still be running then; that is the caller's promise when it asks for one.
-    if (mode == kOrdinary) in_stream_order();
-    else asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    if (mode == kOrdinary) asm volatile("griddepcontrol.wait;\n" ::: "memory");
+    // Where there are spare units the next kernel is let in only when they have gone: its blocks would find both slots of some
+    // SMs taken by them, and settle unevenly (128 raw heads x 8 K rows: 80 us, 92 with the next kernel let in at once).
+    if (!kSpares) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    // the block's head, and its place among the head's blocks
+    int bh = blockIdx.z * Hkv + blockIdx.y, split = blockIdx.x, n_split = gridDim.x;   // as if every head had one unit
+    Units u = {bh, 0, 0};
+    if (kSpares) {
+        const int heads = B * Hkv, spare = bh - heads;
+        u = plan_units(core_len, heads, cap, spare < 0 ? bh : -1, spare, lane);
+        if (u.head < 0) return;   // a spare unit that no head needs: nothing read, nothing written
+        n_split *= 1 + u.extra;
+        if (spare >= 0) split += (1 + spare - u.begin) * (int)gridDim.x;
+        bh = u.head;
+    }
     const int len = max(min(core_len[bh], cap), 0);
     const int tiles_total = (len + kTile - 1) / kTile;
     const int tiles_per_split = (tiles_total + n_split - 1) / n_split;
@@ -251,7 +301,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     // q^T as the B operand of every k-step: b0 = q[head g][16ks + 2tig, +1], b1 = same + 8
     uint32_t qb[8][2];
     {
-        const __nv_bfloat16* qh = q + ((size_t)b * Hq + (size_t)h * G + g) * kD;
+        const __nv_bfloat16* qh = q + ((size_t)bh * G + g) * kD;
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
             // read through L2: under a chained launch q was written while this kernel was already running
@@ -345,6 +395,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
         if (nxt < my_tiles)
             issue_tile(wbase + (i % kStages) * kStageBytes, kh, vh, ch, (t0 + warp + nxt * kWarps) * kTile, len, lane, soff);
         cp_async_commit();
+        if (kSpares && i == 0) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     }
     cp_async_wait<0>();
 
@@ -407,8 +458,11 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     // and no single block pulling all partials through its own port); the members stay until all have read.
     cg::cluster_group cluster = cg::this_cluster();
     const int csize = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
-    const int n_clusters = n_split / csize, cidx = split / csize;   // clusters per head, this one's index
-    float* my_part = part + ((size_t)bh * n_clusters + cidx) * kPartStride;
+    const int n_clusters = n_split / csize, cidx = split / csize;   // clusters of the head, this one's index
+    // partials: every head's own unit in turn, then the spare units; a unit leaves one for each of its clusters
+    const int per_unit = kSpares ? (int)gridDim.x / csize : n_clusters;
+    const int first = bh * per_unit, more = (B * Hkv + u.begin) * per_unit;
+    float* my_part = part + (size_t)(cidx + (!kSpares || cidx < per_unit ? first : more - per_unit)) * kPartStride;
     const bool direct = n_clusters == 1;   // this cluster holds the whole head: its fold is the result
     const int slice = (G * (kD / 4) + csize - 1) / csize;
     cluster.sync();
@@ -445,7 +499,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
         }
         if (direct) {
             const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
-            store_out4(out + ((size_t)b * Hq + (size_t)h * G + hd) * kD + d4, acc, inv);
+            store_out4(out + ((size_t)bh * G + hd) * kD + d4, acc, inv);
         } else {
             *reinterpret_cast<float4*>(my_part + hd * kD + d4) = acc;
             if (d4 == 0) { my_part[8 * kD + hd] = gm; my_part[8 * kD + 8 + hd] = lsum; }
@@ -456,7 +510,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     if (direct || crank != 0) return;
 
     // ---- several partials per head: the last block to arrive merges them ----
-    ticket_and_merge(part, tickets, bh, n_clusters, G, Hq, b, h, out, &sh_last);
+    ticket_and_merge<kSpares>(part, first, more, per_unit, n_clusters, tickets, bh, G, out, &sh_last);
 }
 
 // Block split of one head: how many blocks stream it, and how they are grouped into clusters.
@@ -464,17 +518,17 @@ struct SplitPlan { int n_split, cluster; };
 // Largest number of clusters of c blocks (c = 2..16) that are resident at once, two blocks per SM: fit[c].
 struct Resident { int sms; int fit[kMaxCluster + 1]; };
 
-inline int head_slots(long long heads, int cap) {   // most partials a head can leave in global memory
+inline int head_slots(long long heads, int cap) {   // most partials the own unit of a head can leave in global memory
     const int by_rows = (cap + 63) / 64;
     const int s = heads >= kMaxSlots ? 1 : (int)(kMaxSlots / heads);
     return s < by_rows ? s : (by_rows < 1 ? 1 : by_rows);
 }
-// Partials a launch can leave.  It grows with the number of heads and with the capacity, so that a workspace for the largest batch
-// serves every smaller one (more than kMaxTickets heads have one cluster each and leave none).
+// Partials a launch can leave, the spare units' among them.  It grows with the number of heads and with the capacity, so that a
+// workspace for the largest batch serves every smaller one.
 inline size_t all_slots(long long heads, int cap) {
     const long long by_rows = cap < 64 ? 1 : (cap + 63) / 64, split = heads * by_rows;
     const long long several = split < kMaxSlots ? split : kMaxSlots, own = heads < kMaxTickets ? heads : kMaxTickets;
-    return (size_t)(several > own ? several : own);
+    return 2 * (size_t)(several > own ? several : own);
 }
 
 // The rules and what they were measured against (us per layer, Llama-shaped heads of 128 columns, 2 x 148 block slots; the
@@ -513,6 +567,14 @@ inline SplitPlan plan_for(long long heads, int cap, bool raw, const Resident& re
     return {c * (k < 1 ? 1 : k), c};
 }
 
+// Spare units (plan_units) for a batch whose blocks may otherwise get thousands of rows to stream.  Among equal heads they cost
+// 0.5 us (16 x 8 heads of 8 K capacity 42.9 -> 43.4), up to 7 % where a block has little to do.  16 x 8 heads, one sequence long and the
+// others short: 32 K of 32 K 134 -> 43 us, 4 K of 4 K 22.6 -> 18.9, raw 32 K 220 -> 58; not below 1 K rows a block (8 K of 8 K over
+// 4 x 8 heads, eight blocks each, 16.5 -> 18.9) and not for two sequences, whose longer one can only gain half (34.8 -> 34.3).
+inline bool has_spares(int B, int Hkv, int cap, int n_split) {
+    return B > 2 && (long long)B * Hkv <= kMaxTickets && cap >= 4096 && cap > 1024 * n_split;
+}
+
 }  // namespace dm
 
 bool decode_mma_supported(const DecodeArgs& a) {
@@ -541,8 +603,11 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
         int v = 0;
         cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
         res.sms = v < 1 ? 1 : v;
-        cudaFuncSetAttribute(dm::decode_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dm::kSmemBytes);
-        const bool wide = cudaFuncSetAttribute(dm::decode_mma_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        bool wide = true;
+        for (auto kernel : {dm::decode_mma_kernel<false>, dm::decode_mma_kernel<true>}) {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dm::kSmemBytes);
+            wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess && wide;
+        }
         for (int c = 2; c <= dm::kMaxCluster; ++c) {
             cudaLaunchConfig_t probe = {};
             probe.gridDim = dim3(c, 1, 1);
@@ -555,7 +620,7 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
             probe.numAttrs = 1;
             int n_clusters = 0;
             res.fit[c] = 0;
-            if ((c <= 8 || wide) && cudaOccupancyMaxActiveClusters(&n_clusters, dm::decode_mma_kernel, &probe) == cudaSuccess) res.fit[c] = n_clusters;
+            if ((c <= 8 || wide) && cudaOccupancyMaxActiveClusters(&n_clusters, dm::decode_mma_kernel<false>, &probe) == cudaSuccess) res.fit[c] = n_clusters;
         }
         (void)cudaGetLastError();   // a refused opt-in or probe is not an error of this call
     });
@@ -564,7 +629,8 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
     float* part = (float*)((char*)a.ws + decode_mma_counter_bytes());
     const float scale = (a.scale == 0.f ? 1.f / sqrtf((float)a.d) : a.scale) * 1.4426950408889634f;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(plan.n_split, a.Hkv, a.B);
+    const bool spares = dm::has_spares(a.B, a.Hkv, a.cap, plan.n_split);
+    cfg.gridDim = dim3(plan.n_split, a.Hkv, spares ? 2 * a.B : a.B);
     cfg.blockDim = dim3(dm::kWarps * 32);
     cfg.dynamicSmemBytes = dm::kSmemBytes;
     cfg.stream = st;
@@ -577,9 +643,9 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
     cfg.numAttrs = 2;
     const int mode = (a.flags & SC_FLAG_OVERLAP_CHAIN) ? dm::kChained : (a.flags & SC_FLAG_OVERLAP_PREV) ? dm::kOverlapped : dm::kOrdinary;
     note_launches(1);
-    return own_error(cudaLaunchKernelEx(&cfg, dm::decode_mma_kernel, (const __nv_bfloat16*)a.q, a.Hq, a.Hkv,
+    return own_error(cudaLaunchKernelEx(&cfg, spares ? dm::decode_mma_kernel<true> : dm::decode_mma_kernel<false>, (const __nv_bfloat16*)a.q, a.Hq, a.Hkv,
                                         (const __nv_bfloat16*)a.core_k, (const __nv_bfloat16*)a.core_v, a.count, a.cap,
-                                        a.core_len, scale, plan.n_split, mode, (__nv_bfloat16*)a.out, part, tickets));
+                                        a.core_len, scale, a.B, mode, (__nv_bfloat16*)a.out, part, tickets));
 }
 
 }  // namespace sc
