@@ -536,18 +536,30 @@ inline size_t all_slots(long long heads, int cap) {
 // block in advance -- which cost more than anything else, 10 to 30 % of every batched or long launch):
 //   - one cluster per head, as wide as lets the clusters of all heads be resident at once: 128 heads x 3.4 K rows, 2 blocks
 //     each, 51.6 -> 41.2; 56 heads x 6.3 K, 5, 43.7 -> 33.9; 32 x 6.3 K, 8, 31.9 -> 22.5; 24 x 12.6 K, 10, 45.7 -> 31.9; 16 x 25 K, 12,
-//     47.0 -> 36.0; 8 x 34 K, 16, 40.2 -> 27.8.  (13 fits 16 heads too and is 3 to 9 % slower than 12.)
+//     47.0 -> 36.0; 8 x 34 K, 16, 40.2 -> 27.8.  More than 12 only where
+//     16 would fit: 16 heads, for which 13 do and 14 do not, 13 blocks instead of 12: 4 to 25 K rows 1 to 2 % faster, 2.1 K rows 8.3 -> 8.9.
 //   - fewer blocks for short capacities, whose time is the fold and the barrier: 8 heads x 0.5 K rows of 1 K capacity: 9 blocks
 //     4.5, 16 blocks 5.0; x 2.1 K of 4 K: 12 blocks 6.1, 16 blocks 6.6; from 8 K of capacity on 16.
 //   - several clusters per head where few heads would leave blocks with thousands of rows: 4 heads x 34 K rows, 3 x 16, 19.7 (one: 21;
 //     21.1 to 43.6 before); not below, the ticket and the merge cost 2: 4 heads x 8.5 K, one cluster 9.2, three 11.1.
-//   - more heads than any cluster width fits: one block per head (256 heads x 3.4 K rows: 82.1, split in two 83.2, 94.0 before).
-//   - a cache without counts is a raw one, whose heads are full and alike: one block per SM outside clusters keeps HBM
-//     busiest (32 heads x 64 K rows, 4 each, 157; 8 each in clusters 166; 192 before; 8 heads x 131 K: 83.5 against 116.9).
+//   - more heads than any cluster width fits: one block per head (256 heads x 3.4 K rows: 82.1, split in two 83.2, 94.0 before); where
+//     they are up to 15 % more than two per SM, which leaves a last round nearly empty, clusters of three (320 heads x 7 K rows:
+//     210 -> 176; 368: 214 -> 204, but with 3.4 K rows 110 -> 120; 320 x 2 K rows of 4 K 68 -> 74).
+//   - a cache without counts is a raw one, whose heads are mostly full: one block per SM outside clusters keeps HBM
+//     busiest (32 heads x 64 K rows, 4 each, 157; 8 each in clusters 166; 192 before; 8 heads x 131 K: 83.5 against 116.9).  From 75
+//     heads on that is one block each; where it leaves more SMs idle in its last round than clusters of two or three would,
+//     those are taken: 76 heads x 8 K rows 60.7 -> 54.4, 88 63.3 -> 60.3, 176 123 -> 113, 200 137 -> 131, 320 232 -> 206 (104 to 152
+//     and 296 heads: one block each is best).
 inline SplitPlan plan_for(long long heads, int cap, bool raw, const Resident& res) {
     const int by_rows = (cap + 4 * kTile - 1) / (4 * kTile);   // at least 64 rows per split
     if (raw && cap >= 8192) {
         int s = heads >= res.sms ? 1 : (int)(res.sms / heads);
+        if (s == 1) {   // one block each, or a cluster of two or three where its rounds of one block per SM are a tenth fuller
+            const auto rounds = [&](long long blocks) { return (blocks + res.sms - 1) / res.sms; };
+            for (int w = 2; w <= 3; ++w)
+                if ((heads <= res.fit[w] || 20 * heads > 21 * res.sms) && 10 * w * rounds(heads * s) > 11 * s * rounds(heads * w)) s = w;
+            return {s, s};
+        }
         const int slots = head_slots(heads, cap);
         s = s < 16 ? s : 16 * (s / 16);
         if (s > slots) s = slots;
@@ -558,7 +570,8 @@ inline SplitPlan plan_for(long long heads, int cap, bool raw, const Resident& re
     if (limit > kMaxCluster) limit = kMaxCluster;
     int c = 1;
     for (int w = 2; w <= limit; ++w)
-        if (w != 13 && heads <= res.fit[w]) c = w;
+        if (heads <= res.fit[w] && (w <= 12 || heads <= res.fit[kMaxCluster])) c = w;
+    if (heads > 2 * res.sms && 20 * heads <= 46 * res.sms && cap >= 8192) c = 3;
     if (c < kMaxCluster) return {c, c};
     int k = (cap + kMaxCluster * kCapRowsPerBlock - 1) / (kMaxCluster * kCapRowsPerBlock);   // clusters per head
     if (k > res.fit[c] / heads) k = (int)(res.fit[c] / heads);
@@ -570,9 +583,10 @@ inline SplitPlan plan_for(long long heads, int cap, bool raw, const Resident& re
 // Spare units (plan_units) for a batch whose blocks may otherwise get thousands of rows to stream.  Among equal heads they cost
 // 0.5 us (16 x 8 heads of 8 K capacity 42.9 -> 43.4), up to 7 % where a block has little to do.  16 x 8 heads, one sequence long and the
 // others short: 32 K of 32 K 134 -> 43 us, 4 K of 4 K 22.6 -> 18.9, raw 32 K 220 -> 58; not below 1 K rows a block (8 K of 8 K over
-// 4 x 8 heads, eight blocks each, 16.5 -> 18.9) and not for two sequences, whose longer one can only gain half (34.8 -> 34.3).
+// 4 x 8 heads, eight blocks each, 16.5 -> 18.9) and not for two sequences, whose longer one can only gain half (34.8 -> 34.3), and for
+// heads of one block each only from 8 K on (344 heads x 2 K of 4 K 69.5 -> 71.4).
 inline bool has_spares(int B, int Hkv, int cap, int n_split) {
-    return B > 2 && (long long)B * Hkv <= kMaxTickets && cap >= 4096 && cap > 1024 * n_split;
+    return B > 2 && (long long)B * Hkv <= kMaxTickets && cap >= (n_split == 1 ? 8192 : 4096) && cap > 1024 * n_split;
 }
 
 }  // namespace dm

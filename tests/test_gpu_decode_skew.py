@@ -104,3 +104,14 @@ def test_a_long_sequence_does_not_hold_up_the_batch():
     H, G = 8, 4
     skewed, even = _us(_layer([32768] + [1024] * 15, 32768, H, 1), H, G), _us(_layer([3008] * 16, 32768, H, 1), H, G)
     assert skewed < 2 * even, (skewed, even)
+
+
+@pytest.mark.parametrize("B,H,G,cap,raw", [(19, 4, 2, 8192, True), (11, 8, 1, 8200, True), (22, 8, 1, 8192, True), (38, 8, 1, 8192, True),
+                                           (38, 8, 4, 8200, False), (42, 8, 1, 8192, False), (2, 8, 4, 7300, False), (1, 8, 4, 5300, False)])
+def test_more_heads_than_seats(B, H, G, cap, raw):
+    """Where a block per head would leave SMs idle in the last round: clusters of two and three; and widths that are passed over."""
+    lens = [cap - 37 * b for b in range(B)]
+    y = _layer(lens, cap, H, B)
+    q = torch.randn((B, H * G, 128), generator=torch.Generator(device=DEV).manual_seed(B), device=DEV).bfloat16()
+    got = binding.decode_attn(q, y, use_count=not raw)
+    assert_close_vectors(to_f64(got), _reference(q, y, raw), TOL[torch.bfloat16], f"{B} x {H} x {G}, capacity {cap}")
