@@ -681,8 +681,10 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
             const long long ctas = (long long)((G * a.m + kT - 1) / kT) * a.Hkv * a.B;
             const int half_tiles = ((a.cap + kT - 1) / kT + 1) / 2;
             int n_split = 1;
-            for (int c = rep == 1 && half_tiles < 8 ? 4 : 2; c <= kMaxSplit; ++c)
+            for (int c = rep == 1 && half_tiles < 8 ? 4 : 2; c <= kMaxSplit; ++c) {
+                if (c > 8 && half_tiles < (c < 12 ? 2 * c : c)) continue;   // a second round of the fold for less than a tile
                 if (ctas <= fit[c] && (half_tiles + c - 1) / c < (half_tiles + n_split - 1) / n_split) n_split = c;
+            }
             p.n_split = n_split;
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)((G * a.m + kT - 1) / kT) * n_split, a.Hkv, a.B);
