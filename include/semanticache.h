@@ -413,8 +413,9 @@ SC_API sc_status sc_append_layers(const sc_append_layer* layers /*DEVICE [L]*/, 
  * process exits, whether or not this entry point is ever called.  The call itself performs no
  * cudaMalloc / cudaFree and calls no allocating routine.
  *
- *   - Shapes whose workspace (sc_decode_workspace_bytes) exceeds SC_STATIC_SCRATCH_BYTES are
- *     rejected with SC_ERR_CAPACITY before anything is enqueued; use sc_decode_attn for those.
+ *   - Shapes whose workspace (sc_decode_workspace_bytes, less the 2 KB of its arrival counters)
+ *     exceeds SC_STATIC_SCRATCH_BYTES are rejected with SC_ERR_CAPACITY before anything is
+ *     enqueued; use sc_decode_attn for those.
  *     For d = 128 the limit admits B * Hq * min(64, ceil(cap / 512)) up to about 16000, e.g.
  *     16 sequences of 32 query heads with 8K rows of capacity each.
  *   - The first call on each GPU looks up the array's device address (a short host-side set-up,

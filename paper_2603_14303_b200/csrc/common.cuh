@@ -160,6 +160,7 @@ struct DecodeArgs {
 };
 cudaError_t launch_decode_generic(const DecodeArgs& a, cudaStream_t st);
 size_t decode_generic_ws_bytes(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t cap);
+size_t decode_mma_counter_bytes();
 
 struct PrefillArgs {   // Eq. 4 with a block of m queries per head
     const void* q; sc_dtype dt; int32_t B, Hq, Hkv, m, d;

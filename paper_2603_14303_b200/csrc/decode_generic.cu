@@ -205,7 +205,7 @@ combine_generic(int64_t heads, int d, int n_split, const float* __restrict__ par
 
 size_t decode_generic_ws_bytes(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t cap) {
     (void)Hkv;
-    return sizeof(float) * (size_t)B * Hq * generic_splits(cap) * (d + 2) + 256;
+    return decode_mma_counter_bytes() + sizeof(float) * (size_t)B * Hq * generic_splits(cap) * (d + 2) + 256;
 }
 
 template <typename T>
@@ -216,8 +216,9 @@ static cudaError_t run(const DecodeArgs& a, cudaStream_t st) {
     const int64_t blocks = (int64_t)n_split * a.Hkv * groups * a.B;
     if (blocks > 0x7fffffff) return cudaErrorInvalidConfiguration;
     const unsigned grid = (unsigned)blocks;
-    // partials are read and written in pairs of floats; a workspace need only be aligned to one (256 spare bytes cover the step)
-    float* part = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(a.ws) + 7) & ~(uintptr_t)7);
+    // Partials lie behind the tensor-core kernel's counters, which have to stay zero for a later call with this workspace.  They
+    // are read and written in pairs of floats; a workspace need only be aligned to one (256 spare bytes cover the step).
+    float* part = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(a.ws) + decode_mma_counter_bytes() + 7) & ~(uintptr_t)7);
     cudaError_t e = launch_in_order(a.d <= 128 ? decode_generic<T, 4> : decode_generic<T, 8>, dim3(grid), kDecWarps * 32, 0, st,
                                     (const T*)a.q, a.Hq, a.Hkv, a.d, (const T*)a.core_k, (const T*)a.core_v, a.count, a.cap,
                                     a.core_len, scale, n_split, part);

@@ -14,7 +14,8 @@
 
 // The scratch itself.  In host code this name is only a handle for the runtime's symbol table,
 // never an address a kernel may be given; the device address is looked up per GPU below.
-static __device__ __align__(256) unsigned char g_static_scratch[SC_STATIC_SCRATCH_BYTES];
+static constexpr size_t kCounterRoom = 2048;   // the arrival counters' place comes on top
+static __device__ __align__(256) unsigned char g_static_scratch[SC_STATIC_SCRATCH_BYTES + kCounterRoom];
 
 namespace {
 
@@ -44,7 +45,6 @@ cudaError_t static_scratch(void** out) {
 
 namespace sc {
 bool decode_mma_supported(const DecodeArgs& a);
-size_t decode_mma_counter_bytes();
 }  // namespace sc
 
 extern "C" sc_status sc_decode_attn_static(const void* q, sc_dtype dt, int32_t B, int32_t Hq, int32_t Hkv,
@@ -61,7 +61,7 @@ extern "C" sc_status sc_decode_attn_static(const void* q, sc_dtype dt, int32_t B
     if (flags & (SC_FLAG_OVERLAP_PREV | SC_FLAG_OVERLAP_CHAIN)) return SC_ERR_INVALID_ARG;
     if (B == 0) return SC_OK;
     const size_t need = sc_decode_workspace_bytes(B, Hq, Hkv, d, cap);
-    if (need > (size_t)SC_STATIC_SCRATCH_BYTES) return SC_ERR_CAPACITY;   // problem too large for the fixed array
+    if (need > SC_STATIC_SCRATCH_BYTES + kCounterRoom) return SC_ERR_CAPACITY;   // problem too large for the fixed array
     void* scratch = nullptr;
     if (static_scratch(&scratch) != cudaSuccess) return SC_ERR_CUDA;
     // The array still holds whatever the previous call (or an aborted one) left.  Only the arrival
@@ -75,5 +75,5 @@ extern "C" sc_status sc_decode_attn_static(const void* q, sc_dtype dt, int32_t B
             return SC_ERR_CUDA;
     }
     return sc_decode_attn(q, dt, B, Hq, Hkv, d, core_k, core_v, count, cap, core_len, scale, flags, out, scratch,
-                          (size_t)SC_STATIC_SCRATCH_BYTES, status, stream);
+                          SC_STATIC_SCRATCH_BYTES + kCounterRoom, status, stream);
 }

@@ -1,5 +1,5 @@
-"""The float32 calls: a decode workspace that starts on any float, and a launch that the runtime refuses, which is an error of
-its own call only."""
+"""The generic calls: a decode workspace that starts on any float and is shared with the tensor-core kernel, and a launch that
+the runtime refuses, which is an error of its own call only."""
 import ctypes
 
 import pytest
@@ -40,3 +40,22 @@ def test_a_refused_launch_is_not_an_error_of_the_next_call():
     code = binding.lib().sc_prefill_attn(none, binding.SC_F32, 1 << 20, 1 << 13, 1 << 13, 1, 40, none, none, None, 8, none, 0.0, 0, none, None, None)
     assert code == binding.SC_ERR_CUDA
     assert_close_vectors(to_f64(binding.decode_attn(q, y)), ref, TOL[torch.float32], "decode")
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_one_workspace_for_both_kinds_of_kernel(dtype):
+    # the batch's long heads meet through counters in front of the workspace, which the generic kernels have to leave alone
+    B, H, cap, d = 4, 2, 9000, 128
+    g = torch.Generator(device=DEV).manual_seed(3)
+    rand = lambda *shape: torch.randn(shape, generator=g, device=DEV)
+    k, v = rand(B, H, cap, d), rand(B, H, cap, d)
+    count = torch.randint(1, 9, (B, H, cap), generator=g, device=DEV, dtype=torch.int32)
+    lens = torch.tensor([[9000], [300], [20], [0]], dtype=torch.int32, device=DEV).expand(B, H).contiguous()
+    y = binding.CompressedLayer(k.bfloat16(), v.bfloat16(), count, lens)
+    z = binding.CompressedLayer(k.to(dtype), v.to(dtype), count, lens)
+    q = rand(B, 4 * H, d)
+    ws = binding.decode_workspace(B, 4 * H, H, d, cap, DEV)
+    want = binding.decode_attn(q.bfloat16(), y)
+    for _ in range(2):
+        binding.decode_attn(q.to(dtype), z, workspace=ws, flags=binding.SC_FLAG_GENERIC)
+        assert torch.equal(binding.decode_attn(q.bfloat16(), y, workspace=ws), want)
