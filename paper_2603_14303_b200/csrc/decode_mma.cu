@@ -581,12 +581,13 @@ inline SplitPlan plan_for(long long heads, int cap, bool raw, const Resident& re
 }
 
 // Spare units (plan_units) for a batch whose blocks may otherwise get thousands of rows to stream.  Among equal heads they cost
-// 0.5 us (16 x 8 heads of 8 K capacity 42.9 -> 43.4), up to 7 % where a block has little to do.  16 x 8 heads, one sequence long and the
-// others short: 32 K of 32 K 134 -> 43 us, 4 K of 4 K 22.6 -> 18.9, raw 32 K 220 -> 58; not below 1 K rows a block (8 K of 8 K over
-// 4 x 8 heads, eight blocks each, 16.5 -> 18.9) and not for two sequences, whose longer one can only gain half (34.8 -> 34.3), and for
-// heads of one block each only from 8 K on (344 heads x 2 K of 4 K 69.5 -> 71.4).
-inline bool has_spares(int B, int Hkv, int cap, int n_split) {
-    return B > 2 && (long long)B * Hkv <= kMaxTickets && cap >= (n_split == 1 ? 8192 : 4096) && cap > 1024 * n_split;
+// 0.3 to 0.7 us (16 x 8 heads of 8 K capacity 42.9 -> 43.4; raw, 8 K rows, 40 to 72 heads up to 7 %); wide clusters find no room beside
+// the others and come last (4 x 8 heads of 13 K, eight blocks each, 13.7 -> 14.4), so they need more rows to be worth it.  One
+// sequence long, the others short, 16 x 8 heads: 32 K of 32 K 134 -> 43 us, 4 K of 4 K 22.6 -> 18.9, raw 32 K 220 -> 57; 4 x 8 heads,
+// 32 K 46.7 -> 33.8.  Not for two sequences, whose longer one can only gain half (34.8 -> 34.3), and for heads of one block each only
+// from 8 K on (344 heads x 2 K of 4 K 69.5 -> 71.4).
+inline bool has_spares(int B, int Hkv, int cap, int n_split, bool raw) {
+    return B > 2 && (long long)B * Hkv <= kMaxTickets && cap >= (n_split == 1 ? 8192 : 4096) && cap > (raw || n_split <= 2 ? 1024 : 2048) * n_split;
 }
 
 }  // namespace dm
@@ -643,7 +644,7 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
     float* part = (float*)((char*)a.ws + decode_mma_counter_bytes());
     const float scale = (a.scale == 0.f ? 1.f / sqrtf((float)a.d) : a.scale) * 1.4426950408889634f;
     cudaLaunchConfig_t cfg = {};
-    const bool spares = dm::has_spares(a.B, a.Hkv, a.cap, plan.n_split);
+    const bool spares = dm::has_spares(a.B, a.Hkv, a.cap, plan.n_split, a.count == nullptr);
     cfg.gridDim = dim3(plan.n_split, a.Hkv, spares ? 2 * a.B : a.B);
     cfg.blockDim = dim3(dm::kWarps * 32);
     cfg.dynamicSmemBytes = dm::kSmemBytes;
