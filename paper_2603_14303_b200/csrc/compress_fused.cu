@@ -20,32 +20,24 @@
 //      from the cluster numbers (kept as bf16: comparing two of them gives the 1.0 or 0.0 the product wants), K and V come
 //      transposed from their staged rows (ldmatrix.trans), mma.m16n8k16 adds up in fp32 (products with 1 and 0 are exact).
 //      Sixteen clusters of more than one token at a time, over the tokens from their first seed to the end of their last
-//      segment only; each warp takes a quarter of the columns.  Sums are scaled by 1/|S|, rounded once and stored.  Clusters of one token are copied bit for bit; a sum that is not finite (0 * inf would reach other
-//      clusters) sends the sixteen clusters to a loop over their members.
+//      segment only; each warp takes a quarter of the columns.  Sums are scaled by 1/|S|, rounded once and stored.  Clusters
+//      of one token are copied bit for bit; a sum that is not finite (0 * inf would reach other clusters) sends the sixteen
+//      clusters to a loop over their members.
 //
 // What bounds it: one launch over 32 layers x 8 heads x 32K tokens takes 1105 us on resident inputs (4.9 TB/s); copies
 // of the kernel with steps left out take 707 us (loads only), 834 (loads, steps 1 and 2) and 1025 (all but the
 // stores of the means), so step 3's shared-memory traffic and arithmetic are the largest part above the loads, then the stores.
 // A tile of 129..256 tokens spends 12 K cycles on step 2 and holds up the look-back of the tiles behind it.
-// The kernel before this one clustered every segment with one warp's mma.sync tiles and greedy pass and added up member
-// rows on the CUDA cores, nine warps and five block barriers a tile, 13 K warp instructions per 128 tokens (6.5 K here):
-// 1395 us; 16 sequences x 16K, lognormal chunks, 8 heads, per layer 500 us, 300 here; 4 x 64K in chunks of 128 with
-// sc_chunk 794 and 578.
-// Of that: masks, segment bounds and seeds without branches per lane, and the code for negative thresholds in instances
-// of its own, 16 x 16K 633 -> 612 us for two layers, chunks of 128 tokens 738 -> 589 (a settled long tile 19 K -> 12 K cycles);
-// clusters of one token out of the product, chunks of 8 tokens -7 %, 16 x 16K -3 %, 32K -1 %.
-// Measured and not taken: sums over member rows in cluster order instead of the product, 1245 us; keys and values released
-// and pooled separately so that the next keys load earlier, +13 %; L2 prefetch of the next tile, +5 %; a second service
-// warp (96 registers a thread), worse throughout; eight pooling warps (72 registers), +1 %; means written to their seeds'
-// staged rows and copied out in 16-byte pieces, +3 %, and +5 % with the offset awaited only before the copy; products of
-// long tiles by mma.sync, 16 x 16K +8 %; mbarrier waits with a suspend-time hint and tickets staggered between heads, no
-// change.  One step out of line or not moves a workload by up to 5 % either way.
+// Why these steps: one product per tile and decision rounds take 6.5 K warp instructions per 128 tokens, a warp per segment with
+// mma.sync tiles, the greedy pass and sums of member rows on the CUDA cores took 13 K: 32 layers 1395 us; 16 sequences x 16K,
+// lognormal chunks, 500 us a layer against 300; 4 x 64K in chunks of 128 794 against 578.  Sums over member rows in cluster
+// order in place of the product: 1245 us.
 //
 // Offsets: a prefix sum over the tiles of each head by decoupled look-back over per-tile status words; tickets are handed
 // out in order, so every predecessor is held by a running block and the bounded wait cannot starve.  A block draws its
-// next ticket only when its tile's count is out and its offset known: drawn with the staging, one tile earlier, a tile
-// waited unstarted in a block that itself waited, and held up its successors (16 x 16K: 711 -> 666 us for two layers; chunks of
-// 128 tokens: 884 -> 781).  Tickets go round the (layer, sequence, head) units.  The last block to finish zeroes the
+// next ticket only when its tile's count is out and its offset known: drawn one tile earlier, a tile waits unstarted in a
+// block that itself waits, and holds up its successors (16 x 16K, two layers 666 us against 711; chunks of 128 tokens 781
+// against 884).  Tickets go round the (layer, sequence, head) units.  The last block to finish zeroes the
 // status words and counters, so a workspace that was zero before the call is zero again after it.  One launch may
 // serve several layers (sc_compress_layers).
 #include <cuda.h>
@@ -71,21 +63,18 @@ constexpr int kShortRows = SC_TILE_ROWS;          // 128
 constexpr int kHalfShort = kShortRows * kHalfRow; // 16384: distance between the column halves of a short tile
 constexpr int kHalfLong = kMaxRows * kHalfRow;    // 32768: ... of a long one
 constexpr int kVOff = 2 * kHalfShort;             // short: K | V, long = one tensor
-constexpr int kBitOff = 2 * kHalfLong;            // uint32[256][8]: earlier-neighbour bits of a long tile's rows
-constexpr int kNormOff = kBitOff;                 // float[128]: norms of a short tile's rows (no bits are stored for it)
-constexpr int kLongNormOff = kBitOff + kMaxRows * 32;        // float[256]
-// behind the norms, once the bits are in registers:
-constexpr int kRankOff = kBitOff + 1024;                     // bf16[256]: cluster of each token (whole numbers to 256 are exact), see rank_slot
-constexpr int kCntOff = kRankOff + kMaxRows * 2;                 // int32[256]: tokens of each cluster
+constexpr int kNormOff = 2 * kHalfLong;           // float[256]: norms of the tile's rows
+constexpr int kRankOff = kNormOff + kMaxRows * 4;            // bf16[256]: cluster of each token (whole numbers to 256 are exact), see rank_slot
+constexpr int kCntOff = kRankOff + kMaxRows * 2;             // int32[256]: tokens of each cluster
 constexpr int kSeedOff = kCntOff + kMaxRows * 4;             // uint8[256]: the cluster's seed
 constexpr int kListOff = kSeedOff + kMaxRows;                // uint8[256]: the clusters of more than one token, in order
 constexpr int kEndOff = kListOff + kMaxRows;                 // uint16[256]: end of the seed's segment
-constexpr int kMiscOff = kLongNormOff + kMaxRows * 4;        // seeds[8], members[8]; starts[2][4]; geo[2][8]; base, P, tmem slot, flags
+constexpr int kMiscOff = kEndOff + kMaxRows * 2;             // seeds[8], members[8]; starts[2][4]; geo[2][8]; base, P, tmem slot, flags
 constexpr int kBarOff = kMiscOff + 64 + 32 + 64 + 32;
 constexpr int kSmemBytes = kBarOff + 64;
 constexpr int kTmemCols = 128;                    // one 128 x 128 fp32 accumulator per block (three blocks per SM: 384 of 512 columns)
 constexpr int kBlocksPerSm = 3;
-static_assert(kEndOff + kMaxRows * 2 <= kLongNormOff && kRankOff % 16 == 0 && kMiscOff % 16 == 0 && kBarOff % 8 == 0, "alignment");
+static_assert(kRankOff % 16 == 0 && kCntOff % 16 == 0 && kMiscOff % 16 == 0 && kBarOff % 8 == 0, "alignment");
 static_assert(kSmemBytes <= 76800, "three blocks per SM need <= 75 KB each");
 
 enum Mode { kCountOnly = 0, kLookBack = 1 };
@@ -93,7 +82,8 @@ enum Geo { gB = 0, gH = 1, gT = 2, gNseg = 3, gRow0 = 4, gR = 5, gLast = 6, gLay
 
 constexpr uint32_t kFlagAggregate = 1u << 30, kFlagPrefix = 2u << 30, kValueMask = (1u << 30) - 1;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // every wait gives up after 2 s
-constexpr int kPollGroups = 2;                               // the look-back reads 64 predecessors per poll (4 and 8 measured slower, 1 slower on short chunks)
+// The look-back reads 64 predecessors per poll (4 and 8 groups measured slower, 1 slower on short chunks).
+constexpr int kPollGroups = 2;
 constexpr int kCtlWords = 64;                                // ticket, done counter, padding
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -353,7 +343,7 @@ __device__ __noinline__ int settle_short_tile(unsigned char* smem, const uint32_
 template <bool kAnyTau>
 __device__ __noinline__ int settle_long_tile(unsigned char* smem, int R, uint32_t tmem, uint32_t phase_u, float tau, bool wait_failed,
                                              int32_t* as, int row0, uint32_t* publish, int* sh_p) {
-    float* norm = reinterpret_cast<float*>(smem + kLongNormOff);
+    float* norm = reinterpret_cast<float*>(smem + kNormOff);
     const uint32_t sbase = smem_u32(smem), bar_u = sbase + kBarOff + 16;
     const int tid = threadIdx.x, lane = tid & 31, q = tid >> 5;
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
@@ -400,8 +390,8 @@ __device__ __noinline__ int settle_long_tile(unsigned char* smem, int R, uint32_
 }
 
 // Step 3 for sixteen clusters whose sums are not all finite: each lane one column of the warp's quarter, member by member.
-__device__ __noinline__ void pool_by_members(const unsigned char* tensor, int hs, const unsigned char* smem, bool listed, int m, int n_multi, int t_lo, int t_hi,
-                                             __nv_bfloat16* dst, int room, int warp, int lane) {
+__device__ __noinline__ void pool_by_members(const unsigned char* tensor, int hs, const unsigned char* smem, bool listed, int m,
+                                             int n_multi, int t_lo, int t_hi, __nv_bfloat16* dst, int room, int warp, int lane) {
     const int* cnt = reinterpret_cast<const int*>(smem + kCntOff);
     const int col = warp * 32 + lane;
     for (int x = 16 * m; x < min(16 * m + 16, n_multi); ++x) {
