@@ -14,7 +14,11 @@
  *     counter, per-GPU launch geometry looked up on first use, and, for sc_decode_attn_static
  *     only, its fixed scratch array with the per-GPU address of that array.
  *   - All work is enqueued on `stream` (a cudaStream_t passed as void*; NULL = default stream).
- *     Calls return after enqueueing; they never synchronise.
+ *     Calls return after enqueueing; they never synchronise.  Kernels are launched with programmatic
+ *     stream serialization and wait for the kernel before them in the stream.  That is the order of
+ *     an ordinary launch, provided that a kernel of the caller's own which is launched with that
+ *     attribute also waits (griddepcontrol.wait) before it ends: one that never does would let the
+ *     calls behind it pass the kernels in front of it.
  *   - The return value reports host-side validation only (SC_OK, SC_ERR_INVALID_ARG,
  *     SC_ERR_UNSUPPORTED, SC_ERR_CUDA for a failed launch; sc_decode_attn_static alone also
  *     returns SC_ERR_CAPACITY from the host for a shape beyond its fixed scratch).  Conditions found on the device
@@ -63,22 +67,22 @@ typedef enum { SC_BF16 = 0, SC_F32 = 1 } sc_dtype;
                                   caller promises that nothing this call READS before it writes (q, cores,
                                   count, core_len; for sc_compress K, V and the chunk plan) is written by
                                   any kernel of the unbroken run of overlapped launches before it, nor by
-                                  the kernel just before that run.  Every write of the call (out,
-                                  workspace, status; for sc_compress also cores, count, core_len, assign)
-                                  is ordered behind the completion of the kernel before it, and so on
-                                  back along the run: sc_decode_attn calls of one run may therefore share
-                                  their workspace and out buffers; sc_compress calls of one run must not
-                                  share a workspace or outputs (it writes throughout).  Independent
+                                  the kernel just before that run.  sc_decode_attn orders every write (out,
+                                  workspace, status) behind the completion of the kernel before it, and so
+                                  on back along the run: calls of one run may share their workspace and out
+                                  buffers.  sc_compress writes throughout and waits for the kernel before it
+                                  only at its end: its workspace and outputs must not be used by any kernel
+                                  of the run before it nor by the kernel just before that run.  Independent
                                   calls, e.g. the layers of an attention-only benchmark, then run back to
                                   back without the launch gap.  A call without the flag orders itself
-                                  after everything enqueued before it, as usual. */
+                                  after everything enqueued before it, as usual (see the general rules). */
 #define SC_FLAG_OVERLAP_CHAIN 8u /* sc_decode_attn only: as SC_FLAG_OVERLAP_PREV, except that q MAY be the
                                   product of the kernel just before this call (layer l+1's query follows
-                                  from layer l's output).  The kernel starts early, sends its share of the
-                                  cores on its way (first tiles to shared memory, the rest to L2), waits
-                                  for the preceding kernel to complete and only then reads q.  The cores,
-                                  count and core_len are still read early and fall under the promise
-                                  above.  Ignored (ordinary launch) on the generic path. */
+                                  from layer l's output).  The kernel starts early, requests the first
+                                  tiles of its cores, waits for the preceding kernel to complete and only
+                                  then reads q.  The cores, count and core_len are still read early and
+                                  fall under the promise above.  Ignored (ordinary launch) on the generic
+                                  path. */
 
 #define SC_FLAG_CAUSAL_TAIL 16u /* sc_prefill_attn only: the last m rows of every head are the m queries' own
                                   tokens; query i attends to rows t < core_len - (m - 1 - i) */

@@ -1,8 +1,10 @@
-"""ctypes binding of the C-ABI library (``include/semanticache.h``).
+"""Binding of the C-ABI library (``include/semanticache.h``).
 
 Argument marshalling only: torch provides device memory and the current stream, every step
-of the path runs in the library's CUDA kernels.  There is no fallback: if the library has not
-been built, or a call reports an error, an exception is raised.
+of the path runs in the library's CUDA kernels.  The calls made per layer or per token go through a
+small extension (``csrc/native_calls.c``), the others through ctypes; ``lib()`` has the prototypes of
+all exports.  There is no fallback: if the library has not been built, or a call reports an error, an
+exception is raised.
 """
 from __future__ import annotations
 
@@ -243,8 +245,8 @@ def sc_compress_layers(Ks, Vs, plan: "ChunkPlan", tau, outs, workspace, status=N
         at += 7
     prm = _GscParams(float(tau), int(plan.max_chunk_len), int(flags))
     st = _Strides(K0.stride(0), K0.stride(1), K0.stride(2))
-    code = lib().sc_compress_layers(ctypes.cast(rows, ctypes.POINTER(_CompressLayer)), L, st, _dt(K0), B, Hkv, n, d, _ptr(plan.seg_off), _ptr(plan.seq_seg_off),
-                                    _ptr(plan.n_seg), _ptr(plan.tile_seg), _ptr(plan.seq_tile_cnt), plan.n_tile_cap,
+    code = lib().sc_compress_layers(ctypes.cast(rows, ctypes.POINTER(_CompressLayer)), L, st, _dt(K0), B, Hkv, n, d,
+                                    _ptr(plan.seg_off), _ptr(plan.seq_seg_off), _ptr(plan.n_seg), _ptr(plan.tile_seg), _ptr(plan.seq_tile_cnt), plan.n_tile_cap,
                                     ctypes.byref(prm), cap, _ptr(workspace),
                                     workspace.numel() * workspace.element_size(), _ptr(status), _stream(K0))
     _check("sc_compress_layers", code)

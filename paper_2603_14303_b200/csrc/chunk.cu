@@ -58,7 +58,7 @@ __device__ __noinline__ int last_delimiter(const int32_t* ids, int lo, int hi, c
 #pragma unroll
         for (int i = 0; i < kLookUnroll; ++i) tok[i] = ids[min(p0 + i * kChunkThreads, hi - 1)];
         unsigned hits = 0u;
-        for (int k = 0; k < D.n; ++k) {   // (one delimiter against all: the other way round each comparison waits for its own fetch of the id)
+        for (int k = 0; k < D.n; ++k) {   // (one delimiter against all tokens: the other way round every comparison waits for its id)
             const int32_t id = D.id[k];
 #pragma unroll
             for (int i = 0; i < kLookUnroll; ++i) hits |= (tok[i] == id ? 1u : 0u) << i;
@@ -283,7 +283,8 @@ cudaError_t launch_chunk(const ChunkArgs& a, cudaStream_t st) {
     D.n = a.n_delim;
     for (int i = 0; i < SC_MAX_DELIMS; ++i) D.id[i] = (i < a.n_delim) ? a.delim[i] : 0;
     const int span = div_up(tps, kMaxSpans), spans = div_up(tps, span);
-    cudaError_t e = launch_in_order(span == 1 ? chunk_flags<true> : chunk_flags<false>, dim3(a.B * spans), kChunkThreads, 0, st, a.token_ids, a.n, tps, span, D, a.max_chunk_len, flags, tile_cnt);
+    cudaError_t e = launch_in_order(span == 1 ? chunk_flags<true> : chunk_flags<false>, dim3(a.B * spans), kChunkThreads, 0, st, a.token_ids,
+                                    a.n, tps, span, D, a.max_chunk_len, flags, tile_cnt);
     if (e != cudaSuccess) return e;
     note_launches(2);
     return launch_in_order(chunk_write_pack, dim3(a.B), kPackThreads, 0, st, (const uint8_t*)flags, (const int32_t*)tile_cnt, a.B, a.n, tps,

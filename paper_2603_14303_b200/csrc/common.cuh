@@ -81,10 +81,11 @@ __device__ __forceinline__ void store4(__nv_bfloat16* p, const float4& v) {
 }
 
 // Kernels are launched with programmatic stream serialization: their blocks are set up while the kernel before them in the
-// stream drains, and in_stream_order(), the first thing they do, holds them until it is complete and its writes are
-// visible: the order of an ordinary launch without its gap (one decode call over 2K tokens after another 8.2 -> 6.0 us; 8 small
-// sc_prefill_attn and 8 sc_append_layers calls in a row 238 -> 211).  Only then does a kernel let the next
-// one be set up, so whatever starts early after it may still count on everything before it being complete.
+// stream drains, and in_stream_order() holds them until it is complete and its writes are visible: the order of an
+// ordinary launch without its gap (one decode call over 2K tokens after another 8.2 -> 6.0 us; 8 small sc_prefill_attn and 8
+// sc_append_layers calls in a row 238 -> 211).  Only then does a kernel let the next one be set up, so whatever starts early
+// after it may still count on everything before it being complete.  (The steps of the budget search and the kernels of
+// global clustering are ordinary launches.)
 __device__ __forceinline__ void in_stream_order() {
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");

@@ -531,25 +531,24 @@ inline size_t all_slots(long long heads, int cap) {
     return 2 * (size_t)(several > own ? several : own);
 }
 
-// The rules and what they were measured against (us per layer, Llama-shaped heads of 128 columns, 2 x 148 block slots; the
-// plan before took splits from the capacity alone, up to 256 a head in several waves, and asked L2 for up to 1 MB per
-// block in advance -- which cost more than anything else, 10 to 30 % of every batched or long launch):
+// The rules and what they were measured against (us per layer, Llama-shaped heads of 128 columns, 2 x 148 block slots; "->" is
+// from a plan that took splits from the capacity alone, in several waves, and asked L2 for each block's rows in advance):
 //   - one cluster per head, as wide as lets the clusters of all heads be resident at once: 128 heads x 3.4 K rows, 2 blocks
 //     each, 51.6 -> 41.2; 56 heads x 6.3 K, 5, 43.7 -> 33.9; 32 x 6.3 K, 8, 31.9 -> 22.5; 24 x 12.6 K, 10, 45.7 -> 31.9; 16 x 25 K, 12,
-//     47.0 -> 36.0; 8 x 34 K, 16, 40.2 -> 27.8.  More than 12 only where
-//     16 would fit: 16 heads, for which 13 do and 14 do not, 13 blocks instead of 12: 4 to 25 K rows 1 to 2 % faster, 2.1 K rows 8.3 -> 8.9.
+//     47.0 -> 36.0; 8 x 34 K, 16, 40.2 -> 27.8.  More than 12 only where 16 would fit: 16 heads, for which 13 do and 14 do not, 13
+//     blocks against 12: 4 to 25 K rows 1 to 2 % faster, 2.1 K rows 8.9 against 8.3.
 //   - fewer blocks for short capacities, whose time is the fold and the barrier: 8 heads x 0.5 K rows of 1 K capacity: 9 blocks
 //     4.5, 16 blocks 5.0; x 2.1 K of 4 K: 12 blocks 6.1, 16 blocks 6.6; from 8 K of capacity on 16.
 //   - several clusters per head where few heads would leave blocks with thousands of rows: 4 heads x 34 K rows, 3 x 16, 19.7 (one: 21;
 //     21.1 to 43.6 before); not below, the ticket and the merge cost 2: 4 heads x 8.5 K, one cluster 9.2, three 11.1.
-//   - more heads than any cluster width fits: one block per head (256 heads x 3.4 K rows: 82.1, split in two 83.2, 94.0 before); where
-//     they are up to 15 % more than two per SM, which leaves a last round nearly empty, clusters of three (320 heads x 7 K rows:
-//     210 -> 176; 368: 214 -> 204, but with 3.4 K rows 110 -> 120; 320 x 2 K rows of 4 K 68 -> 74).
+//   - more heads than any cluster width fits: one block per head (256 heads x 3.4 K rows: 82.1, split in two 83.2); where they
+//     are up to 15 % more than two per SM, which leaves a last round nearly empty, clusters of three (one block and three: 320
+//     heads x 7 K rows 210, 176; 368 214, 204, but with 3.4 K rows 110, 120; 320 x 2 K rows of 4 K 68, 74).
 //   - a cache without counts is a raw one, whose heads are mostly full: one block per SM outside clusters keeps HBM
-//     busiest (32 heads x 64 K rows, 4 each, 157; 8 each in clusters 166; 192 before; 8 heads x 131 K: 83.5 against 116.9).  From 75
+//     busiest (32 heads x 64 K rows, 4 each, 157; 8 each in clusters 166; 8 heads x 131 K: 83.5 against 116.9).  From 75
 //     heads on that is one block each; where it leaves more SMs idle in its last round than clusters of two or three would,
-//     those are taken: 76 heads x 8 K rows 60.7 -> 54.4, 88 63.3 -> 60.3, 176 123 -> 113, 200 137 -> 131, 320 232 -> 206 (104 to 152
-//     and 296 heads: one block each is best).
+//     those are taken (one block and two or three: 76 heads x 8 K rows 60.7, 54.4; 88 63.3, 60.3; 176 123, 113; 200 137, 131; 320
+//     232, 206; at 104 to 152 and 296 heads one block is best).
 inline SplitPlan plan_for(long long heads, int cap, bool raw, const Resident& res) {
     const int by_rows = (cap + 4 * kTile - 1) / (4 * kTile);   // at least 64 rows per split
     if (raw && cap >= 8192) {
