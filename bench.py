@@ -361,7 +361,7 @@ def run_ours(args):
     comp_ms = sum_c / args.steps
     comp_gbs = cbytes / (comp_ms * 1e-3) / 1e9
     launch_text = {"chain": "cuda graphs; within a decode step layer l+1's query is layer l's output and the launches are "
-                            "chained (SC_FLAG_OVERLAP_CHAIN: cores prefetched under the previous layer, query read after it)",
+                            "chained (SC_FLAG_OVERLAP_CHAIN: first tiles of the cores requested under the previous layer, query read after it)",
                    "serial": "cuda graphs; dependent per-layer launches in plain stream order"}[main_mode]
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": args.gpus, "steps": args.steps,
@@ -434,7 +434,30 @@ def run_ours(args):
     sampler.stop()
     if not args.no_cpu_baseline and args.gpus == 1:
         line["cpu_baseline"] = cpu_baseline(w, budget_s=args.cpu_budget)
-    print(json.dumps(line))
+    print(json.dumps({"detail": line}), file=sys.stderr)
+    print(json.dumps(headline(line)))
+
+
+# What the one line on standard output holds (about 2 KB, so that it survives in the tail of a log); the whole record, the
+# launch modes, sweeps and extras among it, goes to standard error as {"detail": ...}.
+HEADLINE = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling", "vs_baseline",
+            "dtype", "data", "config", "decode_tokens_per_s", "compress_ms_per_32k_ctx", "gpu_launches", "clocks")
+HEADLINE_PARTS = {
+    "e2e": ("value", "unit", "h2d_bytes_per_step", "d2h_bytes_per_step", "steps", "ms_per_step"),
+    "roofline": ("kernel", "bound", "achieved", "peak", "unit", "frac", "bytes_per_launch", "us_per_launch", "traffic"),
+    "roofline_compress": ("kernel", "bound", "achieved", "peak", "unit", "frac", "bytes_per_launch", "us_per_launch", "traffic"),
+    "cpu_baseline": ("value", "unit", "cores", "kind", "threads_available", "compress_s_per_layer", "decode_s_per_layer_step"),
+}
+
+
+def headline(line):
+    short = lambda v: float(f"{v:.8g}") if isinstance(v, float) else v
+    out = {k: short(line[k]) for k in HEADLINE}
+    for name, keys in HEADLINE_PARTS.items():
+        part = line.get(name)
+        if part is not None:
+            out[name] = {k: short(part[k]) for k in keys if k in part}
+    return out
 
 
 # ------------------------------------------------------------ the five workloads and their sweeps
