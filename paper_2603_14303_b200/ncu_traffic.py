@@ -6,8 +6,8 @@
 reads a CSV written by ``ncu --csv --page raw`` (or ``ncu --csv --metrics dram__bytes_read.sum,
 dram__bytes_write.sum``), averages ``dram__bytes_read.sum + dram__bytes_write.sum`` over the captured
 launches of the named kernel and stores the figure in ``profiles/traffic.txt`` (JSON) together with a hash
-of the kernel's source file.  ``lookup`` returns the figure only while that file is unchanged, so a
-benchmark line never quotes counters of a kernel that no longer exists.
+of the kernel's source file, its comments and blanks left out.  ``lookup`` returns the figure only while that
+code is unchanged, so a benchmark line never quotes counters of a kernel that no longer exists.
 """
 from __future__ import annotations
 
@@ -16,6 +16,7 @@ import csv
 import hashlib
 import json
 import os
+import re
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
@@ -32,8 +33,9 @@ def source_hash(stage: str) -> str | None:
     path = os.path.join(HERE, SOURCES[stage])
     if not os.path.exists(path):
         return None
-    with open(path, "rb") as f:
-        return hashlib.sha256(f.read()).hexdigest()[:16]
+    with open(path, encoding="utf-8") as f:
+        code = re.sub(r"//[^\n]*|/\*.*?\*/", " ", f.read(), flags=re.DOTALL)   # (no string of these files holds a comment mark)
+    return hashlib.sha256(" ".join(code.split()).encode()).hexdigest()[:16]
 
 
 def lookup(workload: str, stage: str):

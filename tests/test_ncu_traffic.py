@@ -44,3 +44,14 @@ def test_record_goes_stale_when_the_kernel_source_changes(tmp_path, monkeypatch)
     assert ncu_traffic.lookup("other", "decode") is None
     os.remove(rec)
     assert ncu_traffic.lookup("w", "decode") is None
+
+
+def test_a_comment_does_not_make_a_record_stale(tmp_path, monkeypatch):
+    (tmp_path / "csrc").mkdir()
+    src = tmp_path / "csrc" / "decode_mma.cu"
+    monkeypatch.setattr(ncu_traffic, "HERE", str(tmp_path))
+    hashes = []
+    for text in ("int a = 1;  // one\n/* block\n of two */ int b;", "int a = 1;\n  int b; // other", "int a = 2;\n int b;"):
+        src.write_text(text)
+        hashes.append(ncu_traffic.source_hash("decode"))
+    assert hashes[0] == hashes[1] != hashes[2]
