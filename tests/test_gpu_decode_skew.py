@@ -115,3 +115,36 @@ def test_more_heads_than_seats(B, H, G, cap, raw):
     q = torch.randn((B, H * G, 128), generator=torch.Generator(device=DEV).manual_seed(B), device=DEV).bfloat16()
     got = binding.decode_attn(q, y, use_count=not raw)
     assert_close_vectors(to_f64(got), _reference(q, y, raw), TOL[torch.bfloat16], f"{B} x {H} x {G}, capacity {cap}")
+
+
+@pytest.mark.parametrize("flag", [binding.SC_FLAG_OVERLAP_PREV, binding.SC_FLAG_OVERLAP_CHAIN])
+def test_overlapped_launches_with_spare_units(flag):
+    """Layers of one skewed batch, eager and from a graph, with one workspace: the same bits as launches in plain stream order."""
+    H, G, B = 8, 4, 4
+    ys = [_layer([30000, 900, 40, 2500], 32768, H, i, False) for i in range(5)]
+    q = torch.randn((B, H * G, 128), generator=torch.Generator(device=DEV).manual_seed(1), device=DEV).bfloat16()
+    ws = binding.decode_workspace(B, H * G, H, 128, 32768, DEV)
+
+    def layers(flags, outs):
+        x = q
+        for y, o in zip(ys, outs):
+            r = binding.decode_attn(x, y, out=o, workspace=ws, flags=flags)
+            x = r if flag == binding.SC_FLAG_OVERLAP_CHAIN else q
+        return outs
+
+    want = layers(0, [torch.empty_like(q) for _ in ys])
+    torch.cuda.synchronize()
+    outs = [torch.empty_like(q) for _ in ys]
+    for _ in range(3):
+        layers(flag, outs)
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(outs, want))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        layers(flag, outs)
+    for o in outs:
+        o.zero_()
+    graph.replay()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert all(torch.equal(a, b) for a, b in zip(outs, want))
