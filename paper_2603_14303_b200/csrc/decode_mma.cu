@@ -234,7 +234,11 @@ __device__ __forceinline__ Units plan_units(const int32_t* __restrict__ core_len
     return u;
 }
 
-template <bool kSpares>   // the launch has spare units (the code for them costs the others 0.2 us)
+// kSpares: the launch has spare units (the code for them costs the others 0.2 us).
+// kPair: up to four query heads.  The second product's eight columns then hold the heads' leading parts and, four columns on, their
+// remainders, so one product does for both; the queries stand in the first product's columns twice, which gives the lanes
+// of either half the scores they need.
+template <bool kSpares, bool kPair>
 __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm)
 decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __nv_bfloat16* __restrict__ core_k,
                   const __nv_bfloat16* __restrict__ core_v, const int32_t* __restrict__ count, int cap,
@@ -301,18 +305,19 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     // q^T as the B operand of every k-step: b0 = q[head g][16ks + 2tig, +1], b1 = same + 8
     uint32_t qb[8][2];
     {
-        const __nv_bfloat16* qh = q + ((size_t)bh * G + g) * kD;
+        const int hd = kPair ? g & 3 : g;
+        const __nv_bfloat16* qh = q + ((size_t)bh * G + hd) * kD;
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {
             // read through L2: under a chained launch q was written while this kernel was already running
-            qb[ks][0] = (g < G) ? __ldcg(reinterpret_cast<const uint32_t*>(qh + ks * 16 + 2 * tig)) : 0u;
-            qb[ks][1] = (g < G) ? __ldcg(reinterpret_cast<const uint32_t*>(qh + ks * 16 + 2 * tig + 8)) : 0u;
+            qb[ks][0] = (hd < G) ? __ldcg(reinterpret_cast<const uint32_t*>(qh + ks * 16 + 2 * tig)) : 0u;
+            qb[ks][1] = (hd < G) ? __ldcg(reinterpret_cast<const uint32_t*>(qh + ks * 16 + 2 * tig + 8)) : 0u;
         }
     }
     float o[8][4];
 #pragma unroll
     for (int mt = 0; mt < 8; ++mt) { o[mt][0] = o[mt][1] = o[mt][2] = o[mt][3] = 0.f; }
-    float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;   // heads 2tig and 2tig+1
+    float m0 = -INFINITY, m1 = -INFINITY, l0 = 0.f, l1 = 0.f;   // columns 2tig and 2tig+1
 
     // per-lane ldmatrix row/chunk selectors
     const int lm_j = lane >> 3, lm_r = lane & 7;
@@ -377,8 +382,8 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
         const uint32_t r_hi = pack_bf16x2(w2 - bf16_lo(p_hi), w3 - bf16_hi(p_hi));
         l0 += (bf16_lo(p_lo) + bf16_lo(r_lo)) + (bf16_lo(p_hi) + bf16_lo(r_hi));
         l1 += (bf16_hi(p_lo) + bf16_hi(r_lo)) + (bf16_hi(p_hi) + bf16_hi(r_hi));
-        const uint32_t pb0 = movmatrix_trans(p_lo), pb1 = movmatrix_trans(p_hi);
-        const uint32_t rb0 = movmatrix_trans(r_lo), rb1 = movmatrix_trans(r_hi);
+        const uint32_t pb0 = movmatrix_trans(kPair && tig >= 2 ? r_lo : p_lo), pb1 = movmatrix_trans(kPair && tig >= 2 ? r_hi : p_hi);
+        const uint32_t rb0 = kPair ? 0u : movmatrix_trans(r_lo), rb1 = kPair ? 0u : movmatrix_trans(r_hi);
 
         // O^T += V^T . P^T
 #pragma unroll
@@ -387,7 +392,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
             const int c = 2 * mt + v_csel;
             ldmatrix_x4_trans(st + kTileBytes + v_row * kRowBytes + ((c ^ (v_row & 7)) << 4), a0, a1, a2, a3);
             mma_bf16(o[mt], a0, a1, a2, a3, pb0, pb1);
-            mma_bf16(o[mt], a0, a1, a2, a3, rb0, rb1);
+            if (!kPair) mma_bf16(o[mt], a0, a1, a2, a3, rb0, rb1);
         }
         __syncwarp();
         // the stage just consumed takes the tile three ahead
@@ -435,6 +440,10 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
         for (int w2 = 0; w2 < kWarps; ++w2) {
             const float4 v = *reinterpret_cast<const float4*>(slabs + w2 * (8 * kD) + e4 * 4);
             acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
+            if (kPair) {   // the remainders' part
+                const float4 r = *reinterpret_cast<const float4*>(slabs + w2 * (8 * kD) + 4 * kD + e4 * 4);
+                acc.x += r.x; acc.y += r.y; acc.z += r.z; acc.w += r.w;
+            }
         }
         *reinterpret_cast<float4*>(blk + e4 * 4) = acc;
     }
@@ -618,7 +627,8 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
         cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
         res.sms = v < 1 ? 1 : v;
         bool wide = true;
-        for (auto kernel : {dm::decode_mma_kernel<false>, dm::decode_mma_kernel<true>}) {
+        for (auto kernel : {dm::decode_mma_kernel<false, false>, dm::decode_mma_kernel<true, false>, dm::decode_mma_kernel<false, true>,
+                            dm::decode_mma_kernel<true, true>}) {
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dm::kSmemBytes);
             wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess && wide;
         }
@@ -634,7 +644,7 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
             probe.numAttrs = 1;
             int n_clusters = 0;
             res.fit[c] = 0;
-            if ((c <= 8 || wide) && cudaOccupancyMaxActiveClusters(&n_clusters, dm::decode_mma_kernel<false>, &probe) == cudaSuccess) res.fit[c] = n_clusters;
+            if ((c <= 8 || wide) && cudaOccupancyMaxActiveClusters(&n_clusters, dm::decode_mma_kernel<false, false>, &probe) == cudaSuccess) res.fit[c] = n_clusters;
         }
         (void)cudaGetLastError();   // a refused opt-in or probe is not an error of this call
     });
@@ -656,8 +666,11 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
     cfg.attrs = attr;
     cfg.numAttrs = 2;
     const int mode = (a.flags & SC_FLAG_OVERLAP_CHAIN) ? dm::kChained : (a.flags & SC_FLAG_OVERLAP_PREV) ? dm::kOverlapped : dm::kOrdinary;
+    const bool pair = a.Hq / a.Hkv <= 4;
+    const auto kernel = spares ? (pair ? dm::decode_mma_kernel<true, true> : dm::decode_mma_kernel<true, false>)
+                               : (pair ? dm::decode_mma_kernel<false, true> : dm::decode_mma_kernel<false, false>);
     note_launches(1);
-    return own_error(cudaLaunchKernelEx(&cfg, spares ? dm::decode_mma_kernel<true> : dm::decode_mma_kernel<false>, (const __nv_bfloat16*)a.q, a.Hq, a.Hkv,
+    return own_error(cudaLaunchKernelEx(&cfg, kernel, (const __nv_bfloat16*)a.q, a.Hq, a.Hkv,
                                         (const __nv_bfloat16*)a.core_k, (const __nv_bfloat16*)a.core_v, a.count, a.cap,
                                         a.core_len, scale, a.B, mode, (__nv_bfloat16*)a.out, part, tickets));
 }
