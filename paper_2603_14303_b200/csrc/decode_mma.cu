@@ -26,6 +26,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "umma.cuh"
 
 namespace sc {
 
@@ -43,7 +44,8 @@ constexpr int kRowBytes = kD * 2;               // 256
 constexpr int kTileBytes = kTile * kRowBytes;   // 4096 per K or V tile
 constexpr int kStageBytes = 2 * kTileBytes + 64;  // K, V, 16 counts
 constexpr int kWarpBytes = kStages * kStageBytes;
-constexpr int kSmemBytes = kWarps * kWarpBytes;
+constexpr int kRecvBytes = (8 * (kD / 4) + 16) * 16 + 16 * 64;   // what the blocks of a cluster hand each other: slices of O (rounded up), m and l
+constexpr int kSmemBytes = kWarps * kWarpBytes + kRecvBytes;
 constexpr int kPartStride = 8 * kD + 16;        // floats per (b, h, split): acc[8 heads][128], m[8], l[8]
 constexpr int kCtasPerSm = 2;                   // two kernels (consecutive layers) can be co-resident
 constexpr float kMaxSlack = 8.f;                // log2 units a score may exceed the running maximum before it is raised
@@ -60,6 +62,11 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int sr
 }
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src, int src_bytes) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, int rank) {
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(addr), "r"(rank));
+    return a;
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -143,25 +150,28 @@ __device__ __forceinline__ void issue_tile(uint32_t stage, const __nv_bfloat16* 
     }
 }
 
-// Several partials per head in global memory (one per cluster, or per block outside clusters): the last block
-// to arrive merges the `n_parts` of them: the first `n_first` lie in the slots from `first` on, the others from `more` on.  All threads of the block call
-// it.  The cluster barrier / fence before the call orders this block's partial stores before its
-// ticket, whose release makes them visible to whoever reads the ticket with acquire (the last arrival); that
-// block's other threads are ordered behind its thread 0 by the barrier below and read the partials from L2.
+// Several partials per head in global memory (one per cluster, or per block outside clusters).  The blocks that hold the same
+// elements [e_lo, e_hi) of them share a ticket; the last one to arrive merges the `n_parts` partials' elements: the first
+// `n_first` partials lie in the slots from `first` on, the others from `more` on.  All threads of the block call it.  The fence and the
+// barrier order this block's partial stores before its ticket, whose release makes them visible to whoever reads
+// the ticket with acquire (the last arrival); that block's other threads are ordered behind its thread 0 by the second barrier
+// and read the partials from L2.
 template <bool kSpares>
-__device__ __forceinline__ void ticket_and_merge(const float* __restrict__ part, int first, int more, int n_first, int n_parts, int32_t* __restrict__ tickets,
-                                                 int bh, int G, __nv_bfloat16* __restrict__ out, int* sh_last_p) {
+__device__ __forceinline__ void ticket_and_merge(const float* __restrict__ part, int first, int more, int n_first, int n_parts, int32_t* __restrict__ ticket,
+                                                 int arrivals, int e_lo, int e_hi, int bh, int G, __nv_bfloat16* __restrict__ out, int* sh_last_p) {
+    __threadfence();
+    __syncthreads();
     if (threadIdx.x == 0) {
         int t;
-        asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;\n" : "=r"(t) : "l"(tickets + bh) : "memory");
-        *sh_last_p = (t == n_parts - 1);
-        if (*sh_last_p) tickets[bh] = 0;   // leave the counter ready for the next call
+        asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;\n" : "=r"(t) : "l"(ticket) : "memory");
+        *sh_last_p = (t == arrivals - 1);
+        if (*sh_last_p) *ticket = 0;   // leave the counter ready for the next call
     }
     __syncthreads();
     if (!*sh_last_p) return;
     // One thread per (head, four output columns); the partials are folded sixteen at a time, all of a
     // group's loads in flight together (one round trip to L2 per group).
-    for (int e4 = threadIdx.x; e4 < G * (kD / 4); e4 += kWarps * 32) {
+    for (int e4 = e_lo + threadIdx.x; e4 < e_hi; e4 += kWarps * 32) {
         const int hd = e4 / (kD / 4), d4 = (e4 % (kD / 4)) * 4;
         float gm = -INFINITY, lsum = 0.f;
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -243,11 +253,12 @@ __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm)
 decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __nv_bfloat16* __restrict__ core_k,
                   const __nv_bfloat16* __restrict__ core_v, const int32_t* __restrict__ count, int cap,
                   const int32_t* __restrict__ core_len, float scale_log2, int B, int mode,
-                  __nv_bfloat16* __restrict__ out, float* __restrict__ part, int32_t* __restrict__ tickets) {
+                  __nv_bfloat16* __restrict__ out, float* __restrict__ part, int32_t* __restrict__ tickets, int32_t* status) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ float sh_m[kWarps][8];
     __shared__ float sh_l[kWarps][8];
     __shared__ int sh_last;
+    __shared__ __align__(8) unsigned long long sh_bar;   // what the cluster's blocks hand this one has arrived
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, tig = lane & 3;
@@ -259,6 +270,18 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     // Where there are spare units the next kernel is let in only when they have gone: its blocks would find both slots of some
     // SMs taken by them, and settle unevenly (128 raw heads x 8 K rows: 80 us, 92 with the next kernel let in at once).
     if (!kSpares) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    // Block r of the cluster folds slice r of the head's (head, column) pairs, [e_lo, e_hi), and
+    // is handed that slice by every block (see the fold).
+    const int csize = (int)cg::this_cluster().num_blocks(), crank = (int)cg::this_cluster().block_rank();
+    const int slice = (G * (kD / 4) + csize - 1) / csize;
+    const int e_lo = min(crank * slice, G * (kD / 4)), e_hi = min(e_lo + slice, G * (kD / 4));
+    if (threadIdx.x == 0) {
+        umma::mbar_init(smem_u32(&sh_bar), 1);
+        umma::mbar_fence_init();
+        umma::mbar_expect_tx(smem_u32(&sh_bar), (uint32_t)(csize * ((e_hi - e_lo) * 16 + 64)));   // (m and l come to a block without a slice too)
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");   // (the wait is in front of the first access to another block's shared memory)
     // the block's head, and its place among the head's blocks
     int bh = blockIdx.z * Hkv + blockIdx.y, split = blockIdx.x, n_split = gridDim.x;   // as if every head had one unit
     Units u = {bh, 0, 0};
@@ -431,9 +454,16 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
         slab[(2 * tig + 1) * kD + d0 + 8] = o[mt][3] * f1;
     }
     __syncthreads();
-    // ---- block partial (m, l, O) into this block's shared memory, behind the warps' slabs ----
+    // ---- the splits of one thread-block cluster are folded through distributed shared memory ----
+    // Block r of the cluster folds slice r of the (head, column) pairs.  Every block adds up its warps' slabs and hands each slice, and
+    // its m and l, straight to the block that folds it (st.async, counted by that block's mbarrier): a block waits for what it
+    // folds and for nothing else, reads it from its own shared memory and may leave.  32 dependent layers of 8 heads x
+    // 8.3 K rows 325 us; with plain stores and a cluster barrier 339; reading out of the members' shared memory between two
+    // cluster barriers 350.  28 layers of 4 x 34 K rows 499, 501, 520; one call over 8 x 0.5 K rows 5.2 each.
+    float4* recv_o = reinterpret_cast<float4*>(smem + kWarps * kWarpBytes);   // [csize][slice]
+    float* recv_ml = reinterpret_cast<float*>(smem + kWarps * kWarpBytes + (8 * (kD / 4) + 16) * 16);   // [csize][m of 8 heads, l of 8 heads]
+    asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");   // every block of the cluster has started
     const float* slabs = reinterpret_cast<const float*>(smem);
-    float* blk = reinterpret_cast<float*>(smem) + kWarps * (8 * kD);   // [8][128] O, [8] m, [8] l
     for (int e4 = threadIdx.x; e4 < G * (kD / 4); e4 += kWarps * 32) {
         float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
@@ -445,10 +475,13 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
                 acc.x += r.x; acc.y += r.y; acc.z += r.z; acc.w += r.w;
             }
         }
-        *reinterpret_cast<float4*>(blk + e4 * 4) = acc;
+        const int to = e4 / slice;
+        const uint32_t bar_to = mapa(smem_u32(&sh_bar), to), dst = mapa(smem_u32(recv_o + crank * slice + (e4 - to * slice)), to);
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];\n"
+                     ::"r"(dst), "r"(__float_as_uint(acc.x)), "r"(__float_as_uint(acc.y)), "r"(__float_as_uint(acc.z)), "r"(__float_as_uint(acc.w)), "r"(bar_to) : "memory");
     }
-    if (threadIdx.x < 8) {
-        const int hd = threadIdx.x;
+    for (int x = threadIdx.x; x < csize * 8; x += kWarps * 32) {
+        const int hd = x & 7;
         float bm = -INFINITY, bl = 0.f;
 #pragma unroll
         for (int w2 = 0; w2 < kWarps; ++w2) bm = fmaxf(bm, sh_m[w2][hd]);
@@ -457,42 +490,34 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
             const float mw = sh_m[w2][hd];
             bl += (mw == -INFINITY) ? 0.f : sh_l[w2][hd] * fast_exp2(mw - bm);
         }
-        blk[8 * kD + hd] = bm;
-        blk[8 * kD + 8 + hd] = bl;
+        const uint32_t bar_to = mapa(smem_u32(&sh_bar), x >> 3), dst = mapa(smem_u32(recv_ml + crank * 16 + hd * 2), x >> 3);
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];\n"
+                     ::"r"(dst), "r"(__float_as_uint(bm)), "r"(__float_as_uint(bl)), "r"(bar_to) : "memory");
     }
-
-    // ---- the splits of one thread-block cluster are folded through distributed shared memory ----
-    // Every block of the cluster folds its own slice of the (head, column) pairs, reading that slice of
-    // every member's partial straight out of the member's shared memory (no trip through L2, no counter,
-    // and no single block pulling all partials through its own port); the members stay until all have read.
-    cg::cluster_group cluster = cg::this_cluster();
-    const int csize = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
     const int n_clusters = n_split / csize, cidx = split / csize;   // clusters of the head, this one's index
     // partials: every head's own unit in turn, then the spare units; a unit leaves one for each of its clusters
     const int per_unit = kSpares ? (int)gridDim.x / csize : n_clusters;
     const int first = bh * per_unit, more = (B * Hkv + u.begin) * per_unit;
     float* my_part = part + (size_t)(cidx + (!kSpares || cidx < per_unit ? first : more - per_unit)) * kPartStride;
     const bool direct = n_clusters == 1;   // this cluster holds the whole head: its fold is the result
-    const int slice = (G * (kD / 4) + csize - 1) / csize;
-    cluster.sync();
+    if (direct && warp > 0 && e_lo + warp * 32 >= e_hi) return;   // nothing to fold for this warp (one stays until all has arrived)
+    const bool got = umma::mbar_wait<true>(smem_u32(&sh_bar), 0);
     // Nothing has been written to global memory so far (the block partials live in shared memory).  Under
     // an overlapped launch every global write of this kernel (out, cluster partials, arrival counters) is
     // ordered behind the completion of the kernel before it, which ordered its own writes behind its
     // predecessor in the same way: completion is transitive along a run of overlapped launches, and they
     // may share workspace and out buffers.  (A no-op for an ordinary launch and after the wait above.)
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    for (int i = threadIdx.x; i < slice; i += kWarps * 32) {
-        const int e4 = crank * slice + i;
-        if (e4 >= G * (kD / 4)) break;
+    if (!got) set_status(status, SC_ERR_TIMEOUT);
+    for (int e4 = e_lo + threadIdx.x; e4 < e_hi; e4 += kWarps * 32) {
         const int hd = e4 / (kD / 4), d4 = (e4 % (kD / 4)) * 4;
         float mv[kMaxCluster], lv[kMaxCluster];
         float4 ov[kMaxCluster];
 #pragma unroll
         for (int j = 0; j < kMaxCluster; ++j) {
-            const float* pb = cluster.map_shared_rank(blk, j < csize ? j : 0);
-            mv[j] = j < csize ? pb[8 * kD + hd] : -INFINITY;
-            lv[j] = j < csize ? pb[8 * kD + 8 + hd] : 0.f;
-            ov[j] = j < csize ? *reinterpret_cast<const float4*>(pb + hd * kD + d4) : make_float4(0.f, 0.f, 0.f, 0.f);
+            mv[j] = j < csize ? recv_ml[j * 16 + 2 * hd] : -INFINITY;
+            lv[j] = j < csize ? recv_ml[j * 16 + 2 * hd + 1] : 0.f;
+            ov[j] = j < csize ? recv_o[j * slice + e4 - e_lo] : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         float gm = mv[0];
 #pragma unroll
@@ -511,15 +536,15 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
             store_out4(out + ((size_t)bh * G + hd) * kD + d4, acc, inv);
         } else {
             *reinterpret_cast<float4*>(my_part + hd * kD + d4) = acc;
-            if (d4 == 0) { my_part[8 * kD + hd] = gm; my_part[8 * kD + 8 + hd] = lsum; }
+            if (d4 == 0 || e4 == e_lo) { my_part[8 * kD + hd] = gm; my_part[8 * kD + 8 + hd] = lsum; }   // (the same values from every slice of the head)
         }
     }
-    if (!direct) __threadfence();   // this block's slice of the cluster partial, before the cluster's ticket
-    cluster.sync();   // every member's shared memory has been read: they may leave
-    if (direct || crank != 0) return;
+    if (direct) return;
 
-    // ---- several partials per head: the last block to arrive merges them ----
-    ticket_and_merge<kSpares>(part, first, more, per_unit, n_clusters, tickets, bh, G, out, &sh_last);
+    // ---- several partials per head: the last block to arrive merges them, slice by slice where there are counters enough ----
+    const bool by_slice = B * Hkv * csize <= kMaxTickets;
+    ticket_and_merge<kSpares>(part, first, more, per_unit, n_clusters, tickets + (by_slice ? bh * csize + crank : bh), by_slice ? n_clusters : n_clusters * csize,
+                              by_slice ? e_lo : 0, by_slice ? e_hi : G * (kD / 4), bh, G, out, &sh_last);
 }
 
 // Block split of one head: how many blocks stream it, and how they are grouped into clusters.
@@ -672,7 +697,7 @@ cudaError_t launch_decode_mma(const DecodeArgs& a, cudaStream_t st) {
     note_launches(1);
     return own_error(cudaLaunchKernelEx(&cfg, kernel, (const __nv_bfloat16*)a.q, a.Hq, a.Hkv,
                                         (const __nv_bfloat16*)a.core_k, (const __nv_bfloat16*)a.core_v, a.count, a.cap,
-                                        a.core_len, scale, a.B, mode, (__nv_bfloat16*)a.out, part, tickets));
+                                        a.core_len, scale, a.B, mode, (__nv_bfloat16*)a.out, part, tickets, a.status));
 }
 
 }  // namespace sc

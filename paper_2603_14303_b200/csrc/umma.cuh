@@ -35,15 +35,24 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0u;
 }
+// The same for data that other blocks of the cluster hand in.
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0u;
+}
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // every wait gives up after 2 s
 // Bounded wait for the phase with the given parity; false if it gave up.
+template <bool kCluster = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    if (mbar_try_wait(bar, parity)) return true;
+    const auto done = [&] { return kCluster ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
+    if (done()) return true;
     const unsigned long long t0 = global_ns();
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 256; ++i)
-            if (mbar_try_wait(bar, parity)) return true;
+            if (done()) return true;
         if (global_ns() - t0 > kWaitLimitNs) return false;
     }
 }
