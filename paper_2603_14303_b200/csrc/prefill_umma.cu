@@ -4,28 +4,29 @@
 // step this is a dense contraction: the G query heads that share a KV head times the m queries give
 // G*m rows against the same cores, so it runs on the tcgen05 tensor cores (bf16, d = 128):
 //   one CTA = 128 query rows of one (sequence, KV head), walking the head's cores 128 at a time;
-//   warp 0     TMA: the query tile once, then K and V tiles into a three-stage ring (128-byte swizzle);
-//   warp 1     issues the MMAs: S = Q K^T into one of two score buffers in tensor memory (two tiles ahead
+//   warps 0, 2 TMA: the query tile once, then K and V tiles into rings of three (128-byte swizzle); warp 2 log2(count) too;
+//   warp 1     issues the MMAs: S = Q K^T into one of three score buffers in tensor memory (three tiles ahead
 //              of the weighted sum), then O += P V with P read from tensor memory and V as an MN-major
 //              operand straight from its [keys x dims] tile;
-//   warps 2-9  softmax, two threads per query row (= tensor-memory lane; each owns half of a tile's keys and
-//              half of the accumulator's columns, the row maximum is exchanged through shared memory):
-//              x = S * scale*log2(e) + log2(count), masks (head length, optional causal tail), running
-//              maximum raised lazily (the accumulator row is rescaled in tensor memory only then; the tile's
-//              maximum is taken as a bound: largest raw product * scale + largest log2(count) of the tile),
-//              P = 2^(x - m) as a bf16 pair (leading part + remainder) written back over the scores it
-//              came from: the 32 fp32 columns of a chunk of scores become 16 columns of packed leading
-//              parts and 16 of remainders, so P is double-buffered like S and never touches shared
-//              memory; finally O / l -> bf16 -> global.
+//   warps 4-19 softmax, two groups of eight warps that take the key tiles in turn, two threads per query row
+//              (= tensor-memory lane; each owns half of the tile's keys):
+//              x = S * scale*log2(e) + log2(count), masks (head length, optional causal tail), P = 2^(x - m) as a bf16 pair
+//              (leading part + remainder) written back over the scores it came from: the 32 fp32 columns of a chunk of scores
+//              become 16 columns of packed leading parts and 16 of remainders, so P never touches shared memory.
+//              The row's reference m is raised lazily (the accumulator row is rescaled in tensor memory only then; the
+//              tile's maximum is taken as a bound: largest raw product * scale + largest log2(count) of the tile) and is
+//              settled tile by tile: a group looks at its tile's maxima, waits until the other has settled the tile before,
+//              settles its own and goes on to the weights beside the other group; finally O / l -> bf16 -> global.
 // When the launch has too few CTAs to fill the GPU (few query rows: speculative decoding, short chunks), the keys
 // of a head are split over the CTAs of a thread-block cluster: each walks its share of the key tiles, leaves its
 // unnormalised (m, l, O) in its own shared memory, and after a cluster barrier every CTA folds a slice of the
 // query rows out of all members' shared memory (distributed shared memory) and writes that slice of the output.
-// What bounds it: the softmax of a tile (its arithmetic on packed pairs, one exponential per score) with the weighted sum
-// issued twice for the bf16 pair behind it.  4 layers x 512 causal queries per head over 8.5 K cores: 538 -> 489 us when the
-// tile's counts were requested a tile ahead (480 cycles per tile), one barrier per tile instead of two, the scores were
-// read from tensor memory once and two scores went through each fma and add (one at a time: 523 us).  Tried: the two
-// groups of four warps on alternate tiles with a row per thread and an accumulator each, 569 us.
+// What bounds it: shared memory.  A key tile's operands (64 KB for the scores, twice 32 KB for the pair of weights) and its copies
+// (64 KB) are 1536 clocks at 128 bytes, and the tensor cores need 1632; the MMA warp is busy 2300 of the 2530 clocks a tile takes.
+// 4 layers x 512 causal queries per head over 8.5 K cores 522 -> 461 us, 2 x 256 133 -> 110 against two score buffers and eight
+// softmax warps on one tile at a time, whose softmax (3500 clocks with one warp-instruction every 3 clocks per scheduler) was
+// the bound.  Two query tiles per CTA with a score buffer and an accumulator each: 480; the same with a 64-key
+// double buffer 562.  MMAs issued by a branch of one thread take 62 clocks each, by an elected lane of a converged warp 27.
 // Cluster width: as many CTAs per query tile as let every cluster of the launch be resident at once (asked of the
 // occupancy query: on this GPU 15 clusters of 8 or 9, 11 of 10, 7 of 11 to 16); powers of two up to 8 before.  8 queries per
 // head, 8 KV heads: 10 instead of 8 CTAs, 29 -> 24 us per layer with the above (four replicas of the rows, see kRep: 19); 16 clusters: 7 instead of 8 (which took
@@ -50,13 +51,13 @@ namespace cg = cooperative_groups;
 constexpr int kT = 128;                       // query rows per CTA, keys per tile
 constexpr int kHalf = kT * 128;               // 16384 bytes: one 64-column half of a [128 x 128] bf16 tile
 constexpr int kTile = 2 * kHalf;              // 32768
-constexpr int kThreads = 320;                 // warp 0: TMA, warp 1: MMA + tensor memory, warps 2-9: softmax
-constexpr int kTmemCols = 512;                // S0 | S1 | O (128 columns each; P overwrites S in place), rounded up to a power of two
-constexpr int kColS = 0, kColO = 256;
-constexpr int kStages = 3;                    // K/V ring
-constexpr int kSmQ = 0, kSmK = kTile, kSmV = (1 + kStages) * kTile, kSmLc = (1 + 2 * kStages) * kTile, kSmMx = kSmLc + 2 * kT * 4,
+constexpr int kThreads = 640;                 // warps 0, 2: TMA, warp 1: MMA + tensor memory, warps 4-19: softmax
+constexpr int kTmemCols = 512;                // S0 | S1 | S2 | O (128 columns each; P overwrites S in place)
+constexpr int kColS = 0, kColO = 384;
+constexpr int kStages = 3;                    // K and V rings, score buffers
+constexpr int kSmQ = 0, kSmK = kTile, kSmV = (1 + kStages) * kTile, kSmLc = (1 + 2 * kStages) * kTile, kSmMx = kSmLc + kStages * kT * 4,
               kSmBar = kSmMx + 2 * kT * 4;
-constexpr int kSmemBytes = kSmBar + 256;
+constexpr int kSmemBytes = kSmBar + 304;
 constexpr int kMaxSplit = 16;                 // CTAs that share one query tile: a cluster (more than 8 needs the non-portable opt-in)
 constexpr float kMaxSlack = 8.f;              // log2 units a score may exceed the running maximum before it is raised
 static_assert(kSmemBytes <= 232448, "shared memory of one CTA");
@@ -104,9 +105,9 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
         : "memory");
 }
 // D[tmem] (+)= A[tmem] * B[smem]: A's rows are tensor-memory lanes, two 16-bit elements of the contraction
-// axis per 32-bit column; one thread issues.
-__device__ __forceinline__ void mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, bool accumulate) {
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
+// axis per 32-bit column; a whole converged warp calls it, one elected lane issues.
+__device__ __forceinline__ void mma_bf16_ts_warp(uint32_t tmem_d, uint32_t tmem_a, uint64_t bdesc, uint32_t idesc, bool accumulate) {
+    asm volatile("{\n.reg .pred p, e;\nelect.sync _|e, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
                  ::"r"(tmem_d), "r"(tmem_a), "l"(bdesc), "r"(idesc), "r"((uint32_t)accumulate) : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory"); }
@@ -142,7 +143,7 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
 }
 
 // kRep: how often the query rows stand in the tile's 128 lanes.  Up to 32 (64) rows they do so four times (twice), and each
-// replica takes a quarter (half) of every key tile -- its weights of the other keys are zero --, so that all eight softmax warps work
+// replica takes a quarter (half) of every key tile -- its weights of the other keys are zero --, so that all softmax warps work
 // and a thread has 16 (32) scores a tile instead of 64; the replicas are folded at the end like the CTAs of a split.
 template <int kRep>
 __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_constant__ Params p) {
@@ -152,33 +153,27 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     const int G = p.Hq / p.Hkv, bh = b * p.Hkv + h;
     const int rows_total = G * p.m;                           // query rows of this (sequence, KV head)
     const uint32_t sbase = smem_u32(smem);
-    float* lc_s = reinterpret_cast<float*>(smem + kSmLc);     // [2][128] log2(count) of the tile's keys
-    float* ls_s = reinterpret_cast<float*>(smem + kSmMx);     // [2][128] at the end: each half's row sum
-    int* lcm_s = reinterpret_cast<int*>(smem + kSmBar + 128);  // [2][4] largest log2(count) of a tile, per writing warp (float bits)
+    float* lc_s = reinterpret_cast<float*>(smem + kSmLc);     // [3][128] log2(count) of a tile's keys
     const uint32_t bar0 = sbase + kSmBar;
-    const uint32_t q_full = bar0, kv_full0 = bar0 + 8, kv_empty0 = bar0 + 32, s_full0 = bar0 + 56, p_full0 = bar0 + 72,
-                   pv_done0 = bar0 + 88;
-    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kSmBar + 104);
-    volatile int* sh_fail = reinterpret_cast<volatile int*>(smem + kSmBar + 108);
-    volatile int* sh_fail_sm = reinterpret_cast<volatile int*>(smem + kSmBar + 112);   // set by the softmax warps only
-    volatile int* sh_issued = reinterpret_cast<volatile int*>(smem + kSmBar + 116);
+    // three of each, by key tile: K, V, log2(count) landed; K spent; scores ready; weights ready; weights (and V) spent, O holds the tile
+    const uint32_t q_full = bar0, k_full0 = bar0 + 8, v_full0 = bar0 + 32, lc_full0 = bar0 + 56, k_empty0 = bar0 + 80, s_full0 = bar0 + 104,
+                   p_full0 = bar0 + 128, pv_done0 = bar0 + 152, ref0 = bar0 + 176;   // ref: [4 x 32 rows][tile & 1] the tile's reference is settled
+    float* lcm_s = reinterpret_cast<float*>(smem + kSmBar + 240);                      // [3] largest log2(count) of a tile
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + kSmBar + 252);
+    volatile int* sh_fail = reinterpret_cast<volatile int*>(smem + kSmBar + 256);
+    volatile int* sh_issued = reinterpret_cast<volatile int*>(smem + kSmBar + 260);   // key tiles whose K, and whose V, was requested
+    volatile int* sh_fail_pair = reinterpret_cast<volatile int*>(smem + kSmBar + 268);   // [8] set by the two warps of 32 rows of a group
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    if (tid == 0) {
-        mbar_init(q_full, 1);
-        for (int s = 0; s < kStages; ++s) {
-            mbar_init(kv_full0 + 8 * s, 1);
-            mbar_init(kv_empty0 + 8 * s, 1);
-        }
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(s_full0 + 8 * s, 1);
-            mbar_init(p_full0 + 8 * s, 8);
-            mbar_init(pv_done0 + 8 * s, 1);
-        }
+    if (warp == 0) {
+        if (lane < 30) mbar_init(bar0 + 8 * lane, lane >= 22 ? 2 : lane >= 16 && lane < 19 ? 8 : 1);   // ref: a row's two warps; weights: a group's eight
         mbar_fence_init();
-        *sh_fail = 0; *sh_fail_sm = 0; *sh_issued = 0;
+        if (lane < 8) sh_fail_pair[lane] = 0;
+        if (lane == 0) { *sh_fail = 0; sh_issued[0] = 0; sh_issued[1] = 0; }
+    } else if (warp == 2 && lane < 3) {
+        prefetch_map(lane == 0 ? &p.map_q : lane == 1 ? &p.map_k : &p.map_v);
     }
-    if (warp == 1) tmem_alloc(sbase + kSmBar + 104, kTmemCols);
+    if (warp == 1) tmem_alloc(sbase + kSmBar + 252, kTmemCols);
     fence_before_sync();
     __syncthreads();
     fence_after_sync();
@@ -198,202 +193,246 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
         return;
     }
     if (warp == 0) {
-        if (lane == 0 && nt > 0) {   // ---- TMA producer ----
+        if (lane == 0 && nt > 0) {   // ---- TMA producer: queries and keys (a key tile's place is free long before a value tile's) ----
             mbar_expect_tx(q_full, kTile);
             for (int c = 0; c < kRep; ++c) {   // (boxes of 128 / kRep rows)
                 tma_load_4d(sbase + kSmQ + c * (kHalf / kRep), &p.map_q, 0, (int)q_row0, 0, 0, q_full);
                 tma_load_4d(sbase + kSmQ + kHalf + c * (kHalf / kRep), &p.map_q, 64, (int)q_row0, 0, 0, q_full);
             }
-            const int row_base = bh * p.cap + t_lo * kT;
             for (int t = 0; t < nt; ++t) {
-                const int s = t % kStages;
-                if (t >= kStages && !mbar_wait(kv_empty0 + 8 * s, ((t / kStages) - 1) & 1)) { *sh_fail = 1; break; }
-                mbar_expect_tx(kv_full0 + 8 * s, 2 * kTile);
-                const uint32_t dk = sbase + kSmK + s * kTile, dv = sbase + kSmV + s * kTile;
-                tma_load_4d(dk, &p.map_k, 0, row_base + t * kT, 0, 0, kv_full0 + 8 * s);
-                tma_load_4d(dk + kHalf, &p.map_k, 64, row_base + t * kT, 0, 0, kv_full0 + 8 * s);
-                tma_load_4d(dv, &p.map_v, 0, row_base + t * kT, 0, 0, kv_full0 + 8 * s);
-                tma_load_4d(dv + kHalf, &p.map_v, 64, row_base + t * kT, 0, 0, kv_full0 + 8 * s);
-                *sh_issued = t + 1;
+                const int s = t % kStages, round = t / kStages, at = bh * p.cap + (t_lo + t) * kT;
+                if (round > 0 && !mbar_wait(k_empty0 + 8 * s, (round - 1) & 1)) { *sh_fail = 1; break; }
+                mbar_expect_tx(k_full0 + 8 * s, kTile);
+                tma_load_4d(sbase + kSmK + s * kTile, &p.map_k, 0, at, 0, 0, k_full0 + 8 * s);
+                tma_load_4d(sbase + kSmK + s * kTile + kHalf, &p.map_k, 64, at, 0, 0, k_full0 + 8 * s);
+                sh_issued[0] = t + 1;
             }
+        }
+    } else if (warp == 2) {
+        // ---- TMA producer: values; and log2(count) of the tile's keys, whose counts are requested a tile ahead ----
+        const int32_t* cnt = p.count ? p.count + (size_t)bh * p.cap : nullptr;
+        int c[4];
+        auto request_counts = [&](int t) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = (t_lo + t) * kT + u * 32 + lane;
+                c[u] = cnt != nullptr && t < nt && j < len ? cnt[j] : 1;
+            }
+        };
+        request_counts(0);
+        for (int t = 0; t < nt; ++t) {
+            const int s = t % kStages, round = t / kStages, at = bh * p.cap + (t_lo + t) * kT;
+            // (when the weighted sum of the tile before in this place is complete, its counts have been read as well)
+            if (round > 0 && !__all_sync(kFull, mbar_wait(pv_done0 + 8 * s, (round - 1) & 1))) { *sh_fail = 1; break; }
+            if (lane == 0) {
+                mbar_expect_tx(v_full0 + 8 * s, kTile);
+                tma_load_4d(sbase + kSmV + s * kTile, &p.map_v, 0, at, 0, 0, v_full0 + 8 * s);
+                tma_load_4d(sbase + kSmV + s * kTile + kHalf, &p.map_v, 64, at, 0, 0, v_full0 + 8 * s);
+                sh_issued[1] = t + 1;
+            }
+            int top = 0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float lc = lg2((float)max(c[u], 1));
+                lc_s[s * kT + u * 32 + lane] = lc;
+                top = max(top, __float_as_int(lc));   // lc >= 0: the bits order like the values
+            }
+            top = __reduce_max_sync(kFull, top);
+            if (lane == 0) lcm_s[s] = __int_as_float(top);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(lc_full0 + 8 * s);
+            request_counts(t + 1);
         }
     } else if (warp == 1) {
-        if (lane == 0 && nt > 0) {   // ---- MMA issuer ----
+        if (nt > 0) {   // ---- MMA issuer (the whole warp, one elected lane) ----
             constexpr uint32_t idesc_qk = instr_desc_bf16(kT, kT, false, false);   // Q and K both K-major
             constexpr uint32_t idesc_pv = instr_desc_bf16(kT, kT, false, true);    // P K-major (tensor memory), V MN-major
-            const uint32_t aq = sbase + kSmQ;
-            auto issue_qk = [&](int t) {   // S[t & 1] = Q K_t^T
-                const uint32_t bk = sbase + kSmK + (t % kStages) * kTile;
+            const auto arrived = [&](uint32_t bar, int parity) { return __all_sync(kFull, mbar_wait(bar, parity & 1)); };
+            auto issue_qk = [&](int s) {   // S = Q K^T
+                const uint64_t qd = smem_desc_sw128(sbase + kSmQ, 16, 1024), kd = smem_desc_sw128(sbase + kSmK + s * kTile, 16, 1024);
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {
-                    const uint32_t off = (ks >> 2) * kHalf + (ks & 3) * 32;
-                    mma_bf16_ss(tmem + kColS + (t & 1) * kT, smem_desc_sw128(aq + off, 16, 1024), smem_desc_sw128(bk + off, 16, 1024),
-                                idesc_qk, ks > 0);
+                    const uint32_t off = ((ks >> 2) * kHalf + (ks & 3) * 32) >> 4;
+                    mma_bf16_ss_warp(tmem + kColS + s * kT, qd + off, kd + off, idesc_qk, ks > 0);
                 }
-                mma_commit(s_full0 + 8 * (t & 1));
+                mma_commit_warp(k_empty0 + 8 * s);
+                mma_commit_warp(s_full0 + 8 * s);
             };
-            bool ok = mbar_wait(q_full, 0) && mbar_wait(kv_full0, 0);
-            if (ok) { fence_after_sync(); issue_qk(0); }
-            if (ok && nt > 1) {
-                ok = mbar_wait(kv_full0 + 8, 0);
-                if (ok) { fence_after_sync(); issue_qk(1); }
-            }
-            for (int t = 0; t < nt && ok; ++t) {
-                const int sb = t & 1;
-                ok = mbar_wait(p_full0 + 8 * sb, (t >> 1) & 1);   // the weights of tile t are in tensor memory
+            bool ok = arrived(q_full, 0);
+            for (int t = 0; t < min(nt, kStages) && ok; ++t) {
+                ok = arrived(k_full0 + 8 * t, 0);
                 if (!ok) break;
                 fence_after_sync();
-                const uint32_t bv = sbase + kSmV + (t % kStages) * kTile;
-                const uint32_t pcol = tmem + kColS + sb * kT;
+                issue_qk(t);
+            }
+            for (int t = 0; t < nt && ok; ++t) {
+                const int s = t % kStages, round = t / kStages;
+                ok = arrived(v_full0 + 8 * s, round) && arrived(p_full0 + 8 * s, round);   // the weights of tile t are in tensor memory
+                if (!ok) break;
+                fence_after_sync();
+                const uint64_t vd = smem_desc_sw128(sbase + kSmV + s * kTile, kHalf, 1024);   // MN-major, 16 key rows a step
+                const uint32_t pcol = tmem + kColS + s * kT;
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks) {   // sixteen keys per instruction: eight packed columns of P
-                    const uint64_t vdesc = smem_desc_sw128(bv + ks * 16 * 128, kHalf, 1024);   // V: MN-major, 16 key rows down
                     const uint32_t pa = pcol + (ks >> 1) * 32 + (ks & 1) * 8;                  // leading parts; remainders 16 columns on
-                    mma_bf16_ts(tmem + kColO, pa, vdesc, idesc_pv, t > 0 || ks > 0);
-                    mma_bf16_ts(tmem + kColO, pa + 16, vdesc, idesc_pv, true);
+                    mma_bf16_ts_warp(tmem + kColO, pa, vd + ((ks * 16 * 128) >> 4), idesc_pv, t > 0 || ks > 0);
+                    mma_bf16_ts_warp(tmem + kColO, pa + 16, vd + ((ks * 16 * 128) >> 4), idesc_pv, true);
                 }
-                mma_commit(kv_empty0 + 8 * (t % kStages));   // K and V of this stage are spent
-                mma_commit(pv_done0 + 8 * sb);               // P of this buffer is spent, O holds tile t
-                if (t + 2 < nt) {   // the scores two tiles ahead go where this tile's scores and weights were
-                    ok = mbar_wait(kv_full0 + 8 * ((t + 2) % kStages), ((t + 2) / kStages) & 1) &&
-                         mbar_wait(pv_done0 + 8 * sb, (t >> 1) & 1);
+                mma_commit_warp(pv_done0 + 8 * s);   // P of this buffer and V of this stage are spent, O holds tile t
+                if (t + kStages < nt) {   // the scores three tiles ahead go where this tile's scores and weights were
+                    ok = arrived(k_full0 + 8 * s, round + 1) && arrived(pv_done0 + 8 * s, round);
                     if (!ok) break;
                     fence_after_sync();
-                    issue_qk(t + 2);
+                    issue_qk(s);
                 }
             }
-            if (!ok) *sh_fail = 1;
+            if (!ok && lane == 0) *sh_fail = 1;
         }
-    } else {
-        // ---- softmax: two threads per query row (= tensor-memory lane), each owning 64 of a tile's 128 keys
-        //      and 64 of the accumulator's 128 columns; warps 2-5 take the first halves, warps 6-9 the second ----
-        const int q = warp & 3, r = q * 32 + lane, wg = (warp - 2) >> 2;
+    } else if (warp >= 4) {
+        // ---- softmax: warps 4-11 take the even key tiles, warps 12-19 the odd ones; two threads per query row (= tensor-memory
+        //      lane), each owning half of a tile's keys (of the replica's share) ----
+        const int grp = (warp - 4) >> 3, q = warp & 3, r = q * 32 + lane, wg = ((warp - 4) >> 2) & 1;
         constexpr int kRows = kT / kRep, kKeys = 64 / kRep;   // rows of a replica; keys of a tile per thread
+        constexpr int kHold = kKeys > 32 ? 32 : kKeys;        // scores kept in registers (the others are read again)
         const int col0 = (r / kRows) * kRows + wg * kKeys;    // the first of them (a replica has as many keys as rows)
         const int row = qt * kT + r % kRows;                  // row among the G*m of this head group
         const bool row_ok = row < rows_total;
         const int qi = row % p.m;                             // which of the m queries
         const int vis = p.causal ? len - (p.m - 1 - qi) : len;   // keys this row sees: [0, vis)
         const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-        const int32_t* cnt = p.count ? p.count + (size_t)bh * p.cap : nullptr;
-        float m_run = -INFINITY, l_run = 0.f;                 // l_run: this thread's keys only
+        const int pair = grp * 4 + q;                         // the two warps of these 32 rows in this group
+        float* ref_s = reinterpret_cast<float*>(smem + kSmMx);      // [128] the rows' references
+        float* mx_s = ref_s + kT;                                   // [128] a maximum on its way, where a reference is raised
+        float m_mine = -INFINITY, l_run = 0.f;                // l_run: the weights of this thread's keys, relative to m_mine
         bool failed = false;
         const bool idle = qt * kT + (q * 32) % kRows >= rows_total;     // none of the warp's rows exists: it only keeps step
         const float2 scale2 = make_float2(p.scale_log2, p.scale_log2);
-        // log2(count) of a tile's keys, one key per thread of the first four warps.  The counts of the next tile are requested
-        // a tile ahead and published behind this tile's barrier, when nobody reads that buffer any more.
-        auto count_of = [&](int t) { const int j = (t_lo + t) * kT + r; return cnt != nullptr && t < nt && j < len ? cnt[j] : 1; };
-        auto publish_counts = [&](int t, int c) {
-            const float lc = lg2((float)max(c, 1));
-            lc_s[(t & 1) * kT + r] = lc;
-            const int top = __reduce_max_sync(kFull, __float_as_int(lc));   // lc >= 0: the bits order like the values
-            if (lane == 0) lcm_s[(t & 1) * 4 + q] = top;
+        const auto pair_sync = [&] { asm volatile("bar.sync %0, 64;\n" ::"r"(1 + pair) : "memory"); };
+        const auto pair_any = [&](bool mine) {
+            uint32_t out;
+            asm volatile("{\n.reg .pred p, r;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.or.pred r, %2, 64, p;\nselp.u32 %0, 1, 0, r;\n}\n"
+                         : "=r"(out) : "r"(mine ? 1u : 0u), "r"(1 + pair) : "memory");
+            return out != 0u;
         };
-        if (wg == 0) publish_counts(0, count_of(0));
-        for (int t = 0; t < nt; ++t) {
-            const int s = t & 1, st = t % kStages, j0 = (t_lo + t) * kT, jw = j0 + col0;   // jw: first key of this thread
-            const int next_count = wg == 0 ? count_of(t + 1) : 1;
-            if (!mbar_wait(s_full0 + 8 * s, (t >> 1) & 1)) { *sh_fail = 1; *sh_fail_sm = 1; }
+        for (int t = grp; t < nt; t += 2) {
+            const int s = t % kStages, round = t / kStages, j0 = (t_lo + t) * kT, jw = j0 + col0;   // jw: first key of this thread
+            const uint32_t s_addr = lane_addr + kColS + s * kT + col0;
+            bool lost = !mbar_wait(s_full0 + 8 * s, round & 1) || !mbar_wait(lc_full0 + 8 * s, round & 1);
+            __syncwarp();
             fence_after_sync();
-            // pass 1: the row's largest raw product in this tile (each thread its half, then the two are exchanged).  That times
-            // the scale plus the tile's largest log2(count) bounds the row's largest score: any reference at or above the
-            // true maximum serves the softmax, and this one is at most log2 of the largest count above it.  (A scale that
-            // is not positive takes the smallest product.)
-            uint32_t g[kKeys];
+            // pass 1: the largest raw product of the thread's keys.  That times the scale plus the tile's largest log2(count) bounds
+            // its largest score: any reference at or above the true maximum serves the softmax, and this one is at most log2 of
+            // the largest count above it.  (A scale that is not positive takes the smallest product.)
+            uint32_t g[kHold];
             const bool all_seen = __all_sync(kFull, jw + kKeys <= vis);   // none of these keys is masked for any row of the warp
             float mx = -INFINITY;
             if (!idle) {
-                if constexpr (kRep == 4) {
-                    tmem_ld16(lane_addr + kColS + s * kT + col0, g);
-                } else {
 #pragma unroll
-                    for (int k = 0; k < kKeys; k += 32) tmem_ld32(lane_addr + kColS + s * kT + col0 + k, *reinterpret_cast<uint32_t(*)[32]>(&g[k]));
+                for (int c = kKeys / kHold - 1; c >= 0; --c) {   // (the first piece stays in registers, the other is read again)
+                    if constexpr (kHold == 16) tmem_ld16(s_addr, g);
+                    else tmem_ld32(s_addr + c * 32, g);
+                    tmem_ld_wait();
+                    if (!(p.scale_log2 > 0.f)) {
+#pragma unroll
+                        for (int k = 0; k < kHold; ++k)
+                            if (jw + c * 32 + k < vis) mx = fmaxf(mx, -__uint_as_float(g[k]));
+                    } else if (all_seen) {
+                        float m4[4] = {mx, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                        for (int k = 0; k < kHold; k += 8)
+#pragma unroll
+                            for (int x = 0; x < 4; ++x) m4[x] = max3(m4[x], __uint_as_float(g[k + x]), __uint_as_float(g[k + 4 + x]));
+                        mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < kHold; ++k)
+                            if (jw + c * 32 + k < vis) mx = fmaxf(mx, __uint_as_float(g[k]));
+                    }
                 }
-                tmem_ld_wait();
-                if (!(p.scale_log2 > 0.f)) {
-#pragma unroll
-                    for (int k = 0; k < kKeys; ++k)
-                        if (jw + k < vis) mx = fmaxf(mx, -__uint_as_float(g[k]));
-                } else if (all_seen) {
-                    float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-                    for (int k = 0; k < kKeys; k += 8)
-#pragma unroll
-                        for (int x = 0; x < 4; ++x) m4[x] = max3(m4[x], __uint_as_float(g[k + x]), __uint_as_float(g[k + 4 + x]));
-                    mx = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
-                } else {
-#pragma unroll
-                    for (int k = 0; k < kKeys; ++k)
-                        if (jw + k < vis) mx = fmaxf(mx, __uint_as_float(g[k]));
-                }
+                if (mx != -INFINITY) mx = fmaf(mx, fabsf(p.scale_log2), lcm_s[s]);
             }
-            // The halves' maxima [2][128] go where the tile's keys were: their product is complete, and the stage is filled again
-            // only after every warp has handed in this tile's weights (behind the proxy fence below).
-            float* mx_s = reinterpret_cast<float*>(smem + kSmK + st * kTile);
-            mx_s[wg * kT + r] = mx;
             // Rows of the stage past the head's end hold whatever lies behind the cores (0 * NaN would poison
             // the second product): this row's threads clear its V row.  K rows need nothing, their scores are masked.
-            if (j0 + r >= len) {
+            if (j0 + kT > len) {
+                lost = !mbar_wait(v_full0 + 8 * s, round & 1) || lost;
+                if (j0 + r >= len) {
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
-                    *reinterpret_cast<uint4*>(smem + kSmV + st * kTile + wg * kHalf + r * 128 + u * 16) = make_uint4(0u, 0u, 0u, 0u);
+                    for (int u = 0; u < 8; ++u)
+                        *reinterpret_cast<uint4*>(smem + kSmV + s * kTile + wg * kHalf + r * 128 + u * 16) = make_uint4(0u, 0u, 0u, 0u);
+                }
+                fence_async_proxy();   // for the tensor core's reads
+                __syncwarp();
             }
-            asm volatile("bar.sync 2, 256;\n" ::: "memory");   // both halves' maxima and this tile's log2(count) are in place
-            if (*sh_fail_sm) { failed = true; break; }
-            if (wg == 0 && t + 1 < nt) publish_counts(t + 1, next_count);
+            // The row's reference is settled tile by tile, by either group in its turn: the tile before has settled its own.
+            if (t > 0) lost = !mbar_wait(ref0 + 16 * q + 8 * ((t - 1) & 1), ((t - 1) >> 1) & 1) || lost;
+            float m = t > 0 ? ref_s[r] : -INFINITY;
+            if (lost) { *sh_fail = 1; sh_fail_pair[pair] = 1; }
+            if (t == 0) (wg == 0 ? mx_s : ref_s)[r] = mx;       // (there is no reference to read yet)
+            const bool raise_any = pair_any(!idle && mx > m + kMaxSlack);   // also the first finite score (m = -inf)
+            if (sh_fail_pair[pair]) { failed = true; break; }
+            if (raise_any) {
+                if (t > 0) {
+                    (wg == 0 ? mx_s : ref_s)[r] = mx;           // (both threads of the row have read the reference, nobody else does yet)
+                    pair_sync();
+                }
+                mx = fmaxf(mx, (wg == 0 ? ref_s : mx_s)[r]);
+                const bool raise = mx > m + kMaxSlack;          // same in the row's two threads
+                const float f = raise ? ex2(m - mx) : 1.f;      // 0 when nothing had been seen
+                if (raise) m = mx;
+                if (wg == 0) ref_s[r] = m;
+                // the accumulator may be touched only between two weighted sums: the one before must be complete (this tile's
+                // cannot start before this warp has handed in its weights)
+                if (t > 0 && !idle) {
+                    if (!mbar_wait(pv_done0 + 8 * ((t - 1) % kStages), ((t - 1) / kStages) & 1)) { *sh_fail = 1; sh_fail_pair[pair] = 1; }
+                    __syncwarp();
+                    fence_after_sync();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t o[16];
+                        tmem_ld16(lane_addr + kColO + wg * 64 + c * 16, o);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * f);
+                        tmem_st16(lane_addr + kColO + wg * 64 + c * 16, o);
+                    }
+                    tmem_st_wait();
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(ref0 + 16 * q + 8 * (t & 1));
             if (!idle) {
+                if (m != m_mine) {   // the row sum follows the reference
+                    l_run = m_mine == -INFINITY ? 0.f : l_run * ex2(m_mine - m);
+                    m_mine = m;
+                }
                 if (kRep > 1) {   // the weights of the other replicas' keys
                     const uint32_t zero[16] = {0u};
 #pragma unroll
                     for (int c = kRows; c < kT; c += 32) tmem_st16(lane_addr + kColS + s * kT + (((r / kRows) * kRows + c) & (kT - 1)) + wg * 16, zero);
                 }
-                mx = fmaxf(mx, mx_s[(wg ^ 1) * kT + r]);
-                if (mx != -INFINITY) {
-                    const int top = max(max(lcm_s[s * 4], lcm_s[s * 4 + 1]), max(lcm_s[s * 4 + 2], lcm_s[s * 4 + 3]));
-                    mx = fmaf(mx, fabsf(p.scale_log2), __int_as_float(top));
-                }
-                const bool raise = mx > m_run + kMaxSlack;      // also the first finite score (m_run = -inf); same in both threads
-                if (__any_sync(kFull, raise)) {
-                    const float f = raise ? ex2(m_run - mx) : 1.f;   // 0 when nothing had been seen
-                    // the accumulator may be touched only between two weighted sums: the previous one must be complete
-                    // (this tile's cannot start before this warp has handed in its weights)
-                    if (t > 0 && !mbar_wait(pv_done0 + 8 * ((t - 1) & 1), ((t - 1) >> 1) & 1)) { *sh_fail = 1; *sh_fail_sm = 1; }
-                    fence_after_sync();
-                    if (t > 0) {
-#pragma unroll
-                        for (int c = 0; c < 2; ++c) {
-                            uint32_t o[32];
-                            tmem_ld32(lane_addr + kColO + wg * 64 + c * 32, o);
-                            tmem_ld_wait();
-#pragma unroll
-                            for (int k = 0; k < 32; ++k) o[k] = __float_as_uint(__uint_as_float(o[k]) * f);
-                            tmem_st32(lane_addr + kColO + wg * 64 + c * 32, o);
-                        }
-                        tmem_st_wait();
-                    }
-                    l_run *= f;
-                    if (raise) m_run = mx;
-                }
                 // pass 2: weights, as bf16 pairs (leading part + remainder), back into the score buffer's columns: the 32 score
                 // columns of a chunk become 16 columns of packed leading parts and 16 of remainders
-                const float mref = m_run == -INFINITY ? 0.f : m_run;
+                const float mref = m == -INFINITY ? 0.f : m;
                 const float2 nref2 = make_float2(-mref, -mref);
                 // (the row sum takes the weights before the split: the pair carries sixteen bits of each, the difference
                 // is below 2^-17 of the sum)
                 float2 l2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-                for (int c = 0; c < (kRep == 1 ? 2 : 1); ++c) {
-                    constexpr int kChunk = kRep == 4 ? 16 : 32;
-                    uint32_t hi[kChunk / 2], lo[kChunk / 2];
+                for (int c = 0; c < kKeys / 16; ++c) {
+                    if (kKeys > kHold && c == kHold / 16) {
+                        if constexpr (kHold == 32) tmem_ld32(s_addr + 32, g);
+                        tmem_ld_wait();
+                    }
+                    uint32_t hi[8], lo[8];
 #pragma unroll
-                    for (int k = 0; k < kChunk; k += 4) {
-                        const float4 lc = *reinterpret_cast<const float4*>(lc_s + s * kT + col0 + c * 32 + k);
-                        const uint32_t* gk = g + c * 32 + k;
+                    for (int k = 0; k < 16; k += 4) {
+                        const float4 lc = *reinterpret_cast<const float4*>(lc_s + s * kT + col0 + c * 16 + k);
+                        const uint32_t* gk = g + (c * 16) % kHold + k;
                         const float2 x0 = add2(fma2(make_float2(__uint_as_float(gk[0]), __uint_as_float(gk[1])), scale2, make_float2(lc.x, lc.y)), nref2);
                         const float2 x1 = add2(fma2(make_float2(__uint_as_float(gk[2]), __uint_as_float(gk[3])), scale2, make_float2(lc.z, lc.w)), nref2);
                         float2 w0 = make_float2(ex2(x0.x), ex2(x0.y)), w1 = make_float2(ex2(x1.x), ex2(x1.y));
                         if (!all_seen) {
-                            const int j = jw + c * 32 + k;
+                            const int j = jw + c * 16 + k;
                             w0.x = j < vis ? w0.x : 0.f; w0.y = j + 1 < vis ? w0.y : 0.f;
                             w1.x = j + 2 < vis ? w1.x : 0.f; w1.y = j + 3 < vis ? w1.y : 0.f;
                         }
@@ -405,54 +444,53 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
                         hi[k >> 1] = p0; hi[(k >> 1) + 1] = p1;
                         lo[k >> 1] = pack2(r0, r1); lo[(k >> 1) + 1] = pack2(r2, r3);
                     }
-                    if constexpr (kRep == 4) {   // two threads share a chunk of 32 columns
-                        tmem_st8(lane_addr + kColS + s * kT + q * 32 + wg * 8, hi);
-                        tmem_st8(lane_addr + kColS + s * kT + q * 32 + 16 + wg * 8, lo);
-                    } else {
-                        tmem_st16(lane_addr + kColS + s * kT + col0 + c * 32, hi);
-                        tmem_st16(lane_addr + kColS + s * kT + col0 + c * 32 + 16, lo);
-                    }
+                    // (sixteen keys: half a chunk of 32 columns, which the two threads of a row share where there are four replicas)
+                    const uint32_t at = lane_addr + kColS + s * kT + (col0 & ~31) + (c >> 1) * 32 + ((kRep == 4 ? wg : c) & 1) * 8;
+                    tmem_st8(at, hi);
+                    tmem_st8(at + 16, lo);
                 }
                 l_run += (l2[0].x + l2[0].y) + (l2[1].x + l2[1].y);
                 tmem_st_wait();
             }
             fence_before_sync();      // this thread's accesses to tensor memory
-            fence_async_proxy();      // a cleared V row, for the tensor core's reads; the maxima, for the copies to come
             __syncwarp();
             if (lane == 0) mbar_arrive(p_full0 + 8 * s);
         }
-        // ---- O / l -> bf16 -> global: each thread its 64 columns; l is the sum of the row's two partial sums ----
-        if (!failed && nt > 0) {
-            if (!mbar_wait(pv_done0 + 8 * ((nt - 1) & 1), ((nt - 1) >> 1) & 1)) { *sh_fail = 1; failed = true; }
+        // ---- O / l -> bf16 -> global: each thread 32 columns of its row; l is the sum of the row's four partial sums ----
+        bool ok = nt > 0 && !failed;
+        if (ok) {
+            ok = __all_sync(kFull, mbar_wait(pv_done0 + 8 * ((nt - 1) % kStages), ((nt - 1) / kStages) & 1));
+            if (!ok) *sh_fail = 1;
             fence_after_sync();
         }
-        asm volatile("bar.sync 2, 256;\n" ::: "memory");   // nobody still reads the last tile's maxima
-        ls_s[wg * kT + r] = l_run;
-        asm volatile("bar.sync 1, 256;\n" ::: "memory");
-        const float l_row = l_run + ls_s[(wg ^ 1) * kT + r];
+        const auto rows_sync = [&] { asm volatile("bar.sync %0, 128;\n" ::"r"(9 + q) : "memory"); };   // the four warps of these 32 rows
+        rows_sync();   // the last reference is settled
+        const float m_row = nt > 0 ? ref_s[r] : -INFINITY;
+        float* ls_s = reinterpret_cast<float*>(smem + kSmK + 2 * kTile);   // [4][128] (all keys are spent)
+        ls_s[(grp * 2 + wg) * kT + r] = m_mine == -INFINITY ? 0.f : l_run * ex2(m_mine - m_row);
+        rows_sync();
+        const float l_row = (ls_s[r] + ls_s[kT + r]) + (ls_s[2 * kT + r] + ls_s[3 * kT + r]);
+        const int ocol = (grp * 2 + wg) * 32;
+        uint32_t o[32];
+        if (ok) {
+            tmem_ld32(lane_addr + kColO + ocol, o);
+            tmem_ld_wait();
+        } else {
+#pragma unroll
+            for (int k = 0; k < 32; ++k) o[k] = 0u;
+        }
         if (kRep == 1 && n_split == 1) {
-            __nv_bfloat16* orow = p.out + (size_t)(q_row0 + r) * 128 + wg * 64;
+            __nv_bfloat16* orow = p.out + (size_t)(q_row0 + r) * 128 + ocol;
             const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
+            if (row_ok) {
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t o[32];
-                if (nt > 0 && !failed) {
-                    tmem_ld32(lane_addr + kColO + wg * 64 + c * 32, o);
-                    tmem_ld_wait();
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) o[k] = 0u;
-                }
-                if (row_ok) {
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        uint4 v;
-                        v.x = pack2(__uint_as_float(o[8 * u]) * inv, __uint_as_float(o[8 * u + 1]) * inv);
-                        v.y = pack2(__uint_as_float(o[8 * u + 2]) * inv, __uint_as_float(o[8 * u + 3]) * inv);
-                        v.z = pack2(__uint_as_float(o[8 * u + 4]) * inv, __uint_as_float(o[8 * u + 5]) * inv);
-                        v.w = pack2(__uint_as_float(o[8 * u + 6]) * inv, __uint_as_float(o[8 * u + 7]) * inv);
-                        *reinterpret_cast<uint4*>(orow + c * 32 + u * 8) = v;
-                    }
+                for (int u = 0; u < 4; ++u) {
+                    uint4 v;
+                    v.x = pack2(__uint_as_float(o[8 * u]) * inv, __uint_as_float(o[8 * u + 1]) * inv);
+                    v.y = pack2(__uint_as_float(o[8 * u + 2]) * inv, __uint_as_float(o[8 * u + 3]) * inv);
+                    v.z = pack2(__uint_as_float(o[8 * u + 4]) * inv, __uint_as_float(o[8 * u + 5]) * inv);
+                    v.w = pack2(__uint_as_float(o[8 * u + 6]) * inv, __uint_as_float(o[8 * u + 7]) * inv);
+                    *reinterpret_cast<uint4*>(orow + u * 8) = v;
                 }
             }
         } else {
@@ -460,25 +498,14 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             float* part_o = reinterpret_cast<float*>(smem + kSmK);      // [128 rows][32 float4], float4 index ^ (row & 31)
             float* part_ml = reinterpret_cast<float*>(smem + kSmV);     // [128] m, [128] l; the folded replicas' [128] m, [128] l
 #pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                uint32_t o[32];
-                if (nt > 0 && !failed) {
-                    tmem_ld32(lane_addr + kColO + wg * 64 + c * 32, o);
-                    tmem_ld_wait();
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) o[k] = 0u;
-                }
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                    const int c4 = wg * 16 + c * 8 + u;
-                    *reinterpret_cast<uint4*>(part_o + r * 128 + ((c4 ^ (r & 31)) << 2)) = make_uint4(o[4 * u], o[4 * u + 1], o[4 * u + 2], o[4 * u + 3]);
-                }
+            for (int u = 0; u < 8; ++u) {
+                const int c4 = ocol / 4 + u;
+                *reinterpret_cast<uint4*>(part_o + r * 128 + ((c4 ^ (r & 31)) << 2)) = make_uint4(o[4 * u], o[4 * u + 1], o[4 * u + 2], o[4 * u + 3]);
             }
-            if (wg == 0) { part_ml[r] = (nt > 0 && !failed) ? m_run : -INFINITY; part_ml[kT + r] = (nt > 0 && !failed) ? l_row : 0.f; }
+            if (grp == 0 && wg == 0) { part_ml[r] = ok ? m_row : -INFINITY; part_ml[kT + r] = ok ? l_row : 0.f; }
             if (kRep > 1) {   // the replicas of a row into the first, one thread per (row, four output columns)
-                asm volatile("bar.sync 1, 256;\n" ::: "memory");
-                for (int it = tid - 64; it < kRows * 32; it += 256) {
+                asm volatile("bar.sync 13, 512;\n" ::: "memory");
+                for (int it = tid - 128; it < kRows * 32; it += 512) {
                     const int fr = it >> 5, c4 = it & 31;
                     float gm = -INFINITY, lsum = 0.f;
                     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -487,10 +514,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
 #pragma unroll
                     for (int j = 0; j < kRep; ++j) {
                         const float mj = part_ml[fr + kRows * j], w = mj == -INFINITY ? 0.f : ex2(mj - gm);
-                        const float4 o = *reinterpret_cast<const float4*>(part_o + (fr + kRows * j) * 128 + ((c4 ^ (fr & 31)) << 2));
+                        const float4 ov = *reinterpret_cast<const float4*>(part_o + (fr + kRows * j) * 128 + ((c4 ^ (fr & 31)) << 2));
                         lsum = fmaf(w, part_ml[kT + fr + kRows * j], lsum);
-                        acc.x = fmaf(w, o.x, acc.x); acc.y = fmaf(w, o.y, acc.y);
-                        acc.z = fmaf(w, o.z, acc.z); acc.w = fmaf(w, o.w, acc.w);
+                        acc.x = fmaf(w, ov.x, acc.x); acc.y = fmaf(w, ov.y, acc.y);
+                        acc.z = fmaf(w, ov.z, acc.z); acc.w = fmaf(w, ov.w, acc.w);
                     }
                     *reinterpret_cast<float4*>(part_o + fr * 128 + ((c4 ^ (fr & 31)) << 2)) = acc;   // (read by this thread only)
                     if (c4 == 0) { part_ml[2 * kT + fr] = gm; part_ml[3 * kT + fr] = lsum; }
@@ -500,9 +527,10 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
     }
     if (kRep > 1 || n_split > 1) {
         cg::cluster_group cluster = cg::this_cluster();
+        __syncwarp();
         fence_before_sync();
         cluster.sync();   // every member's partial is in its shared memory
-        if (warp >= 2) {
+        if (warp >= 4) {
             // this CTA folds query rows [split * R, (split + 1) * R) of the tile, R = 128 / n_split rounded up: one thread per
             // (row, four output columns), reading that piece of every member's partial, four or eight members at a time
             const float* part_o = reinterpret_cast<const float*>(smem + kSmK);
@@ -511,7 +539,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             const int R = (kRows + n_split - 1) / n_split, r_end = min(min((split + 1) * R, kRows), rows_total - qt * kT);
             const auto fold_rows = [&](auto width) {   // `width` partials at a time
                 constexpr int kFold = decltype(width)::value;
-                for (int it = tid - 64; it < R * 32; it += 256) {
+                for (int it = tid - 128; it < R * 32; it += 512) {
                     const int r = split * R + (it >> 5), c4 = it & 31;
                     if (r >= r_end) break;
                     float gm = -INFINITY, lsum = 0.f;
@@ -553,15 +581,18 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             if (n_split <= 4) fold_rows(std::integral_constant<int, 4>());
             else fold_rows(std::integral_constant<int, 8>());
         }
+        __syncwarp();
         cluster.sync();   // every member's shared memory has been read: they may leave
     }
     __syncthreads();
     if (*sh_fail) {   // a wait gave up: report it and give copies still in flight one more bounded wait
         if (tid == 0) {
             set_status(p.status, SC_ERR_TIMEOUT);
-            const int issued = *sh_issued;
             if (nt > 0) mbar_wait(q_full, 0);
-            for (int t = max(issued - kStages, 0); t < issued; ++t) mbar_wait(kv_full0 + 8 * (t % kStages), (t / kStages) & 1);
+            for (int u = 0; u < 2; ++u) {
+                const int issued = sh_issued[u];
+                for (int t = max(issued - kStages, 0); t < issued; ++t) mbar_wait((u ? v_full0 : k_full0) + 8 * (t % kStages), (t / kStages) & 1);
+            }
         }
         __syncthreads();
     }
