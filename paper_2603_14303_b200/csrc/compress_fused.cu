@@ -24,9 +24,13 @@
 //      of one token are copied bit for bit; a sum that is not finite (0 * inf would reach other clusters) sends the sixteen
 //      clusters to a loop over their members.
 //
-// What bounds it: one launch over 32 layers x 8 heads x 32K tokens takes 1105 us on resident inputs (4.9 TB/s); copies
-// of the kernel with steps left out take 707 us (loads only), 834 (loads, steps 1 and 2) and 1025 (all but the
-// stores of the means), so step 3's shared-memory traffic and arithmetic are the largest part above the loads, then the stores.
+// What bounds it: the latency of a tile's serial steps, three tiles to an SM; an instruction of a warp takes 6 clocks (issue slots
+// 34 % used, tensor pipe 24 %, shared memory about half), so chains of dependent instructions count: four shift chains
+// instead of one in sim_word, four in the check of the sums and steps 1 and 2 of a short tile in line took 8 layers x 8 heads x 32K tokens
+// from 303 to 291 us (one launch per layer 117 -> 110 for two, chunks of 8 tokens 345 -> 333, of 128 508 -> 485).  Nothing may spill:
+// shared memory leaves the L1 cache 28 KB, a spilled word is a trip to L2, and variants with 4 to 80 bytes of stack lost 5 to 10 %.
+// Copies of an earlier form with steps left out, 32 layers on resident inputs, 1105 us: 707 (loads only), 834 (loads, steps 1 and 2), 1025
+// (all but the stores of the means).
 // A tile of 129..256 tokens spends 12 K cycles on step 2 and holds up the look-back of the tiles behind it.
 // Why these steps: one product per tile and decision rounds take 6.5 K warp instructions per 128 tokens, a warp per segment with
 // mma.sync tiles, the greedy pass and sums of member rows on the CUDA cores took 13 K: 32 layers 1395 us; 16 sequences x 16K,
@@ -147,20 +151,22 @@ __device__ __forceinline__ void umma_gram_block(uint32_t kbase, int hs, int mb, 
 }
 
 // Bits over 32 columns: bit c = (thr_c - G_c < 0), thr_c = norm_c * tni.  The sign of each difference is shifted in
-// behind the others, from the last column to the first; a difference of zero (Sim == tau) and one that is not a
+// behind the others, from the last column of a byte to the first; a difference of zero (Sim == tau) and one that is not a
 // number give no bit.
 __device__ __forceinline__ uint32_t sim_word(const uint32_t (&g)[32], const float* norm_c, float tni) {
-    uint32_t w = 0u;
+    uint32_t w[4] = {0u, 0u, 0u, 0u};   // a byte each: four chains of eight shifts side by side
     const float4* nc = reinterpret_cast<const float4*>(norm_c);
 #pragma unroll
-    for (int k4 = 7; k4 >= 0; --k4) {
-        const float4 nv = nc[k4];
-        const float n4[4] = {nv.x, nv.y, nv.z, nv.w};
+    for (int half = 1; half >= 0; --half)
 #pragma unroll
-        for (int k = 3; k >= 0; --k)
-            w = __funnelshift_l(__float_as_uint(fmaf(n4[k], tni, -__uint_as_float(g[k4 * 4 + k]))), w, 1);
-    }
-    return w;
+        for (int x = 0; x < 4; ++x) {
+            const float4 nv = nc[2 * x + half];
+            const float n4[4] = {nv.x, nv.y, nv.z, nv.w};
+#pragma unroll
+            for (int k = 3; k >= 0; --k)
+                w[x] = __funnelshift_l(__float_as_uint(fmaf(n4[k], tni, -__uint_as_float(g[x * 8 + half * 4 + k]))), w[x], 1);
+        }
+    return __byte_perm(__byte_perm(w[0], w[1], 0x0040), __byte_perm(w[2], w[3], 0x0040), 0x5410);
 }
 // A negative threshold: a zero-norm key has Sim = 0 > tau.
 __device__ __forceinline__ uint32_t sim_word_neg(const uint32_t (&g)[32], const float* norm_c, float tni) {
@@ -285,7 +291,7 @@ __device__ __forceinline__ float diagonal(const uint32_t (&g)[32], int lane) {
 // Steps 1 and 2 for a tile of up to 128 rows, thread i = row i (the product of its keys is complete).  `starts`: bit words of the
 // rows that start a segment.
 template <bool kAnyTau>
-__device__ __noinline__ int settle_short_tile(unsigned char* smem, const uint32_t* starts, int R, uint32_t tmem, uint32_t phase_u, float tau,
+__device__ __forceinline__ int settle_short_tile(unsigned char* smem, const uint32_t* starts, int R, uint32_t tmem, uint32_t phase_u, float tau,
                                                  bool wait_failed, int32_t* as, int row0, uint32_t* publish, int* sh_p) {
     float* norm = reinterpret_cast<float*>(smem + kNormOff);
     const int i = threadIdx.x, lane = i & 31, q = i >> 5;
@@ -464,14 +470,14 @@ __device__ __forceinline__ void pool_tile(unsigned char* smem, int hs, int P, __
                 mma_bf16(acc[t][3], a0, a1, a2, a3, b2, b3);
             }
         }
-        float check = 0.f;   // stays zero as long as every sum is finite
+        float check[4] = {0.f, 0.f, 0.f, 0.f};   // stay zero as long as every sum is finite
 #pragma unroll
         for (int t = 0; t < NT; ++t)
 #pragma unroll
             for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-                for (int x = 0; x < 4; ++x) check = fmaf(acc[t][nt][x], 0.f, check);
-        if (__any_sync(kFull, !(check == 0.f))) {
+                for (int x = 0; x < 4; ++x) check[x] = fmaf(acc[t][nt][x], 0.f, check[x]);
+        if (__any_sync(kFull, !((check[0] + check[1]) + (check[2] + check[3]) == 0.f))) {
             const int t_lo = k_lo * 16;
             pool_by_members(smem, hs, smem, NT > 1, m, n_multi, t_lo, t_hi, dst_k, room, warp, lane);
             if (NT > 1) pool_by_members(smem + kVOff, hs, smem, NT > 1, m, n_multi, t_lo, t_hi, dst_v, room, warp, lane);
