@@ -2,22 +2,26 @@
 // three kernels per layer -- GSC per segment, prefix sum of cluster counts per (b, head),
 // mean-pool merge per segment.  CUDA-core arithmetic in fp32; serves SC_F32 and is the
 // cross-check of the fused bf16 path.
-// One warp per segment; bounded by the latency of its loads, so all rows of a segment of up to 32 tokens are in flight at
-// once: clustering keeps them in registers for every seed, the merge adds them, eight at a time, to its clusters' sums in shared memory.
-// 8 heads x 8K tokens of fp32, chunks of 20 / 8 tokens (caches cold): clustering 43 / 34 us -> 29 / 20, merge 35 / 41 -> 30 / 31
-// against eight and four rows in flight, which longer segments, larger heads and segments of many clusters still
-// take (101 and 83 us with one row at a time).  Clustering: 128 registers of rows leave three blocks of four warps per SM; four blocks spill, +8 %.
+// One warp per segment, a block of its own (blocks of four warps ran as long as their longest segment, in two uneven waves: scheduler
+// partitions were busy 17 to 52 thousand of 62 thousand clocks; the whole path for 8 heads x 8K tokens 89.9 -> 85.3 us).
+// Bounded by the latency of its loads, so all rows of a segment of up to 32 tokens are in flight at
+// once: clustering keeps them in registers for every seed, the merge takes them in the order of their clusters, eight at a time.
+// 8 heads x 8K tokens of fp32, chunks of 20 / 8 tokens (caches cold): clustering 43 / 34 us -> 29 / 20
+// against eight and four rows in flight, which longer segments and larger heads still
+// take (101 us with one row at a time).  Clustering: 128 registers of rows leave three warps per scheduler; four spill, +8 %.
 // The eight lanes of a row group share out the sums of their rows (seven shuffles and one division for eight rows; with
-// 24 and eight, 34 / 39 us).  Merge: the rows in registers and a sum over them per cluster, 35 / 52 us.
+// 24 and eight, 34 / 39 us).  Merge: in cluster order a sum is one set of registers; added to the clusters' sums in shared memory
+// row by row (a load, an addition and a store that wait for one another) the path takes 85.8 us against 80.4; K and V of
+// a segment in one warp 82.4, and chunks of 128 tokens 280 against 250 (they leave too few warps).
 #include "common.cuh"
 
 namespace sc {
 
-constexpr int kGenWarps = 4;
-constexpr int kGenBlocks = 3;      // per SM (168 registers a thread): a short segment's rows are kept in registers
+constexpr int kGenWarps = 1;
+constexpr int kGenBlocks = 12;     // per SM (168 registers a thread): a short segment's rows are kept in registers
 constexpr int kShortSeg = 32;      // rows of a short segment (d <= 128)
-constexpr int kMergeSlots = 16;    // clusters of a short segment summed up in shared memory (8 KB per warp)
-constexpr int kMergeBlocks = 6;
+constexpr int kMergeRows = 8;     // rows of a short segment requested together
+constexpr int kMergeBlocks = 24;
 
 // Sums over the eight lanes of a row group: x[q] of every lane in, the sum for q = lane % R out (R = 8, 4, 2).
 template <int R>
@@ -210,8 +214,8 @@ scan_generic(int Hkv, const int32_t* __restrict__ seq_seg_off, int seg_stride,
 }
 
 // Eq. 3 for one segment of K or of V per warp: fp32 sums in token order, one divide, one rounding.  A lane owns four
-// columns (eight where d > 128).  Beyond 32 tokens, 16 clusters (8 KB of sums per warp, six blocks per SM) or 128
-// columns a cluster's members come from ballots over the segment's assignments, four rows requested together.
+// columns (eight where d > 128).  Beyond 32 tokens or 128 columns a cluster's members come from ballots over the segment's
+// assignments, four rows requested together.
 template <typename T, int kPer>
 __global__ void __launch_bounds__(kGenWarps * 32, kMergeBlocks)
 merge_generic(const T* __restrict__ K, const T* __restrict__ V, sc_strides st, int B, int Hkv, int n, int d,
@@ -219,7 +223,7 @@ merge_generic(const T* __restrict__ K, const T* __restrict__ V, sc_strides st, i
               const int32_t* __restrict__ assign, const int32_t* __restrict__ seg_core_off,
               T* __restrict__ core_k, T* __restrict__ core_v, int32_t* __restrict__ count, int cap) {
     constexpr int kWords = SC_MAX_CHUNK_LEN / 32;
-    __shared__ __align__(16) float4 sums[kGenWarps][kPer == 1 ? kMergeSlots : 1][32];
+    __shared__ uint8_t order[kGenWarps][32];
     in_stream_order();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int n_seg = min(*n_seg_p, seg_stride);
@@ -244,40 +248,48 @@ merge_generic(const T* __restrict__ K, const T* __restrict__ V, sc_strides st, i
             continue;
         }
         if constexpr (kPer == 1) {
-            const int own = lane < l ? as[lane] - r : -1;
-            const unsigned seeds = __ballot_sync(kFull, own == lane);
-            if (l <= kShortSeg && __popc(seeds) <= kMergeSlots) {
-                // rows in token order, eight requested together, each added to its cluster's sum in shared memory (a lane
-                // touches its own four columns only); a cluster's first row starts the sum
+            if (l <= kShortSeg) {
+                // the tokens in order of their clusters: place p of that order holds a token and whether it is its cluster's last
+                const int own = lane < l ? as[lane] - r : -1;
+                int before = 0, place = 0, last = 0;
+                for (unsigned todo = __ballot_sync(kFull, own == lane); todo; todo &= todo - 1) {
+                    const unsigned members = __ballot_sync(kFull, own == __ffs(todo) - 1);
+                    if ((members >> lane) & 1u) { place = before + __popc(members & ((1u << lane) - 1u)); last = members >> lane == 1u ? 32 : 0; }
+                    before += __popc(members);
+                }
+                if (lane < l) order[w][place] = (uint8_t)(lane | last);
+                __syncwarp();
+                const int at = order[w][lane];   // (places from l on are not used)
+                // rows in that order, eight requested together: a cluster's sum needs one register set, a first row starts it
                 const bool on = lane * 4 < d;
-                const int rank = __popc(seeds & ((1u << (own & 31)) - 1u));
-                for (int j0 = 0; j0 < l; j0 += 8) {
-                    float4 v[8];
+                float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+                int cnt = 0;
+                for (int p0 = 0; p0 < l; p0 += kMergeRows) {
+                    float4 v[kMergeRows];
 #pragma unroll
-                    for (int x = 0; x < 8; ++x) v[x] = on && j0 + x < l ? load4(rows + (int64_t)(j0 + x) * st.n) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int x = 0; x < kMergeRows; ++x) {
+                        const int token = __shfl_sync(kFull, at, (p0 + x) & 31) & 31;
+                        v[x] = on && p0 + x < l ? load4(rows + (int64_t)token * st.n) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
 #pragma unroll
-                    for (int x = 0; x < 8; ++x) {
-                        if (j0 + x >= l) break;
-                        float4* to = &sums[w][__shfl_sync(kFull, rank, j0 + x)][lane];
-                        if (!((seeds >> (j0 + x)) & 1u)) {
-                            const float4 t = *to;
-                            v[x].x += t.x; v[x].y += t.y; v[x].z += t.z; v[x].w += t.w;
+                    for (int x = 0; x < kMergeRows; ++x) {
+                        if (p0 + x >= l) break;
+                        sum = cnt == 0 ? v[x] : make_float4(sum.x + v[x].x, sum.y + v[x].y, sum.z + v[x].z, sum.w + v[x].w);
+                        ++cnt;
+                        if (!(__shfl_sync(kFull, at, (p0 + x) & 31) & 32)) continue;
+                        if (row < cap) {
+                            if (cnt > 1) {
+                                const float fc = (float)cnt;
+                                sum = make_float4(sum.x / fc, sum.y / fc, sum.z / fc, sum.w / fc);
+                            }
+                            if (on) store4(cores + (int64_t)row * d, sum);
+                            if (lane == 0 && !is_v) count[obase + row] = cnt;
                         }
-                        *to = v[x];
+                        cnt = 0;
+                        ++row;
                     }
                 }
-                int c = 0;
-                for (unsigned todo = seeds; todo; todo &= todo - 1, ++c, ++row) {
-                    const int cnt = __popc(__ballot_sync(kFull, own == __ffs(todo) - 1));
-                    if (row >= cap) break;
-                    float4 v = sums[w][c][lane];
-                    if (cnt > 1) {
-                        const float fc = (float)cnt;
-                        v = make_float4(v.x / fc, v.y / fc, v.z / fc, v.w / fc);
-                    }
-                    if (on) store4(cores + (int64_t)row * d, v);
-                    if (lane == 0 && !is_v) count[obase + row] = cnt;
-                }
+                __syncwarp();   // the order is read: the next segment's may be written
                 continue;
             }
         }
@@ -350,7 +362,7 @@ static cudaError_t run(const CompressArgs& a, cudaStream_t st) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int grid = sms * 16;
+    const int grid = sms * 64;
     auto gsc = a.d <= 128 ? gsc_generic<T, 4> : gsc_generic<T, 8>;
     cudaError_t e = launch_in_order(gsc, dim3(grid), kGenWarps * 32, 0, st, (const T*)a.K, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off,
                                     a.n_seg, seg_stride, a.tau, a.tau_dev, a.skip, assign, seg_p);

@@ -1,16 +1,16 @@
 // Generic decode path for Eq. 4 (any dtype, d <= 256 multiple of 8).  One block serves one (sequence, KV head, split of
-// its cores, up to four of its query heads); its four warps take 32-row tiles in turn: eight lanes per row form the
+// its cores, up to four of its query heads); its eight warps take 32-row tiles in turn: eight lanes per row form the
 // scores (four rows at a time, sixteen requested ahead), one lane per row takes part in the online softmax in
 // fp32, and for the weighted sum a lane owns four columns of every row, sixteen rows requested together.  A second kernel combines the splits in order.
 // Serves SC_F32 and cross-checks the tensor-core bf16 kernel.
 // Bounded by the latency of its loads: 2162 cores x 8 heads of fp32, 16 splits: 217 + 18 us when a warp served one query
-// head row by row (each row a dependent chain of load, five shuffles and two exponentials), 19 + 7 us like this (37 + 7 with
-// eight rows requested at a time).
+// head row by row (each row a dependent chain of load, five shuffles and two exponentials), 14 + 7 us like this (20 + 7 with
+// four warps, of which one had two tiles; 37 + 7 with eight rows requested at a time).
 #include "common.cuh"
 
 namespace sc {
 
-constexpr int kDecWarps = 4;
+constexpr int kDecWarps = 8;
 constexpr int kDecHeads = 4;    // query heads per block
 constexpr int kDecMaxD = 256;
 
@@ -21,7 +21,7 @@ __host__ __device__ inline int generic_splits(int cap) {
 
 // NC: the most 32-column pieces a row has (4 or 8).
 template <typename T, int NC>
-__global__ void __launch_bounds__(kDecWarps * 32)
+__global__ void __launch_bounds__(kDecWarps * 32, 1)
 decode_generic(const T* __restrict__ q, int Hq, int Hkv, int d, const T* __restrict__ core_k,
                const T* __restrict__ core_v, const int32_t* __restrict__ count, int cap,
                const int32_t* __restrict__ core_len, float scale_log2, int n_split, float* __restrict__ part) {
