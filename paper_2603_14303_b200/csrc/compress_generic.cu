@@ -40,6 +40,14 @@ __device__ __forceinline__ float group_sums(float (&x)[R], int lane) {
     return x[0];
 }
 
+// A vote of lanes that decide for row (their group of eight) R + lane % R, as bits by row.
+template <int R>
+__device__ __forceinline__ unsigned by_row(unsigned votes) {
+    if (R == 4) return (votes & 15u) | ((votes >> 4) & 0xf0u) | ((votes >> 8) & 0xf00u) | ((votes >> 12) & 0xf000u);
+    if (R == 2) return (votes & 3u) | ((votes >> 6) & 12u) | ((votes >> 12) & 48u) | ((votes >> 18) & 192u);
+    return votes;
+}
+
 // Algorithm 1 for a segment of at most 4 R rows: all of them are requested at once and stay in registers, R per group of
 // eight lanes; only the seeds' rows are read again.  A lane decides for row (its group) R + lane % R.  Same sums in the
 // same order as the loop for longer ones.
@@ -68,10 +76,7 @@ __device__ __forceinline__ int short_segment(int l, float tau, int32_t* as, int 
         for (int q = 0; q < R; ++q) x[q] = dot(seed, v[q]);
         const float prod = group_sums<R>(x, lane);
         const float sim = (ni == 0.f || nj == 0.f) ? 0.f : prod / (ni * nj);
-        unsigned hits = __ballot_sync(kFull, sim > tau);   // group g's rows in byte g
-        if (R == 4) hits = (hits & 15u) | ((hits >> 4) & 0xf0u) | ((hits >> 8) & 0xf00u) | ((hits >> 12) & 0xf000u);
-        if (R == 2) hits = (hits & 3u) | ((hits >> 6) & 12u) | ((hits >> 12) & 48u) | ((hits >> 18) & 192u);
-        hits &= open;
+        const unsigned hits = by_row<R>(__ballot_sync(kFull, sim > tau)) & open;
         if ((hits >> lane) & 1u) mine = i;
         open &= ~hits;
     }
@@ -127,17 +132,19 @@ gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d
                 continue;
             }
         }
-        for (int j0 = 0; j0 < l; j0 += 8) {
-            float4 v0[NC], v1[NC];
-            load_row(j0 + rsub, j0 + rsub < l, v0);
-            load_row(j0 + 4 + rsub, j0 + 4 + rsub < l, v1);
-            float d0 = dot(v0, v0), d1 = dot(v1, v1);
+        // longer: kRows rows at a time; a lane decides for row j0 + row_of (in pairs of lanes, or fours)
+        constexpr int R = NC == 4 ? 4 : 2, kRows = 4 * R;
+        const int row_of = rsub * R + lane % R;
+        const bool speaks = sub < R;   // one lane of those that decide for the same row
+        for (int j0 = 0; j0 < l; j0 += kRows) {
+            float4 v[R][NC];
+            float x[R];
 #pragma unroll
-            for (int o = 1; o < 8; o <<= 1) { d0 += __shfl_xor_sync(kFull, d0, o); d1 += __shfl_xor_sync(kFull, d1, o); }
-            if (sub == 0) {
-                if (j0 + rsub < l) norms[w][j0 + rsub] = sqrtf(d0);
-                if (j0 + 4 + rsub < l) norms[w][j0 + 4 + rsub] = sqrtf(d1);
-            }
+            for (int q = 0; q < R; ++q) load_row(j0 + rsub * R + q, j0 + rsub * R + q < l, v[q]);
+#pragma unroll
+            for (int q = 0; q < R; ++q) x[q] = dot(v[q], v[q]);
+            const float nn = group_sums<R>(x, lane);
+            if (speaks && j0 + row_of < l) norms[w][j0 + row_of] = sqrtf(nn);
         }
         __syncwarp();
         unsigned word = 0;  // lane c holds the assigned bits of tokens 32c .. 32c+31
@@ -152,29 +159,22 @@ gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d
             float4 seed[NC];
             load_row(i, true, seed);
             const float ni = norms[w][i];
-            for (int j0 = (i + 1) & ~7; j0 < l; j0 += 8) {   // eight tokens of one word
-                const unsigned open = (~__shfl_sync(kFull, word, j0 >> 5)) >> (j0 & 31);
-                const bool on0 = j0 + rsub > i && j0 + rsub < l && ((open >> rsub) & 1u);
-                const bool on1 = j0 + 4 + rsub > i && j0 + 4 + rsub < l && ((open >> (4 + rsub)) & 1u);
-                if (!__any_sync(kFull, on0 || on1)) continue;
-                float4 v0[NC], v1[NC];
-                load_row(j0 + rsub, on0, v0);
-                load_row(j0 + 4 + rsub, on1, v1);
-                float d0 = dot(seed, v0), d1 = dot(seed, v1);
+            for (int j0 = (i + 1) & ~(kRows - 1); j0 < l; j0 += kRows) {   // kRows tokens of one word
+                unsigned open = (~__shfl_sync(kFull, word, j0 >> 5)) >> (j0 & 31) & ((1u << kRows) - 1u);
+                if (j0 <= i) open &= ~0u << (i + 1 - j0);
+                if (l - j0 < kRows) open &= (1u << (l - j0)) - 1u;
+                if (open == 0u) continue;
+                float4 v[R][NC];
+                float x[R];
 #pragma unroll
-                for (int o = 1; o < 8; o <<= 1) { d0 += __shfl_xor_sync(kFull, d0, o); d1 += __shfl_xor_sync(kFull, d1, o); }
-                const float n0 = on0 ? norms[w][j0 + rsub] : 0.f, n1 = on1 ? norms[w][j0 + 4 + rsub] : 0.f;
-                const float s0 = (ni == 0.f || n0 == 0.f) ? 0.f : d0 / (ni * n0);
-                const float s1 = (ni == 0.f || n1 == 0.f) ? 0.f : d1 / (ni * n1);
-                const bool hit0 = on0 && s0 > tau, hit1 = on1 && s1 > tau;
-                const unsigned b0 = __ballot_sync(kFull, hit0) & 0x01010101u, b1 = __ballot_sync(kFull, hit1) & 0x01010101u;
-                const unsigned hits = ((b0 | (b0 >> 7) | (b0 >> 14) | (b0 >> 21)) & 15u) |
-                                      (((b1 | (b1 >> 7) | (b1 >> 14) | (b1 >> 21)) & 15u) << 4);
+                for (int q = 0; q < R; ++q) load_row(j0 + rsub * R + q, (open >> (rsub * R + q)) & 1u, v[q]);
+#pragma unroll
+                for (int q = 0; q < R; ++q) x[q] = dot(seed, v[q]);
+                const float prod = group_sums<R>(x, lane), nj = j0 + row_of < l ? norms[w][j0 + row_of] : 0.f;
+                const float sim = (ni == 0.f || nj == 0.f) ? 0.f : prod / (ni * nj);
+                const unsigned hits = by_row<R>(__ballot_sync(kFull, sim > tau)) & open;
                 if (lane == (j0 >> 5)) word |= hits << (j0 & 31);
-                if (sub == 0) {
-                    if (hit0) as[j0 + rsub] = r + i;
-                    if (hit1) as[j0 + 4 + rsub] = r + i;
-                }
+                if (speaks && ((hits >> row_of) & 1u)) as[j0 + row_of] = r + i;
             }
         }
         if (lane == 0) seg_p[(int64_t)h * seg_stride + s] = p;
