@@ -7,8 +7,7 @@
 // Bounded by the latency of its loads, so all rows of a segment of up to 32 tokens are in flight at
 // once: clustering keeps them in registers for every seed, the merge takes them in the order of their clusters, eight at a time.
 // 8 heads x 8K tokens of fp32, chunks of 20 / 8 tokens (caches cold): clustering 43 / 34 us -> 29 / 20
-// against eight and four rows in flight, which longer segments and larger heads still
-// take (101 us with one row at a time).  Clustering: 128 registers of rows leave three warps per scheduler; four spill, +8 %.
+// against eight and four rows in flight (101 us with one row at a time).  Clustering: 128 registers of rows leave three warps per scheduler; four spill, +8 %.
 // The eight lanes of a row group share out the sums of their rows (seven shuffles and one division for eight rows; with
 // 24 and eight, 34 / 39 us).  Merge: in cluster order a sum is one set of registers; added to the clusters' sums in shared memory
 // row by row (a load, an addition and a store that wait for one another) the path takes 85.8 us against 80.4; K and V of
@@ -84,9 +83,10 @@ __device__ __forceinline__ int short_segment(int l, float tau, int32_t* as, int 
     return p;
 }
 
-// Algorithm 1 for one segment per warp.  Longer segments' rows are read straight from global memory, eight at a time: lanes 8r .. 8r + 7
-// form the product of row r (of four) with the seed's row, which they hold in registers.  NC: the most 32-column pieces
-// a row has (4 or 8).
+// Algorithm 1 for one segment per warp.  Longer segments' rows are read straight from global memory, 32 at a time (16 where d > 128),
+// eight lanes a row, against the seed's row, which they hold in registers; rows already assigned are not read.  The whole path for
+// 8 heads x 8K tokens of fp32 in chunks of 128: eight rows at a time 250 us, sixteen 200, 32 178; of 60: 169, 148, 139.  NC: the
+// most 32-column pieces a row has (4 or 8).
 template <typename T, int NC>
 __global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks)
 gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d,
@@ -133,7 +133,7 @@ gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d
             }
         }
         // longer: kRows rows at a time; a lane decides for row j0 + row_of (in pairs of lanes, or fours)
-        constexpr int R = NC == 4 ? 4 : 2, kRows = 4 * R;
+        constexpr int R = NC == 4 ? 8 : 4, kRows = 4 * R;
         const int row_of = rsub * R + lane % R;
         const bool speaks = sub < R;   // one lane of those that decide for the same row
         for (int j0 = 0; j0 < l; j0 += kRows) {
@@ -160,7 +160,7 @@ gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d
             load_row(i, true, seed);
             const float ni = norms[w][i];
             for (int j0 = (i + 1) & ~(kRows - 1); j0 < l; j0 += kRows) {   // kRows tokens of one word
-                unsigned open = (~__shfl_sync(kFull, word, j0 >> 5)) >> (j0 & 31) & ((1u << kRows) - 1u);
+                unsigned open = (~__shfl_sync(kFull, word, j0 >> 5)) >> (j0 & 31) & (0xffffffffu >> (32 - kRows));
                 if (j0 <= i) open &= ~0u << (i + 1 - j0);
                 if (l - j0 < kRows) open &= (1u << (l - j0)) - 1u;
                 if (open == 0u) continue;
