@@ -263,25 +263,33 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, tig = lane & 3;
     const int G = Hq / Hkv;
-    // An ordinary launch waits here for the kernel before it.  Under an overlapped one the next kernel may start beside
-    // this one, and whatever this block reads before its own griddepcontrol.wait below (core_len, cores, counts) must not
-    // be written by a kernel that may still be running then; that is the caller's promise when it asks for one.
-    if (mode == kOrdinary) asm volatile("griddepcontrol.wait;\n" ::: "memory");
-    // Where there are spare units the next kernel is let in only when they have gone: its blocks would find both slots of some
-    // SMs taken by them, and settle unevenly (128 raw heads x 8 K rows: 80 us, 92 with the next kernel let in at once).
-    if (!kSpares) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    // Block r of the cluster folds slice r of the head's (head, column) pairs, [e_lo, e_hi), and
-    // is handed that slice by every block (see the fold).
+    // Block r of the cluster folds slice r of the head's (head, column) pairs, [e_lo, e_hi), and is handed that slice by every
+    // block (see the fold).
     const int csize = (int)cg::this_cluster().num_blocks(), crank = (int)cg::this_cluster().block_rank();
     const int slice = (G * (kD / 4) + csize - 1) / csize;
     const int e_lo = min(crank * slice, G * (kD / 4)), e_hi = min(e_lo + slice, G * (kD / 4));
-    if (threadIdx.x == 0) {
-        umma::mbar_init(smem_u32(&sh_bar), 1);
-        umma::mbar_fence_init();
-        umma::mbar_expect_tx(smem_u32(&sh_bar), (uint32_t)(csize * ((e_hi - e_lo) * 16 + 64)));   // (m and l come to a block without a slice too)
+    const auto set_up = [&] {
+        if (threadIdx.x == 0) {
+            umma::mbar_init(smem_u32(&sh_bar), 1);
+            umma::mbar_fence_init();
+            umma::mbar_expect_tx(smem_u32(&sh_bar), (uint32_t)(csize * ((e_hi - e_lo) * 16 + 64)));   // (m and l come to a block without a slice too)
+        }
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");   // (the wait is in front of the first access to another block's shared memory)
+    };
+    // An ordinary launch waits here for the kernel before it.  Under an overlapped one the next kernel may start beside
+    // this one, and whatever this block reads before its own griddepcontrol.wait below (core_len, cores, counts) must not
+    // be written by a kernel that may still be running then; that is the caller's promise when it asks for one.  An ordinary
+    // launch sets its barrier up before it waits (200 calls over 8 x 0.5 K rows from a graph 4.13 -> 3.72 us each, 4.32 when
+    // the fold read the members' shared memory), an overlapped one lets the next kernel in first (32 dependent layers 325, 332 the other way).
+    if (mode == kOrdinary) {
+        set_up();
+        asm volatile("griddepcontrol.wait;\n" ::: "memory");
     }
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory");   // (the wait is in front of the first access to another block's shared memory)
+    // Where there are spare units the next kernel is let in only when they have gone: its blocks would find both slots of some
+    // SMs taken by them, and settle unevenly (128 raw heads x 8 K rows: 80 us, 92 with the next kernel let in at once).
+    if (!kSpares) asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
+    if (mode != kOrdinary) set_up();
     // the block's head, and its place among the head's blocks
     int bh = blockIdx.z * Hkv + blockIdx.y, split = blockIdx.x, n_split = gridDim.x;   // as if every head had one unit
     Units u = {bh, 0, 0};
