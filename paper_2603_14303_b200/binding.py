@@ -290,14 +290,17 @@ def sc_compress_global(K, V, tau, core_k, core_v, count, core_len, workspace, as
 
 def sc_decode_attn(q, core_k, core_v, count, core_len, out, workspace, scale=0.0, status=None, flags=0):
     """Raw sc_decode_attn for one layer and one decode step."""
-    _need_cuda(q, core_k, core_v, count, core_len, out, workspace)
+    if not (q.is_cuda and core_k.is_cuda and core_v.is_cuda and core_len.is_cuda and out.is_cuda and workspace.is_cuda
+            and (count is None or count.is_cuda)):   # (a call is short of 4 us on the device: in line, 0.3 us less than a loop)
+        raise ValueError("device tensors required")
     B, Hq, d = q.shape
     _, Hkv, cap, _ = core_k.shape
     assert q.is_contiguous() and out.is_contiguous() and core_k.is_contiguous() and core_v.is_contiguous()
     code = _native().decode_attn(q.data_ptr(), _dt(q), B, Hq, Hkv, d, core_k.data_ptr(), core_v.data_ptr(), _ptr(count), cap,
                                  core_len.data_ptr(), float(scale), int(flags), out.data_ptr(), workspace.data_ptr(),
-                                 _bytes(workspace), _ptr(status), _stream(q))
-    _check("sc_decode_attn", code)
+                                 workspace.nbytes, _ptr(status), _stream(q))
+    if code != SC_OK:
+        raise ScError("sc_decode_attn", code)
 
 
 def sc_prefill_attn(q, core_k, core_v, count, core_len, out, scale=0.0, status=None, flags=0):
@@ -502,11 +505,11 @@ def decode_workspace(B, Hq, Hkv, d, cap, device) -> torch.Tensor:
 def decode_attn(q, layer: CompressedLayer, out=None, workspace=None, scale: float = 0.0, status=None, flags=0,
                 use_count: bool = True):
     """One decode step of Proportional Attention over one layer's cores."""
-    B, Hq, d = q.shape
-    _, Hkv, cap, _ = layer.core_k.shape
     if out is None:
         out = torch.empty_like(q)
     if workspace is None:
+        B, Hq, d = q.shape
+        _, Hkv, cap, _ = layer.core_k.shape
         workspace = decode_workspace(B, Hq, Hkv, d, cap, q.device)
     sc_decode_attn(q, layer.core_k, layer.core_v, layer.count if use_count else None, layer.core_len, out,
                    workspace, scale, status, flags)
