@@ -10,7 +10,7 @@
 //      memory (the 128-byte-swizzled layout the TMA boxes wrote is the K-major operand layout; three such products, one
 //      after the other, for a tile of 129..256 tokens).  Thread i owns row i; it reads only the columns its warp's rows
 //      can need and keeps, as bits in registers, which EARLIER tokens of its segment it is similar to (Sim > tau decided as
-//      |k_c| (tau |k_i|) - G < 0: one fma and one funnel shift that collects its sign per pair).
+//      |k_c| (tau |k_i|) - G < 0: half an instruction of two fmas and one funnel shift that collects its sign per pair).
 //   2. Algorithm 1 for all rows at once, in rounds: a row with an earlier neighbour that is a seed is a member, a row
 //      whose earlier neighbours are all members is a seed.  Both facts are final once true, the lowest open row is
 //      decided in every round, so the rounds end and give exactly the sequential pass's partition; chunks that are unions
@@ -137,10 +137,11 @@ __device__ __forceinline__ bool team_any(bool mine) {
     return out != 0u;
 }
 
-// One 128 x 128 block of K.K^T of the staged keys: rows of 128-row block mb against rows of block nb (column halves `hs` bytes
+// One 128 x 128 block of -K.K^T of the staged keys (the product negates its first operand, so that sim_word adds pairs of
+// accumulators to its products: the two-at-a-time fma takes no negated operand): rows of 128-row block mb against rows of block nb (column halves `hs` bytes
 // apart).  One thread issues the eight instructions; the mbarrier gets one arrival when they are complete.
 __device__ __forceinline__ void umma_gram_block(uint32_t kbase, int hs, int mb, int nb, uint32_t tmem, uint32_t bar) {
-    constexpr uint32_t idesc = umma::instr_desc_bf16(128, 128, false, false);
+    constexpr uint32_t idesc = umma::instr_desc_bf16(128, 128, false, false, true);
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
         const uint32_t off = (ks >> 2) * hs + (ks & 3) * 32;
@@ -150,10 +151,11 @@ __device__ __forceinline__ void umma_gram_block(uint32_t kbase, int hs, int mb, 
     umma::mma_commit(bar);
 }
 
-// Bits over 32 columns: bit c = (thr_c - G_c < 0), thr_c = norm_c * tni.  The sign of each difference is shifted in
+// Bits over 32 columns: bit c = (thr_c - G_c < 0), thr_c = norm_c * tni; g holds -G.  The sign of each difference is shifted in
 // behind the others, from the last column of a byte to the first; a difference of zero (Sim == tau) and one that is not a
-// number give no bit.
-__device__ __forceinline__ uint32_t sim_word(const uint32_t (&g)[32], const float* norm_c, float tni) {
+// number give no bit.  Two differences per instruction: 4 x 64K in chunks of 128, two layers, 553 -> 521 us (chunks of 20: the same).
+__device__ __forceinline__ uint32_t sim_word(const uint32_t (&g)[32], const float* norm_c, float tni1) {
+    const float2 tni = make_float2(tni1, tni1);
     uint32_t w[4] = {0u, 0u, 0u, 0u};   // a byte each: four chains of eight shifts side by side
     const float4* nc = reinterpret_cast<const float4*>(norm_c);
 #pragma unroll
@@ -161,10 +163,13 @@ __device__ __forceinline__ uint32_t sim_word(const uint32_t (&g)[32], const floa
 #pragma unroll
         for (int x = 0; x < 4; ++x) {
             const float4 nv = nc[2 * x + half];
-            const float n4[4] = {nv.x, nv.y, nv.z, nv.w};
-#pragma unroll
-            for (int k = 3; k >= 0; --k)
-                w[x] = __funnelshift_l(__float_as_uint(fmaf(n4[k], tni, -__uint_as_float(g[x * 8 + half * 4 + k]))), w[x], 1);
+            const uint32_t* gk = g + x * 8 + half * 4;
+            const float2 hi = umma::fma2(make_float2(nv.z, nv.w), tni, make_float2(__uint_as_float(gk[2]), __uint_as_float(gk[3])));
+            const float2 lo = umma::fma2(make_float2(nv.x, nv.y), tni, make_float2(__uint_as_float(gk[0]), __uint_as_float(gk[1])));
+            w[x] = __funnelshift_l(__float_as_uint(hi.y), w[x], 1);
+            w[x] = __funnelshift_l(__float_as_uint(hi.x), w[x], 1);
+            w[x] = __funnelshift_l(__float_as_uint(lo.y), w[x], 1);
+            w[x] = __funnelshift_l(__float_as_uint(lo.x), w[x], 1);
         }
     return __byte_perm(__byte_perm(w[0], w[1], 0x0040), __byte_perm(w[2], w[3], 0x0040), 0x5410);
 }
@@ -174,7 +179,7 @@ __device__ __forceinline__ uint32_t sim_word_neg(const uint32_t (&g)[32], const 
 #pragma unroll
     for (int k = 0; k < 32; ++k) {
         const float thr = norm_c[k] * tni;
-        w |= (__uint_as_float(g[k]) > thr || thr == 0.f ? 1u : 0u) << k;
+        w |= (-__uint_as_float(g[k]) > thr || thr == 0.f ? 1u : 0u) << k;
     }
     return w;
 }
@@ -274,7 +279,7 @@ __device__ __forceinline__ int settle_rows(const uint32_t (&e)[NR][4 * NR], cons
     return P;
 }
 
-// The diagonal of a diagonal block = squared norms: thread (warp q, lane) owns row 32 q + lane of the block.  `g` holds the
+// The diagonal of a diagonal block = squared norms, negated (a key without length: zero of either sign): thread (warp q, lane) owns row 32 q + lane of the block.  `g` holds the
 // 32 columns of the warp's own rows; this lane's element is picked by the bits of the lane number.
 __device__ __forceinline__ float diagonal(const uint32_t (&g)[32], int lane) {
     uint32_t t[16];
@@ -319,7 +324,7 @@ __device__ __forceinline__ int settle_short_tile(unsigned char* smem, const uint
     uint32_t g[32];
     umma::tmem_ld32(lane_addr + q * 32, g);   // the columns of the warp's own rows
     umma::tmem_ld_wait();
-    norm[i] = sqrtf(diagonal(g, lane));
+    norm[i] = sqrtf(fabsf(diagonal(g, lane)));
     const bool act[1] = {i < R};
     if (team_any(wait_failed)) return -1;   // (the norms are in place)
     const float tni = tau * norm[i];
@@ -372,7 +377,7 @@ __device__ __noinline__ int settle_long_tile(unsigned char* smem, int R, uint32_
         if (mb == nb) {
             umma::tmem_ld32(lane_addr + q * 32, g);
             umma::tmem_ld_wait();
-            norm[i] = sqrtf(diagonal(g, lane));
+            norm[i] = sqrtf(fabsf(diagonal(g, lane)));
             if (team_any(wait_failed)) return -1;   // (the norms are in place)
         }
         const float tni = tau * norm[i];

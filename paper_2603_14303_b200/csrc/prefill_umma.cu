@@ -128,13 +128,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
     asm("max.f32 %0, %1, %2, %3;\n" : "=f"(y) : "f"(a), "f"(b), "f"(c));
     return y;
 }
-// Two fp32 operations per instruction.
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-    float2 y;
-    asm("{\n.reg .b64 a, b, c, y;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nmov.b64 c, {%6, %7};\nfma.rn.f32x2 y, a, b, c;\nmov.b64 {%0, %1}, y;\n}\n"
-        : "=f"(y.x), "=f"(y.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return y;
-}
 __device__ __forceinline__ float2 add2(float2 a, float2 b) {
     float2 y;
     asm("{\n.reg .b64 a, b, y;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nadd.rn.f32x2 y, a, b;\nmov.b64 {%0, %1}, y;\n}\n"

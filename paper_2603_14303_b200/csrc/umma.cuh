@@ -98,11 +98,18 @@ __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t saddr, uint32_t lbo
     d |= 2ull << 61;
     return d;
 }
+// Two fp32 operations per instruction.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 y;
+    asm("{\n.reg .b64 a, b, c, y;\nmov.b64 a, {%2, %3};\nmov.b64 b, {%4, %5};\nmov.b64 c, {%6, %7};\nfma.rn.f32x2 y, a, b, c;\nmov.b64 {%0, %1}, y;\n}\n"
+        : "=f"(y.x), "=f"(y.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return y;
+}
 // Instruction descriptor for kind::f16 with bf16 operands and fp32 accumulation.
-// Bits: [4,6) accumulator format (1 = f32), [7,10) A format (1 = bf16), [10,13) B format, [15] A is MN-major,
+// Bits: [4,6) accumulator format (1 = f32), [7,10) A format (1 = bf16), [10,13) B format, [13] A negated, [15] A is MN-major,
 // [16] B is MN-major, [17,23) N >> 3, [24,29) M >> 4.
-__host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N, bool a_mn_major, bool b_mn_major) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn_major ? 1u : 0u) << 15) | ((b_mn_major ? 1u : 0u) << 16) |
+__host__ __device__ constexpr uint32_t instr_desc_bf16(int M, int N, bool a_mn_major, bool b_mn_major, bool a_negated = false) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((a_negated ? 1u : 0u) << 13) | ((a_mn_major ? 1u : 0u) << 15) | ((b_mn_major ? 1u : 0u) << 16) |
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
