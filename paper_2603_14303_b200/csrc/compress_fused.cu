@@ -25,7 +25,7 @@
 //      clusters to a loop over their members.
 //
 // What bounds it: the latency of a tile's serial steps, three tiles to an SM; an instruction of a warp takes 6 clocks (issue slots
-// 34 % used, tensor pipe 24 %, shared memory about half), so chains of dependent instructions count: four shift chains
+// 36 % used, tensor pipe 27 %, shared memory about half), so chains of dependent instructions count: four shift chains
 // instead of one in sim_word, four in the check of the sums and steps 1 and 2 of a short tile in line took 8 layers x 8 heads x 32K tokens
 // from 303 to 291 us (one launch per layer 117 -> 110 for two, chunks of 8 tokens 345 -> 333, of 128 508 -> 485).  Nothing may spill:
 // shared memory leaves the L1 cache 28 KB, a spilled word is a trip to L2, and variants with 4 to 80 bytes of stack lost 5 to 10 %.
