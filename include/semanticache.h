@@ -308,6 +308,7 @@ SC_API sc_status sc_compress_global(const void* K, const void* V, sc_strides kv_
  *   workspace  at least sc_decode_workspace_bytes(B, Hq, Hkv, d, cap) bytes.  It holds the
  *              split partials and a few arrival counters; the counters must be zero on entry
  *              and are left zero on exit, so zero the workspace once after allocating it.
+ *   status     SC_ERR_TIMEOUT if a bounded wait inside the kernel gave up; the outputs it was for are not a number then
  */
 SC_API size_t sc_decode_workspace_bytes(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t cap);
 

@@ -25,8 +25,7 @@
 
 #include <mutex>
 
-#include "common.cuh"
-#include "umma.cuh"
+#include "decode_fold.cuh"
 
 namespace sc {
 
@@ -50,7 +49,6 @@ constexpr int kPartStride = 8 * kD + 16;        // floats per (b, h, split): acc
 constexpr int kCtasPerSm = 2;                   // two kernels (consecutive layers) can be co-resident
 constexpr float kMaxSlack = 8.f;                // log2 units a score may exceed the running maximum before it is raised
 constexpr int kMergeGroup = 16;                 // cluster partials folded per round by the merging block
-constexpr int kMaxCluster = 16;                 // blocks per cluster (more than 8 needs the non-portable opt-in)
 constexpr int kCapRowsPerBlock = 1408;          // rows of capacity per block from which a head gets another cluster (heads are usually half full or less)
 constexpr int kMaxSlots = 160;                  // partials in global memory over the launch's own units (at least one per head)
 constexpr int kMaxTickets = 512;                // heads of a launch whose blocks may meet through global memory
@@ -62,11 +60,6 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int sr
 }
 __device__ __forceinline__ void cp_async4(uint32_t dst, const void* src, int src_bytes) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ uint32_t mapa(uint32_t addr, int rank) {
-    uint32_t a;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(addr), "r"(rank));
-    return a;
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
@@ -97,11 +90,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 }
 __device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
-__device__ __forceinline__ float fast_exp2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
-    return y;
-}
 __device__ __forceinline__ float fast_log2(float x) {
     float y;
     asm("lg2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
@@ -485,8 +473,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
         }
         const int to = e4 / slice;
         const uint32_t bar_to = mapa(smem_u32(&sh_bar), to), dst = mapa(smem_u32(recv_o + crank * slice + (e4 - to * slice)), to);
-        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];\n"
-                     ::"r"(dst), "r"(__float_as_uint(acc.x)), "r"(__float_as_uint(acc.y)), "r"(__float_as_uint(acc.z)), "r"(__float_as_uint(acc.w)), "r"(bar_to) : "memory");
+        hand_over(dst, bar_to, acc);
     }
     for (int x = threadIdx.x; x < csize * 8; x += kWarps * 32) {
         const int hd = x & 7;
@@ -499,8 +486,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
             bl += (mw == -INFINITY) ? 0.f : sh_l[w2][hd] * fast_exp2(mw - bm);
         }
         const uint32_t bar_to = mapa(smem_u32(&sh_bar), x >> 3), dst = mapa(smem_u32(recv_ml + crank * 16 + hd * 2), x >> 3);
-        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];\n"
-                     ::"r"(dst), "r"(__float_as_uint(bm)), "r"(__float_as_uint(bl)), "r"(bar_to) : "memory");
+        hand_over(dst, bar_to, bm, bl);
     }
     const int n_clusters = n_split / csize, cidx = split / csize;   // clusters of the head, this one's index
     // partials: every head's own unit in turn, then the spare units; a unit leaves one for each of its clusters
@@ -509,7 +495,7 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     float* my_part = part + (size_t)(cidx + (!kSpares || cidx < per_unit ? first : more - per_unit)) * kPartStride;
     const bool direct = n_clusters == 1;   // this cluster holds the whole head: its fold is the result
     if (direct && warp > 0 && e_lo + warp * 32 >= e_hi) return;   // nothing to fold for this warp (one stays until all has arrived)
-    const bool got = umma::mbar_wait<true>(smem_u32(&sh_bar), 0);
+    const bool got = slices_arrived(smem_u32(&sh_bar));
     // Nothing has been written to global memory so far (the block partials live in shared memory).  Under
     // an overlapped launch every global write of this kernel (out, cluster partials, arrival counters) is
     // ordered behind the completion of the kernel before it, which ordered its own writes behind its
@@ -519,40 +505,24 @@ decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __
     if (!got) set_status(status, SC_ERR_TIMEOUT);
     for (int e4 = e_lo + threadIdx.x; e4 < e_hi; e4 += kWarps * 32) {
         const int hd = e4 / (kD / 4), d4 = (e4 % (kD / 4)) * 4;
-        float mv[kMaxCluster], lv[kMaxCluster];
-        float4 ov[kMaxCluster];
-#pragma unroll
-        for (int j = 0; j < kMaxCluster; ++j) {
-            mv[j] = j < csize ? recv_ml[j * 16 + 2 * hd] : -INFINITY;
-            lv[j] = j < csize ? recv_ml[j * 16 + 2 * hd + 1] : 0.f;
-            ov[j] = j < csize ? recv_o[j * slice + e4 - e_lo] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        float gm = mv[0];
-#pragma unroll
-        for (int j = 1; j < kMaxCluster; ++j) gm = fmaxf(gm, mv[j]);
-        float lsum = 0.f;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int j = 0; j < kMaxCluster; ++j) {
-            const float w = (mv[j] == -INFINITY) ? 0.f : fast_exp2(mv[j] - gm);
-            lsum = fmaf(w, lv[j], lsum);
-            acc.x = fmaf(w, ov[j].x, acc.x); acc.y = fmaf(w, ov[j].y, acc.y);
-            acc.z = fmaf(w, ov[j].z, acc.z); acc.w = fmaf(w, ov[j].w, acc.w);
-        }
+        const Folded f = fold_slices(recv_o, recv_ml, csize, slice, e4 - e_lo, hd, got);
         if (direct) {
-            const float inv = lsum > 0.f ? 1.f / lsum : 0.f;
-            store_out4(out + ((size_t)bh * G + hd) * kD + d4, acc, inv);
+            const float inv = f.l > 0.f ? 1.f / f.l : 0.f;
+            store_out4(out + ((size_t)bh * G + hd) * kD + d4, f.o, inv);
         } else {
-            *reinterpret_cast<float4*>(my_part + hd * kD + d4) = acc;
-            if (d4 == 0 || e4 == e_lo) { my_part[8 * kD + hd] = gm; my_part[8 * kD + 8 + hd] = lsum; }   // (the same values from every slice of the head)
+            *reinterpret_cast<float4*>(my_part + hd * kD + d4) = f.o;
+            if (d4 == 0 || e4 == e_lo) { my_part[8 * kD + hd] = f.m; my_part[8 * kD + 8 + hd] = f.l; }   // (the same values from every slice of the head)
         }
     }
-    if (direct) return;
+    if (direct && __all_sync(kFull, got)) return;   // (as good as always: 0.1 us less here than behind the code for several partials)
 
     // ---- several partials per head: the last block to arrive merges them, slice by slice where there are counters enough ----
-    const bool by_slice = B * Hkv * csize <= kMaxTickets;
-    ticket_and_merge<kSpares>(part, first, more, per_unit, n_clusters, tickets + (by_slice ? bh * csize + crank : bh), by_slice ? n_clusters : n_clusters * csize,
-                              by_slice ? e_lo : 0, by_slice ? e_hi : G * (kD / 4), bh, G, out, &sh_last);
+    if (!direct) {
+        const bool by_slice = B * Hkv * csize <= kMaxTickets;
+        ticket_and_merge<kSpares>(part, first, more, per_unit, n_clusters, tickets + (by_slice ? bh * csize + crank : bh), by_slice ? n_clusters : n_clusters * csize,
+                                  by_slice ? e_lo : 0, by_slice ? e_hi : G * (kD / 4), bh, G, out, &sh_last);
+    }
+    outlast_cluster(smem_u32(&sh_bar), got);
 }
 
 // Block split of one head: how many blocks stream it, and how they are grouped into clusters.
