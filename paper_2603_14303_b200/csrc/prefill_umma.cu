@@ -450,14 +450,17 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             if (lane == 0) mbar_arrive(p_full0 + 8 * s);
         }
         // ---- O / l -> bf16 -> global: each thread 32 columns of its row; l is the sum of the row's four partial sums ----
-        bool ok = nt > 0 && !failed;
-        if (ok) {
-            ok = __all_sync(kFull, mbar_wait(pv_done0 + 8 * ((nt - 1) % kStages), ((nt - 1) / kStages) & 1));
-            if (!ok) *sh_fail = 1;
+        // The group that took the last tile waits for the last weighted sum.  (The other one could not: while the sum three tiles
+        // before is not complete, the parity of that place's barrier reads as if the last one were.)  It knows through rows_sync.
+        if (nt > 0 && !failed && grp == ((nt - 1) & 1)) {
+            if (!__all_sync(kFull, mbar_wait(pv_done0 + 8 * ((nt - 1) % kStages), ((nt - 1) / kStages) & 1))) { *sh_fail = 1; sh_fail_pair[pair] = 1; }
             fence_after_sync();
+            fence_before_sync();
         }
         const auto rows_sync = [&] { asm volatile("bar.sync %0, 128;\n" ::"r"(9 + q) : "memory"); };   // the four warps of these 32 rows
-        rows_sync();   // the last reference is settled
+        rows_sync();   // the last reference is settled, O is complete
+        fence_after_sync();
+        const bool ok = nt > 0 && !sh_fail_pair[q] && !sh_fail_pair[4 + q];
         const float m_row = nt > 0 ? ref_s[r] : -INFINITY;
         float* ls_s = reinterpret_cast<float*>(smem + kSmK + 2 * kTile);   // [4][128] (all keys are spent)
         ls_s[(grp * 2 + wg) * kT + r] = m_mine == -INFINITY ? 0.f : l_run * ex2(m_mine - m_row);
