@@ -1,16 +1,16 @@
 // Generic decode path for Eq. 4 (any dtype, d <= 256 multiple of 8).  One block serves one (sequence, KV head, split of
-// its cores, up to four of its query heads); its eight warps take 32-row tiles in turn: eight lanes per row form the
+// its cores, up to four of its query heads); its warps take 32-row tiles in turn: eight lanes per row form the
 // scores (four rows at a time, sixteen requested ahead), one lane per row takes part in the online softmax in
 // fp32, and for the weighted sum a lane owns four columns of every row, sixteen rows requested together.  A second kernel combines the splits in order.
 // Serves SC_F32 and cross-checks the tensor-core bf16 kernel.
 // Bounded by the latency of its loads: 2162 cores x 8 heads of fp32, 16 splits: 217 + 18 us when a warp served one query
-// head row by row (each row a dependent chain of load, five shuffles and two exponentials), 14 + 7 us like this (20 + 7 with
-// four warps, of which one had two tiles; 37 + 7 with eight rows requested at a time).
+// head row by row (each row a dependent chain of load, five shuffles and two exponentials), 14 + 7 us like this (37 + 7 with
+// eight rows requested at a time).  Eight warps or four per block: see run().
 #include "common.cuh"
 
 namespace sc {
 
-constexpr int kDecWarps = 8;
+constexpr int kCombineWarps = 4;
 constexpr int kDecHeads = 4;    // query heads per block
 constexpr int kDecMaxD = 256;
 
@@ -20,8 +20,9 @@ __host__ __device__ inline int generic_splits(int cap) {
 }
 
 // NC: the most 32-column pieces a row has (4 or 8).
-template <typename T, int NC>
-__global__ void __launch_bounds__(kDecWarps * 32, 1)
+// Eight warps have an SM to themselves (bounds (256, 1); left to itself the compiler takes 80 registers and spills: 23 us for 16).
+template <typename T, int NC, int kDecWarps>
+__global__ void __launch_bounds__(kDecWarps * 32, kDecWarps == 8 ? 1 : 0)
 decode_generic(const T* __restrict__ q, int Hq, int Hkv, int d, const T* __restrict__ core_k,
                const T* __restrict__ core_v, const int32_t* __restrict__ count, int cap,
                const int32_t* __restrict__ core_len, float scale_log2, int n_split, float* __restrict__ part) {
@@ -126,7 +127,7 @@ decode_generic(const T* __restrict__ q, int Hq, int Hkv, int d, const T* __restr
         }
         __syncwarp();   // the next tile's scores overwrite the weights
     }
-    // the four warps' (m, l, O), in order
+    // the warps' (m, l, O), in order
 #pragma unroll
     for (int g = 0; g < kDecHeads; ++g) {
         const float lw = warp_sum(l[g]);
@@ -160,11 +161,11 @@ decode_generic(const T* __restrict__ q, int Hq, int Hkv, int d, const T* __restr
 
 // One warp per query head: the splits' weights from one pair of loads per lane, then their sums in order.
 template <typename T>
-__global__ void __launch_bounds__(kDecWarps * 32)
+__global__ void __launch_bounds__(kCombineWarps * 32)
 combine_generic(int64_t heads, int d, int n_split, const float* __restrict__ part, T* __restrict__ out) {
-    __shared__ float sw[kDecWarps][64];
+    __shared__ float sw[kCombineWarps][64];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t hd = (int64_t)blockIdx.x * kDecWarps + w;
+    const int64_t hd = (int64_t)blockIdx.x * kCombineWarps + w;
     in_stream_order();
     if (hd >= heads) return;
     const float* pr = part + hd * n_split * (d + 2);
@@ -219,12 +220,22 @@ static cudaError_t run(const DecodeArgs& a, cudaStream_t st) {
     // Partials lie behind the tensor-core kernel's counters, which have to stay zero for a later call with this workspace.  They
     // are read and written in pairs of floats; a workspace need only be aligned to one (256 spare bytes cover the step).
     float* part = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(a.ws) + decode_mma_counter_bytes() + 7) & ~(uintptr_t)7);
-    cudaError_t e = launch_in_order(a.d <= 128 ? decode_generic<T, 4> : decode_generic<T, 8>, dim3(grid), kDecWarps * 32, 0, st,
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // A launch of no more blocks than SMs leaves each block an SM, which eight warps use better: float32, 8 heads x 4 K rows of 8 K
+    // 19.7 -> 16.1 us, bf16 with d = 256 38.3 -> 29.4.  Where there are more, blocks of four warps, of which an SM holds three
+    // to five with their starts and folds beside the others' loads: 16 sequences x 8 heads x 4 K rows, float32 211 -> 135, bf16
+    // with d = 64 283 -> 113, with d = 256 429 -> 282; just above the line, 10 heads x 4 K rows, 23.9 -> 22.7.
+    const bool alone = blocks <= sms;
+    const auto kernel = a.d <= 128 ? (alone ? decode_generic<T, 4, 8> : decode_generic<T, 4, 4>)
+                                   : (alone ? decode_generic<T, 8, 8> : decode_generic<T, 8, 4>);
+    cudaError_t e = launch_in_order(kernel, dim3(grid), (alone ? 8 : 4) * 32, 0, st,
                                     (const T*)a.q, a.Hq, a.Hkv, a.d, (const T*)a.core_k, (const T*)a.core_v, a.count, a.cap,
                                     a.core_len, scale, n_split, part);
     if (e != cudaSuccess) return e;
     const int64_t heads = (int64_t)a.B * a.Hq;
-    e = launch_in_order(combine_generic<T>, dim3(div_up(heads, kDecWarps)), kDecWarps * 32, 0, st, heads, a.d, n_split,
+    e = launch_in_order(combine_generic<T>, dim3(div_up(heads, kCombineWarps)), kCombineWarps * 32, 0, st, heads, a.d, n_split,
                               (const float*)part, (T*)a.out);
     if (e != cudaSuccess) return e;
     note_launches(2);
