@@ -12,6 +12,8 @@
 // 24 and eight, 34 / 39 us).  Merge: in cluster order a sum is one set of registers; added to the clusters' sums in shared memory
 // row by row (a load, an addition and a store that wait for one another) the path takes 85.8 us against 80.4; K and V of
 // a segment in one warp 82.4, and chunks of 128 tokens 280 against 250 (they leave too few warps).
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace sc {
@@ -362,9 +364,14 @@ static cudaError_t run(const CompressArgs& a, cudaStream_t st) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int grid = sms * 64;
+    // A warp takes two segments in turn; how many there are is known on the device only.  A run and its delimiter are three rows or
+    // more as a rule (where they are not, a warp takes further ones), and blocks without any cost 0.5 us per thousand: 8 heads x 64
+    // tokens of float32 8.6 us for the three kernels, 22 with 64 blocks per SM whatever the input; a pair to four rows 11.8, a
+    // pair to two the same as to three up to 128 tokens and 0.1 to 1.5 us more above.
+    const int64_t pairs = (int64_t)a.B * a.Hkv * a.n / 3 + 1, most = (int64_t)sms * 64;
+    const unsigned gsc_grid = (unsigned)std::min(pairs, most), merge_grid = (unsigned)std::min(2 * pairs, most);
     auto gsc = a.d <= 128 ? gsc_generic<T, 4> : gsc_generic<T, 8>;
-    cudaError_t e = launch_in_order(gsc, dim3(grid), kGenWarps * 32, 0, st, (const T*)a.K, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off,
+    cudaError_t e = launch_in_order(gsc, dim3(gsc_grid), kGenWarps * 32, 0, st, (const T*)a.K, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off,
                                     a.n_seg, seg_stride, a.tau, a.tau_dev, a.skip, assign, seg_p);
     if (e != cudaSuccess) return e;
     e = launch_in_order(scan_generic, dim3(a.B * a.Hkv), 256, 0, st, a.Hkv, a.seq_seg_off, seg_stride, (const int32_t*)seg_p,
@@ -374,7 +381,7 @@ static cudaError_t run(const CompressArgs& a, cudaStream_t st) {
         note_launches(2);
         return cudaSuccess;
     }
-    e = launch_in_order(a.d <= 128 ? merge_generic<T, 1> : merge_generic<T, 2>, dim3(grid), kGenWarps * 32, 0, st, (const T*)a.K,
+    e = launch_in_order(a.d <= 128 ? merge_generic<T, 1> : merge_generic<T, 2>, dim3(merge_grid), kGenWarps * 32, 0, st, (const T*)a.K,
                               (const T*)a.V, a.st, a.B, a.Hkv, a.n, a.d, a.seg_off, a.n_seg, seg_stride, (const int32_t*)assign,
                               (const int32_t*)seg_core_off, (T*)a.core_k, (T*)a.core_v, a.count, a.cap);
     if (e != cudaSuccess) return e;
