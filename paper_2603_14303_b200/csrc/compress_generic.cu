@@ -13,6 +13,7 @@
 // row by row (a load, an addition and a store that wait for one another) the path takes 85.8 us against 80.4; K and V of
 // a segment in one warp 82.4, and chunks of 128 tokens 280 against 250 (they leave too few warps).
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -85,10 +86,13 @@ __device__ __forceinline__ int short_segment(int l, float tau, int32_t* as, int 
     return p;
 }
 
-// Algorithm 1 for one segment per warp.  Longer segments' rows are read straight from global memory, 32 at a time (16 where d > 128),
-// eight lanes a row, against the seed's row, which they hold in registers; rows already assigned are not read.  The whole path for
-// 8 heads x 8K tokens of fp32 in chunks of 128: eight rows at a time 250 us, sixteen 200, 32 178; of 60: 169, 148, 139.  NC: the
-// most 32-column pieces a row has (4 or 8).
+// Algorithm 1 for one segment per warp.  Longer segments' rows are read straight from global memory, 32 at a time, eight lanes a
+// row, against the seed's row, which they hold in registers; rows already assigned are not read.  The whole path for
+// 8 heads x 8K tokens of fp32 in chunks of 128: eight rows at a time 250 us, sixteen 200, 32 178; of 60: 169, 148, 139.  Where d > 128
+// sixteen rows of fp32 (8 x 8K in chunks of 128 on the average: eight 482 us, sixteen 384), but eight for segments of up to 32 rows, whose
+// places in a batch are mostly empty (8 heads x 128 tokens in chunks of 8: eight 24.4, sixteen 26.3), and eight of bf16, which
+// spends its time on instructions and not on loads (4 x 8 x 8K, chunks of 8: 489 and 590; of 128: 848 and 944).  NC:
+// the most 32-column pieces a row has (4 or 8).
 template <typename T, int NC>
 __global__ void __launch_bounds__(kGenWarps * 32, kGenBlocks)
 gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d,
@@ -134,51 +138,58 @@ gsc_generic(const T* __restrict__ K, sc_strides st, int B, int Hkv, int n, int d
                 continue;
             }
         }
-        // longer: kRows rows at a time; a lane decides for row j0 + row_of (in pairs of lanes, or fours)
-        constexpr int R = NC == 4 ? 8 : 4, kRows = 4 * R;
-        const int row_of = rsub * R + lane % R;
-        const bool speaks = sub < R;   // one lane of those that decide for the same row
-        for (int j0 = 0; j0 < l; j0 += kRows) {
-            float4 v[R][NC];
-            float x[R];
-#pragma unroll
-            for (int q = 0; q < R; ++q) load_row(j0 + rsub * R + q, j0 + rsub * R + q < l, v[q]);
-#pragma unroll
-            for (int q = 0; q < R; ++q) x[q] = dot(v[q], v[q]);
-            const float nn = group_sums<R>(x, lane);
-            if (speaks && j0 + row_of < l) norms[w][j0 + row_of] = sqrtf(nn);
-        }
-        __syncwarp();
-        unsigned word = 0;  // lane c holds the assigned bits of tokens 32c .. 32c+31
-        int p = 0;
-        for (int i = 0; i < l; ++i) {
-            const unsigned wi = __shfl_sync(kFull, word, i >> 5);
-            if ((wi >> (i & 31)) & 1u) continue;
-            ++p;
-            if (lane == (i >> 5)) word |= 1u << (i & 31);
-            if (lane == 0) as[i] = r + i;
-            if (i + 1 >= l) break;
-            float4 seed[NC];
-            load_row(i, true, seed);
-            const float ni = norms[w][i];
-            for (int j0 = (i + 1) & ~(kRows - 1); j0 < l; j0 += kRows) {   // kRows tokens of one word
-                unsigned open = (~__shfl_sync(kFull, word, j0 >> 5)) >> (j0 & 31) & (0xffffffffu >> (32 - kRows));
-                if (j0 <= i) open &= ~0u << (i + 1 - j0);
-                if (l - j0 < kRows) open &= (1u << (l - j0)) - 1u;
-                if (open == 0u) continue;
+        // longer: 4 R rows at a time; a lane decides for row j0 + row_of (in pairs of lanes, or fours)
+        const auto longer = [&](auto rows_per_group) {
+            constexpr int R = decltype(rows_per_group)::value, kRows = 4 * R;
+            const int row_of = rsub * R + lane % R;
+            const bool speaks = sub < R;   // one lane of those that decide for the same row
+            for (int j0 = 0; j0 < l; j0 += kRows) {
                 float4 v[R][NC];
                 float x[R];
-#pragma unroll
-                for (int q = 0; q < R; ++q) load_row(j0 + rsub * R + q, (open >> (rsub * R + q)) & 1u, v[q]);
-#pragma unroll
-                for (int q = 0; q < R; ++q) x[q] = dot(seed, v[q]);
-                const float prod = group_sums<R>(x, lane), nj = j0 + row_of < l ? norms[w][j0 + row_of] : 0.f;
-                const float sim = (ni == 0.f || nj == 0.f) ? 0.f : prod / (ni * nj);
-                const unsigned hits = by_row<R>(__ballot_sync(kFull, sim > tau)) & open;
-                if (lane == (j0 >> 5)) word |= hits << (j0 & 31);
-                if (speaks && ((hits >> row_of) & 1u)) as[j0 + row_of] = r + i;
+    #pragma unroll
+                for (int q = 0; q < R; ++q) load_row(j0 + rsub * R + q, j0 + rsub * R + q < l, v[q]);
+    #pragma unroll
+                for (int q = 0; q < R; ++q) x[q] = dot(v[q], v[q]);
+                const float nn = group_sums<R>(x, lane);
+                if (speaks && j0 + row_of < l) norms[w][j0 + row_of] = sqrtf(nn);
             }
-        }
+            __syncwarp();
+            unsigned word = 0;  // lane c holds the assigned bits of tokens 32c .. 32c+31
+            int p = 0;
+            for (int i = 0; i < l; ++i) {
+                const unsigned wi = __shfl_sync(kFull, word, i >> 5);
+                if ((wi >> (i & 31)) & 1u) continue;
+                ++p;
+                if (lane == (i >> 5)) word |= 1u << (i & 31);
+                if (lane == 0) as[i] = r + i;
+                if (i + 1 >= l) break;
+                float4 seed[NC];
+                load_row(i, true, seed);
+                const float ni = norms[w][i];
+                for (int j0 = (i + 1) & ~(kRows - 1); j0 < l; j0 += kRows) {   // kRows tokens of one word
+                    unsigned open = (~__shfl_sync(kFull, word, j0 >> 5)) >> (j0 & 31) & (0xffffffffu >> (32 - kRows));
+                    if (j0 <= i) open &= ~0u << (i + 1 - j0);
+                    if (l - j0 < kRows) open &= (1u << (l - j0)) - 1u;
+                    if (open == 0u) continue;
+                    float4 v[R][NC];
+                    float x[R];
+    #pragma unroll
+                    for (int q = 0; q < R; ++q) load_row(j0 + rsub * R + q, (open >> (rsub * R + q)) & 1u, v[q]);
+    #pragma unroll
+                    for (int q = 0; q < R; ++q) x[q] = dot(seed, v[q]);
+                    const float prod = group_sums<R>(x, lane), nj = j0 + row_of < l ? norms[w][j0 + row_of] : 0.f;
+                    const float sim = (ni == 0.f || nj == 0.f) ? 0.f : prod / (ni * nj);
+                    const unsigned hits = by_row<R>(__ballot_sync(kFull, sim > tau)) & open;
+                    if (lane == (j0 >> 5)) word |= hits << (j0 & 31);
+                    if (speaks && ((hits >> row_of) & 1u)) as[j0 + row_of] = r + i;
+                }
+            }
+            return p;
+        };
+        int p;
+        if constexpr (NC == 4) p = longer(std::integral_constant<int, 8>());
+        else if constexpr (sizeof(T) == 2) p = longer(std::integral_constant<int, 2>());
+        else p = l <= 32 ? longer(std::integral_constant<int, 2>()) : longer(std::integral_constant<int, 4>());
         if (lane == 0) seg_p[(int64_t)h * seg_stride + s] = p;
         __syncwarp();
     }
