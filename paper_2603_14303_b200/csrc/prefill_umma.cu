@@ -8,7 +8,7 @@
 //   warp 1     issues the MMAs: S = Q K^T into one of three score buffers in tensor memory (three tiles ahead
 //              of the weighted sum), then O += P V with P read from tensor memory and V as an MN-major
 //              operand straight from its [keys x dims] tile;
-//   warps 4-19 softmax, two groups of eight warps that take the key tiles in turn, two threads per query row
+//   warps 4-19 softmax, two groups of eight warps that take the key tiles in turn (one, warps 4-11, where there is one tile), two threads per query row
 //              (= tensor-memory lane; each owns half of the tile's keys):
 //              x = S * scale*log2(e) + log2(count), masks (head length, optional causal tail), P = 2^(x - m) as a bf16 pair
 //              (leading part + remainder) written back over the scores it came from: the 32 fp32 columns of a chunk of scores
@@ -35,6 +35,7 @@
 // A CUDA-core kernel (one warp per query) serves other dtypes and head sizes.
 #include <cooperative_groups.h>
 
+#include <algorithm>
 #include <mutex>
 #include <type_traits>
 
@@ -51,7 +52,6 @@ namespace cg = cooperative_groups;
 constexpr int kT = 128;                       // query rows per CTA, keys per tile
 constexpr int kHalf = kT * 128;               // 16384 bytes: one 64-column half of a [128 x 128] bf16 tile
 constexpr int kTile = 2 * kHalf;              // 32768
-constexpr int kThreads = 640;                 // warps 0, 2: TMA, warp 1: MMA + tensor memory, warps 4-19: softmax
 constexpr int kTmemCols = 512;                // S0 | S1 | S2 | O (128 columns each; P overwrites S in place)
 constexpr int kColS = 0, kColO = 384;
 constexpr int kStages = 3;                    // K and V rings, score buffers
@@ -138,8 +138,9 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
 // kRep: how often the query rows stand in the tile's 128 lanes.  Up to 32 (64) rows they do so four times (twice), and each
 // replica takes a quarter (half) of every key tile -- its weights of the other keys are zero --, so that all softmax warps work
 // and a thread has 16 (32) scores a tile instead of 64; the replicas are folded at the end like the CTAs of a split.
-template <int kRep>
-__global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_constant__ Params p) {
+// kGroups: groups of softmax warps, one or two.
+template <int kRep, int kGroups>
+__global__ void __launch_bounds__(128 + 256 * kGroups, 1) prefill_umma_kernel(const __grid_constant__ Params p) {
     extern __shared__ __align__(1024) unsigned char smem[];   // the swizzle pattern repeats every 1024 bytes
     const int n_split = p.n_split, split = blockIdx.x % n_split;   // the CTAs of a cluster are consecutive in x
     const int qt = blockIdx.x / n_split, h = blockIdx.y, b = blockIdx.z;
@@ -282,9 +283,9 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             if (!ok && lane == 0) *sh_fail = 1;
         }
     } else if (warp >= 4) {
-        // ---- softmax: warps 4-11 take the even key tiles, warps 12-19 the odd ones; two threads per query row (= tensor-memory
+        // ---- softmax: warps 4-11 take the even key tiles, warps 12-19 the odd ones (one group: all); two threads per query row (= tensor-memory
         //      lane), each owning half of a tile's keys (of the replica's share) ----
-        const int grp = (warp - 4) >> 3, q = warp & 3, r = q * 32 + lane, wg = ((warp - 4) >> 2) & 1;
+        const int grp = kGroups == 1 ? 0 : (warp - 4) >> 3, q = warp & 3, r = q * 32 + lane, wg = ((warp - 4) >> 2) & 1;
         constexpr int kRows = kT / kRep, kKeys = 64 / kRep;   // rows of a replica; keys of a tile per thread
         constexpr int kHold = kKeys > 32 ? 32 : kKeys;        // scores kept in registers (the others are read again)
         const int col0 = (r / kRows) * kRows + wg * kKeys;    // the first of them (a replica has as many keys as rows)
@@ -307,7 +308,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
                          : "=r"(out) : "r"(mine ? 1u : 0u), "r"(1 + pair) : "memory");
             return out != 0u;
         };
-        for (int t = grp; t < nt; t += 2) {
+        for (int t = grp; t < nt; t += kGroups) {
             const int s = t % kStages, round = t / kStages, j0 = (t_lo + t) * kT, jw = j0 + col0;   // jw: first key of this thread
             const uint32_t s_addr = lane_addr + kColS + s * kT + col0;
             bool lost = !mbar_wait(s_full0 + 8 * s, round & 1) || !mbar_wait(lc_full0 + 8 * s, round & 1);
@@ -449,38 +450,40 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             __syncwarp();
             if (lane == 0) mbar_arrive(p_full0 + 8 * s);
         }
-        // ---- O / l -> bf16 -> global: each thread 32 columns of its row; l is the sum of the row's four partial sums ----
+        // ---- O / l -> bf16 -> global: each thread 32 (one group: 64) columns of its row; l is the sum of the row's four (two) partial sums ----
         // The group that took the last tile waits for the last weighted sum.  (The other one could not: while the sum three tiles
         // before is not complete, the parity of that place's barrier reads as if the last one were.)  It knows through rows_sync.
-        if (nt > 0 && !failed && grp == ((nt - 1) & 1)) {
+        if (nt > 0 && !failed && grp == (nt - 1) % kGroups) {
             if (!__all_sync(kFull, mbar_wait(pv_done0 + 8 * ((nt - 1) % kStages), ((nt - 1) / kStages) & 1))) { *sh_fail = 1; sh_fail_pair[pair] = 1; }
             fence_after_sync();
             fence_before_sync();
         }
-        const auto rows_sync = [&] { asm volatile("bar.sync %0, 128;\n" ::"r"(9 + q) : "memory"); };   // the four warps of these 32 rows
+        const auto rows_sync = [&] { asm volatile("bar.sync %0, %1;\n" ::"r"(9 + q), "n"(64 * kGroups) : "memory"); };   // the warps of these 32 rows
         rows_sync();   // the last reference is settled, O is complete
         fence_after_sync();
         const bool ok = nt > 0 && !sh_fail_pair[q] && !sh_fail_pair[4 + q];
         const float m_row = nt > 0 ? ref_s[r] : -INFINITY;
-        float* ls_s = reinterpret_cast<float*>(smem + kSmK + 2 * kTile);   // [4][128] (all keys are spent)
+        float* ls_s = reinterpret_cast<float*>(smem + kSmK + 2 * kTile);   // [2 kGroups][128] (all keys are spent)
         ls_s[(grp * 2 + wg) * kT + r] = m_mine == -INFINITY ? 0.f : l_run * ex2(m_mine - m_row);
         rows_sync();
-        const float l_row = (ls_s[r] + ls_s[kT + r]) + (ls_s[2 * kT + r] + ls_s[3 * kT + r]);
-        const int ocol = (grp * 2 + wg) * 32;
-        uint32_t o[32];
+        const float l_row = kGroups == 1 ? ls_s[r] + ls_s[kT + r] : (ls_s[r] + ls_s[kT + r]) + (ls_s[2 * kT + r] + ls_s[3 * kT + r]);
+        constexpr int kOut = 64 / kGroups;   // columns of a thread
+        const int ocol = (grp * 2 + wg) * kOut;
+        uint32_t o[kOut];
         if (ok) {
-            tmem_ld32(lane_addr + kColO + ocol, o);
+#pragma unroll
+            for (int c = 0; c < kOut; c += 32) tmem_ld32(lane_addr + kColO + ocol + c, *reinterpret_cast<uint32_t(*)[32]>(&o[c]));
             tmem_ld_wait();
         } else {
 #pragma unroll
-            for (int k = 0; k < 32; ++k) o[k] = 0u;
+            for (int k = 0; k < kOut; ++k) o[k] = 0u;
         }
         if (kRep == 1 && n_split == 1) {
             __nv_bfloat16* orow = p.out + (size_t)(q_row0 + r) * 128 + ocol;
             const float inv = l_row > 0.f ? 1.f / l_row : 0.f;
             if (row_ok) {
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
+                for (int u = 0; u < kOut / 8; ++u) {
                     uint4 v;
                     v.x = pack2(__uint_as_float(o[8 * u]) * inv, __uint_as_float(o[8 * u + 1]) * inv);
                     v.y = pack2(__uint_as_float(o[8 * u + 2]) * inv, __uint_as_float(o[8 * u + 3]) * inv);
@@ -494,14 +497,14 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             float* part_o = reinterpret_cast<float*>(smem + kSmK);      // [128 rows][32 float4], float4 index ^ (row & 31)
             float* part_ml = reinterpret_cast<float*>(smem + kSmV);     // [128] m, [128] l; the folded replicas' [128] m, [128] l
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
+            for (int u = 0; u < kOut / 4; ++u) {
                 const int c4 = ocol / 4 + u;
                 *reinterpret_cast<uint4*>(part_o + r * 128 + ((c4 ^ (r & 31)) << 2)) = make_uint4(o[4 * u], o[4 * u + 1], o[4 * u + 2], o[4 * u + 3]);
             }
             if (grp == 0 && wg == 0) { part_ml[r] = ok ? m_row : -INFINITY; part_ml[kT + r] = ok ? l_row : 0.f; }
             if (kRep > 1) {   // the replicas of a row into the first, one thread per (row, four output columns)
-                asm volatile("bar.sync 13, 512;\n" ::: "memory");
-                for (int it = tid - 128; it < kRows * 32; it += 512) {
+                asm volatile("bar.sync 13, %0;\n" ::"n"(256 * kGroups) : "memory");
+                for (int it = tid - 128; it < kRows * 32; it += 256 * kGroups) {
                     const int fr = it >> 5, c4 = it & 31;
                     float gm = -INFINITY, lsum = 0.f;
                     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -535,7 +538,7 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_umma_kernel(const __grid_
             const int R = (kRows + n_split - 1) / n_split, r_end = min(min((split + 1) * R, kRows), rows_total - qt * kT);
             const auto fold_rows = [&](auto width) {   // `width` partials at a time
                 constexpr int kFold = decltype(width)::value;
-                for (int it = tid - 128; it < R * 32; it += 512) {
+                for (int it = tid - 128; it < R * 32; it += 256 * kGroups) {
                     const int r = split * R + (it >> 5), c4 = it & 31;
                     if (r >= r_end) break;
                     float gm = -INFINITY, lsum = 0.f;
@@ -670,14 +673,15 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
         int* fit = fit_of[dev];
         std::call_once(once_of[dev], [&] {
             bool wide = true;
-            for (auto kernel : {prefill_umma_kernel<1>, prefill_umma_kernel<2>, prefill_umma_kernel<4>}) {
+            for (auto kernel : {prefill_umma_kernel<1, 2>, prefill_umma_kernel<2, 2>, prefill_umma_kernel<4, 2>, prefill_umma_kernel<1, 1>, prefill_umma_kernel<2, 1>,
+                                prefill_umma_kernel<4, 1>}) {
                 cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
                 wide = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess && wide;
             }
             for (int c = 2; c <= (wide ? kMaxSplit : 8); ++c) {
                 cudaLaunchConfig_t probe = {};
                 probe.gridDim = dim3(c, 1, 1);
-                probe.blockDim = dim3(kThreads);
+                probe.blockDim = dim3(128 + 256 * 2);
                 probe.dynamicSmemBytes = kSmemBytes;
                 cudaLaunchAttribute pa[1];
                 pa[0].id = cudaLaunchAttributeClusterDimension;
@@ -685,7 +689,7 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
                 probe.attrs = pa;
                 probe.numAttrs = 1;
                 int n_clusters = 0;
-                if (cudaOccupancyMaxActiveClusters(&n_clusters, prefill_umma_kernel<1>, &probe) == cudaSuccess) fit[c] = n_clusters;
+                if (cudaOccupancyMaxActiveClusters(&n_clusters, prefill_umma_kernel<1, 2>, &probe) == cudaSuccess) fit[c] = n_clusters;
             }
             (void)cudaGetLastError();   // a refused opt-in or probe is not an error of this call
         });
@@ -715,7 +719,15 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
             p.n_split = n_split;
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = dim3((unsigned)((G * a.m + kT - 1) / kT) * n_split, a.Hkv, a.B);
-            cfg.blockDim = dim3(kThreads);
+            // One group of softmax warps where a CTA is likely to have a single key tile, or two of few rows folded over a cluster anyway:
+            // 384 threads start 0.3 us sooner than 640, and a second group has nothing, or little, to do.  8 heads, one query over 266
+            // rows of 512: 8.3 us with two groups, 8.0 with one; 128 causal ones over 394: 11.9, 11.4; 28 rows over 2162 on 16 CTAs 9.5, 9.1.  With more tiles two: 32 queries
+            // over 2162 rows 14.3, 14.6; 64 over 130, two tiles of one CTA, 9.8, 10.5.  Likely: five eighths of the capacity, a
+            // little more than the half that compressed heads fill, and a causal block's own tokens.
+            const long long likely = (causal ? (long long)std::max(a.cap - a.m, 0) * 5 / 8 + a.m : (long long)a.cap * 5 / 8);
+            const long long each = ((likely + kT - 1) / kT + n_split - 1) / n_split;
+            const bool one_group = each <= (rep > 1 && n_split > 1 ? 2 : 1);
+            cfg.blockDim = dim3(128 + 256 * (one_group ? 1 : 2));
             cfg.dynamicSmemBytes = kSmemBytes;
             cfg.stream = st;
             cudaLaunchAttribute attr[2];
@@ -726,7 +738,8 @@ cudaError_t launch_prefill(const PrefillArgs& a, cudaStream_t st) {
             cfg.attrs = attr;
             cfg.numAttrs = 2;
             note_launches(1);
-            return own_error(cudaLaunchKernelEx(&cfg, rep == 4 ? prefill_umma_kernel<4> : rep == 2 ? prefill_umma_kernel<2> : prefill_umma_kernel<1>, p));
+            return own_error(cudaLaunchKernelEx(&cfg, one_group ? (rep == 4 ? prefill_umma_kernel<4, 1> : rep == 2 ? prefill_umma_kernel<2, 1> : prefill_umma_kernel<1, 1>)
+                                                         : (rep == 4 ? prefill_umma_kernel<4, 2> : rep == 2 ? prefill_umma_kernel<2, 2> : prefill_umma_kernel<1, 2>), p));
         }
     }
     const unsigned blocks = (unsigned)((q_rows + 3) / 4);
