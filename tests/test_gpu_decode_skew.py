@@ -53,7 +53,12 @@ def _reference(q, y, raw):
     ([9000, 9000, 9000, 9001], 9001, 8, 4, True, True),     # raw caches: equal, and not
     ([30000, 1000, 1000, 1000], 30000, 8, 4, True, True),
     ([12000] + [800] * 9, 12000, 8, 4, True, False),        # 80 raw heads
-    ([12000] + [300] * 40, 12000, 4, 4, True, True)])       # 164 raw heads
+    ([12000] + [300] * 40, 12000, 4, 4, True, True),        # 164 raw heads
+    # more blocks of clusters than counters, several clusters per long head: a head's blocks share one
+    ([9000, 4000] + [300] * 38, 9000, 8, 4, False, True),   # 320 heads, clusters of three
+    ([200] * 20 + [9000] + [0] * 17, 9000, 8, 7, False, False),   # 304
+    ([8200] + [100] * 20 + [5000], 8200, 8, 1, True, True),       # 176 raw heads, clusters of three
+    ([100] * 39 + [8200], 8200, 8, 4, True, False)])              # 320, of two
 def test_lengths_far_apart(lens, cap, H, G, raw, equal):
     y = _layer(lens, cap, H, len(lens), equal)
     ws = binding.decode_workspace(len(lens), H * G, H, 128, cap, DEV)
