@@ -31,7 +31,9 @@
 // shared memory leaves the L1 cache 28 KB, a spilled word is a trip to L2, and variants with 4 to 80 bytes of stack lost 5 to 10 %.
 // Copies of an earlier form with steps left out, 32 layers on resident inputs, 1105 us: 707 (loads only), 834 (loads, steps 1 and 2), 1025
 // (all but the stores of the means).
-// A tile of 129..256 tokens spends 12 K cycles on step 2 and holds up the look-back of the tiles behind it.
+// A tile of 129..256 tokens holds up the look-back of the tiles behind it with its three products.  In short inputs, whose time is one such
+// tile's, steps 1 and 2 of the short tiles in line cost 0.3 to 0.6 us (8 heads x 512 tokens with chunks over 128: 12.8 us with those
+// steps out of line, 13.5); 32 layers x 32K tokens gain 26 us by them, 4 x 64K in chunks of 128 23 of 547.
 // Why these steps: one product per tile and decision rounds take 6.5 K warp instructions per 128 tokens, a warp per segment with
 // mma.sync tiles, the greedy pass and sums of member rows on the CUDA cores took 13 K: 32 layers 1395 us; 16 sequences x 16K,
 // lognormal chunks, 500 us a layer against 300; 4 x 64K in chunks of 128 794 against 578.  Sums over member rows in cluster

@@ -12,7 +12,8 @@
 // Warps are merged in a fixed order through shared memory into one (m, l, O) partial per block.
 // The splits of a head form a thread-block cluster and fold their partials through distributed shared memory, each
 // block its own slice of the output (no partial leaves the SMs).  Where a head has several clusters, or blocks outside
-// clusters, partials go to global memory and the last one of a head to arrive (atomic ticket, no waiting) merges them.
+// clusters, partials go to global memory and the last one to arrive (atomic ticket, no waiting) merges them, slice by slice
+// where there are counters enough, else a head at once.
 // How many splits: plan_for.  In a batch the blocks that the plan gives a head are one unit; a head much longer than the mean
 // of the launch gets more units (plan_units), so that a long sequence among short ones is not streamed by a few blocks.
 // Every order is fixed, so results are bit-reproducible.
@@ -51,7 +52,7 @@ constexpr float kMaxSlack = 8.f;                // log2 units a score may exceed
 constexpr int kMergeGroup = 16;                 // cluster partials folded per round by the merging block
 constexpr int kCapRowsPerBlock = 1408;          // rows of capacity per block from which a head gets another cluster (heads are usually half full or less)
 constexpr int kMaxSlots = 160;                  // partials in global memory over the launch's own units (at least one per head)
-constexpr int kMaxTickets = 512;                // heads of a launch whose blocks may meet through global memory
+constexpr int kMaxTickets = 512;                // arrival counters: one per head and slice where these are enough, else one per head
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -235,7 +236,8 @@ __device__ __forceinline__ Units plan_units(const int32_t* __restrict__ core_len
 // kSpares: the launch has spare units (the code for them costs the others 0.2 us).
 // kPair: up to four query heads.  The second product's eight columns then hold the heads' leading parts and, four columns on, their
 // remainders, so one product does for both; the queries stand in the first product's columns twice, which gives the lanes
-// of either half the scores they need.
+// of either half the scores they need.  The remainders' part then has accumulators of its own, which rounds less: of 98304 outputs over 4 x 64K
+// raw rows 246 are not the bf16 nearest to the value in 64 bits, 410 with both parts in one accumulator (16 x 16K cores: 930 and 966 of 393216).
 template <bool kSpares, bool kPair>
 __global__ void __launch_bounds__(kWarps * 32, kCtasPerSm)
 decode_mma_kernel(const __nv_bfloat16* __restrict__ q, int Hq, int Hkv, const __nv_bfloat16* __restrict__ core_k,
@@ -613,7 +615,7 @@ size_t decode_mma_counter_bytes() { return sizeof(int32_t) * dm::kMaxTickets; }
 
 size_t decode_mma_ws_bytes(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t cap) {
     (void)Hq; (void)d;
-    // tickets (one per (b, head), zero between calls) + partials
+    // arrival counters (zero between calls) + partials
     return 256 + decode_mma_counter_bytes() + sizeof(float) * dm::all_slots((long long)B * Hkv, cap) * dm::kPartStride;
 }
 

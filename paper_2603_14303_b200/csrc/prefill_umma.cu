@@ -23,7 +23,7 @@
 // query rows out of all members' shared memory (distributed shared memory) and writes that slice of the output.
 // What bounds it: shared memory.  A key tile's operands (64 KB for the scores, twice 32 KB for the pair of weights) and its copies
 // (64 KB) are 1536 clocks at 128 bytes, and the tensor cores need 1632; the MMA warp is busy 2300 of the 2530 clocks a tile takes.
-// 4 layers x 512 causal queries per head over 8.5 K cores 522 -> 461 us, 2 x 256 133 -> 110 against two score buffers and eight
+// 4 layers x 512 causal queries per head over 8.5 K cores 520 -> 467 us, one layer x 256 65 -> 54 against two score buffers and eight
 // softmax warps on one tile at a time, whose softmax (3500 clocks with one warp-instruction every 3 clocks per scheduler) was
 // the bound.  Two query tiles per CTA with a score buffer and an accumulator each: 480; the same with a 64-key
 // double buffer 562.  MMAs issued by a branch of one thread take 62 clocks each, by an elected lane of a converged warp 27.

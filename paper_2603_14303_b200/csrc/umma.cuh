@@ -1,7 +1,7 @@
 // Thin wrappers over the sm_100a tensor-core path used by the dense contractions of this library:
 // TMA tile loads (cp.async.bulk.tensor, no multicast), mbarriers with bounded waits, tensor memory
-// (TMEM) allocation, tcgen05.mma issued by one thread with both operands in shared memory, and
-// tcgen05.ld for the epilogue.  One CTA per tile (cta_group::1).
+// (TMEM) allocation, tcgen05.mma with both operands in shared memory, issued by one thread or by an elected lane of a whole
+// warp, and tcgen05.ld for the epilogue.  One CTA per tile (cta_group::1).
 #pragma once
 
 #include <cuda.h>
